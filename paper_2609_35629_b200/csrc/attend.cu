@@ -134,6 +134,7 @@ template <int G, bool kAll, bool kStatic, bool kHalf>
 __global__ void __launch_bounds__(kAttendThreads, 1)
 attend_kernel(AttendParams p)
 {
+    step_wait();
     extern __shared__ __align__(1024) unsigned char smem[];
     using S = Smem<G>;
     int *seg_prefix = reinterpret_cast<int *>(smem + S::seg_prefix);
@@ -576,6 +577,7 @@ template <int kParts, bool kStatic>
 __global__ void __launch_bounds__(kParts * 32)
 merge_kernel(AttendParams p, int attend_grid)
 {
+    step_wait();
     __shared__ float red_m[kParts], red_l[kParts];
     __shared__ __align__(16) float red_acc[kParts][kHeadDim];
     const int G = p.bv.group;
@@ -682,11 +684,11 @@ cudaError_t launch_attend_g(const AttendParams &p, bool all_heads, bool static_s
     cudaError_t err = ensure_dynamic_smem(fns[which], (int)smem, done[which]);
     if (err != cudaSuccess) return err;
     if (all_heads) {
-        if (static_split) return launch_kernel(attend_kernel<G, true, true, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
-        return launch_kernel(attend_kernel<G, true, false, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
+        if (static_split) return launch_step(attend_kernel<G, true, true, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
+        return launch_step(attend_kernel<G, true, false, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
     }
-    if (static_split) return launch_kernel(attend_kernel<G, false, true, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
-    return launch_kernel(attend_kernel<G, false, false, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
+    if (static_split) return launch_step(attend_kernel<G, false, true, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
+    return launch_step(attend_kernel<G, false, false, kHalf>, dim3(grid), dim3(kAttendThreads), smem, s, p);
 }
 
 }  // namespace
@@ -707,9 +709,9 @@ cudaError_t launch_merge(const AttendParams &p, bool static_split, int attend_gr
     // few pairs: many partials each (16 warps share them); many pairs: a handful each
     const dim3 blocks(p.bv.group, p.n_pairs);
     const bool wide = static_split || p.n_pairs * 8 <= attend_grid;
-    if (static_split) return launch_kernel(merge_kernel<16, true>, blocks, dim3(16 * 32), 0, s, p, attend_grid);
-    if (wide) return launch_kernel(merge_kernel<16, false>, blocks, dim3(16 * 32), 0, s, p, attend_grid);
-    return launch_kernel(merge_kernel<4, false>, blocks, dim3(4 * 32), 0, s, p, attend_grid);
+    if (static_split) return launch_step(merge_kernel<16, true>, blocks, dim3(16 * 32), 0, s, p, attend_grid);
+    if (wide) return launch_step(merge_kernel<16, false>, blocks, dim3(16 * 32), 0, s, p, attend_grid);
+    return launch_step(merge_kernel<4, false>, blocks, dim3(4 * 32), 0, s, p, attend_grid);
 }
 
 cudaError_t launch_attend(const AttendParams &p, bool all_heads, bool static_split, int grid, cudaStream_t s)

@@ -294,6 +294,7 @@ __device__ __forceinline__ Words8 ldg256(const void *p)
 __global__ void __launch_bounds__(kLsThreads)
 latent_score_kernel(LatentScoreParams p)
 {
+    step_wait();
     constexpr int kQPitchW = (kRowBytes + 16) / 4;                  // words per staged query (+16 bytes: conflict-free LDS.128)
     __shared__ __align__(16) uint32_t q_s[kHeads * kQPitchW];
     __shared__ __align__(16) uint32_t words_s[kLsThreads / 32][kHeads][16];
@@ -412,6 +413,7 @@ template <int kT>
 __global__ void __launch_bounds__(kT, kT >= 512 ? 1 : 1024 / kT)
 latent_select_kernel(PlanInputs in)
 {
+    step_wait();
     __shared__ HeadSmemT<kRowDim> sm;
     trace_mark(in.trace, 1, 0);
     select_head<kT, kT >= 512 ? 4 : 2, false, kRowDim>(in, blockIdx.x, sm);
@@ -455,6 +457,7 @@ struct LatentPlanSmem {
 __global__ void __launch_bounds__(kLpThreads)
 latent_plan_kernel(LatentPlanParams p)
 {
+    step_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LatentPlanSmem &sm = *reinterpret_cast<LatentPlanSmem *>(smem_raw);
     const int b = blockIdx.x, tid = threadIdx.x;
@@ -642,6 +645,7 @@ template <bool kAll>
 __global__ void __launch_bounds__(kLfThreads, 1)
 latent_attend_kernel(LatentAttendParams p)
 {
+    step_wait();
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int pv_role = warp >> 2, gw = warp & 3, gt = gw * 32 + lane;
@@ -974,6 +978,7 @@ constexpr int kLmThreads = 512;
 __global__ void __launch_bounds__(kLmThreads)
 latent_merge_kernel(const float *partials, const uint32_t *pair_prefix, int n_seqs, int n_heads, int grid, float *out, int32_t *status)
 {
+    step_wait();
     __shared__ float red[kLmThreads / 32];
     __shared__ float4 part_acc[3][128];
     __shared__ float part_l[3][128];
@@ -1141,26 +1146,26 @@ int latent_attend_and_merge(const santapp_latent_geom *geom, const santapp_laten
             if (dense) {
                 if ((err = ensure_dynamic_smem((const void *)latent_attend_kernel<true>, kLfSmemBytes, done_sp_all)) != cudaSuccess)
                     return note_cuda_failure(err, "latent attend attribute");
-                err = launch_kernel(latent_attend_kernel<true>, dim3(L.grid), dim3(kLfThreads), kLfSmemBytes, s, ap);
+                err = launch_step(latent_attend_kernel<true>, dim3(L.grid), dim3(kLfThreads), kLfSmemBytes, s, ap);
             } else {
                 if ((err = ensure_dynamic_smem((const void *)latent_attend_kernel<false>, kLfSmemBytes, done_sp_sel)) != cudaSuccess)
                     return note_cuda_failure(err, "latent attend attribute");
-                err = launch_kernel(latent_attend_kernel<false>, dim3(L.grid), dim3(kLfThreads), kLfSmemBytes, s, ap);
+                err = launch_step(latent_attend_kernel<false>, dim3(L.grid), dim3(kLfThreads), kLfSmemBytes, s, ap);
             }
         } else if (dense) {
             if ((err = ensure_dynamic_smem((const void *)latent_attend_tc_kernel<true>, kTcSmemBytes, done_tc_all)) != cudaSuccess)
                 return note_cuda_failure(err, "latent attend attribute");
-            err = launch_kernel(latent_attend_tc_kernel<true>, dim3(L.grid), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
+            err = launch_step(latent_attend_tc_kernel<true>, dim3(L.grid), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
         } else {
             if ((err = ensure_dynamic_smem((const void *)latent_attend_tc_kernel<false>, kTcSmemBytes, done_tc_sel)) != cudaSuccess)
                 return note_cuda_failure(err, "latent attend attribute");
-            err = launch_kernel(latent_attend_tc_kernel<false>, dim3(L.grid), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
+            err = launch_step(latent_attend_tc_kernel<false>, dim3(L.grid), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
         }
         if (err != cudaSuccess) return note_cuda_failure(err, "latent attend launch");
         ++launches;
     }
     if (mask & SANTAPP_STAGE_MERGE) {
-        err = launch_kernel(latent_merge_kernel, dim3(geom->n_heads, geom->n_seqs), dim3(kLmThreads), 0, s,
+        err = launch_step(latent_merge_kernel, dim3(geom->n_heads, geom->n_seqs), dim3(kLmThreads), 0, s,
                             (const float *)ap.partials, (const uint32_t *)ap.pair_prefix, geom->n_seqs, geom->n_heads, L.grid, out,
                             status);
         if (err != cudaSuccess) return note_cuda_failure(err, "latent merge launch");
@@ -1326,7 +1331,7 @@ int santapp_latent_decode_attn(const santapp_latent_geom *geom, const santapp_la
         sp.tiles_per_warp = (int)std::min<long long>(std::max<long long>((blocks1 + slots - 1) / slots, 1), 64);
         const dim3 grid((teams->max_teams_per_seq + kLsTeamsPerBlock * sp.tiles_per_warp - 1) / (kLsTeamsPerBlock * sp.tiles_per_warp),
                         geom->n_seqs);
-        if ((err = launch_kernel(latent_score_kernel, grid, dim3(kLsThreads), 0, s, sp)) != cudaSuccess)
+        if ((err = launch_step(latent_score_kernel, grid, dim3(kLsThreads), 0, s, sp)) != cudaSuccess)
             return note_cuda_failure(err, "latent score launch");
         ++launches;
     }
@@ -1367,8 +1372,8 @@ int santapp_latent_decode_attn(const santapp_latent_geom *geom, const santapp_la
         in.dbg_union_rows = nullptr;
         in.trace = dbg ? reinterpret_cast<unsigned long long *>(dbg->trace) : nullptr;
         const int n_heads = geom->n_seqs * geom->n_heads;
-        if (n_heads <= L.grid) err = launch_kernel(latent_select_kernel<512>, dim3(n_heads), dim3(512), 0, s, in);
-        else                   err = launch_kernel(latent_select_kernel<256>, dim3(n_heads), dim3(256), 0, s, in);
+        if (n_heads <= L.grid) err = launch_step(latent_select_kernel<512>, dim3(n_heads), dim3(512), 0, s, in);
+        else                   err = launch_step(latent_select_kernel<256>, dim3(n_heads), dim3(256), 0, s, in);
         if (err != cudaSuccess) return note_cuda_failure(err, "latent select launch");
         ++launches;
 
@@ -1391,7 +1396,7 @@ int santapp_latent_decode_attn(const santapp_latent_geom *geom, const santapp_la
         static std::atomic<unsigned long long> done_plan;
         if ((err = ensure_dynamic_smem((const void *)latent_plan_kernel, (int)sizeof(LatentPlanSmem), done_plan)) != cudaSuccess)
             return note_cuda_failure(err, "latent plan attribute");
-        if ((err = launch_kernel(latent_plan_kernel, dim3(geom->n_seqs), dim3(kLpThreads), sizeof(LatentPlanSmem), s, pp)) != cudaSuccess)
+        if ((err = launch_step(latent_plan_kernel, dim3(geom->n_seqs), dim3(kLpThreads), sizeof(LatentPlanSmem), s, pp)) != cudaSuccess)
             return note_cuda_failure(err, "latent plan launch");
         ++launches;
     }

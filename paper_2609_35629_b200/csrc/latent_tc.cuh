@@ -135,6 +135,7 @@ template <bool kAll>
 __global__ void __launch_bounds__(kTcThreads, 1)
 latent_attend_tc_kernel(LatentAttendParams p, int32_t *status)
 {
+    step_wait();
     extern __shared__ __align__(1024) unsigned char smem_tc[];
     unsigned char *smem = smem_tc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

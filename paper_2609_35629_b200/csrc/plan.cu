@@ -23,6 +23,7 @@ struct PlanKernelSmem {
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(PlanParams p, int max_words)
 {
+    step_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PlanKernelSmem &sm = *reinterpret_cast<PlanKernelSmem *>(smem_raw);
     const int pair = blockIdx.x, tid = threadIdx.x;
@@ -45,6 +46,7 @@ plan_kernel(PlanParams p, int max_words)
 __global__ void __launch_bounds__(256)
 dense_plan_kernel(PlanParams p)
 {
+    step_wait();
     const uint32_t all_heads = (1u << p.in.bv.group) - 1u;
     const int pair = blockIdx.x * blockDim.x + threadIdx.x;
     if (pair < 2) p.plan.tail_counter[pair] = 0;
@@ -77,6 +79,7 @@ dense_plan_kernel(PlanParams p)
 __global__ void __launch_bounds__(1024)
 pair_prefix_kernel(PlanView plan, int n_pairs)
 {
+    step_wait();
     __shared__ int scan[33];
     int64_t carry = 0;
     for (int base = 0; base < n_pairs; base += (int)blockDim.x) {
@@ -98,17 +101,17 @@ cudaError_t launch_plan(const PlanParams &p, int max_teams_per_seq, cudaStream_t
     static std::atomic<unsigned long long> done;
     cudaError_t err = ensure_dynamic_smem((const void *)plan_kernel, (int)smem, done);
     if (err != cudaSuccess) return err;
-    return launch_kernel(plan_kernel, dim3(p.n_pairs), dim3(kPlanThreads), smem, s, p, (max_teams_per_seq + 31) / 32);
+    return launch_step(plan_kernel, dim3(p.n_pairs), dim3(kPlanThreads), smem, s, p, (max_teams_per_seq + 31) / 32);
 }
 
 cudaError_t launch_dense_plan(const PlanParams &p, cudaStream_t s)
 {
-    return launch_kernel(dense_plan_kernel, dim3((p.n_pairs + 255) / 256), dim3(256), 0, s, p);
+    return launch_step(dense_plan_kernel, dim3((p.n_pairs + 255) / 256), dim3(256), 0, s, p);
 }
 
 cudaError_t launch_pair_prefix(const PlanParams &p, cudaStream_t s)
 {
-    return launch_kernel(pair_prefix_kernel, dim3(1), dim3(1024), 0, s, p.plan, p.n_pairs);
+    return launch_step(pair_prefix_kernel, dim3(1), dim3(1024), 0, s, p.plan, p.n_pairs);
 }
 
 }  // namespace santapp

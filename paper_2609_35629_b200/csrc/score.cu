@@ -80,6 +80,7 @@ template <int G, bool kHalf>
 __global__ void __launch_bounds__(kScoreThreads, 2)
 score32_kernel(ScoreParams p)
 {
+    step_wait();
     __shared__ uint4 philox_words[kScoreThreads / 32][32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, c = lane & 3;
@@ -164,6 +165,7 @@ template <int G, bool kHalf>
 __global__ void __launch_bounds__(kScoreThreads, 2)
 score32_flat_kernel(ScoreParams p)
 {
+    step_wait();
     extern __shared__ uint4 score_ring[];
     __shared__ uint4 philox_words[kScoreThreads / 32][32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -327,12 +329,12 @@ cudaError_t launch_score32_g(const ScoreParams &p, int max_teams, cudaStream_t s
     const long long ctas1 = (long long)((max_teams + kScoreTeamsPerCta - 1) / kScoreTeamsPerCta) * p.n_pairs;
     if (ctas1 < 2 * attend_grid_size()) {
         dim3 grid((max_teams + kScoreTeamsPerCta - 1) / kScoreTeamsPerCta, p.n_pairs);
-        return launch_kernel(score32_kernel<G, kHalf>, grid, dim3(kScoreThreads), 0, s, p);
+        return launch_step(score32_kernel<G, kHalf>, grid, dim3(kScoreThreads), 0, s, p);
     }
     static std::atomic<unsigned long long> done;
     cudaError_t e = ensure_dynamic_smem((const void *)score32_flat_kernel<G, kHalf>, kScoreRingBytes, done);
     if (e != cudaSuccess) return e;
-    return launch_kernel(score32_flat_kernel<G, kHalf>, dim3(2 * attend_grid_size()), dim3(kScoreThreads), kScoreRingBytes, s, p);
+    return launch_step(score32_flat_kernel<G, kHalf>, dim3(2 * attend_grid_size()), dim3(kScoreThreads), kScoreRingBytes, s, p);
 }
 
 }  // namespace
