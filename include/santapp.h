@@ -181,9 +181,8 @@ int santapp_build_teams_sizes(const santapp_geom *geom, const int32_t *prompt_le
  *   teams                host struct of device pointers, out: every array is overwritten; the
  *                        host scalars are filled in
  *   workspace            device, >= sizes.build_workspace_bytes; contents undefined afterwards
- * The call copies the (n_seqs + 1)-entry offset tables to the device with cudaMemcpyAsync from
- * pageable memory, which orders after prior work on `stream`; it is a preparation call, outside
- * the per-token path.
+ * The (n_seqs + 1)-entry offset tables travel to the device inside kernel arguments; it is a
+ * preparation call, outside the per-token path.
  */
 int santapp_build_teams(const santapp_geom *geom, const int32_t *prompt_len_host,
                         const void *k_prompt, const void *v_prompt,
@@ -253,9 +252,8 @@ int32_t santapp_kmeans_parent_count(int32_t prompt_len, int32_t parent_size);
  * most of the fit; with opts->no_host_poll = 1 it never waits and enqueues every step up to the
  * limit instead (the result is the same: a stopped fit's later steps do nothing). In that mode the
  * call may be issued during a stream capture and the graph replayed: the per-sequence tables made
- * from the host arrays travel inside kernel arguments, nothing is copied from host memory. (The
- * other preparation calls that take host arrays -- the builders and santapp_assign_parents -- copy
- * their tables from host memory that is gone when they return: they must not be captured.)
+ * from the host arrays travel inside kernel arguments, nothing is copied from host memory (the other
+ * preparation calls that take host arrays do the same).
  */
 typedef struct santapp_kmeans_opts {
     int32_t batch_size;           /* paper: 4096 */

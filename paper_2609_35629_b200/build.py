@@ -7,7 +7,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 SOURCES = ["api.cu", "build_teams.cu", "build_parents.cu", "kmeans.cu", "score.cu", "headplan.cu", "plan.cu", "attend.cu", "latent.cu"]
-HEADERS = [os.path.join(CSRC, h) for h in ("common.cuh", "pairplan.cuh", "headplan.cuh", "score_tile.cuh", "build_util.cuh", "latent_tc.cuh")] \
+HEADERS = [os.path.join(CSRC, h) for h in ("common.cuh", "pairplan.cuh", "headplan.cuh", "score_tile.cuh", "build_util.cuh", "select_rows.cuh", "latent_tc.cuh")] \
     + [os.path.join(ROOT, "include", h) for h in ("santapp.h", "santapp_latent.h")]
 OUT = os.path.join(HERE, "libsantapp.so")
 
@@ -25,7 +25,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         newest = max(os.path.getmtime(f) for f in srcs + HEADERS + [os.path.abspath(__file__)])
         if os.path.getmtime(OUT) >= newest:
             return OUT
-    cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
+    cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "--threads", "0", "-std=c++17",
            "-Xcompiler", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
            "-o", OUT] + srcs
     if os.environ.get("SANTAPP_TUNE"):

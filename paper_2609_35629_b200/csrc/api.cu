@@ -237,11 +237,9 @@ int build_records(const santapp_geom *geom, const int32_t *prompt_len_host, cons
         const int parents = (N + geom->parent_size - 1) / geom->parent_size;
         if (parents > max_parents) max_parents = parents;
     }
-    const size_t ob = sizeof(int64_t) * ((size_t)geom->n_seqs + 1);
-    cudaError_t err = cudaMemcpyAsync(teams->seq_row_off, row_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy seq_row_off");
-    err = cudaMemcpyAsync(teams->seq_team_off, team_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy seq_team_off");
+    cudaError_t err = launch_tables({row_off, team_off, nullptr}, {teams->seq_row_off, teams->seq_team_off, nullptr}, geom->n_seqs + 1,
+                                    teams->rep_abs_max, geom->n_kv_heads * geom->n_seqs, s);
+    if (err != cudaSuccess) return cuda_fail(err, "offset tables");
 
     teams->rows_total = sz.rows_total;
     teams->teams_total = sz.teams_total;
@@ -261,12 +259,14 @@ int build_records(const santapp_geom *geom, const int32_t *prompt_len_host, cons
     p.team_row_start = teams->team_row_start;
     p.row_token = teams->row_token;
     p.team_count = teams->team_count;
-    p.owner = static_cast<uint16_t *>(workspace);
+    p.rep_abs_max = teams->rep_abs_max;
     p.max_parents_per_seq = max_parents;
     err = mean_groups ? launch_build_groups_mean(p, s) : launch_build_teams(p, s);
     if (err != cudaSuccess) return cuda_fail(err, "build launch");
-    err = launch_rep_abs_max(p.bv, p.rep_keys, teams->rep_abs_max, s);
-    if (err != cudaSuccess) return cuda_fail(err, "rep_abs_max launch");
+    if (mean_groups) {                                          // (the team builder raises it as it goes)
+        err = launch_rep_abs_max(p.bv, sz.max_teams_per_seq, p.rep_keys, teams->rep_abs_max, s);
+        if (err != cudaSuccess) return cuda_fail(err, "rep_abs_max launch");
+    }
     return SANTAPP_OK;
 }
 
@@ -348,10 +348,8 @@ int santapp_assign_parents(const santapp_geom *geom, const int32_t *prompt_len_h
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     int64_t *d_row_off = reinterpret_cast<int64_t *>(ws);
     int64_t *d_cen_off = reinterpret_cast<int64_t *>(ws + align_up(ob));
-    cudaError_t err = cudaMemcpyAsync(d_row_off, row_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy row offsets");
-    err = cudaMemcpyAsync(d_cen_off, cen_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy centre offsets");
+    cudaError_t err = launch_tables({row_off, cen_off, nullptr}, {d_row_off, d_cen_off, nullptr}, geom->n_seqs + 1, nullptr, 0, s);
+    if (err != cudaSuccess) return cuda_fail(err, "offset tables");
     AssignParams p;
     p.n_seqs = geom->n_seqs;
     p.n_kv = geom->n_kv_heads;
@@ -432,13 +430,10 @@ static int build_parent_records(const santapp_geom *geom, const int32_t *prompt_
     }
     const ParentLayout L = parent_layout(B, geom->n_kv_heads, sz.rows_total, label_off[B], sz.teams_total);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
-    const size_t ob = sizeof(int64_t) * ((size_t)B + 1);
-    cudaError_t err = cudaMemcpyAsync(teams->seq_row_off, row_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy seq_row_off");
-    err = cudaMemcpyAsync(teams->seq_team_off, team_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy seq_team_off");
-    err = cudaMemcpyAsync(ws + L.label_off, label_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "copy label offsets");
+    cudaError_t err = launch_tables({row_off, team_off, label_off},
+                                    {teams->seq_row_off, teams->seq_team_off, reinterpret_cast<int64_t *>(ws + L.label_off)}, B + 1,
+                                    teams->rep_abs_max, geom->n_kv_heads * B, s);
+    if (err != cudaSuccess) return cuda_fail(err, "offset tables");
 
     teams->rows_total = sz.rows_total;
     teams->teams_total = sz.teams_total;
@@ -474,7 +469,7 @@ static int build_parent_records(const santapp_geom *geom, const int32_t *prompt_
     p.dest = reinterpret_cast<int32_t *>(ws + L.dest);
     err = launch_build_teams_parents(p, s);
     if (err != cudaSuccess) return cuda_fail(err, "build_teams_parents launch");
-    err = launch_rep_abs_max(p.bv, p.rep_keys, teams->rep_abs_max, s);
+    err = launch_rep_abs_max(p.bv, sz.max_teams_per_seq, p.rep_keys, teams->rep_abs_max, s);
     if (err != cudaSuccess) return cuda_fail(err, "rep_abs_max launch");
     return SANTAPP_OK;
 }

@@ -235,7 +235,8 @@ int current_stage_mask();
 // Host launchers (each returns the cudaError_t of its launches).
 // ---------------------------------------------------------------------------------------------
 cudaError_t launch_score32(const ScoreParams &p, int max_teams_per_seq, cudaStream_t s);
-cudaError_t launch_rep_abs_max(const BatchView &bv, const uint16_t *rep_keys, float *rep_abs_max, cudaStream_t s);
+// raises rep_abs_max (zero, or a bound so far) to the pair's largest |element|
+cudaError_t launch_rep_abs_max(const BatchView &bv, int max_teams_per_seq, const uint16_t *rep_keys, float *rep_abs_max, cudaStream_t s);
 cudaError_t launch_headplan(const PlanInputs &in, cudaStream_t s);
 cudaError_t launch_plan(const PlanParams &p, int max_teams_per_seq, cudaStream_t s);
 cudaError_t launch_pair_prefix(const PlanParams &p, cudaStream_t s);
@@ -258,9 +259,11 @@ struct BuildParams {
     uint16_t *k_packed, *v_packed, *rep_keys;
     int32_t *team_row_start, *row_token;
     int32_t *team_count;                    // [n_kv][n_seqs] or null
-    uint16_t *owner;                        // workspace [n_kv][rows_total]: team index inside the parent
+    float *rep_abs_max;                     // [n_kv][n_seqs], zero before the kernel
     int max_parents_per_seq;
 };
+// The batch's offset tables on the device (up to three of `entries` values each; null: none), and n_zero floats set to 0.
+cudaError_t launch_tables(const int64_t *const (&host)[3], int64_t *const (&dev)[3], int entries, float *zero, int n_zero, cudaStream_t s);
 cudaError_t launch_build_teams(const BuildParams &p, cudaStream_t s);
 cudaError_t launch_build_groups_mean(const BuildParams &p, cudaStream_t s);
 

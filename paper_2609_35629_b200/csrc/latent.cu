@@ -25,11 +25,11 @@
 #include <algorithm>
 #include <vector>
 
-#include "build_util.cuh"
 #include "common.cuh"
 #include "headplan.cuh"
 #include "santapp_latent.h"
 #include "score_tile.cuh"
+#include "select_rows.cuh"
 
 using namespace santapp;
 
@@ -59,188 +59,87 @@ struct LatentBuildParams {
     const uint16_t *rows_prompt;
     uint16_t *rows_packed, *rep_rows;
     int32_t *team_row_start, *row_token;
-    float *rep_abs_max;
-    uint8_t *owner;                 // workspace [rows_total]
+    float *rep_abs_max;             // zero before the kernel
     int max_parents_per_seq;
 };
 
-constexpr int kLbThreads = 128;
+// A warp per parent (at most 32 rows), everything in one kernel: the parent's rows keep their range of the packed
+// order, so its owners give its row offsets and packed rows at once. Rows go through shared memory (asynchronous
+// copies, 18 KB of 16 rows on their way per warp, ten warps per SM); distances over the latent columns and the
+// selection: select_rows.cuh. Bound by memory: 1152 bytes in and 1152 * (1 + R / P) out per row. The fp64
+// version in three kernels (block per parent, scan, pack) took 1309 us for 32 sequences of 8192.
+constexpr int kLbPitch = kRowDim / 2 + 4;                   // words per staged row: ldmatrix without bank conflicts
+constexpr int kLbWarps = 2;
+template <int kRows>
+struct LatentBuildSmem {
+    __align__(16) uint32_t rows[kRows * kLbPitch];
+    float dist[kRows * (kRows + 1)];
+    int rep_of[kMaxP];
+};
 
-// Squared distance between two rows' latent parts in fp64: dims in increasing order, multiply
-// and add rounded separately (the order the records are defined with).
-__device__ __forceinline__ double latent_sqdist(const uint32_t *a, const uint32_t *b)
+template <int kRows>
+__global__ void __launch_bounds__(kLbWarps * 32)
+latent_build_kernel(LatentBuildParams p)
 {
-    double s = 0.0;
-#pragma unroll 8
-    for (int w = 0; w < kLatDim / 2; ++w) {
-        const uint32_t x = a[w], y = b[w];
-        const double e0 = __dsub_rn((double)bf16_lo(x), (double)bf16_lo(y));
-        const double e1 = __dsub_rn((double)bf16_hi(x), (double)bf16_hi(y));
-        s = __dadd_rn(s, __dmul_rn(e0, e0));
-        s = __dadd_rn(s, __dmul_rn(e1, e1));
-    }
-    return s;
-}
-
-// One block per (parent, sequence).
-__global__ void __launch_bounds__(kLbThreads)
-latent_build_parent_kernel(LatentBuildParams p)
-{
-    constexpr int kPitch = kRowDim / 2 + 1;                 // words per staged row (+1: conflict-free column walks)
-    __shared__ uint32_t rows[kMaxP * kPitch];
-    __shared__ double mu[kLatDim];
-    __shared__ double mind[kMaxP];
-    __shared__ ValIdx scratch[33];
-    __shared__ int owner[kMaxP], count[kMaxP], rep_of[kMaxP];
-    __shared__ unsigned char is_rep[kMaxP];
-
-    const int parent = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-    const int64_t row0 = p.lv.seq_row_off[b];
-    const int N = (int)(p.lv.seq_row_off[b + 1] - row0);
-    const int P = p.parent_size;
-    const int first = parent * P;
-    if (first >= N) return;
-    const int nC = min(P, N - first);
-    const int r = min(p.reps, nC);
-
-    const uint32_t *src = reinterpret_cast<const uint32_t *>(p.rows_prompt) + (size_t)(row0 + first) * (kRowDim / 2);
-    for (int e = tid; e < nC * (kRowDim / 2); e += kLbThreads) rows[(e / (kRowDim / 2)) * kPitch + e % (kRowDim / 2)] = src[e];
-    for (int i = tid; i < nC; i += kLbThreads) { is_rep[i] = 0; count[i] = 0; }
-    __syncthreads();
-
-    // parent mean of the latent columns: rows added in token order, then one division
-    for (int d = tid; d < kLatDim; d += kLbThreads) {
-        double s = 0.0;
-        for (int i = 0; i < nC; ++i) {
-            const uint32_t word = rows[i * kPitch + (d >> 1)];
-            s = __dadd_rn(s, (double)((d & 1) ? bf16_hi(word) : bf16_lo(word)));
-        }
-        mu[d] = __ddiv_rn(s, (double)nC);
-    }
-    __syncthreads();
-
-    // first representative: the row whose latent is nearest the mean
-    {
-        ValIdx best = {INFINITY, INT_MAX};
-        for (int i = tid; i < nC; i += kLbThreads) {
-            double s = 0.0;
-            const uint32_t *row = rows + i * kPitch;
-            for (int w = 0; w < kLatDim / 2; ++w) {
-                const uint32_t word = row[w];
-                const double e0 = __dsub_rn((double)bf16_lo(word), mu[2 * w]);
-                const double e1 = __dsub_rn((double)bf16_hi(word), mu[2 * w + 1]);
-                s = __dadd_rn(s, __dmul_rn(e0, e0));
-                s = __dadd_rn(s, __dmul_rn(e1, e1));
-            }
-            ValIdx c = {s, i};
-            best = pick<true>(best, c);
-        }
-        best = block_arg<true>(best, scratch);
-        if (tid == 0) { rep_of[0] = best.i; is_rep[best.i] = 1; }
-    }
-    __syncthreads();
-
-    // farthest-first representatives with the running nearest-representative assignment
-    for (int i = tid; i < nC; i += kLbThreads) { mind[i] = INFINITY; owner[i] = 0; }
-    for (int u = 0; u < r; ++u) {
-        const uint32_t *ref = rows + rep_of[u] * kPitch;
-        ValIdx far = {-2.0, INT_MAX};
-        for (int i = tid; i < nC; i += kLbThreads) {
-            const double dist = latent_sqdist(rows + i * kPitch, ref);
-            if (dist < mind[i]) { mind[i] = dist; owner[i] = u; }
-            ValIdx c = {is_rep[i] ? -1.0 : mind[i], i};
-            far = pick<false>(far, c);
-        }
-        if (u + 1 < r) {
-            far = block_arg<false>(far, scratch);
-            if (tid == 0) { rep_of[u + 1] = far.i; is_rep[far.i] = 1; }
-            __syncthreads();
-        }
-    }
-    __syncthreads();
-    for (int u = tid; u < r; u += kLbThreads) owner[rep_of[u]] = u;      // a representative owns its own row
-    __syncthreads();
-    for (int i = tid; i < nC; i += kLbThreads) atomicAdd(&count[owner[i]], 1);
-    __syncthreads();
-
-    uint8_t *owner_out = p.owner + row0 + first;
-    for (int i = tid; i < nC; i += kLbThreads) owner_out[i] = (uint8_t)owner[i];
-    const int64_t team0 = p.lv.seq_team_off[b];
-    const int team_local0 = parent * p.teams_per_full_parent;
-    int32_t *csr = p.team_row_start + team0 + b;
-    if (parent == 0 && tid == 0) csr[0] = 0;
-    for (int u = tid; u < r; u += kLbThreads) csr[1 + team_local0 + u] = count[u];    // sizes; scanned next
-    uint32_t *rep_dst = reinterpret_cast<uint32_t *>(p.rep_rows) + (size_t)(team0 + team_local0) * (kRowDim / 2);
-    for (int e = tid; e < r * (kRowDim / 2); e += kLbThreads)
-        rep_dst[e] = rows[rep_of[e / (kRowDim / 2)] * kPitch + e % (kRowDim / 2)];
-}
-
-// One block per sequence: team sizes -> CSR offsets, and the largest |value| of the representatives.
-__global__ void __launch_bounds__(256)
-latent_scan_kernel(LatentBuildParams p)
-{
-    __shared__ int scratch[33];
-    __shared__ uint32_t red[8];
-    const int b = blockIdx.x;
-    const int64_t team0 = p.lv.seq_team_off[b];
-    const int M = (int)(p.lv.seq_team_off[b + 1] - team0);
-    int32_t *csr = p.team_row_start + team0 + b + 1;
-    int carry = 0;
-    for (int base = 0; base < M; base += 256) {
-        const int g = base + threadIdx.x;
-        const int v = g < M ? csr[g] : 0;
-        int total;
-        const int excl = block_exclusive_scan(v, scratch, total);
-        if (g < M) csr[g] = carry + excl + v;
-        carry += total;
-    }
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(p.rep_rows) + (size_t)team0 * (kRowDim / 2);
-    const int64_t n = (int64_t)M * (kRowDim / 2);
-    uint32_t m = 0u;                                        // bf16 magnitudes order like integers
-    for (int64_t i = threadIdx.x; i < n; i += 256) {
-        const uint32_t v = w[i];
-        m = max(m, max(v & 0x7FFFu, (v >> 16) & 0x7FFFu));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < 8; ++i) m = max(m, red[i]);
-        p.rep_abs_max[b] = __uint_as_float(m << 16);
-    }
-}
-
-// One block per (parent, sequence): stable partition of the parent's rows by team, row copies.
-__global__ void __launch_bounds__(kLbThreads)
-latent_pack_kernel(LatentBuildParams p)
-{
-    __shared__ uint8_t owner[kMaxP];
-    __shared__ int dest[kMaxP];
-    const int parent = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_wait();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    LatentBuildSmem<kRows> &sm = reinterpret_cast<LatentBuildSmem<kRows> *>(smem_raw)[warp];
+    const int parent = blockIdx.x * kLbWarps + warp, b = blockIdx.y;
     const int64_t row0 = p.lv.seq_row_off[b];
     const int N = (int)(p.lv.seq_row_off[b + 1] - row0);
     const int first = parent * p.parent_size;
     if (first >= N) return;
-    const int nC = min(p.parent_size, N - first);
-    for (int i = tid; i < nC; i += kLbThreads) owner[i] = p.owner[row0 + first + i];
-    __syncthreads();
-    const int32_t *csr = p.team_row_start + p.lv.seq_team_off[b] + b;
+    const int nC = min(p.parent_size, N - first), r = min(p.reps, nC);
+    const size_t row_at = (size_t)row0 + first;
+    const uint4 *src = reinterpret_cast<const uint4 *>(p.rows_prompt) + row_at * kRowChunks;
+    uint4 *dst = reinterpret_cast<uint4 *>(p.rows_packed) + row_at * kRowChunks;
+    for (int e = lane; e < nC * kRowChunks; e += 32)
+        copy16_async(shared_addr(sm.rows + (e / kRowChunks) * kLbPitch + (e % kRowChunks) * 4), src + e);
+    copy_async_wait();
+    __syncwarp();
+    int owner, pos;
+    select_small<kRows, kLatDim / 2, kLbPitch, false>(sm.rows, sm.dist, sm.rep_of, nC, r, owner, pos);
+    for (int i = 0; i < nC; ++i) {                          // a row: 72 pieces of 16 bytes
+        const uint4 *row = reinterpret_cast<const uint4 *>(sm.rows + i * kLbPitch);
+        uint4 *to = dst + (size_t)__shfl_sync(0xFFFFFFFFu, pos, i) * kRowChunks;
+        to[lane] = row[lane];
+        to[lane + 32] = row[lane + 32];
+        if (lane < kRowChunks - 64) to[lane + 64] = row[lane + 64];
+    }
+    if (lane < nC) p.row_token[row_at + pos] = first + lane;
+    const int64_t team0 = p.lv.seq_team_off[b];
     const int team_local0 = parent * p.teams_per_full_parent;
-    for (int i = tid; i < nC; i += kLbThreads) {
-        const int u = owner[i];
-        int rank = 0;
-        for (int a = 0; a < i; ++a) rank += (owner[a] == u);
-        dest[i] = csr[team_local0 + u] + rank;              // members in increasing token index
+    int32_t *csr = p.team_row_start + team0 + b + team_local0;
+    int upto = 0;                                           // rows of the teams 0 .. lane
+    for (int i = 0; i < nC; ++i) upto += __shfl_sync(0xFFFFFFFFu, owner, i) <= lane ? 1 : 0;
+    if (lane < r) csr[1 + lane] = first + upto;
+    if (parent == 0 && lane == 0) csr[0] = 0;
+    uint4 *rep_dst = reinterpret_cast<uint4 *>(p.rep_rows) + (size_t)(team0 + team_local0) * kRowChunks;
+    uint32_t m = 0u;                                        // bf16 magnitudes order like integers
+    for (int u = 0; u < r; ++u) {
+        const uint4 *row = reinterpret_cast<const uint4 *>(sm.rows + sm.rep_of[u] * kLbPitch);
+        for (int c = lane; c < kRowChunks; c += 32) {
+            const uint4 w = row[c];
+            rep_dst[(size_t)u * kRowChunks + c] = w;
+            const uint32_t v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) m = max(m, max(v[k] & 0x7FFFu, (v[k] >> 16) & 0x7FFFu));
+        }
     }
-    __syncthreads();
-    const uint4 *src = reinterpret_cast<const uint4 *>(p.rows_prompt) + (size_t)(row0 + first) * kRowChunks;
-    uint4 *dst = reinterpret_cast<uint4 *>(p.rows_packed) + (size_t)row0 * kRowChunks;
-    for (int e = tid; e < nC * kRowChunks; e += kLbThreads) {
-        const int i = e / kRowChunks, c = e - i * kRowChunks;
-        dst[(size_t)dest[i] * kRowChunks + c] = src[e];
-    }
-    for (int i = tid; i < nC; i += kLbThreads) p.row_token[row0 + dest[i]] = first + i;
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if (lane == 0) atomicMax(reinterpret_cast<uint32_t *>(p.rep_abs_max + b), m << 16);
+}
+
+template <int kRows>
+cudaError_t launch_latent_build(const LatentBuildParams &p, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> done;
+    const int smem = (int)sizeof(LatentBuildSmem<kRows>) * kLbWarps;
+    const cudaError_t err = ensure_dynamic_smem((const void *)latent_build_kernel<kRows>, smem, done);
+    if (err != cudaSuccess) return err;
+    return launch_step(latent_build_kernel<kRows>, dim3((p.max_parents_per_seq + kLbWarps - 1) / kLbWarps, p.lv.n_seqs),
+                       dim3(kLbWarps * 32), smem, s, p);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1232,11 +1131,9 @@ int santapp_latent_build_teams(const santapp_latent_geom *geom, const int32_t *p
         team_off[b + 1] = team_off[b] + latent_teams_in_sequence(N, geom->parent_size, geom->reps_per_parent);
         max_parents = std::max(max_parents, (N + geom->parent_size - 1) / geom->parent_size);
     }
-    const size_t ob = sizeof(int64_t) * ((size_t)geom->n_seqs + 1);
-    cudaError_t err = cudaMemcpyAsync(teams->seq_row_off, row_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return note_cuda_failure(err, "copy seq_row_off");
-    err = cudaMemcpyAsync(teams->seq_team_off, team_off, ob, cudaMemcpyHostToDevice, s);
-    if (err != cudaSuccess) return note_cuda_failure(err, "copy seq_team_off");
+    cudaError_t err = launch_tables({row_off, team_off, nullptr}, {teams->seq_row_off, teams->seq_team_off, nullptr}, geom->n_seqs + 1,
+                                    teams->rep_abs_max, geom->n_seqs, s);
+    if (err != cudaSuccess) return note_cuda_failure(err, "offset tables");
     teams->rows_total = sz.rows_total;
     teams->teams_total = sz.teams_total;
     teams->max_teams_per_seq = sz.max_teams_per_seq;
@@ -1253,15 +1150,9 @@ int santapp_latent_build_teams(const santapp_latent_geom *geom, const int32_t *p
     p.team_row_start = teams->team_row_start;
     p.row_token = teams->row_token;
     p.rep_abs_max = teams->rep_abs_max;
-    p.owner = static_cast<uint8_t *>(workspace);
     p.max_parents_per_seq = max_parents;
-    const dim3 grid(max_parents, geom->n_seqs);
-    if ((err = launch_kernel(latent_build_parent_kernel, grid, dim3(kLbThreads), 0, s, p)) != cudaSuccess)
-        return note_cuda_failure(err, "latent build launch");
-    if ((err = launch_kernel(latent_scan_kernel, dim3(geom->n_seqs), dim3(256), 0, s, p)) != cudaSuccess)
-        return note_cuda_failure(err, "latent scan launch");
-    if ((err = launch_kernel(latent_pack_kernel, grid, dim3(kLbThreads), 0, s, p)) != cudaSuccess)
-        return note_cuda_failure(err, "latent pack launch");
+    err = p.parent_size <= 16 ? launch_latent_build<16>(p, s) : launch_latent_build<kMaxP>(p, s);
+    if (err != cudaSuccess) return note_cuda_failure(err, "latent build launch");
     return SANTAPP_OK;
 }
 

@@ -1,0 +1,94 @@
+"""Contiguous records where the fp32 distances decide little or sit at the edges of their tiles: parents of
+every kernel's smallest, largest and odd sizes, one team per key, keys repeated many times, keys whose squares
+leave the range of fp32, and one key far larger than the rest; against the oracle, bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import santapp_oracle as orc
+from paper_2609_35629_b200 import binding as sp
+from paper_2609_35629_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _keys(kind, n, d, rng):
+    x = rng.standard_normal((n, d)).astype(np.float32)
+    if kind == "repeated":                       # few distinct rows: most distances are exactly zero or exactly tied
+        x = x[rng.integers(0, 5, size=n)]
+    elif kind == "zero":
+        x[:] = 0.0
+    elif kind == "huge":                         # squares overflow fp32 (fp64 decides)
+        x *= np.float32(1e25)
+    elif kind == "tiny":                         # squares underflow fp32
+        x *= np.float32(1e-25)
+    elif kind == "outlier":                      # one row a thousand times longer: its error bound dwarfs the others'
+        x[n // 2] *= np.float32(1000.0)
+    elif kind == "offset":                       # a common component much longer than the differences
+        x += np.float32(30.0)
+    elif kind == "integer":                      # exact ties at many distances
+        x = rng.integers(-1, 2, size=(n, d)).astype(np.float32)
+    return x
+
+
+CASES = [(p, r) for p, r in [(1, 1), (5, 1), (8, 2), (16, 4), (16, 16), (17, 17), (24, 8), (32, 32), (33, 11), (64, 8), (65, 13),
+                             (128, 8), (129, 43), (256, 16), (258, 258), (512, 32), (512, 512), (512, 1)]]
+
+
+@pytest.mark.parametrize("P,R", CASES)
+@pytest.mark.parametrize("kind,elem", [("plain", "bf16"), ("plain", "fp16"), ("repeated", "bf16"), ("integer", "fp16"),
+                                       ("outlier", "bf16"), ("offset", "bf16")])
+def test_records_at_every_parent_size(P, R, kind, elem):
+    _check(P, R, kind, elem)
+
+
+@pytest.mark.parametrize("P,R", [(16, 4), (32, 8), (64, 8), (512, 32)])
+@pytest.mark.parametrize("kind", ["zero", "huge", "tiny"])
+def test_records_outside_the_range_of_fp32_squares(P, R, kind):
+    _check(P, R, kind, "bf16")
+
+
+def _check(P, R, kind, elem):
+    rng = np.random.default_rng([P, R, len(kind)])
+    lens, kv = [2 * P + P // 2 + 1, P, max(1, P - 1)], 2
+    n = sum(lens)
+    k_bits = synth.round_bits(np.stack([_keys(kind, n, 128, rng) for _ in range(kv)]), elem)
+    v_bits = synth.round_bits(rng.standard_normal((kv, n, 128)).astype(np.float32), elem)
+    geom = sp.Geometry(len(lens), 2 * kv, kv, 128, P, R, sp.SANTAPP_FP16 if elem == "fp16" else sp.SANTAPP_BF16)
+    t = sp.santapp_build_teams(geom, lens, sp.bf16_bits_to_cuda(k_bits, dtype=geom.torch_dtype), sp.bf16_bits_to_cuda(v_bits, dtype=geom.torch_dtype))
+    torch.cuda.synchronize()
+    csr, token = t.team_row_start.cpu().numpy(), t.row_token.cpu().numpy()
+    kp, vp, rep = (x.view(torch.int16).cpu().numpy().view(np.uint16) for x in (t.k_packed, t.v_packed, t.rep_keys))
+    toff, amax = t.seq_team_off.cpu().numpy(), t.rep_abs_max.cpu().numpy()
+    off = np.concatenate([[0], np.cumsum(lens)])
+    for j in range(kv):
+        for b, N in enumerate(lens):
+            rows = slice(off[b], off[b + 1])
+            ts, tm, reps = orc.build_teams_contiguous(synth.to_f64(k_bits[j, rows], elem), P, R)
+            t0, t1 = int(toff[b]), int(toff[b + 1])
+            assert t.team_count[j, b].item() == t1 - t0 == len(reps)
+            assert np.array_equal(csr[j, t0 + b:t1 + b + 1], ts)
+            assert np.array_equal(token[j, rows], tm)
+            assert np.array_equal(rep[j, t0:t1], k_bits[j, rows][reps])
+            assert np.array_equal(kp[j, rows], k_bits[j, rows][tm]) and np.array_equal(vp[j, rows], v_bits[j, rows][tm])
+            assert amax[j, b] == np.abs(synth.to_f32(k_bits[j, rows][reps], elem)).max()
+
+
+@pytest.mark.parametrize("P,R", [(1, 1), (8, 2), (16, 4), (17, 17), (32, 8), (32, 32)])
+@pytest.mark.parametrize("kind", ["plain", "repeated", "integer", "outlier", "huge", "zero"])
+def test_shared_latent_records_at_every_parent_size(P, R, kind):
+    rng = np.random.default_rng([P, R, len(kind), 1])
+    lens = [3 * P + P // 2 + 1, P, max(1, P - 1)]
+    off = np.concatenate([[0], np.cumsum(lens)])
+    bits = synth.round_bits(_keys(kind, sum(lens), sp.LATENT_ROW, rng))
+    t = sp.santapp_latent_build_teams(sp.LatentGeometry(len(lens), 16, P, R), lens, sp.bf16_bits_to_cuda(bits))
+    torch.cuda.synchronize()
+    csr, token, toff = t.team_row_start.cpu().numpy(), t.row_token.cpu().numpy(), t.seq_team_off.cpu().numpy()
+    packed, rep = (x.view(torch.int16).cpu().numpy().view(np.uint16) for x in (t.rows_packed, t.rep_rows))
+    for b in range(len(lens)):
+        rows = bits[off[b]:off[b + 1]]
+        ts, tm, reps = orc.shared_latent_records(synth.to_f64(rows), sp.LATENT_DIM, P, R)
+        t0, t1 = int(toff[b]), int(toff[b + 1])
+        assert np.array_equal(csr[t0 + b:t1 + b + 1], ts) and np.array_equal(token[off[b]:off[b + 1]], tm)
+        assert np.array_equal(synth.to_f64(rep[t0:t1]), reps) and np.array_equal(packed[off[b]:off[b + 1]], rows[tm])
+        assert t.rep_abs_max[b].item() == np.abs(synth.to_f32(rep[t0:t1])).max()
