@@ -14,6 +14,7 @@
 
 #include "build_util.cuh"
 #include "common.cuh"
+#include "nearest.cuh"
 
 namespace santapp {
 
@@ -24,60 +25,91 @@ constexpr int kThreads = 256;
 __device__ __forceinline__ int clamp_label(int v, int n) { return min(max(v, 0), n - 1); }
 
 // ---- Algorithm 3, assignment step: b_i = argmin_u |k_i - mu_u|^2, ties to the smaller u ----
-constexpr int kAssignThreads = 128;
-constexpr int kAssignPts = 2;             // tokens per thread
-constexpr int kAssignGroup = 8;           // centres per pass
-constexpr int kCentreTile = 16;
-static_assert(kCentreTile % kAssignGroup == 0, "a tile of centres is a whole number of passes");
-
-// A thread holds two tokens and takes eight centres at a time (dist_points: a centre value read from
-// shared memory serves both tokens, a token value is widened once for the eight centres).
+// A block takes 256 tokens and scans all centres (nearest.cuh), which it splits into their 16-bit halves as it
+// brings them into shared memory (a quarter of a row per thread). Only tokens whose bounds leave more than
+// one centre see fp64. 4 x 32768 tokens, 2048 centres: 6.7 ms with every distance in fp64.
 template <bool kHalf>
-__global__ void __launch_bounds__(kAssignThreads)
+__global__ void __launch_bounds__(kNearThreads, 2)
 assign_parents_kernel(AssignParams p)
 {
-    __shared__ __align__(16) double c[kCentreTile][kHeadDim];
-    const int b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    NearSmem &sm = *reinterpret_cast<NearSmem *>(smem_raw);
+    step_wait();
+    const int b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
     const int64_t row0 = p.seq_row_off[b];
-    const int N = (int)(p.seq_row_off[b + 1] - row0);
-    if ((int)(blockIdx.x * kAssignThreads * kAssignPts) >= N) return;
+    const int N = (int)(p.seq_row_off[b + 1] - row0), i0 = blockIdx.x * kNearPoints;
+    if (i0 >= N) return;
     const int64_t c0off = p.seq_centre_off[b];
-    const int n_centres = (int)(p.seq_centre_off[b + 1] - c0off);
-    int i[kAssignPts], arg[kAssignPts];
-    const uint4 *row[kAssignPts];
-    double best[kAssignPts];
-#pragma unroll
-    for (int u = 0; u < kAssignPts; ++u) {
-        i[u] = (blockIdx.x * kAssignPts + u) * kAssignThreads + tid;
-        row[u] = reinterpret_cast<const uint4 *>(p.k_prompt + ((size_t)j * p.rows_total + row0 + min(i[u], N - 1)) * kHeadDim);
-        best[u] = INFINITY;
-        arg[u] = 0;
-    }
+    const int k = (int)(p.seq_centre_off[b + 1] - c0off);
+    const uint16_t *keys = p.k_prompt + ((size_t)j * p.rows_total + row0) * kHeadDim;
     const float *cen = p.centres + ((size_t)j * p.centres_total + c0off) * kHeadDim;
-    for (int base = 0; base < n_centres; base += kCentreTile) {
-        const int nt = min(kCentreTile, n_centres - base);
-        __syncthreads();
-        for (int e = tid; e < nt * kHeadDim; e += kAssignThreads)
-            c[e >> 7][e & 127] = (double)cen[(size_t)base * kHeadDim + e];
-        __syncthreads();
-        for (int t = 0; t < nt; t += kAssignGroup) {
-            // (rows of the tile past nt hold older values; their sums are not looked at)
-            double s[kAssignPts][kAssignGroup];
+    if (tid == 0) sm.largest = 0.f;
+    uint32_t a[2][8][4];
+    near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)min(i0 + i, N - 1) * kHeadDim; }, a);
+    near_scan<kHalf>(sm, a, 0, k, [&](int stage, int base, int n) {
+        const int row = tid >> 2, part = tid & 3;            // 32 values: four 16-byte pieces of each half
+        float nc = 0.f;
+        if (row < n) {
+            const float *src = cen + (size_t)(base + row) * kHeadDim + part * 32;
+            const bool wide = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
 #pragma unroll
-            for (int u = 0; u < kAssignPts; ++u)
+            for (int c = 0; c < 4; ++c) {
+                float v[8];
+                if (wide) {
+                    const float4 v0 = __ldg(reinterpret_cast<const float4 *>(src + 8 * c)), v1 = __ldg(reinterpret_cast<const float4 *>(src + 8 * c + 4));
+                    v[0] = v0.x; v[1] = v0.y; v[2] = v0.z; v[3] = v0.w; v[4] = v1.x; v[5] = v1.y; v[6] = v1.z; v[7] = v1.w;
+                } else {
 #pragma unroll
-                for (int v = 0; v < kAssignGroup; ++v) s[u][v] = 0.0;
-            dist_points<kHalf, kAssignPts, kAssignGroup, kAssignGroup>(row, c + t, s);
+                    for (int e = 0; e < 8; ++e) v[e] = __ldg(src + 8 * c + e);
+                }
+                uint32_t hi[4], mid[4];
 #pragma unroll
-            for (int u = 0; u < kAssignPts; ++u)
-#pragma unroll
-                for (int v = 0; v < kAssignGroup; ++v)
-                    if (t + v < nt && s[u][v] < best[u]) { best[u] = s[u][v]; arg[u] = base + t + v; }
+                for (int e = 0; e < 4; ++e) {
+                    hi[e] = pack_elems<kHalf>(v[2 * e], v[2 * e + 1]);
+                    mid[e] = pack_elems<kHalf>(v[2 * e] - elem_lo<kHalf>(hi[e]), v[2 * e + 1] - elem_hi<kHalf>(hi[e]));
+                    nc = fmaf(v[2 * e], v[2 * e], fmaf(v[2 * e + 1], v[2 * e + 1], nc));
+                }
+                sm.ring[stage][0][near_piece(row, part * 4 + c)] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                sm.ring[stage][1][near_piece(row, part * 4 + c)] = make_uint4(mid[0], mid[1], mid[2], mid[3]);
+            }
+        }
+        nc += __shfl_xor_sync(0xFFFFFFFFu, nc, 1);
+        nc += __shfl_xor_sync(0xFFFFFFFFu, nc, 2);
+        const float bias = row < n ? centre_bias<kHalf>(nc) : CUDART_INF_F;
+        if (row < n && !(bias > -CUDART_INF_F))              // fp32 cannot hold its norm: no part in the products
+            for (int c = 0; c < 4; ++c)
+                sm.ring[stage][0][near_piece(row, part * 4 + c)] = sm.ring[stage][1][near_piece(row, part * 4 + c)] = make_uint4(0u, 0u, 0u, 0u);
+        if (part == 0) {
+            sm.bias[stage][row] = bias;
+            if (row < n && nc <= 1e37f) atomicMax(reinterpret_cast<uint32_t *>(&sm.largest), __float_as_uint(nc));
+        }
+    });
+    __syncthreads();
+    const int i = i0 + tid;
+    const bool live = i < N;
+    const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)min(i, N - 1) * kHeadDim);
+    const NearTop top = sm.top[tid];
+    const float nx = sm.nx[tid];
+    int arg = top.i1;
+    bool all = !(nx <= 1e37f) || !(fabsf(top.t1) < CUDART_INF_F);
+    if (!all && live && !(top.t2 > top.t1 + near_slack<kHalf>(nx, sm.largest))) {
+        float nc = 0.f;
+        for (int d = 0; d < kHeadDim; ++d) { const float v = cen[(size_t)arg * kHeadDim + d]; nc = fmaf(v, v, nc); }
+        const float bar = top.t1 + near_slack<kHalf>(nx, nc);
+        all = !(top.t3 > bar);
+        if (!all && !(top.t2 > bar)) {
+            const double d1 = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim), d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
+            if (d2 < d1 || (d2 == d1 && top.i2 < arg)) arg = top.i2;
         }
     }
-#pragma unroll
-    for (int u = 0; u < kAssignPts; ++u)
-        if (i[u] < N) p.parent_of[(size_t)j * p.rows_total + row0 + i[u]] = arg[u];
+    for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
+        const int l = __ffs(left) - 1;
+        const uint4 *xl = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)x, l));
+        double d;
+        const int u = near_scan_exact<kHalf>(xl, cen, k, d);
+        if (lane == l) arg = u;
+    }
+    if (live) p.parent_of[(size_t)j * p.rows_total + row0 + i] = arg;
 }
 
 // ---- token counts per label ----
@@ -369,12 +401,18 @@ pack_rows_kernel(ParentBuildParams p)
 
 }  // namespace
 
+template <bool kHalf>
+static cudaError_t launch_assign(const AssignParams &p, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> done;
+    const cudaError_t err = ensure_dynamic_smem((const void *)assign_parents_kernel<kHalf>, (int)sizeof(NearSmem), done);
+    if (err != cudaSuccess) return err;
+    return launch_step(assign_parents_kernel<kHalf>, dim3((p.max_rows_per_seq + kNearPoints - 1) / kNearPoints, p.n_seqs, p.n_kv),
+                       dim3(kNearThreads), sizeof(NearSmem), s, p);
+}
 cudaError_t launch_assign_parents(const AssignParams &p, cudaStream_t s)
 {
-    dim3 grid((p.max_rows_per_seq + kAssignThreads * kAssignPts - 1) / (kAssignThreads * kAssignPts), p.n_seqs, p.n_kv);
-    if (p.elem) assign_parents_kernel<true><<<grid, kAssignThreads, 0, s>>>(p);
-    else        assign_parents_kernel<false><<<grid, kAssignThreads, 0, s>>>(p);
-    return cudaGetLastError();
+    return p.elem ? launch_assign<true>(p, s) : launch_assign<false>(p, s);
 }
 
 cudaError_t launch_build_teams_parents(const ParentBuildParams &p, cudaStream_t s)

@@ -305,6 +305,8 @@ struct ParentBuildParams {
 cudaError_t launch_build_teams_parents(const ParentBuildParams &p, cudaStream_t s);
 
 // Minibatch k-means fit (second line of Algorithm 3), one problem per (sequence, KV head).
+struct NearTop;
+constexpr size_t kNearTopBytes = 20;
 struct KmeansState {
     double ewa, ewa_min;                    // averaged per-point inertia and its minimum so far
     int bad, steps, stopped, pad;
@@ -332,10 +334,13 @@ struct KmeansParams {
     double *count;                          // [n_kv][centres_total]
     int32_t *idx, *label;                   // [pairs][batch]
     double *dist;                           // [pairs][batch]
-    double *dist_part;                      // [pairs][assign_split][batch] nearest centre inside each slice of the centres
-    int32_t *label_part;                    // [pairs][assign_split][batch]
-    int assign_split;                       // slices the centres are cut into for the nearest-centre search
-    uint32_t *sorted;                       // [pairs][4096] minibatch slots ordered by (label, slot): label << 12 | slot, padded with ~0
+    uint16_t *centre_hi, *centre_mid;       // [n_kv][centres_total][128] the centres as two 16-bit vectors (nearest.cuh)
+    float *centre_bias;                     // [n_kv][centres_total]
+    NearTop *near_top;                      // [pairs][assign_split][batch] the scan's result inside each slice of the centres
+    float *near_nx;                         // [pairs][batch] squared norms of the minibatch's points
+    int assign_split;                       // slices the centres are cut into for the scan
+    int32_t *sorted;                        // [pairs][4096] the minibatch's points ordered by (label, slot)
+    int32_t *start;                         // [pairs][k_max + 1] where each label starts there
     KmeansState *state;                     // [pairs]
     int *active;                            // [1] fits that still have steps to run
 };

@@ -14,13 +14,13 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "nearest.cuh"
 
 namespace santapp {
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kTile = 16;                 // centres staged per shared-memory tile
 constexpr int kPollEvery = 16;            // steps between two looks at the fits' stop flags
 constexpr uint32_t kTagSample = 1u, kTagStart = 2u, kTagBatch = 3u, kTagMove = 4u;
 
@@ -58,70 +58,45 @@ __device__ __forceinline__ uint32_t km_word(const KmeansParams &p, uint32_t slot
 }
 __device__ __forceinline__ int km_index(uint32_t word, int n) { return (int)(((unsigned long long)word * (unsigned long long)n) >> 32); }
 
-template <bool kHalf>
-__device__ __forceinline__ double sqdist_rows(const uint4 *a, const uint4 *b)
-{
-    double s = 0.0;
-#pragma unroll 4
-    for (int q = 0; q < 16; ++q) {
-        const uint4 x4 = a[q], y4 = b[q];
-        const uint32_t x[4] = {x4.x, x4.y, x4.z, x4.w}, y[4] = {y4.x, y4.y, y4.z, y4.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const double e0 = __dsub_rn((double)elem_lo<kHalf>(x[t]), (double)elem_lo<kHalf>(y[t]));
-            const double e1 = __dsub_rn((double)elem_hi<kHalf>(x[t]), (double)elem_hi<kHalf>(y[t]));
-            s = __dadd_rn(s, __dmul_rn(e0, e0));
-            s = __dadd_rn(s, __dmul_rn(e1, e1));
-        }
-    }
-    return s;
-}
-
 // ---- 1. initialisation sample: head of a Fisher-Yates shuffle ----
-__global__ void __launch_bounds__(kThreads)
-km_perm_identity_kernel(KmeansParams p)
+// Step i of the shuffle swaps entries i and r_i >= i of the index list, so entry i is final after step i, and holds
+// what entry r_i held before it: the value that the last earlier step j with r_j = r_i put there, which is what
+// entry j held before step j, and so on until no earlier step touched the entry (it still holds its own
+// index). The chains are short (about one step), so every entry is found on its own: steps are looked up by
+// target in a hash table in shared memory. One block per pair. (Swapping in order took 60 ns a step, 0.75 ms.)
+constexpr int kSampleThreads = 1024, kSampleBuckets = 8192;
+__host__ __device__ constexpr size_t sample_smem(int n_init)
 {
-    const Pair q = pair_of(p, blockIdx.y, blockIdx.z);
-    const int i = blockIdx.x * kThreads + threadIdx.x;
-    if (i < q.N) p.perm[q.plane + i] = i;
+    return sizeof(int32_t) * ((size_t)kSampleBuckets + (size_t)n_init) + sizeof(uint16_t) * (size_t)n_init;
 }
-
-// One block per pair. The swaps run in order on one lane; when the sequence's index list fits in
-// shared memory (smem_rows entries) it lives there for the shuffle -- a swap then costs two
-// shared-memory round trips instead of two to L2 -- and only the head, the sample, is written out.
-constexpr int kSampleSmemRows = 50 * 1024;
-__global__ void __launch_bounds__(kThreads)
-km_sample_kernel(KmeansParams p, int smem_rows)
+__global__ void __launch_bounds__(kSampleThreads)
+km_sample_kernel(KmeansParams p)
 {
-    extern __shared__ int32_t perm_s[];
+    extern __shared__ int32_t bucket_s[];                     // step + 1 of a bucket's first entry, 0: none
+    step_wait();
     const Pair q = pair_of(p, blockIdx.x, blockIdx.y);
-    const int tid = threadIdx.x, lane = tid & 31;
-    int32_t *perm_g = p.perm + q.plane;                       // (holds the identity when it is used for the shuffle)
-    const bool in_smem = q.N <= smem_rows;
-    if (in_smem)
-        for (int i = tid; i < q.N; i += kThreads) perm_s[i] = i;
+    const int tid = threadIdx.x;
+    int32_t *target_s = bucket_s + kSampleBuckets;            // [n_init] r_i
+    uint16_t *next_s = reinterpret_cast<uint16_t *>(target_s + q.n_init);   // [n_init] step + 1 of the next entry in the bucket
+    for (int u = tid; u < kSampleBuckets; u += kSampleThreads) bucket_s[u] = 0;
     __syncthreads();
-    if (tid < 32) {
-        int32_t *perm = in_smem ? perm_s : perm_g;
-        // the words of 32 positions at a time, the swaps in order on one lane
-        for (int i0 = 0; i0 < q.n_init; i0 += 32) {
-            const int i = i0 + lane;
-            const uint32_t w = i < q.n_init ? km_word(p, (uint32_t)i, kTagSample, q.stream, 0u) : 0u;
-            for (int l = 0; l < 32 && i0 + l < q.n_init; ++l) {
-                const uint32_t wl = __shfl_sync(0xFFFFFFFFu, w, l);
-                if (lane == 0) {
-                    const int at = i0 + l;
-                    const int r = at + km_index(wl, q.N - at);
-                    const int32_t t = perm[at];
-                    perm[at] = perm[r];
-                    perm[r] = t;
-                }
-            }
-        }
+    for (int i = tid; i < q.n_init; i += kSampleThreads) {
+        const int r = i + km_index(km_word(p, (uint32_t)i, kTagSample, q.stream, 0u), q.N - i);
+        target_s[i] = r;
+        next_s[i] = (uint16_t)atomicExch(&bucket_s[r & (kSampleBuckets - 1)], i + 1);
     }
     __syncthreads();
-    if (in_smem)
-        for (int i = tid; i < q.n_init; i += kThreads) perm_g[i] = perm_s[i];
+    for (int i = tid; i < q.n_init; i += kSampleThreads) {
+        int at = target_s[i], before = i;
+        while (true) {
+            int last = -1;
+            for (int e = bucket_s[at & (kSampleBuckets - 1)]; e > 0; e = next_s[e - 1])
+                if (target_s[e - 1] == at && e - 1 < before && e - 1 > last) last = e - 1;
+            if (last < 0) break;
+            at = before = last;
+        }
+        p.perm[q.plane + i] = at;
+    }
     if (tid == 0) p.pick[(size_t)q.id * p.trials_max] = km_index(km_word(p, 0u, kTagStart, q.stream, 0u), q.n_init);
 }
 
@@ -347,182 +322,307 @@ km_accept_kernel(KmeansParams p, int c)
 }
 
 // ---- 3. minibatch steps ----
+// A step is five kernels: the scan for the nearest centres (nearest.cuh), the fp64 distance to the one found,
+// the minibatch ordered by centre, the update, the reassignment of starved centres. The inertia of a
+// minibatch is a sum of `batch` terms in order -- 4096 dependent additions, 20 us -- and only decides whether
+// another step follows, so it is taken by one block per pair beside the next step's scan, which reads nothing
+// that it writes; from the kernel after that on, a fit that has stopped does nothing. At 4 pairs, batch
+// 4096 and 2048 centres a step was 0.94 ms (0.84 of it fp64 distances to every centre).
 __device__ __forceinline__ bool pair_active(const KmeansParams &p, const Pair &q, int t)
 {
     return t < q.t_max && !p.state[q.id].stopped;
 }
 
-// Draw the minibatch and assign each point to its nearest centre (ties to the smaller index). A thread
-// holds two points and takes eight centres at a time (dist_points); every sum still adds its 128
-// terms in order.
-constexpr int kAssignPts = 2;             // points per thread
-constexpr int kAssignBlock = 128 * kAssignPts;
-constexpr int kAssignGroup = 8;           // centres per pass
-static_assert(kTile % kAssignGroup == 0, "a tile of centres is a whole number of passes");
+// Four components of a centre per lane of a warp: the fp64 centre, its 16-bit split and its bound constant.
 template <bool kHalf>
-__global__ void __launch_bounds__(128)
-km_batch_assign_kernel(KmeansParams p, int t)
+__device__ __forceinline__ void store_centre(const KmeansParams &p, size_t centre, const double (&v)[4])
 {
-    __shared__ __align__(16) double c[kTile][kHeadDim];
-    const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
-    if (!pair_active(p, q, t)) return;
-    const int tid = threadIdx.x;
-    int s[kAssignPts], idx[kAssignPts];
-    const uint4 *row[kAssignPts];
-    double best[kAssignPts];
-    int arg[kAssignPts];
+    const int lane = threadIdx.x & 31;
+    uint16_t hi[4], mid[4];
+    float n = 0.f;
 #pragma unroll
-    for (int j = 0; j < kAssignPts; ++j) {
-        s[j] = blockIdx.x * kAssignBlock + j * 128 + tid;
-        idx[j] = km_index(km_word(p, (uint32_t)(s[j] < p.batch ? s[j] : 0), kTagBatch, q.stream, (uint32_t)t), q.N);
-        row[j] = reinterpret_cast<const uint4 *>(p.k_prompt + (q.plane + (size_t)idx[j]) * kHeadDim);
-        best[j] = INFINITY;
-        arg[j] = 0;
+    for (int e = 0; e < 4; ++e) {
+        split_component<kHalf>(v[e], hi[e], mid[e]);
+        n = fmaf((float)v[e], (float)v[e], n);
     }
-    const double *cen = p.centres64 + q.cplane * kHeadDim;
-    // this block searches one slice of the centres (a multiple of kTile each); the slices' results are
-    // compared in slice order afterwards, so ties still go to the smaller centre index
-    const int slice = blockIdx.z;
-    const int per = ((q.k + p.assign_split - 1) / p.assign_split + kTile - 1) / kTile * kTile;
+    n = warp_sum(n);
+    const float bias = centre_bias<kHalf>(n);
+    const bool fits = bias > -CUDART_INF_F;
+    double2 *to = reinterpret_cast<double2 *>(p.centres64 + centre * kHeadDim + 4 * lane);
+    to[0] = make_double2(v[0], v[1]);
+    to[1] = make_double2(v[2], v[3]);
+    auto pack = [&](const uint16_t (&h)[4]) {
+        return fits ? make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16)) : make_uint2(0u, 0u);
+    };
+    reinterpret_cast<uint2 *>(p.centre_hi + centre * kHeadDim)[lane] = pack(hi);
+    reinterpret_cast<uint2 *>(p.centre_mid + centre * kHeadDim)[lane] = pack(mid);
+    if (lane == 0) p.centre_bias[centre] = bias;
+}
+
+// The centres as the start left them, their counts and the fits' state at zero. A warp per centre.
+template <bool kHalf>
+__global__ void __launch_bounds__(kThreads)
+km_prepare_kernel(KmeansParams p)
+{
+    step_wait();
+    const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
+    const int u = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0, 0, 0, 0};
+    if (u >= q.k) return;
+    const double2 *from = reinterpret_cast<const double2 *>(p.centres64 + (q.cplane + u) * kHeadDim + 4 * lane);
+    const double2 v0 = from[0], v1 = from[1];
+    const double v[4] = {v0.x, v0.y, v1.x, v1.y};
+    store_centre<kHalf>(p, q.cplane + u, v);
+    if (lane == 0) p.count[q.cplane + u] = 0.0;
+}
+
+// Averaged inertia of step t and the stopping rule, one block per pair. The sum of the minibatch distances in
+// order runs on one thread over shared memory that all threads filled.
+__device__ __forceinline__ void km_stop_rule(const KmeansParams &p, const Pair &q, int t, double *dist_s)
+{
+    if (t < 0 || !pair_active(p, q, t)) return;
+    const double *dist = p.dist + (size_t)q.id * p.batch;
+    for (int s = threadIdx.x; s < p.batch; s += blockDim.x) dist_s[s] = dist[s];
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double inertia = 0.0;
+#pragma unroll 16
+    for (int s = 0; s < p.batch; ++s) inertia = __dadd_rn(inertia, dist_s[s]);
+    KmeansState &st = p.state[q.id];
+    double alpha = __ddiv_rn(__dmul_rn(2.0, (double)p.batch), __dadd_rn((double)q.N, 1.0));
+    if (alpha > 1.0) alpha = 1.0;
+    const double per_point = __ddiv_rn(inertia, (double)p.batch);
+    const double ewa = t == 0 ? per_point
+                              : __dadd_rn(__dmul_rn(st.ewa, __dsub_rn(1.0, alpha)), __dmul_rn(per_point, alpha));
+    st.ewa = ewa;
+    st.steps += 1;
+    if (t == 0 || ewa < st.ewa_min) { st.ewa_min = ewa; st.bad = 0; }
+    else if (++st.bad >= p.patience) st.stopped = 1;
+}
+
+__global__ void __launch_bounds__(kThreads)
+km_last_stop_rule_kernel(KmeansParams p, int t)
+{
+    __shared__ double dist_s[4096];
+    step_wait();
+    km_stop_rule(p, pair_of(p, blockIdx.x / p.n_kv, blockIdx.x % p.n_kv), t, dist_s);
+}
+
+// Draw the minibatch and scan the centres for each point's nearest: block (256 points, pair, slice of the
+// centres). Blocks of slice `assign_split` take the stopping rule of the step before instead.
+template <bool kHalf>
+__global__ void __launch_bounds__(kNearThreads, 2)
+km_scan_kernel(KmeansParams p, int t)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    NearSmem &sm = *reinterpret_cast<NearSmem *>(smem_raw);
+    __shared__ int idx_s[kNearPoints];
+    step_wait();
+    const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
+    const int slice = blockIdx.z, tid = threadIdx.x;
+    if (slice == p.assign_split) {
+        if (blockIdx.x == 0) km_stop_rule(p, q, t - 1, reinterpret_cast<double *>(smem_raw));
+        return;
+    }
+    if (!pair_active(p, q, t)) return;                      // (a fit that is being stopped now may still be scanned)
+    const int per = ((q.k + p.assign_split - 1) / p.assign_split + kNearTile - 1) / kNearTile * kNearTile;
     const int k_lo = min(slice * per, q.k), k_hi = min(k_lo + per, q.k);
-    for (int base = k_lo; base < k_hi; base += kTile) {
-        const int nt = min(kTile, k_hi - base);
-        __syncthreads();
-        for (int e = tid; e < nt * kHeadDim; e += 128) c[e >> 7][e & 127] = cen[(size_t)base * kHeadDim + e];
-        __syncthreads();
-        for (int u = 0; u < nt; u += kAssignGroup) {
-            // (rows of the tile past nt hold older values; their sums are not looked at)
-            double d[kAssignPts][kAssignGroup];
+    const int s = blockIdx.x * kNearPoints + tid;
+    idx_s[tid] = km_index(km_word(p, (uint32_t)(s < p.batch ? s : 0), kTagBatch, q.stream, (uint32_t)t), q.N);
+    if (slice == 0 && s < p.batch) p.idx[(size_t)q.id * p.batch + s] = idx_s[tid];
+    __syncwarp();
+    const uint16_t *keys = p.k_prompt + q.plane * kHeadDim;
+    uint32_t a[2][8][4];
+    near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)idx_s[i] * kHeadDim; }, a);
+    const uint4 *hi = reinterpret_cast<const uint4 *>(p.centre_hi + q.cplane * kHeadDim);
+    const uint4 *mid = reinterpret_cast<const uint4 *>(p.centre_mid + q.cplane * kHeadDim);
+    const float *bias = p.centre_bias + q.cplane;
+    near_scan<kHalf>(sm, a, k_lo, k_hi, [&](int stage, int base, int n) {
 #pragma unroll
-            for (int j = 0; j < kAssignPts; ++j)
-#pragma unroll
-                for (int v = 0; v < kAssignGroup; ++v) d[j][v] = 0.0;
-            dist_points<kHalf, kAssignPts, kAssignGroup, kAssignGroup>(row, c + u, d);
-#pragma unroll
-            for (int j = 0; j < kAssignPts; ++j)
-#pragma unroll
-                for (int v = 0; v < kAssignGroup; ++v)
-                    if (u + v < nt && d[j][v] < best[j]) { best[j] = d[j][v]; arg[j] = base + u + v; }
+        for (int m = 0; m < kNearTile * 16 / kNearThreads; ++m) {
+            const int e = m * kNearThreads + tid, row = e >> 4, ch = e & 15;
+            if (row < n) {
+                copy16_async(shared_addr(&sm.ring[stage][0][near_piece(row, ch)]), hi + (size_t)base * 16 + e);
+                copy16_async(shared_addr(&sm.ring[stage][1][near_piece(row, ch)]), mid + (size_t)base * 16 + e);
+            }
         }
-    }
-#pragma unroll
-    for (int j = 0; j < kAssignPts; ++j) {
-        if (s[j] >= p.batch) continue;
-        const size_t at = (size_t)q.id * p.batch + s[j];
-        if (slice == 0) p.idx[at] = idx[j];
-        if (p.assign_split == 1) {
-            p.label[at] = arg[j];
-            p.dist[at] = best[j];
-        } else {
-            const size_t pa = ((size_t)q.id * p.assign_split + slice) * p.batch + s[j];
-            p.label_part[pa] = arg[j];
-            p.dist_part[pa] = best[j];
-        }
+        if (tid < kNearTile) sm.bias[stage][tid] = tid < n ? bias[base + tid] : CUDART_INF_F;
+    });
+    if (s < p.batch) {
+        p.near_top[((size_t)q.id * p.assign_split + slice) * p.batch + s] = sm.top[tid];
+        if (slice == 0) p.near_nx[(size_t)q.id * p.batch + s] = sm.nx[tid];
     }
 }
 
-// The nearest centre of each minibatch point over all slices (strictly smaller distance wins, slices in
-// order of the centre index).
-__global__ void __launch_bounds__(128)
-km_assign_reduce_kernel(KmeansParams p, int t)
+// The nearest centre of each minibatch point and the fp64 distance to it: the slices' results merged, the
+// candidates that the bounds leave open compared in fp64. A thread per point.
+constexpr int kResolveThreads = 64;
+template <bool kHalf>
+__global__ void __launch_bounds__(kResolveThreads)
+km_resolve_kernel(KmeansParams p, int t)
 {
+    step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     if (!pair_active(p, q, t)) return;
-    const int s = blockIdx.x * 128 + threadIdx.x;
-    if (s >= p.batch) return;
-    double best = INFINITY;
-    int arg = 0;
-    for (int slice = 0; slice < p.assign_split; ++slice) {
-        const size_t pa = ((size_t)q.id * p.assign_split + slice) * p.batch + s;
-        const double d = p.dist_part[pa];
-        if (d < best) { best = d; arg = p.label_part[pa]; }
+    const int s = blockIdx.x * kResolveThreads + threadIdx.x, lane = threadIdx.x & 31;
+    const bool live = s < p.batch;
+    const size_t at = (size_t)q.id * p.batch + (live ? s : 0);
+    const uint4 *x = reinterpret_cast<const uint4 *>(p.k_prompt + (q.plane + (size_t)p.idx[at]) * kHeadDim);
+    const double *cen = p.centres64 + q.cplane * kHeadDim;
+    NearTop top = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, 0, 0};
+    for (int slice = 0; slice < p.assign_split; ++slice)
+        near_merge(top, p.near_top[((size_t)q.id * p.assign_split + slice) * p.batch + (live ? s : 0)]);
+    const float nx = p.near_nx[at];
+    bool all = !(nx <= 1e37f) || !(fabsf(top.t1) < CUDART_INF_F);
+    int arg = top.i1;
+    double best = CUDART_INF;
+    if (!all) {
+        const float bar = top.t1 + near_slack<kHalf>(nx, p.centre_bias[q.cplane + top.i1] * (1.f + 2.f * kNearErr));
+        all = !(top.t3 > bar);
+        if (!all) {
+            best = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim);
+            if (!(top.t2 > bar)) {
+                const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
+                if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
+            }
+        }
     }
-    const size_t at = (size_t)q.id * p.batch + s;
-    p.label[at] = arg;
-    p.dist[at] = best;
+    for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
+        const int l = __ffs(left) - 1;
+        const uint4 *xl = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)x, l));
+        double d;
+        const int u = near_scan_exact<kHalf>(xl, cen, q.k, d);
+        if (lane == l) { best = d; arg = u; }
+    }
+    if (live) {
+        p.label[at] = arg;
+        p.dist[at] = best;
+    }
 }
 
-// The minibatch's slots ordered by (label, slot), one block per pair: a bitonic sort of the keys
-// label << 12 | slot in shared memory (batch <= 4096; the keys are distinct, so the order is the
-// minibatch order inside every label).
-constexpr int kSortThreads = 1024, kSortKeys = 4096;
+// The minibatch ordered by (label, slot), one block per pair: two stable counting passes over the label's digits
+// (kSortBits each), then where each label starts. A thread holds four consecutive entries; ranks of equal
+// digits come from the warp (in order) and from counts of the warps before. (A bitonic sort of the same
+// keys took 24 us.)
+constexpr int kSortThreads = 1024, kSortKeys = 4096, kSortBits = 7, kSortDigits = 1 << kSortBits, kSortWarps = kSortThreads / 32;
+struct SortSmem {
+    uint32_t key[2][kSortKeys];                             // label << 12 | slot
+    uint16_t count[kSortDigits][kSortWarps + 1];
+    int scan[33];
+};
 __global__ void __launch_bounds__(kSortThreads)
 km_sort_batch_kernel(KmeansParams p, int t)
 {
-    __shared__ uint32_t key_s[kSortKeys];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
+    step_wait();
     const Pair q = pair_of(p, blockIdx.x / p.n_kv, blockIdx.x % p.n_kv);
     if (!pair_active(p, q, t)) return;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int s = tid; s < kSortKeys; s += kSortThreads)
-        key_s[s] = s < p.batch ? ((uint32_t)p.label[(size_t)q.id * p.batch + s] << 12) | (uint32_t)s : 0xFFFFFFFFu;
-    __syncthreads();
-    for (int size = 2; size <= kSortKeys; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int e = tid; e < kSortKeys / 2; e += kSortThreads) {
-                const int lo = 2 * e - (e & (stride - 1)), hi = lo + stride;       // partners of this compare-exchange
-                const bool up = (lo & size) == 0;
-                const uint32_t a = key_s[lo], b = key_s[hi];
-                if ((a > b) == up) { key_s[lo] = b; key_s[hi] = a; }
-            }
-            __syncthreads();
+        sm.key[0][s] = s < p.batch ? ((uint32_t)p.label[(size_t)q.id * p.batch + s] << 12) | (uint32_t)s : 0xFFFFFFFFu;
+    for (int pass = 0; pass < 2; ++pass) {
+        const int shift = 12 + pass * kSortBits;
+        for (int e = tid; e < kSortDigits * (kSortWarps + 1); e += kSortThreads) (&sm.count[0][0])[e] = 0;
+        __syncthreads();
+        uint32_t key[4];
+        int digit[4], rank[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {                       // the warp's 128 entries, 32 at a time in order
+            key[c] = sm.key[pass][warp * 128 + c * 32 + lane];
+            digit[c] = (int)((key[c] >> shift) & (kSortDigits - 1));
+            const unsigned same = __match_any_sync(0xFFFFFFFFu, digit[c]);
+            const int before = sm.count[digit[c]][warp];
+            rank[c] = before + __popc(same & ((1u << lane) - 1u));
+            __syncwarp();
+            if ((same & ((1u << lane) - 1u)) == 0u) sm.count[digit[c]][warp] = (uint16_t)(before + __popc(same));
+            __syncwarp();
         }
+        __syncthreads();
+        // exclusive prefix over (digit, warp): thread = digit * 8 + part of four warps
+        {
+            const int d = tid >> 3, w0 = (tid & 7) * 4;
+            int n[4], sum = 0, total;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) { n[w] = sm.count[d][w0 + w]; sum += n[w]; }
+            int at = block_exclusive_scan(sum, sm.scan, total);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) { sm.count[d][w0 + w] = (uint16_t)at; at += n[w]; }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sm.key[pass ^ 1][sm.count[digit[c]][warp] + rank[c]] = key[c];
+        __syncthreads();
     }
-    for (int s = tid; s < kSortKeys; s += kSortThreads) p.sorted[(size_t)q.id * kSortKeys + s] = key_s[s];
+    const int32_t *idx = p.idx + (size_t)q.id * p.batch;
+    int32_t *start = p.start + (size_t)q.id * (p.k_max + 1);
+    for (int s = tid; s < kSortKeys; s += kSortThreads) {
+        const uint32_t key = sm.key[0][s];
+        const int label = min((int)(key >> 12), q.k);       // (the padding sorts behind every label)
+        const int prev = s > 0 ? min((int)(sm.key[0][s - 1] >> 12), q.k) : -1;
+        for (int u = prev + 1; u <= label; ++u) start[u] = s;
+        if (s == kSortKeys - 1)
+            for (int u = label + 1; u <= q.k; ++u) start[u] = kSortKeys;
+        if (s < p.batch) p.sorted[(size_t)q.id * kSortKeys + s] = idx[key & 4095u];
+    }
 }
 
-// Cumulative-count update: thread (centre, dimension) adds the centre's new points in minibatch
-// order (it finds them in the sorted slots); c <- (c * count + sum) / (count + n).
+// Cumulative-count update, a warp per centre (four dimensions per lane): the centre's new points are added in
+// minibatch order, eight rows requested at a time; c <- (c * count + sum) / (count + n).
 template <bool kHalf>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(128)
 km_batch_update_kernel(KmeansParams p, int t)
 {
+    step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     if (!pair_active(p, q, t)) return;
-    const int u = blockIdx.x * (kThreads / kHeadDim) + threadIdx.x / kHeadDim, d = threadIdx.x % kHeadDim;
-    const bool live = u < q.k;
-    double sum = 0.0, count = 0.0;
-    int n = 0;
-    if (live) {
-        const uint32_t *sorted = p.sorted + (size_t)q.id * kSortKeys;
-        int lo = 0, hi = kSortKeys;                         // first position with label >= u
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if ((sorted[mid] >> 12) >= (uint32_t)u) hi = mid; else lo = mid + 1;
+    const int u = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (u >= q.k) return;
+    const int32_t *start = p.start + (size_t)q.id * (p.k_max + 1);
+    const int lo = start[u], hi = start[u + 1];
+    if (lo == hi) return;
+    const int32_t *point = p.sorted + (size_t)q.id * kSortKeys;
+    const uint2 *keys = reinterpret_cast<const uint2 *>(p.k_prompt + q.plane * kHeadDim) + lane;
+    const double count = p.count[q.cplane + u];
+    const double2 *from = reinterpret_cast<const double2 *>(p.centres64 + (q.cplane + u) * kHeadDim + 4 * lane);
+    const double2 c0 = from[0], c1 = from[1];
+    double sum[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i0 = lo; i0 < hi; i0 += 8) {
+        uint2 w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = __ldg(keys + (size_t)point[min(i0 + i, hi - 1)] * 32);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (i0 + i >= hi) break;
+            sum[0] = __dadd_rn(sum[0], (double)elem_lo<kHalf>(w[i].x));
+            sum[1] = __dadd_rn(sum[1], (double)elem_hi<kHalf>(w[i].x));
+            sum[2] = __dadd_rn(sum[2], (double)elem_lo<kHalf>(w[i].y));
+            sum[3] = __dadd_rn(sum[3], (double)elem_hi<kHalf>(w[i].y));
         }
-        count = p.count[q.cplane + u];
-        const uint16_t *col = p.k_prompt + q.plane * kHeadDim + d;
-        const int32_t *idx = p.idx + (size_t)q.id * p.batch;
-        for (int at = lo; at < kSortKeys && (sorted[at] >> 12) == (uint32_t)u; ++at, ++n)
-            sum = __dadd_rn(sum, elem_to_double<kHalf>(col[(size_t)idx[sorted[at] & 4095u] * kHeadDim]));
     }
-    __syncthreads();                                        // every thread has read its centre's count
-    if (live && n > 0) {
-        const double grown = __dadd_rn(count, (double)n);
-        double *cd = p.centres64 + (q.cplane + (size_t)u) * kHeadDim + d;
-        *cd = __ddiv_rn(__dadd_rn(__dmul_rn(*cd, count), sum), grown);
-        if (d == 0) p.count[q.cplane + u] = grown;
-    }
+    const double grown = __dadd_rn(count, (double)(hi - lo)), c[4] = {c0.x, c0.y, c1.x, c1.y};
+    double v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = __ddiv_rn(__dadd_rn(__dmul_rn(c[e], count), sum[e]), grown);
+    store_centre<kHalf>(p, q.cplane + u, v);
+    if (lane == 0) p.count[q.cplane + u] = grown;
 }
 
-// One block per pair: reassignment of starved centres, averaged inertia, stopping rule. The serial
-// parts (the inertia is the sum of the minibatch distances in order) run on one thread over shared
-// memory that all threads filled.
+// Reassignment of starved centres, one block per pair.
 template <bool kHalf>
 __global__ void __launch_bounds__(kThreads)
-km_control_kernel(KmeansParams p, int t)
+km_reassign_kernel(KmeansParams p, int t)
 {
-    extern __shared__ double ctl_dist[];                    // dist[batch], then int32 slots[batch], move_centre[batch / 2]
+    extern __shared__ int32_t slots[];                      // slots[batch], then move_centre[batch / 2]
     __shared__ int n_move_s;
     __shared__ double cmin_s[kThreads / 32], cmax_s[kThreads / 32];
+    step_wait();
     const Pair q = pair_of(p, blockIdx.x, blockIdx.y);
-    if (!pair_active(p, q, t)) return;
+    if (!(p.ratio > 0.0) || !pair_active(p, q, t)) return;
     const int tid = threadIdx.x;
-    int32_t *slots = reinterpret_cast<int32_t *>(ctl_dist + p.batch), *move_centre = slots + p.batch;
+    int32_t *move_centre = slots + p.batch;
     double *count = p.count + q.cplane;
-    const int32_t *idx = p.idx + (size_t)q.id * p.batch;
     {
-        const double *dist = p.dist + (size_t)q.id * p.batch;
-        for (int s = tid; s < p.batch; s += kThreads) ctl_dist[s] = dist[s];
         double cmin = INFINITY, cmax = 0.0;                 // smallest and largest count: any order gives the same
         for (int u = tid; u < q.k; u += kThreads) {
             const double v = count[u];
@@ -545,7 +645,7 @@ km_control_kernel(KmeansParams p, int t)
             if (cmax_s[w] > cmax) cmax = cmax_s[w];
         }
         const long long period = 10 + (long long)floor(cmin);
-        if (p.ratio > 0.0 && ((long long)t + 1) % period == 0) {
+        if (((long long)t + 1) % period == 0) {
             const double thr = __dmul_rn(p.ratio, cmax);
             const int cap = p.batch / 2;
             double keep_min = INFINITY;
@@ -568,26 +668,11 @@ km_control_kernel(KmeansParams p, int t)
         n_move_s = n_move;
     }
     __syncthreads();
-    const int n_move = n_move_s;
-    for (int e = tid; e < n_move * kHeadDim; e += kThreads) {   // the moved centres jump onto minibatch points
-        const int i = e >> 7, d = e & (kHeadDim - 1);
-        const uint16_t *src = p.k_prompt + (q.plane + (size_t)idx[slots[i]]) * kHeadDim;
-        p.centres64[(q.cplane + (size_t)move_centre[i]) * kHeadDim + d] = elem_to_double<kHalf>(src[d]);
-    }
-    if (tid == 0) {
-        double inertia = 0.0;
-#pragma unroll 8
-        for (int s = 0; s < p.batch; ++s) inertia = __dadd_rn(inertia, ctl_dist[s]);
-        KmeansState &st = p.state[q.id];
-        double alpha = __ddiv_rn(__dmul_rn(2.0, (double)p.batch), __dadd_rn((double)q.N, 1.0));
-        if (alpha > 1.0) alpha = 1.0;
-        const double per_point = __ddiv_rn(inertia, (double)p.batch);
-        const double ewa = t == 0 ? per_point
-                                  : __dadd_rn(__dmul_rn(st.ewa, __dsub_rn(1.0, alpha)), __dmul_rn(per_point, alpha));
-        st.ewa = ewa;
-        st.steps += 1;
-        if (t == 0 || ewa < st.ewa_min) { st.ewa_min = ewa; st.bad = 0; }
-        else if (++st.bad >= p.patience) st.stopped = 1;
+    const int32_t *idx = p.idx + (size_t)q.id * p.batch;
+    for (int i = tid >> 5; i < n_move_s; i += kThreads / 32) {   // the moved centres jump onto minibatch points
+        const uint2 w = reinterpret_cast<const uint2 *>(p.k_prompt + (q.plane + (size_t)idx[slots[i]]) * kHeadDim)[tid & 31];
+        const double v[4] = {(double)elem_lo<kHalf>(w.x), (double)elem_hi<kHalf>(w.x), (double)elem_lo<kHalf>(w.y), (double)elem_hi<kHalf>(w.y)};
+        store_centre<kHalf>(p, q.cplane + move_centre[i], v);
     }
 }
 
@@ -625,15 +710,9 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
     const int B = p.n_seqs, H = p.n_kv, pairs = B * H;
     cudaError_t err;
 #define KM_CHECK() if ((err = cudaGetLastError()) != cudaSuccess) return err
-    const int sample_smem_rows = std::min(p.max_rows_per_seq, kSampleSmemRows);
-    if (p.max_rows_per_seq > sample_smem_rows) {              // some sequence shuffles its index list in global memory
-        km_perm_identity_kernel<<<dim3((p.max_rows_per_seq + kThreads - 1) / kThreads, B, H), kThreads, 0, s>>>(p);
-        KM_CHECK();
-    }
-    if ((err = cudaFuncSetAttribute(km_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(int32_t) * kSampleSmemRows)) != cudaSuccess) return err;
-    km_sample_kernel<<<dim3(B, H), kThreads, sizeof(int32_t) * (size_t)sample_smem_rows, s>>>(p, sample_smem_rows);
-    KM_CHECK();
+    static std::atomic<unsigned long long> sample_done;
+    if ((err = ensure_dynamic_smem((const void *)km_sample_kernel, (int)sample_smem(kMaxSumBlocks * kSumBlock), sample_done)) != cudaSuccess) return err;
+    if ((err = launch_step(km_sample_kernel, dim3(B, H), dim3(kSampleThreads), sample_smem(p.n_init_max), s, p)) != cudaSuccess) return err;
     const dim3 dist_grid((p.n_init_max + kSumBlock - 1) / kSumBlock, (p.trials_max + kDistTrials - 1) / kDistTrials, pairs);
     const size_t draw_smem = sizeof(double) * ((size_t)p.n_init_max + 2 * kMaxSumBlocks);
     if ((err = cudaFuncSetAttribute(km_accept_kernel<kHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)draw_smem)) != cudaSuccess)
@@ -644,24 +723,21 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
         km_accept_kernel<kHalf><<<dim3(B, H), kAcceptThreads, draw_smem, s>>>(p, c);     // ... and the trial points of centre c + 1
         KM_CHECK();
     }
-    if ((err = cudaMemsetAsync(p.count, 0, sizeof(double) * (size_t)H * p.centres_total, s)) != cudaSuccess) return err;
-    if ((err = cudaMemsetAsync(p.state, 0, sizeof(KmeansState) * (size_t)pairs, s)) != cudaSuccess) return err;
-    const size_t control_smem = sizeof(double) * (size_t)p.batch + sizeof(int32_t) * ((size_t)p.batch + (size_t)p.batch / 2 + 1);
-    if ((err = cudaFuncSetAttribute(km_control_kernel<kHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)control_smem)) != cudaSuccess)
-        return err;
-    for (int t = 0; t < p.t_max_max; ++t) {
-        km_batch_assign_kernel<kHalf><<<dim3((p.batch + kAssignBlock - 1) / kAssignBlock, pairs, p.assign_split), 128, 0, s>>>(p, t);
-        KM_CHECK();
-        if (p.assign_split > 1) {
-            km_assign_reduce_kernel<<<dim3((p.batch + 127) / 128, pairs), 128, 0, s>>>(p, t);
-            KM_CHECK();
-        }
-        km_sort_batch_kernel<<<dim3(pairs), kSortThreads, 0, s>>>(p, t);
-        KM_CHECK();
-        km_batch_update_kernel<kHalf><<<dim3((p.k_max + 1) / 2, pairs), kThreads, 0, s>>>(p, t);
-        KM_CHECK();
-        km_control_kernel<kHalf><<<dim3(B, H), kThreads, control_smem, s>>>(p, t);
-        KM_CHECK();
+    const dim3 threads(kThreads);
+    if ((err = launch_step(km_prepare_kernel<kHalf>, dim3((p.k_max + kThreads / 32 - 1) / (kThreads / 32), pairs), threads, 0, s, p)) != cudaSuccess) return err;
+    static std::atomic<unsigned long long> scan_done, sort_done;
+    if ((err = ensure_dynamic_smem((const void *)km_scan_kernel<kHalf>, (int)sizeof(NearSmem), scan_done)) != cudaSuccess) return err;
+    if ((err = ensure_dynamic_smem((const void *)km_sort_batch_kernel, (int)sizeof(SortSmem), sort_done)) != cudaSuccess) return err;
+    const size_t move_smem = sizeof(int32_t) * ((size_t)p.batch + (size_t)p.batch / 2 + 1);
+    const dim3 scan_grid((p.batch + kNearPoints - 1) / kNearPoints, pairs, p.assign_split + 1);
+    const dim3 resolve_grid((p.batch + kResolveThreads - 1) / kResolveThreads, pairs);
+    int t = 0;
+    for (; t < p.t_max_max; ++t) {
+        if ((err = launch_step(km_scan_kernel<kHalf>, scan_grid, dim3(kNearThreads), sizeof(NearSmem), s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_resolve_kernel<kHalf>, resolve_grid, dim3(kResolveThreads), 0, s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_sort_batch_kernel, dim3(pairs), dim3(kSortThreads), sizeof(SortSmem), s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_batch_update_kernel<kHalf>, dim3((p.k_max + 3) / 4, pairs), dim3(128), 0, s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_reassign_kernel<kHalf>, dim3(B, H), threads, move_smem, s, p, t)) != cudaSuccess) return err;
         if (!p.no_host_poll && (t + 1) % kPollEvery == 0 && t + 1 < p.t_max_max) {
             // most fits stop long before the step limit: ask the device how many are still running
             // (the copy into pageable memory returns when it has completed)
@@ -670,9 +746,10 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
             KM_CHECK();
             if ((err = cudaMemcpyAsync(&active, p.active, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return err;
             if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return err;
-            if (active == 0) break;
+            if (active == 0) { ++t; break; }
         }
     }
+    if ((err = launch_step(km_last_stop_rule_kernel, dim3(pairs), threads, 0, s, p, t - 1)) != cudaSuccess) return err;   // counts the last step
     km_finish_kernel<<<dim3((p.k_max * kHeadDim + kThreads - 1) / kThreads, B, H), kThreads, 0, s>>>(p);
     KM_CHECK();
 #undef KM_CHECK

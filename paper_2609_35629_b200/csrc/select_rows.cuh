@@ -86,6 +86,12 @@ __device__ __forceinline__ int warp_arg(double v, int i, bool in)
     }
     return i;
 }
+__device__ __forceinline__ float warp_sum(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
 __device__ __forceinline__ float warp_max(float v)
 {
 #pragma unroll
