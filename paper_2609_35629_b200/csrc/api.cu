@@ -500,7 +500,7 @@ namespace {
 constexpr int kKmeansMaxSample = 28544;     // 223 KB of fp64 running sums (plus their block offsets): up to 9514 centres per sequence
 
 struct KmeansLayout {
-    size_t row_off, cen_off, tabs, perm, closest, cand, part, pick, centres64, count, idx, label, dist, centre_hi, centre_mid, centre_bias, near_top, near_nx, sorted, start, state, active, total;
+    size_t row_off, cen_off, tabs, perm, closest, cand, part, pick, chosen, centres64, count, idx, label, dist, centre_hi, centre_mid, centre_bias, near_top, near_nx, sorted, start, state, active, total;
     int k_max, n_init_max, trials_max, t_max_max, max_rows, assign_split;
     int64_t rows_total, centres_total;
 };
@@ -549,6 +549,7 @@ int kmeans_layout(const santapp_geom *geom, const int32_t *prompt_len_host, cons
     L->cand = take(sizeof(double) * pairs * (size_t)L->trials_max * (size_t)L->n_init_max);
     L->part = take(sizeof(double) * pairs * (size_t)L->trials_max * (((size_t)L->n_init_max + 127) / 128));
     L->pick = take(sizeof(int32_t) * pairs * (size_t)L->trials_max);
+    L->chosen = take(sizeof(int32_t) * H * (size_t)L->centres_total);
     L->centres64 = take(sizeof(double) * H * (size_t)L->centres_total * kHeadDim);
     L->count = take(sizeof(double) * H * (size_t)L->centres_total);
     L->idx = take(sizeof(int32_t) * pairs * (size_t)o->batch_size);
@@ -661,6 +662,7 @@ int santapp_kmeans_fit(const santapp_geom *geom, const int32_t *prompt_len_host,
     p.cand = reinterpret_cast<double *>(ws + L.cand);
     p.part = reinterpret_cast<double *>(ws + L.part);
     p.pick = reinterpret_cast<int32_t *>(ws + L.pick);
+    p.chosen = reinterpret_cast<int32_t *>(ws + L.chosen);
     p.centres64 = reinterpret_cast<double *>(ws + L.centres64);
     p.count = reinterpret_cast<double *>(ws + L.count);
     p.idx = reinterpret_cast<int32_t *>(ws + L.idx);

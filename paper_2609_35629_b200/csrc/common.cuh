@@ -330,6 +330,7 @@ struct KmeansParams {
     double *cand;                           // [pairs][trials_max][n_init_max]
     double *part;                           // [pairs][trials_max][ceil(n_init_max / 128)] block sums of the trials' potentials
     int32_t *pick;                          // [pairs][trials_max]
+    int32_t *chosen;                        // [n_kv][centres_total] sample index of each centre of the start
     double *centres64;                      // [n_kv][centres_total][128]
     double *count;                          // [n_kv][centres_total]
     int32_t *idx, *label;                   // [pairs][batch]

@@ -244,12 +244,7 @@ km_accept_kernel(KmeansParams p, int c)
     __syncthreads();
     const int best = best_s;
     const double *win = cand + (size_t)best * p.n_init_max;
-    if (tid < kHeadDim) {
-        const int32_t *perm = p.perm + q.plane;
-        const int at = p.pick[(size_t)q.id * p.trials_max + best];
-        const uint16_t v = p.k_prompt[(q.plane + (size_t)perm[at]) * kHeadDim + tid];
-        p.centres64[(q.cplane + (size_t)c) * kHeadDim + tid] = elem_to_double<kHalf>(v);
-    }
+    if (tid == 0) p.chosen[q.cplane + (size_t)c] = p.pick[(size_t)q.id * p.trials_max + best];
     // The nearest-centre distances are lowered and kept in shared memory for the draw of the next
     // centre's trial points (inverse CDF over the sample in order). cum_s holds one pad word per
     // block of the sums (point i at i + i / kSumBlock), so that threads that walk different blocks do
@@ -321,6 +316,509 @@ km_accept_kernel(KmeansParams p, int c)
     }
 }
 
+// The greedy start as one kernel: a cluster of blocks per pair that keeps the sample in shared memory (for samples
+// of at most kStartRows rows per block; the two kernels per centre above take larger ones).
+//
+// Only the winning trial's distances are needed in fp64. A trial lowers the potential by the sum over the points
+// of what it takes off their nearest-centre distance, and the products of the rows with the trial points give every
+// such gain within a bound (select_rows.cuh). Per centre the cluster's blocks
+//   1. multiply their rows with the trial points on tensor cores, mark the points that a trial may lower, add up
+//      each trial's largest and smallest possible gain, and exchange the sums (distributed shared memory);
+//   2. take the trial whose smallest gain exceeds every other's largest; if there is none, the potentials are
+//      summed in fp64 for all trials (about one centre in a hundred; trials that drew the same point do not count);
+//   3. evaluate the winner's marked points in fp64 (a handful, after the first hundred centres), lower the
+//      distances, renew the running sums of the blocks of the sums they lie in, and exchange those blocks' sums;
+//   4. add up the blocks and draw the next trial points: the block that owns a drawn point sends its row to all.
+// Left are three cluster barriers a centre and the serial sums (128 terms of a distance, of a block, the blocks;
+// 8 cycles a term). The two kernels per centre took 38 us, 24 of them fp64 distances of every point to every trial.
+constexpr int kStartThreads = 256, kStartWarps = kStartThreads / 32;
+constexpr int kStartBlocks = 6;          // blocks of the sums per thread block: 768 rows of 256 bytes
+constexpr int kStartRows = kStartBlocks * kSumBlock;
+constexpr int kStartTrials = 10;         // 2 + floor(ln k) for every k with a sample of at most 16 * kStartRows
+constexpr int kStartMaxCluster = 16, kStartSums = kStartBlocks * kStartMaxCluster;
+
+struct StartSmem {
+    uint4 rows[kStartRows * 16];                            // 16-byte pieces XOR-swizzled (near_piece)
+    uint4 trial[kStartTrials * 16];
+    double closest[kStartRows];
+    double run[kStartRows];                                 // running sums of the distances inside each block of the sums
+    double tmp[kStartWarps][kSumBlock];
+    double raw[kStartSums];                                 // sums of all the pair's blocks
+    double pre[kStartSums];                                 // ... and their running sums
+    float norm[kStartRows];                                 // squared norms
+    float bar[kStartRows];                                  // norm * (1 - error) - nearest-centre distance
+    float2 gain[kStartMaxCluster][kStartTrials];            // (smallest, largest) gain of a trial over each block's points
+    float2 warp_gain[kStartWarps][kStartTrials];
+    float trial_norm[kStartTrials];
+    int pick[2][kStartTrials];                              // sample indices of the trial points
+    uint32_t touched[kStartBlocks];                         // trials with a marked point in the block
+    int best;
+    uint16_t mask[kStartRows];                              // trials that may lower the point's distance
+};
+static_assert(sizeof(StartSmem) <= 227 * 1024, "shared memory of one block");
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t in_block(uint32_t addr, uint32_t rank)      // the same shared-memory address in another block
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Every thread of the cluster. Not the .aligned forms: lanes may arrive one by one after a divergent branch (a lane that
+// still runs a serial sum while its warp arrives counted the warp twice).
+__device__ __forceinline__ void cluster_barrier()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    __syncwarp();
+}
+
+// Four of a row's values (dimensions 4 * lane ..) as doubles.
+template <bool kHalf>
+__device__ __forceinline__ void row_quad(const uint4 *rows, int i, double (&v)[4])
+{
+    const int lane = threadIdx.x & 31;
+    const uint2 w = reinterpret_cast<const uint2 *>(rows + near_piece(i, lane >> 1))[lane & 1];
+    v[0] = (double)elem_lo<kHalf>(w.x);
+    v[1] = (double)elem_hi<kHalf>(w.x);
+    v[2] = (double)elem_lo<kHalf>(w.y);
+    v[3] = (double)elem_hi<kHalf>(w.y);
+}
+// Squared norm of a row by a warp (an fp32 sum; every lane gets it).
+template <bool kHalf>
+__device__ __forceinline__ float row_norm(const uint4 *rows, int i)
+{
+    const int lane = threadIdx.x & 31;
+    const uint2 w = reinterpret_cast<const uint2 *>(rows + near_piece(i, lane >> 1))[lane & 1];
+    const float a = elem_lo<kHalf>(w.x), b = elem_hi<kHalf>(w.x), c = elem_lo<kHalf>(w.y), d = elem_hi<kHalf>(w.y);
+    return warp_sum(fmaf(a, a, b * b) + fmaf(c, c, d * d));
+}
+
+// src[from .. cnt) added in order to w, one lane; dst gets the running sums (dst may be src). Eight terms are loaded while
+// the eight before them are added.
+__device__ __forceinline__ double run_sums(const double *src, double *dst, int from, int cnt, double w)
+{
+    int u = from;
+    for (; u < cnt && (u & 7); ++u) { w = __dadd_rn(w, src[u]); dst[u] = w; }
+    if (u + 8 <= cnt) {
+        double t[8];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(&t[e]) = *reinterpret_cast<const double2 *>(src + u + e);
+        for (; u + 8 <= cnt; u += 8) {
+            double n[8];
+            const int nx = u + 16 <= cnt ? u + 8 : u;
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(&n[e]) = *reinterpret_cast<const double2 *>(src + nx + e);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { w = __dadd_rn(w, t[e]); t[e] = w; }
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(dst + u + e) = *reinterpret_cast<const double2 *>(&t[e]);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t[e] = n[e];
+        }
+    }
+    for (; u < cnt; ++u) { w = __dadd_rn(w, src[u]); dst[u] = w; }
+    return w;
+}
+
+// The defining distance of two rows, one lane.
+template <bool kHalf>
+__device__ __forceinline__ double start_dist(const uint4 *rows, int i, const uint4 *trial, int l)
+{
+    double s = 0.0;
+#pragma unroll 4
+    for (int c = 0; c < 16; ++c) {
+        const uint4 x4 = rows[near_piece(i, c)], y4 = trial[near_piece(l, c)];
+        const uint32_t x[4] = {x4.x, x4.y, x4.z, x4.w}, y[4] = {y4.x, y4.y, y4.z, y4.w};
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const double e0 = __dsub_rn((double)elem_lo<kHalf>(x[t]), (double)elem_lo<kHalf>(y[t]));
+            const double e1 = __dsub_rn((double)elem_hi<kHalf>(x[t]), (double)elem_hi<kHalf>(y[t]));
+            s = __dadd_rn(s, __dmul_rn(e0, e0));
+            s = __dadd_rn(s, __dmul_rn(e1, e1));
+        }
+    }
+    return s;
+}
+// The same by a warp: every lane widens and squares four dimensions (widening is what a lane on its own would wait
+// for: 8 cycles a value), one adds them up in order. `tmp`: 128 doubles of the warp. Every lane gets it.
+template <bool kHalf>
+__device__ __forceinline__ double start_dist_warp(const uint4 *rows, int i, const double (&y)[4], double *tmp)
+{
+    const int lane = threadIdx.x & 31;
+    double x[4];
+    row_quad<kHalf>(rows, i, x);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        x[e] = __dsub_rn(x[e], y[e]);
+        x[e] = __dmul_rn(x[e], x[e]);
+    }
+    *reinterpret_cast<double2 *>(tmp + 4 * lane) = make_double2(x[0], x[1]);
+    *reinterpret_cast<double2 *>(tmp + 4 * lane + 2) = make_double2(x[2], x[3]);
+    __syncwarp();
+    double s = 0.0;
+    if (lane == 0) {
+        double t[8];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(&t[e]) = *reinterpret_cast<const double2 *>(tmp + e);
+#pragma unroll
+        for (int u = 0; u < kHeadDim; u += 8) {
+            double n[8];
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(&n[e]) = *reinterpret_cast<const double2 *>(tmp + (u + 8 < kHeadDim ? u + 8 : u) + e);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) s = __dadd_rn(s, t[e]);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t[e] = n[e];
+        }
+    }
+    s = __shfl_sync(0xFFFFFFFFu, s, 0);
+    __syncwarp();
+    return s;
+}
+
+template <bool kHalf>
+__global__ void __launch_bounds__(kStartThreads, 1)
+km_start_kernel(KmeansParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    StartSmem &sm = *reinterpret_cast<StartSmem *>(smem_raw);
+    constexpr float kPairErr = 0.5f * kDistErr;             // times the sum of the two squared norms
+    const int n_blk = (int)cluster_size(), rank = (int)cluster_rank();
+    const int pair = blockIdx.x / n_blk, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, c4 = lane & 3;
+    const Pair q = pair_of(p, pair / p.n_kv, pair % p.n_kv);
+    const int nb = (q.n_init + kSumBlock - 1) / kSumBlock;  // blocks of the sums; this thread block's are [b0, b0 + mb)
+    const int per = (nb + n_blk - 1) / n_blk, b0 = min(rank * per, nb), mb = min(per, nb - b0);
+    const int row0 = b0 * kSumBlock, n_rows = max(min(q.n_init - row0, mb * kSumBlock), 0);
+    const int32_t *perm = p.perm + q.plane;
+    const uint4 *keys = reinterpret_cast<const uint4 *>(p.k_prompt + q.plane * kHeadDim);
+    const int n_part = (p.n_init_max + kSumBlock - 1) / kSumBlock;
+    double *part = p.part + (size_t)q.id * p.trials_max * n_part;       // [trial][n_part] block sums, where all trials are summed
+
+    // ---- the block's rows; the first centre as the only trial point ----
+    for (int e = tid; e < n_rows * 16; e += kStartThreads)
+        copy16_async(shared_addr(&sm.rows[near_piece(e >> 4, e & 15)]), keys + (size_t)perm[row0 + (e >> 4)] * 16 + (e & 15));
+    const int first = p.pick[(size_t)q.id * p.trials_max];
+    if (tid < 16) copy16_async(shared_addr(&sm.trial[near_piece(0, tid)]), keys + (size_t)perm[first] * 16 + tid);
+    copy_async_wait();
+    __syncthreads();
+    for (int i = warp; i < mb * kSumBlock; i += kStartWarps) {
+        const float n = i < n_rows ? row_norm<kHalf>(sm.rows, i) : 0.f;
+        if (lane == 0) {
+            sm.norm[i] = n;
+            sm.closest[i] = i < n_rows ? CUDART_INF : 0.0;
+            sm.bar[i] = i < n_rows ? 0.f : CUDART_INF_F;    // (set with the first distances)
+            sm.mask[i] = i < n_rows ? 1 : 0;
+        }
+    }
+    if (tid < kStartBlocks) sm.touched[tid] = tid < mb ? 1u : 0u;
+    if (tid == 0) sm.pick[0][0] = first;
+    cluster_barrier();                                      // every block of the cluster runs: its shared memory may be written
+
+    for (int c = 0; c < q.k; ++c) {
+        const int L = c == 0 ? 1 : q.L;
+        int best = 0;
+        if (c > 0) {
+            // ---- 1. which points a trial may lower, and by how much ----
+            uint32_t bf[2][8][2];                           // the trial points as MMA columns (two groups of eight)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const int t = min(n * 8 + (lane & 7), L - 1);
+#pragma unroll
+                for (int s2 = 0; s2 < 4; ++s2) {
+                    uint32_t r[4];
+                    ldmatrix4(r, shared_addr(&sm.trial[near_piece(t, 4 * s2 + (lane >> 3))]));
+                    bf[n][2 * s2][0] = r[0]; bf[n][2 * s2][1] = r[1]; bf[n][2 * s2 + 1][0] = r[2]; bf[n][2 * s2 + 1][1] = r[3];
+                }
+            }
+            float ny[4], err[4], lo[4], hi[4];              // the thread's columns: 2 c4, 2 c4 + 1, 8 + 2 c4, 9 + 2 c4
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int t = (v >> 1) * 8 + 2 * c4 + (v & 1);
+                const float n = t < L ? sm.trial_norm[t] : 0.f;
+                // (a column that is no trial is never marked; of a norm that fp32 does not hold the product decides nothing)
+                ny[v] = t >= L ? CUDART_INF_F : (n <= 1e37f ? n * (1.f - kPairErr) : -CUDART_INF_F);
+                err[v] = 2.f * kPairErr * n;
+                lo[v] = hi[v] = 0.f;
+            }
+            const int tiles = mb * (kSumBlock / 16);        // a multiple of 8: every warp has the same number, two at a time
+            for (int m0 = warp; m0 < tiles; m0 += 2 * kStartWarps) {
+                const bool two = m0 + kStartWarps < tiles;
+                const int mt[2] = {m0, two ? m0 + kStartWarps : m0};
+                float acc[2][2][4];
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) acc[k][n][0] = acc[k][n][1] = acc[k][n][2] = acc[k][n][3] = 0.f;
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {
+                    uint32_t a[2][4];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) ldmatrix4(a[k], shared_addr(&sm.rows[near_piece(mt[k] * 16 + (lane & 15), 2 * s + (lane >> 4))]));
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        mma_rows<kHalf>(acc[k][0], a[k][0], a[k][1], a[k][2], a[k][3], bf[0][s][0], bf[0][s][1]);
+                        if (L > 8) mma_rows<kHalf>(acc[k][1], a[k][0], a[k][1], a[k][2], a[k][3], bf[1][s][0], bf[1][s][1]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    if (k == 1 && !two) break;
+                    uint32_t bits[2];
+                    float val[2][4];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float bar = sm.bar[mt[k] * 16 + g + 8 * h];
+                        bits[h] = 0u;
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            val[h][v] = fmaf(-2.f, acc[k][v >> 1][2 * h + (v & 1)], bar + ny[v]);
+                            if (!(val[h][v] > 1e-34f)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));     // (1e-34: products that underflow)
+                        }
+                        if (!(bar < CUDART_INF_F)) bits[h] = 0u;     // past the end of the sample
+                    }
+                    if (__any_sync(0xFFFFFFFFu, (bits[0] | bits[1]) != 0u)) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const float e = 2.f * kPairErr * sm.norm[mt[k] * 16 + g + 8 * h];
+#pragma unroll
+                            for (int v = 0; v < 4; ++v)
+                                if ((bits[h] >> ((v >> 1) * 8 + 2 * c4 + (v & 1))) & 1u) {
+                                    hi[v] -= val[h][v];
+                                    lo[v] += fmaxf(-val[h][v] - (e + err[v]), 0.f);
+                                }
+                            bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 1);
+                            bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 2);
+                        }
+                        const uint32_t any = __reduce_or_sync(0xFFFFFFFFu, bits[0] | bits[1]);
+                        if (lane == 0) atomicOr(&sm.touched[mt[k] / (kSumBlock / 16)], any);
+                    }
+                    if (c4 < 2) sm.mask[mt[k] * 16 + g + 8 * c4] = (uint16_t)(c4 ? bits[1] : bits[0]);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (v >= 2 && L <= 8) break;
+#pragma unroll
+                for (int o = 4; o <= 16; o <<= 1) {
+                    lo[v] += __shfl_xor_sync(0xFFFFFFFFu, lo[v], o);
+                    hi[v] += __shfl_xor_sync(0xFFFFFFFFu, hi[v], o);
+                }
+                const int t = (v >> 1) * 8 + 2 * c4 + (v & 1);
+                if (g == 0 && t < L) sm.warp_gain[warp][t] = make_float2(lo[v], hi[v]);
+            }
+            __syncthreads();
+            for (int e = tid; e < L * n_blk; e += kStartThreads) {
+                const int l = e % L, to = e / L;
+                float2 s = sm.warp_gain[0][l];
+#pragma unroll
+                for (int w = 1; w < kStartWarps; ++w) { s.x += sm.warp_gain[w][l].x; s.y += sm.warp_gain[w][l].y; }
+                asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(in_block(shared_addr(&sm.gain[rank][l]), to)), "f"(s.x), "f"(s.y) : "memory");
+            }
+            cluster_barrier();
+            // ---- 2. the winner ----
+            {
+                // every warp for itself; 1e-5: rounding of the fp32 sums; 1e-11: of the fp64 sums that define the potentials
+                float gl = 0.f, gh = 0.f;
+                if (lane < L)
+                    for (int r = 0; r < n_blk; ++r) { gl += sm.gain[r][lane].x; gh += sm.gain[r][lane].y; }
+                const float slack = (float)(1e-11 * sm.pre[nb - 1]);
+                gl = lane < L ? gl * (1.f - 1e-5f) - slack : -CUDART_INF_F;
+                gh = gh * (1.f + 1e-5f);
+                const float top = warp_max(gl);
+                const unsigned at = __ballot_sync(0xFFFFFFFFu, gl == top);
+                best = at ? __ffs(at) - 1 : 0;
+                const int mine = sm.pick[c & 1][min(lane, L - 1)], its = __shfl_sync(0xFFFFFFFFu, mine, best);
+                const bool open = lane < L && !(gh < top) && mine != its;
+                if (__any_sync(0xFFFFFFFFu, open)) {
+                    // all potentials in fp64: each block of the sums in order, then the blocks in order
+                    for (int v = warp; v < L * mb; v += kStartWarps) {
+                        const int l = v / mb, blk = v - l * mb, base = blk * kSumBlock;
+                        double w = sm.raw[b0 + blk];
+                        if ((sm.touched[blk] >> l) & 1u) {
+                            __syncwarp();
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const int i = base + e * 32 + lane;
+                                double t = sm.closest[i];
+                                if ((sm.mask[i] >> l) & 1) {
+                                    const double d = start_dist<kHalf>(sm.rows, i, sm.trial, l);
+                                    if (d < t) t = d;
+                                }
+                                sm.tmp[warp][e * 32 + lane] = t;
+                            }
+                            __syncwarp();
+                            if (lane == 0) w = run_sums(sm.tmp[warp], sm.tmp[warp], 0, min(kSumBlock, n_rows - base), 0.0);
+                        }
+                        if (lane == 0) part[(size_t)l * n_part + b0 + blk] = w;
+                    }
+                    cluster_barrier();                      // (the same decision in every warp of the cluster)
+                    double pot = 0.0;
+                    if (lane < L)
+#pragma unroll 8
+                        for (int blk = 0; blk < nb; ++blk) pot = __dadd_rn(pot, __ldcg(part + (size_t)lane * n_part + blk));
+                    best = 0;
+                    double low = __shfl_sync(0xFFFFFFFFu, pot, 0);
+                    for (int l = 1; l < L; ++l) {
+                        const double v = __shfl_sync(0xFFFFFFFFu, pot, l);
+                        if (v < low) { low = v; best = l; }
+                    }
+                }
+            }
+        }
+        if (rank == 0 && tid == 0) p.chosen[q.cplane + c] = sm.pick[c & 1][best];
+        if (c + 1 == q.k) break;
+        // ---- 3. the winner's distances, a warp per touched block of the sums ----
+        for (int blk = warp; blk < mb; blk += kStartWarps) {
+            if (!((sm.touched[blk] >> best) & 1u)) continue;
+            const int base = blk * kSumBlock, cnt = min(kSumBlock, n_rows - base);
+            unsigned who[4];
+            int m = 0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                who[e] = __ballot_sync(0xFFFFFFFFu, (sm.mask[base + e * 32 + lane] >> best) & 1);
+                m += __popc(who[e]);
+            }
+            int first_at = kSumBlock;                       // first point that gets a smaller distance
+            auto lower = [&](int i, double d) {             // one lane
+                if (!(d < sm.closest[i]) && c > 0) return false;
+                sm.closest[i] = d;
+                // (a norm that fp32 does not hold: the product decides nothing)
+                sm.bar[i] = sm.norm[i] <= 1e37f ? sm.norm[i] * (1.f - kPairErr) - __double2float_ru(d) : -CUDART_INF_F;
+                return true;
+            };
+            if (m <= 3) {
+                double y[4];
+                row_quad<kHalf>(sm.trial, best, y);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    for (unsigned w = who[e]; w; w &= w - 1) {
+                        const int i = base + e * 32 + __ffs(w) - 1;
+                        const double d = start_dist_warp<kHalf>(sm.rows, i, y, sm.tmp[warp]);
+                        const bool did = lane == 0 && lower(i, d);
+                        if (__any_sync(0xFFFFFFFFu, did)) first_at = min(first_at, i - base);
+                    }
+            } else {
+#pragma unroll 1
+                for (int e = 0; e < 4; ++e) {
+                    bool did = false;
+                    if ((sm.mask[base + e * 32 + lane] >> best) & 1)
+                        did = lower(base + e * 32 + lane, start_dist<kHalf>(sm.rows, base + e * 32 + lane, sm.trial, best));
+                    const unsigned any = __ballot_sync(0xFFFFFFFFu, did);
+                    if (any) first_at = min(first_at, e * 32 + __ffs(any) - 1);
+                }
+            }
+            __syncwarp();
+            if (first_at == kSumBlock) continue;
+            double w = 0.0;
+            if (lane == 0) w = run_sums(sm.closest + base, sm.run + base, first_at, cnt, first_at > 0 ? sm.run[base + first_at - 1] : 0.0);
+            w = __shfl_sync(0xFFFFFFFFu, w, 0);
+            if (lane < n_blk)
+                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(in_block(shared_addr(&sm.raw[b0 + blk]), lane)), "d"(w) : "memory");
+        }
+        cluster_barrier();
+        // ---- 4. the blocks' running sums; the next trial points: a warp per draw, in the block that owns it ----
+        if (tid < kStartBlocks) sm.touched[tid] = 0u;
+        if (tid == 0) run_sums(sm.raw, sm.pre, 0, nb, 0.0);
+        __syncthreads();
+        const double total = sm.pre[nb - 1];
+        for (int l = warp; l < q.L; l += kStartWarps) {
+            const uint32_t w = km_word(p, (uint32_t)l, kTagStart, q.stream, (uint32_t)(c + 1));
+            const double target = __dmul_rn(((double)w + 0.5) * (1.0 / 4294967296.0), total);
+            int blk = nb;                                   // first block whose running sum exceeds the target
+            for (int o = 0; o < nb; o += 32) {
+                const unsigned over = __ballot_sync(0xFFFFFFFFu, o + lane < nb && sm.pre[min(o + lane, nb - 1)] > target);
+                if (over) { blk = o + __ffs(over) - 1; break; }
+            }
+            const bool none = blk == nb;                    // rounding left no point beyond the target: the last one
+            if (none) blk = nb - 1;
+            if (blk < b0 || blk >= b0 + mb) continue;
+            const int base = (blk - b0) * kSumBlock, cnt = min(kSumBlock, n_rows - base);
+            int at = cnt - 1;
+            if (!none) {                                    // first point of the block with offset + running sum beyond it
+                const double before = blk > 0 ? sm.pre[blk - 1] : 0.0;
+#pragma unroll
+                for (int e = 3; e >= 0; --e) {
+                    const unsigned over = __ballot_sync(0xFFFFFFFFu, e * 32 + lane < cnt && __dadd_rn(before, sm.run[base + e * 32 + lane]) > target);
+                    if (over) at = e * 32 + __ffs(over) - 1;
+                }
+            }
+            const uint4 piece = sm.rows[near_piece(base + at, lane & 15)];
+            const uint32_t row_to = shared_addr(&sm.trial[near_piece(l, lane & 15)]);
+            for (int to = lane >> 4; to < n_blk; to += 2)
+                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(in_block(row_to, to)), "r"(piece.x), "r"(piece.y), "r"(piece.z),
+                             "r"(piece.w) : "memory");
+            if (lane < n_blk) {
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(in_block(shared_addr(&sm.trial_norm[l]), lane)), "f"(sm.norm[base + at]) : "memory");
+                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(in_block(shared_addr(&sm.pick[(c + 1) & 1][l]), lane)), "r"(row0 + base + at) : "memory");
+            }
+        }
+        cluster_barrier();
+    }
+}
+
+// How many blocks share a pair's sample in km_start_kernel; 0: the sample does not fit, or the device has no room for
+// such a cluster. Sixteen where every pair gets its cluster at once; eight halve the wait of many pairs.
+template <bool kHalf>
+int start_cluster(const KmeansParams &p, int pairs)
+{
+    const int nb = (p.n_init_max + kSumBlock - 1) / kSumBlock;
+    if (nb > kStartSums || p.trials_max > kStartTrials) return 0;
+    const int n_blk = nb <= kStartBlocks * 8 && pairs > 8 ? 8 : kStartMaxCluster;
+    const void *fn = (const void *)km_start_kernel<kHalf>;
+    static std::atomic<unsigned long long> done;
+    if (ensure_dynamic_smem(fn, (int)sizeof(StartSmem), done) != cudaSuccess
+        || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    cudaLaunchAttribute dims;
+    dims.id = cudaLaunchAttributeClusterDimension;
+    dims.val.clusterDim.x = n_blk;
+    dims.val.clusterDim.y = dims.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(pairs * n_blk);
+    cfg.blockDim = dim3(kStartThreads);
+    cfg.dynamicSmemBytes = sizeof(StartSmem);
+    cfg.attrs = &dims;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, km_start_kernel<kHalf>, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return fit > 0 ? n_blk : 0;
+}
+
+template <bool kHalf>
+cudaError_t launch_start(const KmeansParams &p, int pairs, int n_blk, cudaStream_t s)
+{
+    cudaLaunchAttribute dims;
+    dims.id = cudaLaunchAttributeClusterDimension;
+    dims.val.clusterDim.x = n_blk;
+    dims.val.clusterDim.y = dims.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(pairs * n_blk);
+    cfg.blockDim = dim3(kStartThreads);
+    cfg.dynamicSmemBytes = sizeof(StartSmem);
+    cfg.stream = s;
+    cfg.attrs = &dims;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, km_start_kernel<kHalf>, p);
+}
+
 // ---- 3. minibatch steps ----
 // A step is five kernels: the scan for the nearest centres (nearest.cuh), the fp64 distance to the one found,
 // the minibatch ordered by centre, the update, the reassignment of starved centres. The inertia of a
@@ -359,7 +857,7 @@ __device__ __forceinline__ void store_centre(const KmeansParams &p, size_t centr
     if (lane == 0) p.centre_bias[centre] = bias;
 }
 
-// The centres as the start left them, their counts and the fits' state at zero. A warp per centre.
+// The centres that the start chose (sample indices), their counts and the fits' state at zero. A warp per centre.
 template <bool kHalf>
 __global__ void __launch_bounds__(kThreads)
 km_prepare_kernel(KmeansParams p)
@@ -369,9 +867,9 @@ km_prepare_kernel(KmeansParams p)
     const int u = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0, 0, 0, 0};
     if (u >= q.k) return;
-    const double2 *from = reinterpret_cast<const double2 *>(p.centres64 + (q.cplane + u) * kHeadDim + 4 * lane);
-    const double2 v0 = from[0], v1 = from[1];
-    const double v[4] = {v0.x, v0.y, v1.x, v1.y};
+    const int row = p.perm[q.plane + p.chosen[q.cplane + u]];
+    const uint2 w = reinterpret_cast<const uint2 *>(p.k_prompt + (q.plane + row) * kHeadDim)[lane];
+    const double v[4] = {(double)elem_lo<kHalf>(w.x), (double)elem_hi<kHalf>(w.x), (double)elem_lo<kHalf>(w.y), (double)elem_hi<kHalf>(w.y)};
     store_centre<kHalf>(p, q.cplane + u, v);
     if (lane == 0) p.count[q.cplane + u] = 0.0;
 }
@@ -713,15 +1211,20 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
     static std::atomic<unsigned long long> sample_done;
     if ((err = ensure_dynamic_smem((const void *)km_sample_kernel, (int)sample_smem(kMaxSumBlocks * kSumBlock), sample_done)) != cudaSuccess) return err;
     if ((err = launch_step(km_sample_kernel, dim3(B, H), dim3(kSampleThreads), sample_smem(p.n_init_max), s, p)) != cudaSuccess) return err;
-    const dim3 dist_grid((p.n_init_max + kSumBlock - 1) / kSumBlock, (p.trials_max + kDistTrials - 1) / kDistTrials, pairs);
-    const size_t draw_smem = sizeof(double) * ((size_t)p.n_init_max + 2 * kMaxSumBlocks);
-    if ((err = cudaFuncSetAttribute(km_accept_kernel<kHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)draw_smem)) != cudaSuccess)
-        return err;
-    for (int c = 0; c < p.k_max; ++c) {
-        km_candidate_dist_kernel<kHalf><<<dist_grid, kDistThreads, 0, s>>>(p, c);
-        KM_CHECK();
-        km_accept_kernel<kHalf><<<dim3(B, H), kAcceptThreads, draw_smem, s>>>(p, c);     // ... and the trial points of centre c + 1
-        KM_CHECK();
+    const int n_blk = start_cluster<kHalf>(p, pairs);
+    if (n_blk > 0) {
+        if ((err = launch_start<kHalf>(p, pairs, n_blk, s)) != cudaSuccess) return err;
+    } else {
+        const dim3 dist_grid((p.n_init_max + kSumBlock - 1) / kSumBlock, (p.trials_max + kDistTrials - 1) / kDistTrials, pairs);
+        const size_t draw_smem = sizeof(double) * ((size_t)p.n_init_max + 2 * kMaxSumBlocks);
+        if ((err = cudaFuncSetAttribute(km_accept_kernel<kHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)draw_smem)) != cudaSuccess)
+            return err;
+        for (int c = 0; c < p.k_max; ++c) {
+            km_candidate_dist_kernel<kHalf><<<dist_grid, kDistThreads, 0, s>>>(p, c);
+            KM_CHECK();
+            km_accept_kernel<kHalf><<<dim3(B, H), kAcceptThreads, draw_smem, s>>>(p, c);     // ... and the trial points of centre c + 1
+            KM_CHECK();
+        }
     }
     const dim3 threads(kThreads);
     if ((err = launch_step(km_prepare_kernel<kHalf>, dim3((p.k_max + kThreads / 32 - 1) / (kThreads / 32), pairs), threads, 0, s, p)) != cudaSuccess) return err;
