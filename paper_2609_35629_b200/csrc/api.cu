@@ -277,27 +277,32 @@ namespace {
 
 // Workspace of santapp_build_teams_parents. Offsets in bytes.
 struct ParentLayout {
-    size_t label_off, parent_start, parent_cursor, parent_team_base, members, team_of, mind, owner, is_rep,
-        team_cursor, dest, total;
+    size_t label_off, parent_start, parent_team_base, label_hist, rank, members, list[3], list_count, mind, owner, is_rep, total;
+    int chunks;
 };
 
-ParentLayout parent_layout(int n_seqs, int n_kv, int64_t rows_total, int64_t labels_total, int64_t teams_total)
+ParentLayout parent_layout(int n_seqs, int n_kv, int64_t rows_total, int64_t labels_total)
 {
     ParentLayout L;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
     const size_t H = (size_t)n_kv, R = (size_t)rows_total, Lt = (size_t)labels_total;
+    // chunks of a sequence's tokens that are ranked side by side: 32, fewer where there are so many labels that the
+    // chunks' counts would outgrow the tokens
+    L.chunks = (int)std::max<int64_t>(1, std::min<int64_t>(32, 4 * rows_total / labels_total));
     L.label_off = take(sizeof(int64_t) * ((size_t)n_seqs + 1));
     L.parent_start = take(sizeof(int32_t) * H * (Lt + (size_t)n_seqs));
-    L.parent_cursor = take(sizeof(int32_t) * H * Lt);
     L.parent_team_base = take(sizeof(int32_t) * H * Lt);
+    L.label_hist = take(sizeof(int32_t) * H * Lt * (size_t)L.chunks);
+    L.rank = take(sizeof(int32_t) * H * R);
     L.members = take(sizeof(int32_t) * H * R);
-    L.team_of = take(sizeof(int32_t) * H * R);
+    L.list[0] = take(sizeof(int2) * H * (R / 33 + 1));
+    L.list[1] = take(sizeof(int2) * H * (R / 129 + 1));
+    L.list[2] = take(sizeof(int2) * H * (R / 513 + 1));
+    L.list_count = take(sizeof(int32_t) * 3);
     L.mind = take(sizeof(double) * H * R);
     L.owner = take(sizeof(int32_t) * H * R);
     L.is_rep = take(H * R);
-    L.team_cursor = take(sizeof(int32_t) * H * (size_t)teams_total);
-    L.dest = take(sizeof(int32_t) * H * R);
     L.total = off;
     return L;
 }
@@ -390,7 +395,7 @@ int santapp_parent_teams_sizes(const santapp_geom *geom, const int32_t *prompt_l
     if (out->rows_total >= (int64_t)1 << 31 || labels_total >= (int64_t)1 << 31) return SANTAPP_ERR_UNSUPPORTED;
     out->team_row_start_elems = (int64_t)geom->n_kv_heads * (out->teams_total + geom->n_seqs);
     out->build_workspace_bytes =
-        parent_layout(geom->n_seqs, geom->n_kv_heads, out->rows_total, labels_total, out->teams_total).total;
+        parent_layout(geom->n_seqs, geom->n_kv_heads, out->rows_total, labels_total).total;
     return SANTAPP_OK;
 }
 
@@ -429,7 +434,7 @@ static int build_parent_records(const santapp_geom *geom, const int32_t *prompt_
         label_off[b + 1] = label_off[b] + n_parents_host[b];
         if (n_parents_host[b] > max_labels) max_labels = n_parents_host[b];
     }
-    const ParentLayout L = parent_layout(B, geom->n_kv_heads, sz.rows_total, label_off[B], sz.teams_total);
+    const ParentLayout L = parent_layout(B, geom->n_kv_heads, sz.rows_total, label_off[B]);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     cudaError_t err = launch_tables({row_off, team_off, label_off},
                                     {teams->seq_row_off, teams->seq_team_off, reinterpret_cast<int64_t *>(ws + L.label_off)}, B + 1,
@@ -458,20 +463,24 @@ static int build_parent_records(const santapp_geom *geom, const int32_t *prompt_
     p.team_row_start = teams->team_row_start;
     p.row_token = teams->row_token;
     p.team_count = teams->team_count;
+    p.rep_abs_max = teams->rep_abs_max;
+    p.chunks = L.chunks;
     p.parent_start = reinterpret_cast<int32_t *>(ws + L.parent_start);
-    p.parent_cursor = reinterpret_cast<int32_t *>(ws + L.parent_cursor);
     p.parent_team_base = reinterpret_cast<int32_t *>(ws + L.parent_team_base);
+    p.label_hist = reinterpret_cast<int32_t *>(ws + L.label_hist);
+    p.rank = reinterpret_cast<int32_t *>(ws + L.rank);
     p.members = reinterpret_cast<int32_t *>(ws + L.members);
-    p.team_of = reinterpret_cast<int32_t *>(ws + L.team_of);
+    for (int k = 0; k < 3; ++k) p.list[k] = reinterpret_cast<int2 *>(ws + L.list[k]);
+    p.list_count = reinterpret_cast<int32_t *>(ws + L.list_count);
     p.mind = reinterpret_cast<double *>(ws + L.mind);
     p.owner = reinterpret_cast<int32_t *>(ws + L.owner);
     p.is_rep = ws + L.is_rep;
-    p.team_cursor = reinterpret_cast<int32_t *>(ws + L.team_cursor);
-    p.dest = reinterpret_cast<int32_t *>(ws + L.dest);
     err = launch_build_teams_parents(p, s);
     if (err != cudaSuccess) return cuda_fail(err, "build_teams_parents launch");
-    err = launch_rep_abs_max(p.bv, sz.max_teams_per_seq, p.rep_keys, teams->rep_abs_max, s);
-    if (err != cudaSuccess) return cuda_fail(err, "rep_abs_max launch");
+    if (mean_keys) {                                            // (the team builder raises it as it goes)
+        err = launch_rep_abs_max(p.bv, sz.max_teams_per_seq, p.rep_keys, teams->rep_abs_max, s);
+        if (err != cudaSuccess) return cuda_fail(err, "rep_abs_max launch");
+    }
     return SANTAPP_OK;
 }
 

@@ -1,13 +1,14 @@
 // Team records from an arbitrary parent partition (the partition Algorithm 3 returns: parents of
 // any size, in centre order, empty ones omitted), and the nearest-centre assignment that closes
-// Algorithm 3. Preparation path, run once after prefill. As in the contiguous builder, distances
-// are fp64, summed over dimensions in increasing order with separately rounded multiply and add,
-// so exact ties fall the way the paper's tie rules say.
+// Algorithm 3. Preparation path, run once after prefill. As in the contiguous builder, the teams are those of fp64
+// distances summed over dimensions in increasing order with separately rounded multiply and add.
 //
-// Steps: count the tokens of each label; scan the counts into member-list offsets and number the
-// teams (a parent of c tokens yields min(R, c)); list each parent's tokens in increasing index
-// (stable scatter); Algorithm 2 per non-empty parent; scan team sizes into CSR offsets; stable
-// scatter of the tokens by team; copy K/V rows into the team-contiguous layout.
+// Steps: rank every token among the earlier tokens of its label (per chunk of the sequence, side by side) and count
+// the labels of each chunk; scan the counts into member-list offsets, number the teams (a parent of c tokens
+// yields min(R, c)) and list the parents by size; write the member lists; then one kernel per size class does
+// Algorithm 2 and the packed copy of its parents (parent_teams.cuh; a parent's rows are one range of the packed
+// order). 4 x 32K keys in 2048 k-means parents: 1250 us with one block per pair scattering tokens in order, by
+// label and again by team.
 #include <limits.h>
 
 #include <algorithm>
@@ -15,6 +16,7 @@
 #include "build_util.cuh"
 #include "common.cuh"
 #include "nearest.cuh"
+#include "parent_teams.cuh"
 
 namespace santapp {
 
@@ -112,101 +114,187 @@ assign_parents_kernel(AssignParams p)
     if (live) p.parent_of[(size_t)j * p.rows_total + row0 + i] = arg;
 }
 
-// ---- token counts per label ----
-__global__ void __launch_bounds__(kThreads)
-count_labels_kernel(ParentBuildParams p)
+// ---- member lists ----
+// One warp per (chunk of a sequence's tokens, sequence, KV head): the tokens 32 at a time in increasing index; lanes with
+// the same label form a group whose lowest lane moves the label's count, and each lane takes its rank in the
+// group on top of the count before. The chunk's counts go to label_hist. They live in shared memory when they
+// fit (smem_labels of them), else in label_hist itself; a step's labels are requested one step ahead.
+constexpr int kHistSmemLabels = 50 * 1024;                  // 200 KB
+constexpr int kRankThreads = 128;                           // all of them clear and write the counts, the first warp ranks
+__global__ void __launch_bounds__(kRankThreads)
+rank_labels_kernel(ParentBuildParams p, int smem_labels)
 {
-    const int b = blockIdx.y, j = blockIdx.z;
+    extern __shared__ int32_t count_s[];
+    step_wait();
+    const int chunk = blockIdx.x, b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
     const int64_t row0 = p.bv.seq_row_off[b];
     const int N = (int)(p.bv.seq_row_off[b + 1] - row0);
-    const int i = blockIdx.x * kThreads + threadIdx.x;
-    if (i >= N) return;
     const int64_t l0 = p.seq_label_off[b];
     const int n_labels = (int)(p.seq_label_off[b + 1] - l0);
-    const int u = clamp_label(p.parent_of[(size_t)j * p.bv.rows_total + row0 + i], n_labels);
-    atomicAdd(p.parent_cursor + (size_t)j * p.labels_total + l0 + u, 1);
+    const int per = ((N + p.chunks - 1) / p.chunks + 31) / 32 * 32, lo = min(chunk * per, N), hi = min(lo + per, N);
+    const size_t plane = (size_t)j * p.bv.rows_total + row0;
+    int32_t *hist = p.label_hist + ((size_t)j * p.chunks + chunk) * p.labels_total + l0;
+    const bool in_smem = n_labels <= smem_labels;
+    int32_t *count = in_smem ? count_s : hist;
+    for (int u = tid; u < n_labels; u += kRankThreads) count[u] = 0;
+    __syncthreads();
+    if (tid < 32) {
+        const int32_t *lab = p.parent_of + plane;
+        int next = lo + lane < hi ? lab[lo + lane] : 0;
+        for (int i0 = lo; i0 < hi; i0 += 32) {
+            const int i = i0 + lane, mine = next;
+            const bool valid = i < hi;
+            if (i + 32 < hi) next = lab[i + 32];
+            const int u = valid ? clamp_label(mine, n_labels) : -1 - lane;     // idle lanes stay alone
+            const unsigned group = __match_any_sync(0xFFFFFFFFu, u);
+            const int leader = __ffs(group) - 1;
+            int base = 0;
+            if (valid && lane == leader) base = atomicAdd(count + u, __popc(group));
+            base = __shfl_sync(0xFFFFFFFFu, base, leader);  // (also completes a step's updates before the next)
+            if (valid) p.rank[plane + i] = base + __popc(group & ((1u << lane) - 1u));
+        }
+    }
+    __syncthreads();
+    if (in_smem)
+        for (int u = tid; u < n_labels; u += kRankThreads) hist[u] = count_s[u];
 }
 
-// One block per (sequence, KV head): counts -> member-list offsets, team numbering, team count.
-__global__ void __launch_bounds__(kThreads)
+// One block per (sequence, KV head): counts of the chunks -> where each chunk's tokens of a label go in the member
+// list, member-list offsets, team numbering, team count, the row offsets of the slots behind the last team (empty
+// teams), and the parents by size class.
+constexpr int kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads)
 scan_parents_kernel(ParentBuildParams p)
 {
     __shared__ int scratch[33];
-    const int b = blockIdx.x, j = blockIdx.y;
+    step_wait();
+    const int b = blockIdx.x, j = blockIdx.y, tid = threadIdx.x;
     const int64_t l0 = p.seq_label_off[b];
     const int n_labels = (int)(p.seq_label_off[b + 1] - l0);
-    int32_t *cursor = p.parent_cursor + (size_t)j * p.labels_total + l0;
     int32_t *tbase = p.parent_team_base + (size_t)j * p.labels_total + l0;
     int32_t *pstart = p.parent_start + (size_t)j * (p.labels_total + p.bv.n_seqs) + l0 + b;
     int rows_carry = 0, teams_carry = 0;
-    for (int base = 0; base < n_labels; base += kThreads) {
-        const int u = base + threadIdx.x;
-        const int cnt = u < n_labels ? cursor[u] : 0;
-        const int r = min(cnt, p.reps);
+    for (int base = 0; base < n_labels; base += kScanThreads) {
+        const int u = base + tid;
+        int32_t *hist = p.label_hist + (size_t)j * p.chunks * p.labels_total + l0 + u;
+        int cnt = 0;
+        if (u < n_labels)
+            for (int c0 = 0; c0 < p.chunks; c0 += 8) {
+                int h[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) h[c] = c0 + c < p.chunks ? hist[(size_t)(c0 + c) * p.labels_total] : 0;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    if (c0 + c < p.chunks) hist[(size_t)(c0 + c) * p.labels_total] = cnt;
+                    cnt += h[c];
+                }
+            }
         int rows_total, teams_total;
         const int rows_excl = block_exclusive_scan(cnt, scratch, rows_total);
-        const int teams_excl = block_exclusive_scan(r, scratch, teams_total);
+        const int teams_excl = block_exclusive_scan(min(cnt, p.reps), scratch, teams_total);
         if (u < n_labels) {
             pstart[u] = rows_carry + rows_excl;
-            cursor[u] = rows_carry + rows_excl;
             tbase[u] = teams_carry + teams_excl;
+            const int kind = p.mean_keys ? -1 : (cnt <= 32 ? -1 : (cnt <= 128 ? 0 : (cnt <= 512 ? 1 : 2)));
+            if (kind >= 0) p.list[kind][atomicAdd(p.list_count + kind, 1)] = make_int2(b * p.bv.n_kv + j, u);
         }
         rows_carry += rows_total;
         teams_carry += teams_total;
     }
-    if (threadIdx.x == 0) {
+    const int64_t team0 = p.bv.seq_team_off[b];
+    const int slots = (int)(p.bv.seq_team_off[b + 1] - team0);
+    const int N = (int)(p.bv.seq_row_off[b + 1] - p.bv.seq_row_off[b]);
+    int32_t *csr = p.team_row_start + (size_t)j * (p.bv.teams_total + p.bv.n_seqs) + team0 + b;
+    for (int g = teams_carry + tid; g < slots; g += kScanThreads) csr[1 + g] = N;
+    if (tid == 0) {
         pstart[n_labels] = rows_carry;
         p.team_count[(size_t)j * p.bv.n_seqs + b] = teams_carry;
+        csr[0] = 0;
     }
 }
 
-// One block per (sequence, KV head): position of every token in the list ordered by (label, token
-// index). One warp takes the tokens 32 at a time in increasing index; lanes with the same label
-// form a group whose lowest lane reserves the group's slots at the label's cursor, and each lane
-// takes the slot of its rank inside the group. The full-warp shuffle that hands the reserved base
-// round also makes every reservation of one step complete before the next step begins. The
-// cursors are copied into shared memory by the whole block when they fit (smem_labels of them: a
-// step then costs a shared-memory atomic instead of a round trip to L2; they are not needed
-// afterwards), and a step's labels are requested one step ahead.
-//   kInverse: out[position] = token (member lists); otherwise out[token] = position.
-constexpr int kScatterSmemLabels = 50 * 1024;               // cursors that fit in shared memory (200 KB)
-template <bool kInverse>
 __global__ void __launch_bounds__(kThreads)
-stable_scatter_kernel(const int32_t *labels, int32_t *cursors, int32_t *out, const int64_t *seq_row_off,
-                      const int64_t *seq_label_off, int64_t rows_total, int64_t labels_total, int smem_labels)
+members_kernel(ParentBuildParams p)
 {
-    extern __shared__ int32_t cur_s[];
-    const int b = blockIdx.x, j = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-    const int64_t row0 = seq_row_off[b];
-    const int N = (int)(seq_row_off[b + 1] - row0);
-    const int64_t l0 = seq_label_off[b];
-    const int n_labels = (int)(seq_label_off[b + 1] - l0);
-    const int32_t *lab = labels + (size_t)j * rows_total + row0;
-    int32_t *cur = cursors + (size_t)j * labels_total + l0;
-    int32_t *dst = out + (size_t)j * rows_total + row0;
-    const bool in_smem = n_labels <= smem_labels;
-    if (in_smem)
-        for (int u = tid; u < n_labels; u += kThreads) cur_s[u] = cur[u];
-    __syncthreads();
-    if (tid >= 32) return;
-    int next = lane < N ? lab[lane] : 0;
-    for (int i0 = 0; i0 < N; i0 += 32) {
-        const int i = i0 + lane;
-        const bool valid = i < N;
-        const int mine = next;
-        if (i + 32 < N) next = lab[i + 32];
-        const int u = valid ? clamp_label(mine, n_labels) : -1 - lane;         // idle lanes stay alone
-        const unsigned group = __match_any_sync(0xFFFFFFFFu, u);
-        const int leader = __ffs(group) - 1;
-        const int rank = __popc(group & ((1u << lane) - 1u));
-        int base = 0;
-        if (valid && lane == leader) base = in_smem ? atomicAdd(cur_s + u, __popc(group)) : atomicAdd(cur + u, __popc(group));
-        base = __shfl_sync(0xFFFFFFFFu, base, leader);
-        if (valid) {
-            if (kInverse) dst[base + rank] = i;
-            else dst[i] = base + rank;
-        }
+    step_wait();
+    const int b = blockIdx.y, j = blockIdx.z;
+    const int64_t row0 = p.bv.seq_row_off[b];
+    const int N = (int)(p.bv.seq_row_off[b + 1] - row0), i = blockIdx.x * kThreads + threadIdx.x;
+    if (i >= N) return;
+    const int64_t l0 = p.seq_label_off[b];
+    const int n_labels = (int)(p.seq_label_off[b + 1] - l0);
+    const int per = ((N + p.chunks - 1) / p.chunks + 31) / 32 * 32;
+    const size_t plane = (size_t)j * p.bv.rows_total + row0;
+    const int u = clamp_label(p.parent_of[plane + i], n_labels);
+    const int at = p.parent_start[(size_t)j * (p.labels_total + p.bv.n_seqs) + l0 + b + u]
+                   + p.label_hist[((size_t)j * p.chunks + i / per) * p.labels_total + l0 + u] + p.rank[plane + i];
+    p.members[plane + at] = i;
+}
+
+// The parent of label u of (sequence b, KV head j).
+__device__ __forceinline__ void listed_parent(const ParentBuildParams &p, int u, int b, int j, ParentRows &t)
+{
+    const int64_t l0 = p.seq_label_off[b], row0 = p.bv.seq_row_off[b], team0 = p.bv.seq_team_off[b];
+    const int32_t *pstart = p.parent_start + (size_t)j * (p.labels_total + p.bv.n_seqs) + l0 + b;
+    const int tb = p.parent_team_base[(size_t)j * p.labels_total + l0 + u];
+    t.k_prompt = p.k_prompt;
+    t.v_prompt = p.v_prompt;
+    t.k_packed = p.k_packed;
+    t.v_packed = p.v_packed;
+    t.rep_keys = p.rep_keys;
+    t.row_token = p.row_token;
+    t.plane = (size_t)j * p.bv.rows_total + row0;
+    t.s0 = pstart[u];
+    t.nC = pstart[u + 1] - t.s0;
+    t.r = min(p.reps, t.nC);
+    t.members = p.members + t.plane + t.s0;
+    t.csr = p.team_row_start + (size_t)j * (p.bv.teams_total + p.bv.n_seqs) + team0 + b + tb;
+    t.rep0 = (size_t)j * p.bv.teams_total + team0 + tb;
+    t.abs_max = p.rep_abs_max + (size_t)j * p.bv.n_seqs + b;
+}
+
+// Parents of at most 32 rows, a warp per label.
+constexpr int kSmallParentWarps = 2;
+template <bool kHalf>
+__global__ void __launch_bounds__(kSmallParentWarps * 32)
+small_parents_kernel(ParentBuildParams p)
+{
+    __shared__ union { SmallSmem<16> s16; SmallSmem<32> s32; } sm[kSmallParentWarps];
+    step_wait();
+    const int warp = threadIdx.x >> 5, u = blockIdx.x * kSmallParentWarps + warp, b = blockIdx.y, j = blockIdx.z;
+    if (u >= (int)(p.seq_label_off[b + 1] - p.seq_label_off[b])) return;
+    ParentRows t;
+    listed_parent(p, u, b, j, t);
+    if (t.nC == 0 || t.nC > 32) return;                     // empty parents are omitted
+    if (t.nC <= 16) small_parent<16, kHalf>(t, sm[warp].s16);
+    else            small_parent<32, kHalf>(t, sm[warp].s32);
+}
+
+// Parents of 33 to 128 and of 129 to 512 rows: blocks walk the lists.
+template <int kWarps, int kRpt, bool kHalf>
+__global__ void __launch_bounds__(32 * kWarps, 1)
+large_parents_kernel(ParentBuildParams p, int kind)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_wait();
+    const int n = p.list_count[kind];
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+        const int2 e = p.list[kind][i];
+        ParentRows t;
+        listed_parent(p, e.y, e.x / p.bv.n_kv, e.x % p.bv.n_kv, t);
+        large_parent<kWarps, kRpt, kHalf>(t, *reinterpret_cast<LargeSmem<kWarps, kRpt> *>(smem_raw));
+        __syncthreads();
     }
+}
+
+// K and V of one token to a row of the sequence's packed order, by a warp.
+__device__ __forceinline__ void copy_row(const ParentRows &t, int token, int row)
+{
+    const int lane = threadIdx.x & 31;
+    const size_t from = (t.plane + token) * 32 + lane, to = (t.plane + row) * 32 + lane;
+    reinterpret_cast<uint2 *>(t.k_packed)[to] = reinterpret_cast<const uint2 *>(t.k_prompt)[from];
+    reinterpret_cast<uint2 *>(t.v_packed)[to] = reinterpret_cast<const uint2 *>(t.v_prompt)[from];
+    if (lane == 0) t.row_token[t.plane + row] = token;
 }
 
 template <bool kHalf>
@@ -248,29 +336,39 @@ __device__ __forceinline__ double sqdist_grow_row(const uint4 *row, const uint32
     return s;
 }
 
-// Algorithm 2 for one parent of any size. One block per (label, sequence, KV head); the parent's
-// tokens are read through its member list, and the per-member state lives in global memory.
+// Parents of more than 512 rows (and, for the centroid-guided baseline, all parents): rows are read through the member
+// list, the per-member state lives in global memory, every distance is taken in fp64. Blocks walk the list
+// of such parents (mean keys: one block per label).
 template <bool kHalf>
 __global__ void __launch_bounds__(kThreads)
-build_parent_general_kernel(ParentBuildParams p)
+huge_parents_kernel(ParentBuildParams p)
 {
+    __shared__ int scan_s[33], start_s[kMaxParent];
     __shared__ double mu[kHeadDim];
     __shared__ uint32_t ref[64];
     __shared__ ValIdx scratch[33];
     __shared__ int count[kMaxParent];
     __shared__ int rep_pos[kMaxParent];
-    const int u_parent = blockIdx.x, b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x;
-    const int64_t l0 = p.seq_label_off[b];
-    const int n_labels = (int)(p.seq_label_off[b + 1] - l0);
-    if (u_parent >= n_labels) return;
-    const int32_t *pstart = p.parent_start + (size_t)j * (p.labels_total + p.bv.n_seqs) + l0 + b;
-    const int s0 = pstart[u_parent];
-    const int nC = pstart[u_parent + 1] - s0;
-    if (nC == 0) return;                                   // empty parents are omitted
-    const int r = min(p.reps, nC);
-    const int64_t row0 = p.bv.seq_row_off[b];
-    const size_t plane = (size_t)j * p.bv.rows_total + row0;
-    const int32_t *mem = p.members + plane + s0;
+    step_wait();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n_list = p.mean_keys ? 0 : p.list_count[2];
+  for (int li = blockIdx.x; p.mean_keys ? li == (int)blockIdx.x : li < n_list; li += gridDim.x) {
+    int u_parent = blockIdx.x, b = blockIdx.y, j = blockIdx.z;
+    if (!p.mean_keys) {
+        const int2 e = p.list[2][li];
+        u_parent = e.y;
+        b = e.x / p.bv.n_kv;
+        j = e.x % p.bv.n_kv;
+    } else if (u_parent >= (int)(p.seq_label_off[b + 1] - p.seq_label_off[b])) {
+        return;
+    }
+    ParentRows t;
+    listed_parent(p, u_parent, b, j, t);
+    const int s0 = t.s0, nC = t.nC, r = t.r;
+    if (nC == 0) return;                                   // (mean keys) empty parents are omitted
+    const size_t plane = t.plane;
+    const int32_t *mem = t.members;
+    __syncthreads();
     double *mind = p.mind + plane + s0;
     int32_t *owner = p.owner + plane + s0;
     unsigned char *is_rep = p.is_rep + plane + s0;
@@ -291,13 +389,9 @@ build_parent_general_kernel(ParentBuildParams p)
     if (p.mean_keys) {
         // centroid-guided baseline: the parent is one group, routed by its mean stored as a 16-bit
         // element (fp64 -> fp32 to nearest, fp32 -> bf16 or fp16 to nearest even)
-        const int tb = p.parent_team_base[(size_t)j * p.labels_total + l0 + u_parent];
-        const int64_t t0 = p.bv.seq_team_off[b];
-        int32_t *tof = p.team_of + plane;
-        for (int i = tid; i < nC; i += kThreads) tof[mem[i]] = tb;
-        if (tid == 0) p.team_row_start[(size_t)j * (p.bv.teams_total + p.bv.n_seqs) + t0 + b + 1 + tb] = nC;
-        if (tid < kHeadDim)
-            p.rep_keys[((size_t)j * p.bv.teams_total + t0 + tb) * kHeadDim + tid] = double_to_elem<kHalf>(mu[tid]);
+        if (tid == 0) t.csr[1] = s0 + nC;
+        if (tid < kHeadDim) p.rep_keys[t.rep0 * kHeadDim + tid] = double_to_elem<kHalf>(mu[tid]);
+        for (int i = warp; i < nC; i += kThreads / 32) copy_row(t, mem[i], s0 + i);
         return;
     }
 
@@ -338,65 +432,45 @@ build_parent_general_kernel(ParentBuildParams p)
     for (int i = tid; i < nC; i += kThreads) atomicAdd(&count[owner[i]], 1);
     __syncthreads();
 
-    // outputs: team of every token, team sizes (scanned later), representative keys
-    const int tbase = p.parent_team_base[(size_t)j * p.labels_total + l0 + u_parent];
-    int32_t *team_of = p.team_of + plane;
-    for (int i = tid; i < nC; i += kThreads) team_of[mem[i]] = tbase + owner[i];
-    const int64_t team0 = p.bv.seq_team_off[b];
-    int32_t *csr = p.team_row_start + (size_t)j * (p.bv.teams_total + p.bv.n_seqs) + team0 + b;
-    for (int u = tid; u < r; u += kThreads) csr[1 + tbase + u] = count[u];
-    uint32_t *rep_dst = reinterpret_cast<uint32_t *>(p.rep_keys) + ((size_t)j * p.bv.teams_total + team0 + tbase) * 64;
-    for (int e = tid; e < r * 64; e += kThreads)
-        rep_dst[e] = reinterpret_cast<const uint32_t *>(kbase + (size_t)mem[rep_pos[e >> 6]] * 16)[e & 63];
-}
-
-// One block per (sequence, KV head): team sizes -> CSR row offsets; the slots behind the pair's
-// last team are empty teams (offset = prompt length); the cursors of the scatter by team.
-__global__ void __launch_bounds__(kThreads)
-scan_teams_kernel(ParentBuildParams p)
-{
-    __shared__ int scratch[33];
-    const int b = blockIdx.x, j = blockIdx.y;
-    const int64_t team0 = p.bv.seq_team_off[b];
-    const int slots = (int)(p.bv.seq_team_off[b + 1] - team0);
-    const int M = p.team_count[(size_t)j * p.bv.n_seqs + b];
-    const int N = (int)(p.bv.seq_row_off[b + 1] - p.bv.seq_row_off[b]);
-    int32_t *csr = p.team_row_start + (size_t)j * (p.bv.teams_total + p.bv.n_seqs) + team0 + b;
-    int32_t *cursor = p.team_cursor + (size_t)j * p.bv.teams_total + team0;
+    // team sizes -> row offsets; then the rows in member order, a warp's 32 at a time, each at its team's cursor
     int carry = 0;
-    for (int base = 0; base < slots; base += kThreads) {
-        const int g = base + threadIdx.x;
-        const int v = g < M ? csr[1 + g] : 0;
+    for (int u0 = 0; u0 < r; u0 += kThreads) {
+        const int u = u0 + tid, n = u < r ? count[u] : 0;
         int total;
-        const int excl = block_exclusive_scan(v, scratch, total);
-        if (g < slots) {
-            csr[1 + g] = g < M ? carry + excl + v : N;
-            cursor[g] = g < M ? carry + excl : N;
+        const int start = carry + block_exclusive_scan(n, scan_s, total);
+        if (u < r) {
+            start_s[u] = start;
+            t.csr[1 + u] = s0 + start + n;
         }
         carry += total;
     }
-    if (threadIdx.x == 0) csr[0] = 0;
-}
-
-// One warp per row: copy the K/V rows to their packed position.
-__global__ void __launch_bounds__(kThreads)
-pack_rows_kernel(ParentBuildParams p)
-{
-    const int b = blockIdx.y, j = blockIdx.z;
-    const int64_t row0 = p.bv.seq_row_off[b];
-    const int N = (int)(p.bv.seq_row_off[b + 1] - row0);
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-    if (i >= N) return;
-    const size_t plane = (size_t)j * p.bv.rows_total + row0;
-    const int d = p.dest[plane + i];
-    const uint2 *ksrc = reinterpret_cast<const uint2 *>(p.k_prompt) + (plane + i) * 32;
-    const uint2 *vsrc = reinterpret_cast<const uint2 *>(p.v_prompt) + (plane + i) * 32;
-    uint2 *kdst = reinterpret_cast<uint2 *>(p.k_packed) + (plane + d) * 32;
-    uint2 *vdst = reinterpret_cast<uint2 *>(p.v_packed) + (plane + d) * 32;
-    kdst[lane] = ksrc[lane];
-    vdst[lane] = vsrc[lane];
-    if (lane == 0) p.row_token[plane + d] = i;
+    __syncthreads();
+    for (int i0 = 0; i0 < nC; i0 += kThreads) {
+        const int i = i0 + tid;
+        const int own = i < nC ? owner[i] : kMaxParent + lane;    // idle lanes stay alone
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, own);
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        int pos = 0;
+        for (int w = 0; w < kThreads / 32; ++w) {
+            if (w == warp) {
+                if (i < nC) pos = start_s[own] + rank;
+                __syncwarp();
+                if (i < nC && rank == 0) start_s[own] += __popc(peers);
+            }
+            __syncthreads();
+        }
+        for (int l = 0; l < 32 && i0 + warp * 32 + l < nC; ++l) copy_row(t, mem[i0 + warp * 32 + l], s0 + __shfl_sync(0xFFFFFFFFu, pos, l));
+    }
+    uint32_t m = 0u;
+    uint32_t *rep_dst = reinterpret_cast<uint32_t *>(p.rep_keys) + t.rep0 * 64;
+    for (int e = tid; e < r * 64; e += kThreads) {
+        const uint32_t w = reinterpret_cast<const uint32_t *>(kbase + (size_t)mem[rep_pos[e >> 6]] * 16)[e & 63];
+        rep_dst[e] = w;
+        m = max(m, magnitude2(w));
+    }
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if (lane == 0) raise_abs_max<kHalf>(t.abs_max, m);
+  }
 }
 
 }  // namespace
@@ -415,39 +489,41 @@ cudaError_t launch_assign_parents(const AssignParams &p, cudaStream_t s)
     return p.elem ? launch_assign<true>(p, s) : launch_assign<false>(p, s);
 }
 
+template <bool kHalf>
+static cudaError_t launch_parents(const ParentBuildParams &p, cudaStream_t s)
+{
+    const int B = p.bv.n_seqs, H = p.bv.n_kv, sms = attend_grid_size();
+    cudaError_t err;
+    if (p.mean_keys) return launch_step(huge_parents_kernel<kHalf>, dim3(p.max_labels_per_seq, B, H), dim3(kThreads), 0, s, p);
+    // the few large parents first: theirs are the longest blocks
+    if ((err = launch_step(huge_parents_kernel<kHalf>, dim3(sms), dim3(kThreads), 0, s, p)) != cudaSuccess) return err;
+    static std::atomic<unsigned long long> large_done, mid_done;
+    using Large = LargeSmem<8, 2>;
+    using Mid = LargeSmem<4, 1>;
+    if ((err = ensure_dynamic_smem((const void *)large_parents_kernel<8, 2, kHalf>, (int)sizeof(Large), large_done)) != cudaSuccess) return err;
+    if ((err = ensure_dynamic_smem((const void *)large_parents_kernel<4, 1, kHalf>, (int)sizeof(Mid), mid_done)) != cudaSuccess) return err;
+    if ((err = launch_step(large_parents_kernel<8, 2, kHalf>, dim3(sms), dim3(256), sizeof(Large), s, p, 1)) != cudaSuccess) return err;
+    if ((err = launch_step(large_parents_kernel<4, 1, kHalf>, dim3(3 * sms), dim3(128), sizeof(Mid), s, p, 0)) != cudaSuccess) return err;
+    return launch_step(small_parents_kernel<kHalf>, dim3((p.max_labels_per_seq + kSmallParentWarps - 1) / kSmallParentWarps, B, H),
+                       dim3(kSmallParentWarps * 32), 0, s, p);
+}
+
 cudaError_t launch_build_teams_parents(const ParentBuildParams &p, cudaStream_t s)
 {
     const int B = p.bv.n_seqs, H = p.bv.n_kv;
-    cudaError_t err = cudaMemsetAsync(p.parent_cursor, 0, sizeof(int32_t) * (size_t)H * p.labels_total, s);
+    cudaError_t err = cudaMemsetAsync(p.list_count, 0, sizeof(int32_t) * 3, s);
     if (err != cudaSuccess) return err;
     // representative keys of the empty slots are zero
     err = cudaMemsetAsync(p.rep_keys, 0, sizeof(uint16_t) * (size_t)H * p.bv.teams_total * kHeadDim, s);
     if (err != cudaSuccess) return err;
-    count_labels_kernel<<<dim3((p.max_rows_per_seq + kThreads - 1) / kThreads, B, H), kThreads, 0, s>>>(p);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    scan_parents_kernel<<<dim3(B, H), kThreads, 0, s>>>(p);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    // cursors in shared memory when a sequence's labels (teams: at most reps per label) fit
-    const int lab_smem = std::min(p.max_labels_per_seq, kScatterSmemLabels);
-    const long long max_teams = (long long)p.max_labels_per_seq * p.reps;
-    const int team_smem = (int)std::min<long long>(max_teams, kScatterSmemLabels);
-    if ((err = cudaFuncSetAttribute(stable_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(int32_t) * kScatterSmemLabels)) != cudaSuccess) return err;
-    if ((err = cudaFuncSetAttribute(stable_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sizeof(int32_t) * kScatterSmemLabels)) != cudaSuccess) return err;
-    stable_scatter_kernel<true><<<dim3(B, H), kThreads, sizeof(int32_t) * (size_t)lab_smem, s>>>(
-        p.parent_of, p.parent_cursor, p.members, p.bv.seq_row_off, p.seq_label_off, p.bv.rows_total, p.labels_total, lab_smem);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    if (p.bv.elem) build_parent_general_kernel<true><<<dim3(p.max_labels_per_seq, B, H), kThreads, 0, s>>>(p);
-    else           build_parent_general_kernel<false><<<dim3(p.max_labels_per_seq, B, H), kThreads, 0, s>>>(p);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    scan_teams_kernel<<<dim3(B, H), kThreads, 0, s>>>(p);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    stable_scatter_kernel<false><<<dim3(B, H), kThreads, sizeof(int32_t) * (size_t)team_smem, s>>>(
-        p.team_of, p.team_cursor, p.dest, p.bv.seq_row_off, p.bv.seq_team_off, p.bv.rows_total, p.bv.teams_total, team_smem);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    pack_rows_kernel<<<dim3((p.max_rows_per_seq + kThreads / 32 - 1) / (kThreads / 32), B, H), kThreads, 0, s>>>(p);
-    return cudaGetLastError();
+    static std::atomic<unsigned long long> rank_done;
+    const int smem_labels = std::min(p.max_labels_per_seq, kHistSmemLabels);
+    if ((err = ensure_dynamic_smem((const void *)rank_labels_kernel, (int)sizeof(int32_t) * kHistSmemLabels, rank_done)) != cudaSuccess) return err;
+    if ((err = launch_step(rank_labels_kernel, dim3(p.chunks, B, H), dim3(kRankThreads), sizeof(int32_t) * (size_t)smem_labels, s, p, smem_labels)) != cudaSuccess)
+        return err;
+    if ((err = launch_step(scan_parents_kernel, dim3(B, H), dim3(kScanThreads), 0, s, p)) != cudaSuccess) return err;
+    if ((err = launch_step(members_kernel, dim3((p.max_rows_per_seq + kThreads - 1) / kThreads, B, H), dim3(kThreads), 0, s, p)) != cudaSuccess) return err;
+    return p.bv.elem ? launch_parents<true>(p, s) : launch_parents<false>(p, s);
 }
 
 }  // namespace santapp

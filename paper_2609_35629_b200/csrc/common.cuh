@@ -290,17 +290,19 @@ struct ParentBuildParams {
     const int64_t *seq_label_off;           // device [n_seqs + 1]
     uint16_t *k_packed, *v_packed, *rep_keys;
     int32_t *team_row_start, *row_token, *team_count;
+    float *rep_abs_max;                     // [n_kv][n_seqs], zero before the kernels
+    int chunks;                             // pieces a sequence's tokens are ranked in
     // workspace
     int32_t *parent_start;                  // [n_kv][labels_total + n_seqs] member-list offsets
-    int32_t *parent_cursor;                 // [n_kv][labels_total] counts, then scatter cursors
     int32_t *parent_team_base;              // [n_kv][labels_total] first team of each parent
+    int32_t *label_hist;                    // [n_kv][chunks][labels_total] tokens of each label in a chunk, then in the chunks before
+    int32_t *rank;                          // [n_kv][rows_total] rank of a token among those of its label in its chunk
     int32_t *members;                       // [n_kv][rows_total] tokens ordered by (label, index)
-    int32_t *team_of;                       // [n_kv][rows_total] team of each token
-    double *mind;                           // [n_kv][rows_total] distance to the nearest representative
+    int2 *list[3];                          // parents of 33..128, 129..512 and more rows: (pair, label)
+    int32_t *list_count;                    // [3]
+    double *mind;                           // [n_kv][rows_total] (huge parents) distance to the nearest representative
     int32_t *owner;                         // [n_kv][rows_total] its rank inside the parent
     unsigned char *is_rep;                  // [n_kv][rows_total]
-    int32_t *team_cursor;                   // [n_kv][teams_total]
-    int32_t *dest;                          // [n_kv][rows_total] packed position of each token
 };
 cudaError_t launch_build_teams_parents(const ParentBuildParams &p, cudaStream_t s);
 

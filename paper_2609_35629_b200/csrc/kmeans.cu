@@ -525,6 +525,7 @@ km_start_kernel(KmeansParams p)
     }
     if (tid < kStartBlocks) sm.touched[tid] = tid < mb ? 1u : 0u;
     if (tid == 0) sm.pick[0][0] = first;
+    for (int e = tid; e < kStartMaxCluster * kStartTrials; e += kStartThreads) sm.gain[0][e] = make_float2(0.f, 0.f);
     cluster_barrier();                                      // every block of the cluster runs: its shared memory may be written
 
     for (int c = 0; c < q.k; ++c) {
@@ -632,8 +633,12 @@ km_start_kernel(KmeansParams p)
             {
                 // every warp for itself; 1e-5: rounding of the fp32 sums; 1e-11: of the fp64 sums that define the potentials
                 float gl = 0.f, gh = 0.f;
-                if (lane < L)
-                    for (int r = 0; r < n_blk; ++r) { gl += sm.gain[r][lane].x; gh += sm.gain[r][lane].y; }
+#pragma unroll
+                for (int r = 0; r < kStartMaxCluster; ++r) {     // (zero past the cluster's blocks)
+                    const float2 v = sm.gain[r][min(lane, L - 1)];
+                    gl += v.x;
+                    gh += v.y;
+                }
                 const float slack = (float)(1e-11 * sm.pre[nb - 1]);
                 gl = lane < L ? gl * (1.f - 1e-5f) - slack : -CUDART_INF_F;
                 gh = gh * (1.f + 1e-5f);
