@@ -509,8 +509,8 @@ namespace {
 constexpr int kKmeansMaxSample = 28544;     // 223 KB of fp64 running sums (plus their block offsets): up to 9514 centres per sequence
 
 struct KmeansLayout {
-    size_t row_off, cen_off, tabs, perm, closest, cand, part, pick, chosen, centres64, count, idx, label, dist, centre_hi, centre_mid, centre_bias, near_top, near_nx, sorted, start, state, active, total;
-    int k_max, n_init_max, trials_max, t_max_max, max_rows, assign_split;
+    size_t row_off, cen_off, tabs, perm, closest, cand, part, pick, chosen, centres64, count, idx, label, dist, centre_hi, centre_bias, near_top, near_nx, sorted, start, state, active, total;
+    int k_max, n_init_max, trials_max, t_max_max, max_rows, scan_blocks, scan_segs;
     int64_t rows_total, centres_total;
 };
 
@@ -563,15 +563,14 @@ int kmeans_layout(const santapp_geom *geom, const int32_t *prompt_len_host, cons
     L->count = take(sizeof(double) * H * (size_t)L->centres_total);
     L->idx = take(sizeof(int32_t) * pairs * (size_t)o->batch_size);
     L->label = take(sizeof(int32_t) * pairs * (size_t)o->batch_size);
-    L->dist = take(sizeof(double) * pairs * (size_t)o->batch_size);
+    L->dist = take(sizeof(double) * 2 * pairs * (size_t)o->batch_size);
     L->centre_hi = take(sizeof(uint16_t) * H * (size_t)L->centres_total * kHeadDim);
-    L->centre_mid = take(sizeof(uint16_t) * H * (size_t)L->centres_total * kHeadDim);
-    L->centre_bias = take(sizeof(float) * H * (size_t)L->centres_total);
-    // the scan of a minibatch is cut into as many slices of the centres as fit on 148 SMs at once (two blocks each),
-    // but none shorter than two stages of 64
-    const int64_t blocks = (int64_t)pairs * ((o->batch_size + 255) / 256);
-    L->assign_split = std::max(1, (int)std::min<int64_t>(2 * 148 / blocks, L->k_max / 128));
-    L->near_top = take(kNearTopBytes * pairs * (size_t)L->assign_split * (size_t)o->batch_size);
+    L->centre_bias = take(sizeof(float2) * H * (size_t)L->centres_total);
+    // the pairs' scans share the blocks that 148 SMs hold at once (two each); no block takes less than a tile
+    const int tiles = (o->batch_size + 255) / 256, k_tiles = (L->k_max + 63) / 64;
+    L->scan_blocks = std::max(1, std::min((int)(2 * 148 / pairs), tiles * k_tiles));
+    L->scan_segs = L->scan_blocks / tiles + 2;
+    L->near_top = take(kNearTopBytes * pairs * (size_t)L->scan_segs * (size_t)o->batch_size);
     L->near_nx = take(sizeof(float) * pairs * (size_t)o->batch_size);
     L->sorted = take(sizeof(int32_t) * pairs * 4096);
     L->start = take(sizeof(int32_t) * pairs * ((size_t)L->k_max + 1));
@@ -678,12 +677,12 @@ int santapp_kmeans_fit(const santapp_geom *geom, const int32_t *prompt_len_host,
     p.label = reinterpret_cast<int32_t *>(ws + L.label);
     p.dist = reinterpret_cast<double *>(ws + L.dist);
     p.centre_hi = reinterpret_cast<uint16_t *>(ws + L.centre_hi);
-    p.centre_mid = reinterpret_cast<uint16_t *>(ws + L.centre_mid);
-    p.centre_bias = reinterpret_cast<float *>(ws + L.centre_bias);
+    p.centre_bias = reinterpret_cast<float2 *>(ws + L.centre_bias);
     p.near_top = reinterpret_cast<NearTop *>(ws + L.near_top);
     p.near_nx = reinterpret_cast<float *>(ws + L.near_nx);
     p.start = reinterpret_cast<int32_t *>(ws + L.start);
-    p.assign_split = L.assign_split;
+    p.scan_blocks = L.scan_blocks;
+    p.scan_segs = L.scan_segs;
     p.sorted = reinterpret_cast<int32_t *>(ws + L.sorted);
     p.state = reinterpret_cast<KmeansState *>(ws + L.state);
     p.active = reinterpret_cast<int *>(ws + L.active);

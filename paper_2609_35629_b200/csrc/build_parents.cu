@@ -27,7 +27,7 @@ constexpr int kThreads = 256;
 __device__ __forceinline__ int clamp_label(int v, int n) { return min(max(v, 0), n - 1); }
 
 // ---- Algorithm 3, assignment step: b_i = argmin_u |k_i - mu_u|^2, ties to the smaller u ----
-// A block takes 256 tokens and scans all centres (nearest.cuh), which it splits into their 16-bit halves as it
+// A block takes 256 tokens and scans all centres (nearest.cuh), which it rounds to 16 bits as it
 // brings them into shared memory (a quarter of a row per thread). Only tokens whose bounds leave more than
 // one centre see fp64. 4 x 32768 tokens, 2048 centres: 6.7 ms with every distance in fp64.
 template <bool kHalf>
@@ -45,12 +45,11 @@ assign_parents_kernel(AssignParams p)
     const int k = (int)(p.seq_centre_off[b + 1] - c0off);
     const uint16_t *keys = p.k_prompt + ((size_t)j * p.rows_total + row0) * kHeadDim;
     const float *cen = p.centres + ((size_t)j * p.centres_total + c0off) * kHeadDim;
-    if (tid == 0) sm.largest = 0.f;
     uint32_t a[2][8][4];
     near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)min(i0 + i, N - 1) * kHeadDim; }, a);
     near_scan<kHalf>(sm, a, 0, k, [&](int stage, int base, int n) {
         const int row = tid >> 2, part = tid & 3;            // 32 values: four 16-byte pieces of each half
-        float nc = 0.f;
+        float nc = 0.f, m = 0.f;
         if (row < n) {
             const float *src = cen + (size_t)(base + row) * kHeadDim + part * 32;
             const bool wide = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
@@ -64,44 +63,43 @@ assign_parents_kernel(AssignParams p)
 #pragma unroll
                     for (int e = 0; e < 8; ++e) v[e] = __ldg(src + 8 * c + e);
                 }
-                uint32_t hi[4], mid[4];
+                uint32_t hi[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     hi[e] = pack_elems<kHalf>(v[2 * e], v[2 * e + 1]);
-                    mid[e] = pack_elems<kHalf>(v[2 * e] - elem_lo<kHalf>(hi[e]), v[2 * e + 1] - elem_hi<kHalf>(hi[e]));
+                    const float r0 = v[2 * e] - elem_lo<kHalf>(hi[e]), r1 = v[2 * e + 1] - elem_hi<kHalf>(hi[e]);
                     nc = fmaf(v[2 * e], v[2 * e], fmaf(v[2 * e + 1], v[2 * e + 1], nc));
+                    m = fmaf(r0, r0, fmaf(r1, r1, m));
                 }
-                sm.ring[stage][0][near_piece(row, part * 4 + c)] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                sm.ring[stage][1][near_piece(row, part * 4 + c)] = make_uint4(mid[0], mid[1], mid[2], mid[3]);
+                sm.ring[stage][near_piece(row, part * 4 + c)] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             }
         }
-        nc += __shfl_xor_sync(0xFFFFFFFFu, nc, 1);
-        nc += __shfl_xor_sync(0xFFFFFFFFu, nc, 2);
-        const float bias = row < n ? centre_bias<kHalf>(nc) : CUDART_INF_F;
-        if (row < n && !(bias > -CUDART_INF_F))              // fp32 cannot hold its norm: no part in the products
-            for (int c = 0; c < 4; ++c)
-                sm.ring[stage][0][near_piece(row, part * 4 + c)] = sm.ring[stage][1][near_piece(row, part * 4 + c)] = make_uint4(0u, 0u, 0u, 0u);
-        if (part == 0) {
-            sm.bias[stage][row] = bias;
-            if (row < n && nc <= 1e37f) atomicMax(reinterpret_cast<uint32_t *>(&sm.largest), __float_as_uint(nc));
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) {
+            nc += __shfl_xor_sync(0xFFFFFFFFu, nc, o);
+            m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
         }
+        const float bias = row < n ? centre_bias<kHalf>(nc) : CUDART_INF_F;
+        const bool fits = bias > -CUDART_INF_F;              // else: no part in the products
+        if (row < n && !fits)
+            for (int c = 0; c < 4; ++c) sm.ring[stage][near_piece(row, part * 4 + c)] = make_uint4(0u, 0u, 0u, 0u);
+        m = fits ? 1.00001f * sqrtf(m) : 0.f;
+        if (part == 0) sm.bias[stage][row] = make_float2(bias, m);
     });
     __syncthreads();
     const int i = i0 + tid;
     const bool live = i < N;
     const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)min(i, N - 1) * kHeadDim);
     const NearTop top = sm.top[tid];
-    const float nx = sm.nx[tid];
     int arg = top.i1;
-    bool all = !(nx <= 1e37f) || !(fabsf(top.t1) < CUDART_INF_F);
-    if (!all && live && !(top.t2 > top.t1 + near_slack<kHalf>(nx, sm.largest))) {
-        float nc = 0.f;
-        for (int d = 0; d < kHeadDim; ++d) { const float v = cen[(size_t)arg * kHeadDim + d]; nc = fmaf(v, v, nc); }
-        const float bar = top.t1 + near_slack<kHalf>(nx, nc);
-        all = !(top.t3 > bar);
-        if (!all && !(top.t2 > bar)) {
-            const double d1 = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim), d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
-            if (d2 < d1 || (d2 == d1 && top.i2 < arg)) arg = top.i2;
+    const bool all = near_open(top, sm.nx[tid]);
+    if (live && !all && !(top.t2 > top.upper)) {
+        double best = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim);
+        const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
+        if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
+        if (!(top.t3 > top.upper)) {
+            const double d3 = near_exact<kHalf>(x, cen + (size_t)top.i3 * kHeadDim);
+            if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
         }
     }
     for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {

@@ -308,9 +308,10 @@ cudaError_t launch_build_teams_parents(const ParentBuildParams &p, cudaStream_t 
 
 // Minibatch k-means fit (second line of Algorithm 3), one problem per (sequence, KV head).
 struct NearTop;
-constexpr size_t kNearTopBytes = 20;
+constexpr size_t kNearTopBytes = 32;
 struct KmeansState {
     double ewa, ewa_min;                    // averaged per-point inertia and its minimum so far
+    double partial;                         // inertia of the step under way, as far as it is summed
     int bad, steps, stopped, pad;
 };
 struct KmeansParams {
@@ -336,12 +337,12 @@ struct KmeansParams {
     double *centres64;                      // [n_kv][centres_total][128]
     double *count;                          // [n_kv][centres_total]
     int32_t *idx, *label;                   // [pairs][batch]
-    double *dist;                           // [pairs][batch]
-    uint16_t *centre_hi, *centre_mid;       // [n_kv][centres_total][128] the centres as two 16-bit vectors (nearest.cuh)
-    float *centre_bias;                     // [n_kv][centres_total]
-    NearTop *near_top;                      // [pairs][assign_split][batch] the scan's result inside each slice of the centres
+    double *dist;                           // [2][pairs][batch] by parity of the step
+    uint16_t *centre_hi;                    // [n_kv][centres_total][128] the centres rounded to the element type (nearest.cuh)
+    float2 *centre_bias;                    // [n_kv][centres_total] constants of their bounds
+    NearTop *near_top;                      // [pairs][scan_segs][batch] the scan's results
     float *near_nx;                         // [pairs][batch] squared norms of the minibatch's points
-    int assign_split;                       // slices the centres are cut into for the scan
+    int scan_blocks, scan_segs;             // blocks that scan for a pair, and how many of them a point can meet
     int32_t *sorted;                        // [pairs][4096] the minibatch's points ordered by (label, slot)
     int32_t *start;                         // [pairs][k_max + 1] where each label starts there
     KmeansState *state;                     // [pairs]

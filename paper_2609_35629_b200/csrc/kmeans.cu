@@ -325,7 +325,7 @@ km_accept_kernel(KmeansParams p, int c)
 //   1. multiply their rows with the trial points on tensor cores, mark the points that a trial may lower, add up
 //      each trial's largest and smallest possible gain, and exchange the sums (distributed shared memory);
 //   2. take the trial whose smallest gain exceeds every other's largest; if there is none, the potentials are
-//      summed in fp64 for all trials (about one centre in a hundred; trials that drew the same point do not count);
+//      summed in fp64 for all trials (a few centres in two thousand; trials that drew the same point do not count);
 //   3. evaluate the winner's marked points in fp64 (a handful, after the first hundred centres), lower the
 //      distances, renew the running sums of the blocks of the sums they lie in, and exchange those blocks' sums;
 //   4. add up the blocks and draw the next trial points: the block that owns a drawn point sends its row to all.
@@ -375,8 +375,7 @@ __device__ __forceinline__ uint32_t in_block(uint32_t addr, uint32_t rank)      
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// Every thread of the cluster. Not the .aligned forms: lanes may arrive one by one after a divergent branch (a lane that
-// still runs a serial sum while its warp arrives counted the warp twice).
+// Every thread of the cluster; the warp has to be whole (it is brought together first).
 __device__ __forceinline__ void cluster_barrier()
 {
     __syncwarp();
@@ -827,39 +826,40 @@ cudaError_t launch_start(const KmeansParams &p, int pairs, int n_blk, cudaStream
 // ---- 3. minibatch steps ----
 // A step is five kernels: the scan for the nearest centres (nearest.cuh), the fp64 distance to the one found,
 // the minibatch ordered by centre, the update, the reassignment of starved centres. The inertia of a
-// minibatch is a sum of `batch` terms in order -- 4096 dependent additions, 20 us -- and only decides whether
-// another step follows, so it is taken by one block per pair beside the next step's scan, which reads nothing
-// that it writes; from the kernel after that on, a fit that has stopped does nothing. At 4 pairs, batch
-// 4096 and 2048 centres a step was 0.94 ms (0.84 of it fp64 distances to every centre).
+// minibatch is a sum of `batch` terms in order -- 4096 dependent additions, 18 us -- and only decides whether
+// the next step's update is still made. An extra block per pair in each of the five kernels from the update on takes
+// a fifth of it, so it is over when the next update starts and costs no time of its own; from then on a fit
+// that has stopped does nothing. At 4 pairs, batch 4096 and 2048 centres a step was 0.94 ms (0.84 of it fp64
+// distances to every centre).
 __device__ __forceinline__ bool pair_active(const KmeansParams &p, const Pair &q, int t)
 {
     return t < q.t_max && !p.state[q.id].stopped;
 }
 
-// Four components of a centre per lane of a warp: the fp64 centre, its 16-bit split and its bound constant.
+// Four components of a centre per lane of a warp: the fp64 centre, its 16-bit rounding and its bound constants.
 template <bool kHalf>
 __device__ __forceinline__ void store_centre(const KmeansParams &p, size_t centre, const double (&v)[4])
 {
     const int lane = threadIdx.x & 31;
-    uint16_t hi[4], mid[4];
-    float n = 0.f;
+    uint16_t hi[4];
+    float n = 0.f, m = 0.f;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        split_component<kHalf>(v[e], hi[e], mid[e]);
+        hi[e] = double_to_elem<kHalf>(v[e]);
+        const float r = (float)(v[e] - elem_to_double<kHalf>(hi[e]));
         n = fmaf((float)v[e], (float)v[e], n);
+        m = fmaf(r, r, m);
     }
     n = warp_sum(n);
+    m = 1.00001f * sqrtf(warp_sum(m));
     const float bias = centre_bias<kHalf>(n);
     const bool fits = bias > -CUDART_INF_F;
     double2 *to = reinterpret_cast<double2 *>(p.centres64 + centre * kHeadDim + 4 * lane);
     to[0] = make_double2(v[0], v[1]);
     to[1] = make_double2(v[2], v[3]);
-    auto pack = [&](const uint16_t (&h)[4]) {
-        return fits ? make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16)) : make_uint2(0u, 0u);
-    };
-    reinterpret_cast<uint2 *>(p.centre_hi + centre * kHeadDim)[lane] = pack(hi);
-    reinterpret_cast<uint2 *>(p.centre_mid + centre * kHeadDim)[lane] = pack(mid);
-    if (lane == 0) p.centre_bias[centre] = bias;
+    reinterpret_cast<uint2 *>(p.centre_hi + centre * kHeadDim)[lane] =
+        fits ? make_uint2((uint32_t)hi[0] | ((uint32_t)hi[1] << 16), (uint32_t)hi[2] | ((uint32_t)hi[3] << 16)) : make_uint2(0u, 0u);
+    if (lane == 0) p.centre_bias[centre] = make_float2(bias, fits ? m : 0.f);
 }
 
 // The centres that the start chose (sample indices), their counts and the fits' state at zero. A warp per centre.
@@ -870,7 +870,7 @@ km_prepare_kernel(KmeansParams p)
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     const int u = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0, 0, 0, 0};
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0.0, 0, 0, 0, 0};
     if (u >= q.k) return;
     const int row = p.perm[q.plane + p.chosen[q.cplane + u]];
     const uint2 w = reinterpret_cast<const uint2 *>(p.k_prompt + (q.plane + row) * kHeadDim)[lane];
@@ -879,22 +879,31 @@ km_prepare_kernel(KmeansParams p)
     if (lane == 0) p.count[q.cplane + u] = 0.0;
 }
 
-// Averaged inertia of step t and the stopping rule, one block per pair. The sum of the minibatch distances in
-// order runs on one thread over shared memory that all threads filled.
-__device__ __forceinline__ void km_stop_rule(const KmeansParams &p, const Pair &q, int t, double *dist_s)
+// Parts [part, part_end) of kInertiaParts of the inertia of step t, one block per pair; after the last part the averaged
+// inertia and the stopping rule. A part's terms go through shared memory: one thread adds them in order.
+constexpr int kInertiaParts = 5, kInertiaTerms = 4096 / kInertiaParts + 1;
+__device__ __forceinline__ void km_inertia(const KmeansParams &p, const Pair &q, int t, int part, int part_end, double *term_s)
 {
     if (t < 0 || !pair_active(p, q, t)) return;
-    const double *dist = p.dist + (size_t)q.id * p.batch;
-    for (int s = threadIdx.x; s < p.batch; s += blockDim.x) dist_s[s] = dist[s];
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    double inertia = 0.0;
-#pragma unroll 16
-    for (int s = 0; s < p.batch; ++s) inertia = __dadd_rn(inertia, dist_s[s]);
     KmeansState &st = p.state[q.id];
+    const double *dist = p.dist + ((size_t)(t & 1) * p.n_seqs * p.n_kv + q.id) * p.batch;
+    double sum = part > 0 ? st.partial : 0.0;
+    for (; part < part_end; ++part) {
+        const int lo = (int)((long long)part * p.batch / kInertiaParts), n = (int)((long long)(part + 1) * p.batch / kInertiaParts) - lo;
+        __syncthreads();
+        for (int s = threadIdx.x; s < n; s += blockDim.x) term_s[s] = dist[lo + s];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+#pragma unroll 16
+            for (int s = 0; s < n; ++s) sum = __dadd_rn(sum, term_s[s]);
+        }
+    }
+    if (threadIdx.x != 0) return;
+    st.partial = sum;
+    if (part < kInertiaParts) return;
     double alpha = __ddiv_rn(__dmul_rn(2.0, (double)p.batch), __dadd_rn((double)q.N, 1.0));
     if (alpha > 1.0) alpha = 1.0;
-    const double per_point = __ddiv_rn(inertia, (double)p.batch);
+    const double per_point = __ddiv_rn(sum, (double)p.batch);
     const double ewa = t == 0 ? per_point
                               : __dadd_rn(__dmul_rn(st.ewa, __dsub_rn(1.0, alpha)), __dmul_rn(per_point, alpha));
     st.ewa = ewa;
@@ -903,16 +912,32 @@ __device__ __forceinline__ void km_stop_rule(const KmeansParams &p, const Pair &
     else if (++st.bad >= p.patience) st.stopped = 1;
 }
 
+// After the last step: what is left of its inertia (its update and reassignment kernels took two parts).
 __global__ void __launch_bounds__(kThreads)
-km_last_stop_rule_kernel(KmeansParams p, int t)
+km_last_inertia_kernel(KmeansParams p, int t)
 {
-    __shared__ double dist_s[4096];
+    __shared__ double term_s[kInertiaTerms];
     step_wait();
-    km_stop_rule(p, pair_of(p, blockIdx.x / p.n_kv, blockIdx.x % p.n_kv), t, dist_s);
+    km_inertia(p, pair_of(p, blockIdx.x / p.n_kv, blockIdx.x % p.n_kv), t, 2, kInertiaParts, term_s);
 }
 
-// Draw the minibatch and scan the centres for each point's nearest: block (256 points, pair, slice of the
-// centres). Blocks of slice `assign_split` take the stopping rule of the step before instead.
+// A pair's minibatch as tiles of 256 points, its centres as tiles of 64: their products in row-major order are cut
+// into equal ranges, one per block of the pair. A block leaves one NearTop per point and tile of points it touches.
+struct ScanSplit {
+    int k_tiles, units, blocks;
+    __device__ int start(int i) const { return (int)((long long)i * units / blocks); }
+    __device__ int block_of(int unit) const { return (int)(((long long)(unit + 1) * blocks - 1) / units); }
+};
+__device__ __forceinline__ ScanSplit scan_split(const KmeansParams &p, const Pair &q)
+{
+    ScanSplit s;
+    s.k_tiles = (q.k + kNearTile - 1) / kNearTile;
+    s.units = s.k_tiles * ((p.batch + kNearPoints - 1) / kNearPoints);
+    s.blocks = min(p.scan_blocks, s.units);
+    return s;
+}
+
+// Draw the minibatch and scan the centres for each point's nearest.
 template <bool kHalf>
 __global__ void __launch_bounds__(kNearThreads, 2)
 km_scan_kernel(KmeansParams p, int t)
@@ -922,95 +947,121 @@ km_scan_kernel(KmeansParams p, int t)
     __shared__ int idx_s[kNearPoints];
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
-    const int slice = blockIdx.z, tid = threadIdx.x;
-    if (slice == p.assign_split) {
-        if (blockIdx.x == 0) km_stop_rule(p, q, t - 1, reinterpret_cast<double *>(smem_raw));
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x == p.scan_blocks) {
+        km_inertia(p, q, t - 1, 2, 3, reinterpret_cast<double *>(smem_raw));
         return;
     }
-    if (!pair_active(p, q, t)) return;                      // (a fit that is being stopped now may still be scanned)
-    const int per = ((q.k + p.assign_split - 1) / p.assign_split + kNearTile - 1) / kNearTile * kNearTile;
-    const int k_lo = min(slice * per, q.k), k_hi = min(k_lo + per, q.k);
-    const int s = blockIdx.x * kNearPoints + tid;
-    idx_s[tid] = km_index(km_word(p, (uint32_t)(s < p.batch ? s : 0), kTagBatch, q.stream, (uint32_t)t), q.N);
-    if (slice == 0 && s < p.batch) p.idx[(size_t)q.id * p.batch + s] = idx_s[tid];
-    __syncwarp();
+    if (!pair_active(p, q, t)) return;
+    const ScanSplit sp = scan_split(p, q);
+    if ((int)blockIdx.x >= sp.blocks) return;
     const uint16_t *keys = p.k_prompt + q.plane * kHeadDim;
-    uint32_t a[2][8][4];
-    near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)idx_s[i] * kHeadDim; }, a);
     const uint4 *hi = reinterpret_cast<const uint4 *>(p.centre_hi + q.cplane * kHeadDim);
-    const uint4 *mid = reinterpret_cast<const uint4 *>(p.centre_mid + q.cplane * kHeadDim);
-    const float *bias = p.centre_bias + q.cplane;
-    near_scan<kHalf>(sm, a, k_lo, k_hi, [&](int stage, int base, int n) {
+    const float2 *bias = p.centre_bias + q.cplane;
+    const int end = sp.start(blockIdx.x + 1);
+    for (int unit = sp.start(blockIdx.x); unit < end;) {
+        const int tile = unit / sp.k_tiles, k0 = unit - tile * sp.k_tiles, k1 = min(sp.k_tiles, k0 + end - unit);
+        const int s = tile * kNearPoints + tid;
+        idx_s[tid] = km_index(km_word(p, (uint32_t)(s < p.batch ? s : 0), kTagBatch, q.stream, (uint32_t)t), q.N);
+        if (k0 == 0 && s < p.batch) p.idx[(size_t)q.id * p.batch + s] = idx_s[tid];
+        __syncwarp();
+        uint32_t a[2][8][4];
+        near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)idx_s[i] * kHeadDim; }, a);
+        near_scan<kHalf>(sm, a, k0 * kNearTile, min(k1 * kNearTile, q.k), [&](int stage, int base, int n) {
 #pragma unroll
-        for (int m = 0; m < kNearTile * 16 / kNearThreads; ++m) {
-            const int e = m * kNearThreads + tid, row = e >> 4, ch = e & 15;
-            if (row < n) {
-                copy16_async(shared_addr(&sm.ring[stage][0][near_piece(row, ch)]), hi + (size_t)base * 16 + e);
-                copy16_async(shared_addr(&sm.ring[stage][1][near_piece(row, ch)]), mid + (size_t)base * 16 + e);
+            for (int m = 0; m < kNearTile * 16 / kNearThreads; ++m) {
+                const int e = m * kNearThreads + tid, row = e >> 4;
+                if (row < n) copy16_async(shared_addr(&sm.ring[stage][near_piece(row, e & 15)]), hi + (size_t)base * 16 + e);
             }
+            if (tid < kNearTile) sm.bias[stage][tid] = tid < n ? bias[base + tid] : make_float2(CUDART_INF_F, 0.f);
+        });
+        if (s < p.batch) {
+            const int seg = (int)blockIdx.x - sp.block_of(tile * sp.k_tiles);
+            p.near_top[((size_t)q.id * p.scan_segs + seg) * p.batch + s] = sm.top[tid];
+            if (k0 == 0) p.near_nx[(size_t)q.id * p.batch + s] = sm.nx[tid];
         }
-        if (tid < kNearTile) sm.bias[stage][tid] = tid < n ? bias[base + tid] : CUDART_INF_F;
-    });
-    if (s < p.batch) {
-        p.near_top[((size_t)q.id * p.assign_split + slice) * p.batch + s] = sm.top[tid];
-        if (slice == 0) p.near_nx[(size_t)q.id * p.batch + s] = sm.nx[tid];
+        unit += k1 - k0;
+        __syncthreads();                                    // sm.top, sm.nx and idx_s are read
     }
 }
 
-// The nearest centre of each minibatch point and the fp64 distance to it: the slices' results merged, the
-// candidates that the bounds leave open compared in fp64. A thread per point.
-constexpr int kResolveThreads = 64;
+// The nearest centre of each minibatch point and the fp64 distance to it: the scan's results merged, the
+// candidates that the bounds leave open compared in fp64. A warp takes 32 points: the terms of each distance are
+// formed by all lanes (coalesced reads, four conversions a lane), then every lane adds up its own point's in order.
+constexpr int kResolveWarps = 2, kTermPitch = kHeadDim + 1;
 template <bool kHalf>
-__global__ void __launch_bounds__(kResolveThreads)
+__global__ void __launch_bounds__(kResolveWarps * 32)
 km_resolve_kernel(KmeansParams p, int t)
 {
+    extern __shared__ double term_s[];                      // [warps][32][kTermPitch]
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
+    if (blockIdx.x == gridDim.x - 1) {
+        km_inertia(p, q, t - 1, 3, 4, term_s);
+        return;
+    }
     if (!pair_active(p, q, t)) return;
-    const int s = blockIdx.x * kResolveThreads + threadIdx.x, lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, s = blockIdx.x * kResolveWarps * 32 + threadIdx.x;
     const bool live = s < p.batch;
     const size_t at = (size_t)q.id * p.batch + (live ? s : 0);
-    const uint4 *x = reinterpret_cast<const uint4 *>(p.k_prompt + (q.plane + (size_t)p.idx[at]) * kHeadDim);
+    const int point = p.idx[at];
     const double *cen = p.centres64 + q.cplane * kHeadDim;
-    NearTop top = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, 0, 0};
-    for (int slice = 0; slice < p.assign_split; ++slice)
-        near_merge(top, p.near_top[((size_t)q.id * p.assign_split + slice) * p.batch + (live ? s : 0)]);
+    const ScanSplit sp = scan_split(p, q);
+    const int tile = (live ? s : 0) / kNearPoints;
+    const int segs = sp.block_of(tile * sp.k_tiles + sp.k_tiles - 1) - sp.block_of(tile * sp.k_tiles) + 1;
+    NearTop top = near_none(0);
+    for (int seg = 0; seg < segs; ++seg) near_merge(top, p.near_top[((size_t)q.id * p.scan_segs + seg) * p.batch + (live ? s : 0)]);
     const float nx = p.near_nx[at];
-    bool all = !(nx <= 1e37f) || !(fabsf(top.t1) < CUDART_INF_F);
+    const bool all = near_open(top, nx);
     int arg = top.i1;
-    double best = CUDART_INF;
-    if (!all) {
-        const float bar = top.t1 + near_slack<kHalf>(nx, p.centre_bias[q.cplane + top.i1] * (1.f + 2.f * kNearErr));
-        all = !(top.t3 > bar);
-        if (!all) {
-            best = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim);
-            if (!(top.t2 > bar)) {
-                const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
-                if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
-            }
+    double *term = term_s + (size_t)(threadIdx.x >> 5) * 32 * kTermPitch;
+    const uint16_t *keys = p.k_prompt + q.plane * kHeadDim;
+#pragma unroll 4
+    for (int l = 0; l < 32; ++l) {
+        const uint16_t *x = keys + (size_t)__shfl_sync(0xFFFFFFFFu, point, l) * kHeadDim;
+        const double *c = cen + (size_t)__shfl_sync(0xFFFFFFFFu, arg, l) * kHeadDim;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double d = __dsub_rn(elem_to_double<kHalf>(__ldg(x + 32 * e + lane)), c[32 * e + lane]);
+            term[l * kTermPitch + 32 * e + lane] = __dmul_rn(d, d);
+        }
+    }
+    __syncwarp();
+    double best = 0.0;
+#pragma unroll 16
+    for (int d = 0; d < kHeadDim; ++d) best = __dadd_rn(best, term[lane * kTermPitch + d]);
+    if (live && !all) {
+        const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)point * kHeadDim);
+        if (!(top.t2 > top.upper)) {
+            const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
+            if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
+        }
+        if (!(top.t3 > top.upper)) {
+            const double d3 = near_exact<kHalf>(x, cen + (size_t)top.i3 * kHeadDim);
+            if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
         }
     }
     for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
         const int l = __ffs(left) - 1;
-        const uint4 *xl = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)x, l));
+        const uint4 *xl = reinterpret_cast<const uint4 *>(keys + (size_t)__shfl_sync(0xFFFFFFFFu, point, l) * kHeadDim);
         double d;
         const int u = near_scan_exact<kHalf>(xl, cen, q.k, d);
         if (lane == l) { best = d; arg = u; }
     }
     if (live) {
         p.label[at] = arg;
-        p.dist[at] = best;
+        p.dist[((size_t)(t & 1) * p.n_seqs * p.n_kv + q.id) * p.batch + s] = best;
     }
 }
 
 // The minibatch ordered by (label, slot), one block per pair: two stable counting passes over the label's digits
-// (kSortBits each), then where each label starts. A thread holds four consecutive entries; ranks of equal
-// digits come from the warp (in order) and from counts of the warps before. (A bitonic sort of the same
-// keys took 24 us.)
-constexpr int kSortThreads = 1024, kSortKeys = 4096, kSortBits = 7, kSortDigits = 1 << kSortBits, kSortWarps = kSortThreads / 32;
+// (8 bits each: a fit has at most 28544 centres), then where each label starts. A thread holds four entries; ranks of
+// equal digits come from the warp (in order) and from counts of the warps before. (A bitonic sort of the same keys
+// took 24 us.)
+constexpr int kSortThreads = 1024, kSortKeys = 4096, kSortBits = 8, kSortDigits = 1 << kSortBits, kSortWarps = kSortThreads / 32;
 struct SortSmem {
     uint32_t key[2][kSortKeys];                             // label << 12 | slot
-    uint16_t count[kSortDigits][kSortWarps + 1];
+    uint16_t count[kSortDigits][kSortWarps + 2];
     int scan[33];
 };
 __global__ void __launch_bounds__(kSortThreads)
@@ -1019,65 +1070,87 @@ km_sort_batch_kernel(KmeansParams p, int t)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
     step_wait();
-    const Pair q = pair_of(p, blockIdx.x / p.n_kv, blockIdx.x % p.n_kv);
+    const int pairs = p.n_seqs * p.n_kv, pair = blockIdx.x % pairs;
+    const Pair q = pair_of(p, pair / p.n_kv, pair % p.n_kv);
+    if ((int)blockIdx.x >= pairs) {
+        km_inertia(p, q, t - 1, 4, 5, reinterpret_cast<double *>(smem_raw));
+        return;
+    }
     if (!pair_active(p, q, t)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int s = tid; s < kSortKeys; s += kSortThreads)
-        sm.key[0][s] = s < p.batch ? ((uint32_t)p.label[(size_t)q.id * p.batch + s] << 12) | (uint32_t)s : 0xFFFFFFFFu;
+    const int32_t *idx = p.idx + (size_t)q.id * p.batch;
+    uint32_t key[4];                                        // the warp's 128 entries, 32 at a time in order
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int s = warp * 128 + c * 32 + lane;
+        key[c] = s < p.batch ? ((uint32_t)p.label[(size_t)q.id * p.batch + s] << 12) | (uint32_t)s : 0xFFFFFFFFu;
+    }
     for (int pass = 0; pass < 2; ++pass) {
         const int shift = 12 + pass * kSortBits;
-        for (int e = tid; e < kSortDigits * (kSortWarps + 1); e += kSortThreads) (&sm.count[0][0])[e] = 0;
+        for (int e = tid; e < kSortDigits * (kSortWarps + 2) / 2; e += kSortThreads) reinterpret_cast<uint32_t *>(&sm.count[0][0])[e] = 0u;
         __syncthreads();
-        uint32_t key[4];
         int digit[4], rank[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {                       // the warp's 128 entries, 32 at a time in order
-            key[c] = sm.key[pass][warp * 128 + c * 32 + lane];
+        for (int c = 0; c < 4; ++c) {
+            if (pass == 1) key[c] = sm.key[1][warp * 128 + c * 32 + lane];
             digit[c] = (int)((key[c] >> shift) & (kSortDigits - 1));
-            const unsigned same = __match_any_sync(0xFFFFFFFFu, digit[c]);
-            const int before = sm.count[digit[c]][warp];
-            rank[c] = before + __popc(same & ((1u << lane) - 1u));
+            unsigned same = 0xFFFFFFFFu;                    // lanes with the same digit
+#pragma unroll
+            for (int bit = 0; bit < kSortBits; ++bit) {
+                const bool on = (digit[c] >> bit) & 1;
+                const unsigned with = __ballot_sync(0xFFFFFFFFu, on);
+                same &= on ? with : ~with;
+            }
+            const unsigned before = same & ((1u << lane) - 1u);
+            const int base = sm.count[digit[c]][warp];
+            rank[c] = base + __popc(before);
             __syncwarp();
-            if ((same & ((1u << lane) - 1u)) == 0u) sm.count[digit[c]][warp] = (uint16_t)(before + __popc(same));
+            if (before == 0u) sm.count[digit[c]][warp] = (uint16_t)(base + __popc(same));
             __syncwarp();
         }
         __syncthreads();
-        // exclusive prefix over (digit, warp): thread = digit * 8 + part of four warps
+        // exclusive prefix over (digit, warp): thread = digit * 4 + part of eight warps
         {
-            const int d = tid >> 3, w0 = (tid & 7) * 4;
-            int n[4], sum = 0, total;
+            const int d = tid >> 2, w0 = (tid & 3) * 8;
+            int n[8], sum = 0, total;
 #pragma unroll
-            for (int w = 0; w < 4; ++w) { n[w] = sm.count[d][w0 + w]; sum += n[w]; }
+            for (int w = 0; w < 8; ++w) { n[w] = sm.count[d][w0 + w]; sum += n[w]; }
             int at = block_exclusive_scan(sum, sm.scan, total);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) { sm.count[d][w0 + w] = (uint16_t)at; at += n[w]; }
+            for (int w = 0; w < 8; ++w) { sm.count[d][w0 + w] = (uint16_t)at; at += n[w]; }
         }
         __syncthreads();
 #pragma unroll
         for (int c = 0; c < 4; ++c) sm.key[pass ^ 1][sm.count[digit[c]][warp] + rank[c]] = key[c];
         __syncthreads();
     }
-    const int32_t *idx = p.idx + (size_t)q.id * p.batch;
     int32_t *start = p.start + (size_t)q.id * (p.k_max + 1);
-    for (int s = tid; s < kSortKeys; s += kSortThreads) {
-        const uint32_t key = sm.key[0][s];
-        const int label = min((int)(key >> 12), q.k);       // (the padding sorts behind every label)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int s = c * kSortThreads + tid;
+        const uint32_t mine = sm.key[0][s];
+        const int label = min((int)(mine >> 12), q.k);      // (the padding sorts behind every label)
         const int prev = s > 0 ? min((int)(sm.key[0][s - 1] >> 12), q.k) : -1;
         for (int u = prev + 1; u <= label; ++u) start[u] = s;
         if (s == kSortKeys - 1)
             for (int u = label + 1; u <= q.k; ++u) start[u] = kSortKeys;
-        if (s < p.batch) p.sorted[(size_t)q.id * kSortKeys + s] = idx[key & 4095u];
+        if (s < p.batch) p.sorted[(size_t)q.id * kSortKeys + s] = idx[mine & 4095u];
     }
 }
 
 // Cumulative-count update, a warp per centre (four dimensions per lane): the centre's new points are added in
-// minibatch order, eight rows requested at a time; c <- (c * count + sum) / (count + n).
+// minibatch order; c <- (c * count + sum) / (count + n). The next 16 rows are on their way while 16 are added.
 template <bool kHalf>
 __global__ void __launch_bounds__(128)
 km_batch_update_kernel(KmeansParams p, int t)
 {
+    __shared__ double term_s[kInertiaTerms];
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
+    if (blockIdx.x == gridDim.x - 1) {
+        km_inertia(p, q, t, 0, 1, term_s);
+        return;
+    }
     if (!pair_active(p, q, t)) return;
     const int u = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (u >= q.k) return;
@@ -1090,12 +1163,27 @@ km_batch_update_kernel(KmeansParams p, int t)
     const double2 *from = reinterpret_cast<const double2 *>(p.centres64 + (q.cplane + u) * kHeadDim + 4 * lane);
     const double2 c0 = from[0], c1 = from[1];
     double sum[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i0 = lo; i0 < hi; i0 += 8) {
-        uint2 w[8];
+    constexpr int kAhead = 16;
+    int id = point[min(lo + lane, hi - 1)];                 // tokens of the 32 points from `lo` on
+    uint2 next[kAhead];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = __ldg(keys + (size_t)point[min(i0 + i, hi - 1)] * 32);
+    for (int i = 0; i < kAhead; ++i) {
+        const int tok = __shfl_sync(0xFFFFFFFFu, id, i);
+        if (lo + i < hi) next[i] = __ldg(keys + (size_t)tok * 32);
+    }
+    for (int i0 = lo; i0 < hi; i0 += kAhead) {
+        uint2 w[kAhead];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < kAhead; ++i) w[i] = next[i];
+        const bool second = ((i0 - lo) & kAhead) == 0;      // the next 16 are the second half of `id`
+        if (!second) id = point[min(i0 + kAhead + lane, hi - 1)];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            const int tok = __shfl_sync(0xFFFFFFFFu, id, second ? kAhead + i : i);
+            if (i0 + kAhead + i < hi) next[i] = __ldg(keys + (size_t)tok * 32);
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
             if (i0 + i >= hi) break;
             sum[0] = __dadd_rn(sum[0], (double)elem_lo<kHalf>(w[i].x));
             sum[1] = __dadd_rn(sum[1], (double)elem_hi<kHalf>(w[i].x));
@@ -1111,68 +1199,77 @@ km_batch_update_kernel(KmeansParams p, int t)
     if (lane == 0) p.count[q.cplane + u] = grown;
 }
 
-// Reassignment of starved centres, one block per pair.
+// Reassignment of starved centres, one block per pair (and one that takes a part of the inertia).
 template <bool kHalf>
 __global__ void __launch_bounds__(kThreads)
 km_reassign_kernel(KmeansParams p, int t)
 {
-    extern __shared__ int32_t slots[];                      // slots[batch], then move_centre[batch / 2]
-    __shared__ int n_move_s;
+    extern __shared__ __align__(16) int32_t slots[];        // slots[batch], then move_centre[batch / 2]
+    __shared__ int scan_s[33];
     __shared__ double cmin_s[kThreads / 32], cmax_s[kThreads / 32];
     step_wait();
     const Pair q = pair_of(p, blockIdx.x, blockIdx.y);
+    if (blockIdx.z == 1) {
+        km_inertia(p, q, t, 1, 2, reinterpret_cast<double *>(slots));
+        return;
+    }
     if (!(p.ratio > 0.0) || !pair_active(p, q, t)) return;
     const int tid = threadIdx.x;
     int32_t *move_centre = slots + p.batch;
     double *count = p.count + q.cplane;
-    {
-        double cmin = INFINITY, cmax = 0.0;                 // smallest and largest count: any order gives the same
-        for (int u = tid; u < q.k; u += kThreads) {
-            const double v = count[u];
-            if (v < cmin) cmin = v;
-            if (v > cmax) cmax = v;
-        }
+    auto reduce = [&](double v, bool smallest, double *scratch) {     // any order gives the same
         for (int o = 16; o > 0; o >>= 1) {
-            const double a = __shfl_xor_sync(0xffffffffu, cmin, o), b = __shfl_xor_sync(0xffffffffu, cmax, o);
-            if (a < cmin) cmin = a;
-            if (b > cmax) cmax = b;
+            const double w = __shfl_xor_sync(0xffffffffu, v, o);
+            if (smallest ? w < v : w > v) v = w;
         }
-        if ((tid & 31) == 0) { cmin_s[tid >> 5] = cmin; cmax_s[tid >> 5] = cmax; }
+        __syncthreads();
+        if ((tid & 31) == 0) scratch[tid >> 5] = v;
+        __syncthreads();
+        for (int w = 0; w < kThreads / 32; ++w)
+            if (smallest ? scratch[w] < v : scratch[w] > v) v = scratch[w];
+        return v;
+    };
+    double cmin = INFINITY, cmax = 0.0;
+    for (int u = tid; u < q.k; u += kThreads) {
+        const double v = count[u];
+        if (v < cmin) cmin = v;
+        if (v > cmax) cmax = v;
     }
-    __syncthreads();
-    if (tid == 0) {
-        int n_move = 0;
-        double cmin = INFINITY, cmax = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) {
-            if (cmin_s[w] < cmin) cmin = cmin_s[w];
-            if (cmax_s[w] > cmax) cmax = cmax_s[w];
-        }
-        const long long period = 10 + (long long)floor(cmin);
-        if (((long long)t + 1) % period == 0) {
-            const double thr = __dmul_rn(p.ratio, cmax);
-            const int cap = p.batch / 2;
-            double keep_min = INFINITY;
-            for (int u = 0; u < q.k; ++u) {
-                const double v = count[u];
-                if (v < thr && n_move < cap) move_centre[n_move++] = u;
-                else if (v < keep_min) keep_min = v;
-            }
-            if (n_move > 0) {
-                for (int s = 0; s < p.batch; ++s) slots[s] = s;
-                for (int i = 0; i < n_move; ++i) {
-                    const int r = i + km_index(km_word(p, (uint32_t)i, kTagMove, q.stream, (uint32_t)t), p.batch - i);
-                    const int tmp = slots[i];
-                    slots[i] = slots[r];
-                    slots[r] = tmp;
-                }
-                for (int i = 0; i < n_move; ++i) count[move_centre[i]] = keep_min;
-            }
-        }
-        n_move_s = n_move;
+    cmin = reduce(cmin, true, cmin_s);
+    const long long period = 10 + (long long)floor(cmin);
+    if (((long long)t + 1) % period != 0) return;
+    cmax = reduce(cmax, false, cmax_s);
+    // the starved centres in order, at most batch / 2 of them; the smallest count among the others
+    const double thr = __dmul_rn(p.ratio, cmax);
+    const int cap = p.batch / 2;
+    int n_move = 0;
+    double keep_min = INFINITY;
+    for (int u0 = 0; u0 < q.k; u0 += kThreads) {
+        const int u = u0 + tid;
+        const double v = u < q.k ? count[u] : INFINITY;
+        const bool starved = u < q.k && v < thr;
+        int total;
+        const int at = n_move + block_exclusive_scan(starved ? 1 : 0, scan_s, total);
+        if (starved && at < cap) move_centre[at] = u;
+        else if (u < q.k && v < keep_min) keep_min = v;
+        n_move += total;
     }
+    n_move = min(n_move, cap);
+    if (n_move == 0) return;
+    keep_min = reduce(keep_min, true, cmin_s);
+    for (int s = tid; s < p.batch; s += kThreads) slots[s] = s;
     __syncthreads();
+    if (tid == 0)
+        for (int i = 0; i < n_move; ++i) {
+            const int r = i + km_index(km_word(p, (uint32_t)i, kTagMove, q.stream, (uint32_t)t), p.batch - i);
+            const int tmp = slots[i];
+            slots[i] = slots[r];
+            slots[r] = tmp;
+        }
+    __syncthreads();
+    for (int i = tid; i < n_move; i += kThreads) count[move_centre[i]] = keep_min;
     const int32_t *idx = p.idx + (size_t)q.id * p.batch;
-    for (int i = tid >> 5; i < n_move_s; i += kThreads / 32) {   // the moved centres jump onto minibatch points
+    for (int i = tid >> 5; i < n_move; i += kThreads / 32) {     // the moved centres jump onto minibatch points
         const uint2 w = reinterpret_cast<const uint2 *>(p.k_prompt + (q.plane + (size_t)idx[slots[i]]) * kHeadDim)[tid & 31];
         const double v[4] = {(double)elem_lo<kHalf>(w.x), (double)elem_hi<kHalf>(w.x), (double)elem_lo<kHalf>(w.y), (double)elem_hi<kHalf>(w.y)};
         store_centre<kHalf>(p, q.cplane + move_centre[i], v);
@@ -1233,19 +1330,20 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
     }
     const dim3 threads(kThreads);
     if ((err = launch_step(km_prepare_kernel<kHalf>, dim3((p.k_max + kThreads / 32 - 1) / (kThreads / 32), pairs), threads, 0, s, p)) != cudaSuccess) return err;
-    static std::atomic<unsigned long long> scan_done, sort_done;
+    static std::atomic<unsigned long long> scan_done, resolve_done, sort_done;
+    const size_t resolve_smem = sizeof(double) * kResolveWarps * 32 * kTermPitch;
     if ((err = ensure_dynamic_smem((const void *)km_scan_kernel<kHalf>, (int)sizeof(NearSmem), scan_done)) != cudaSuccess) return err;
+    if ((err = ensure_dynamic_smem((const void *)km_resolve_kernel<kHalf>, (int)resolve_smem, resolve_done)) != cudaSuccess) return err;
     if ((err = ensure_dynamic_smem((const void *)km_sort_batch_kernel, (int)sizeof(SortSmem), sort_done)) != cudaSuccess) return err;
-    const size_t move_smem = sizeof(int32_t) * ((size_t)p.batch + (size_t)p.batch / 2 + 1);
-    const dim3 scan_grid((p.batch + kNearPoints - 1) / kNearPoints, pairs, p.assign_split + 1);
-    const dim3 resolve_grid((p.batch + kResolveThreads - 1) / kResolveThreads, pairs);
+    const size_t move_smem = std::max(sizeof(int32_t) * ((size_t)p.batch + (size_t)p.batch / 2 + 1), sizeof(double) * (size_t)kInertiaTerms);
+    const dim3 resolve_grid((p.batch + kResolveWarps * 32 - 1) / (kResolveWarps * 32) + 1, pairs);
     int t = 0;
     for (; t < p.t_max_max; ++t) {
-        if ((err = launch_step(km_scan_kernel<kHalf>, scan_grid, dim3(kNearThreads), sizeof(NearSmem), s, p, t)) != cudaSuccess) return err;
-        if ((err = launch_step(km_resolve_kernel<kHalf>, resolve_grid, dim3(kResolveThreads), 0, s, p, t)) != cudaSuccess) return err;
-        if ((err = launch_step(km_sort_batch_kernel, dim3(pairs), dim3(kSortThreads), sizeof(SortSmem), s, p, t)) != cudaSuccess) return err;
-        if ((err = launch_step(km_batch_update_kernel<kHalf>, dim3((p.k_max + 3) / 4, pairs), dim3(128), 0, s, p, t)) != cudaSuccess) return err;
-        if ((err = launch_step(km_reassign_kernel<kHalf>, dim3(B, H), threads, move_smem, s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_scan_kernel<kHalf>, dim3(p.scan_blocks + 1, pairs), dim3(kNearThreads), sizeof(NearSmem), s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_resolve_kernel<kHalf>, resolve_grid, dim3(kResolveWarps * 32), resolve_smem, s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_sort_batch_kernel, dim3(2 * pairs), dim3(kSortThreads), sizeof(SortSmem), s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_batch_update_kernel<kHalf>, dim3((p.k_max + 3) / 4 + 1, pairs), dim3(128), 0, s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_reassign_kernel<kHalf>, dim3(B, H, 2), threads, move_smem, s, p, t)) != cudaSuccess) return err;
         if (!p.no_host_poll && (t + 1) % kPollEvery == 0 && t + 1 < p.t_max_max) {
             // most fits stop long before the step limit: ask the device how many are still running
             // (the copy into pageable memory returns when it has completed)
@@ -1257,7 +1355,7 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
             if (active == 0) { ++t; break; }
         }
     }
-    if ((err = launch_step(km_last_stop_rule_kernel, dim3(pairs), threads, 0, s, p, t - 1)) != cudaSuccess) return err;   // counts the last step
+    if ((err = launch_step(km_last_inertia_kernel, dim3(pairs), threads, 0, s, p, t - 1)) != cudaSuccess) return err;   // counts the last step
     km_finish_kernel<<<dim3((p.k_max * kHeadDim + kThreads - 1) / kThreads, B, H), kThreads, 0, s>>>(p);
     KM_CHECK();
 #undef KM_CHECK

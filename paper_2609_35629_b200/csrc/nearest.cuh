@@ -2,16 +2,16 @@
 // order, multiply and add rounded separately; ties to the smaller centre index), without evaluating most of
 // the fp64 distances.
 //
-// A centre is the sum of two 16-bit vectors, hi + mid (each component rounded twice to the points' element
-// type: within 2^-17 of it), so x.c comes from tensor cores as two products, and
-//   s_c = |c|^2 - 2 x.c      (the squared distance less |x|^2, the same for every centre)
-// orders the centres up to an error. With S = sum |x_d c_d| <= (|x|^2 + |c|^2) / 2: eight MMAs of 16 values in a
-// row cost at most 8 * 17 * 2^-23 S (see select_rows.cuh), what the split leaves out 2^-17 S, twice both: below
-// kNearErr (|x|^2 + |c|^2). The scan keeps, per point, the two smallest lower bounds s_c - kNearErr |c|^2 with
-// their centres and the third smallest; a centre whose lower bound exceeds the smallest by more than twice the
-// error of that one cannot be nearest. Usually that leaves one; where it leaves two they are compared in
-// fp64, where it leaves more all centres are (with early exit). fp16 halves below 2^-14 lose precision
-// absolutely, which adds a term in |x|; products that underflow fp32 add less than 1e-34.
+// A centre is rounded to a 16-bit vector `hi` (the points' element type); m = |c - hi|. With x.hi from tensor cores,
+//   s_c = |c|^2 - 2 x.hi      (the squared distance less |x|^2, the same for every centre)
+// orders the centres up to an error: what the rounding leaves out is at most 2 |x| m, eight MMAs of 16 values in a
+// row cost at most 8 * 17 * 2^-23 of sum |x_d hi_d| <= (1 + 2^-8) (|x|^2 + |c|^2) / 2 (see select_rows.cuh): together at most
+// E_c = kNearErr (|x|^2 + |c|^2) + 2 |x| m. The scan keeps, per point, the smallest upper bound so far, and of the centres
+// whose lower bound does not exceed it the three smallest lower bounds with their centres and the fourth smallest.
+// Usually one is left at the end; where two or three are, they are compared in fp64, where there are more all centres
+// are (with early exit). (A second product with c - hi would leave fewer open, for twice the MMAs. Keeping the
+// smallest lower bounds whatever the upper one took 79 us instead of 70 for 4 x 4096 points and 2048 centres:
+// every centre was inserted somewhere in a warp.) Products that underflow fp32 add less than 1e-34.
 #pragma once
 #include <math_constants.h>
 
@@ -20,25 +20,36 @@
 
 namespace santapp {
 
-constexpr float kNearErr = 2.6e-5f;
+constexpr float kNearErr = 2.2e-5f;
 constexpr int kNearPoints = 256;         // points per block
 constexpr int kNearThreads = 256;        // 8 warps of 32 points
 constexpr int kNearTile = 64;            // centres per shared-memory stage
 
-struct NearTop {                         // smallest lower bounds of a point, their centres, the third smallest
-    float t1, t2, t3;
-    int i1, i2;
+// Bounds leave out what all centres of a point share (its kNearErr |x|^2): lower s_c - kNearErr |c|^2 - 2 |x| m, and the
+// upper bound with that part counted twice.
+struct NearTop {                         // smallest lower bounds of a point, their centres, the fourth smallest; the smallest upper bound
+    float t1, t2, t3, t4, upper;
+    int i1, i2, i3;
 };
 static_assert(sizeof(NearTop) == kNearTopBytes, "the fit's workspace holds these");
+__device__ __forceinline__ NearTop near_none(int i)
+{
+    return {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, i, i, i};
+}
 __device__ __forceinline__ void near_insert(NearTop &n, float s, int i)
 {
-    if (s < n.t3) {
-        if (s < n.t2) {
-            n.t3 = n.t2;
-            if (s < n.t1) { n.t2 = n.t1; n.i2 = n.i1; n.t1 = s; n.i1 = i; }
-            else { n.t2 = s; n.i2 = i; }
+    if (s < n.t4) {
+        if (s < n.t3) {
+            n.t4 = n.t3;
+            if (s < n.t2) {
+                n.t3 = n.t2; n.i3 = n.i2;
+                if (s < n.t1) { n.t2 = n.t1; n.i2 = n.i1; n.t1 = s; n.i1 = i; }
+                else { n.t2 = s; n.i2 = i; }
+            } else {
+                n.t3 = s; n.i3 = i;
+            }
         } else {
-            n.t3 = s;
+            n.t4 = s;
         }
     }
 }
@@ -46,23 +57,15 @@ __device__ __forceinline__ void near_merge(NearTop &n, const NearTop &o)
 {
     near_insert(n, o.t1, o.i1);
     near_insert(n, o.t2, o.i2);
-    if (o.t3 < n.t3) n.t3 = o.t3;        // not below n.t2: o.t2 has been inserted
+    near_insert(n, o.t3, o.i3);
+    if (o.t4 < n.t4) n.t4 = o.t4;        // not below n.t3: the three before it have been inserted
+    n.upper = fminf(n.upper, o.upper);
 }
-// How far above the smallest lower bound (of a centre with squared norm nc) a rival's may lie.
-template <bool kHalf>
-__device__ __forceinline__ float near_slack(float nx, float nc)
-{
-    return 2.f * kNearErr * (nx + nc) + (kHalf ? 1.4e-6f * sqrtf(nx) : 0.f) + 1e-34f;
-}
+// Whether the bounds say too little, and all centres have to be compared.
+__device__ __forceinline__ bool near_open(const NearTop &n, float nx) { return !(nx <= 1e37f) || !(fabsf(n.t1) < CUDART_INF_F) || !(n.t4 > n.upper); }
 
-// A centre component as hi + mid. A centre with components beyond the element type, or whose squared norm fp32 cannot
-// hold, is stored as zeros with a bound of -inf: it is a candidate of every point.
-template <bool kHalf>
-__device__ __forceinline__ void split_component(double v, uint16_t &hi, uint16_t &mid)
-{
-    hi = double_to_elem<kHalf>(v);
-    mid = double_to_elem<kHalf>(v - elem_to_double<kHalf>(hi));
-}
+// A centre with components beyond the element type, or whose squared norm fp32 cannot hold, is stored as zeros with
+// a bound of -inf: it is a candidate of every point. Else: the lower bound's constant.
 template <bool kHalf>
 __device__ __forceinline__ float centre_bias(float nc) { return nc <= (kHalf ? 4.2e9f : 1e37f) ? nc * (1.f - kNearErr) : -CUDART_INF_F; }
 template <bool kHalf>
@@ -75,9 +78,9 @@ __device__ __forceinline__ uint32_t pack_elems(float lo, float hi)
 }
 
 struct NearSmem {
-    uint4 ring[2][2][kNearTile * 16];    // [stage][hi, mid]: 64 rows of 256 bytes, 16-byte pieces XOR-swizzled
-    float bias[2][kNearTile];
-    float largest;                       // largest squared norm among the centres (fp32 source only)
+    uint4 ring[4][kNearTile * 16];       // stages (and, all of it, the points before the scan): rows of 256 bytes, 16-byte pieces XOR-swizzled
+    float2 bias[2][kNearTile];           // constant of the lower bound, m
+    float list[7][kNearThreads * 4];     // a thread's four points (of which it sees a quarter of the centres): t1 .. t4, i1 .. i3
     NearTop top[kNearPoints];
     float nx[kNearPoints];
 };
@@ -89,7 +92,7 @@ template <bool kHalf, typename RowOf>
 __device__ __forceinline__ void near_load_points(NearSmem &sm, RowOf row_of, uint32_t (&a)[2][8][4])
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint4 *rows = &sm.ring[0][0][0];                        // 64 KB: the whole ring
+    uint4 *rows = &sm.ring[0][0];                           // 64 KB: the whole ring
 #pragma unroll 4
     for (int m = 0; m < 16; ++m) {                          // a warp copies its own 32 rows, two per step
         const int i = warp * 32 + 2 * m + (lane >> 4), ch = lane & 15;
@@ -132,9 +135,40 @@ template <bool kHalf, typename Fill>
 __device__ __forceinline__ void near_scan(NearSmem &sm, const uint32_t (&a)[2][8][4], int k_lo, int k_hi, Fill fill)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane & 3;
-    NearTop top[4];                                         // rows g, g + 8, g + 16, g + 24 of the warp's 32
+    // The thread's points are rows g, g + 8, g + 16, g + 24 of the warp's 32. Their lists are in shared memory: they are
+    // touched rarely, and would not fit in registers beside the points.
+    float reach[4], shared[4], upper[4];                    // 2 |x|, the part of the upper bound that all centres share
+    auto slot = [&](int r) { return &sm.list[0][r * kNearThreads + threadIdx.x]; };
+    constexpr int kWord = kNearThreads * 4;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) top[r] = {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, k_lo, k_lo};
+    for (int r = 0; r < 4; ++r) {
+        float *l = slot(r);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) l[w * kWord] = CUDART_INF_F;
+#pragma unroll
+        for (int w = 4; w < 7; ++w) l[w * kWord] = __int_as_float(k_lo);
+        const float nx = sm.nx[warp * 32 + 8 * r + (lane >> 2)];
+        reach[r] = 2.000002f * sqrtf(nx);
+        shared[r] = fmaf(2.f * kNearErr, nx, 1e-34f);
+        upper[r] = CUDART_INF_F;
+    }
+    auto load = [&](int r) {
+        const float *l = slot(r);
+        return NearTop{l[0], l[kWord], l[2 * kWord], l[3 * kWord], upper[r], __float_as_int(l[4 * kWord]), __float_as_int(l[5 * kWord]),
+                       __float_as_int(l[6 * kWord])};
+    };
+    auto insert = [&](int r, float s, int i) {
+        NearTop n = load(r);
+        near_insert(n, s, i);
+        float *l = slot(r);
+        l[0] = n.t1;
+        l[kWord] = n.t2;
+        l[2 * kWord] = n.t3;
+        l[3 * kWord] = n.t4;
+        l[4 * kWord] = __int_as_float(n.i1);
+        l[5 * kWord] = __int_as_float(n.i2);
+        l[6 * kWord] = __int_as_float(n.i3);
+    };
     fill(0, k_lo, min(kNearTile, k_hi - k_lo));
     asm volatile("cp.async.commit_group;");
     int stage = 0;
@@ -142,50 +176,78 @@ __device__ __forceinline__ void near_scan(NearSmem &sm, const uint32_t (&a)[2][8
         if (base + kNearTile < k_hi) fill(stage ^ 1, base + kNearTile, min(kNearTile, k_hi - base - kNearTile));
         asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
         __syncthreads();
-        const uint32_t hi_a = shared_addr(&sm.ring[stage][0][0]), mid_a = shared_addr(&sm.ring[stage][1][0]);
+        const uint32_t hi_a = shared_addr(&sm.ring[stage][0]);
 #pragma unroll 2
         for (int nt = 0; nt < kNearTile / 8; ++nt) {
-            const int row = nt * 8 + (lane & 7);
-            float ah[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, am[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            float acc[2][2][4];                             // two chains of four MMAs each per group of 16 points
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) acc[m][h][0] = acc[m][h][1] = acc[m][h][2] = acc[m][h][3] = 0.f;
 #pragma unroll
             for (int s2 = 0; s2 < 4; ++s2) {
-                uint32_t bh[4], bm[4];
-                const uint32_t at = (uint32_t)near_piece(row, 4 * s2 + (lane >> 3)) * 16u;
-                ldmatrix4(bh, hi_a + at);
-                ldmatrix4(bm, mid_a + at);
+                uint32_t bh[4];
+                ldmatrix4(bh, hi_a + (uint32_t)near_piece(nt * 8 + (lane & 7), 4 * s2 + (lane >> 3)) * 16u);
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
 #pragma unroll
                     for (int m = 0; m < 2; ++m) {
                         const uint32_t(&f)[4] = a[m][2 * s2 + h];
-                        mma_rows<kHalf>(ah[m], f[0], f[1], f[2], f[3], bh[2 * h], bh[2 * h + 1]);
-                        mma_rows<kHalf>(am[m], f[0], f[1], f[2], f[3], bm[2 * h], bm[2 * h + 1]);
+                        mma_rows<kHalf>(acc[m][h], f[0], f[1], f[2], f[3], bh[2 * h], bh[2 * h + 1]);
                     }
             }
-            const float2 bias = *reinterpret_cast<const float2 *>(&sm.bias[stage][nt * 8 + 2 * c]);
-            const int col = base + nt * 8 + 2 * c;
+            const float4 bias = *reinterpret_cast<const float4 *>(&sm.bias[stage][nt * 8 + 2 * c]);
+            float low[2][4];
+            bool some = false;
 #pragma unroll
             for (int m = 0; m < 2; ++m)
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    near_insert(top[2 * m + (e >> 1)], fmaf(-2.f, ah[m][e] + am[m][e], (e & 1) ? bias.y : bias.x), col + (e & 1));
+                for (int e = 0; e < 4; ++e) {
+                    const int r = 2 * m + (e >> 1);
+                    low[m][e] = fmaf(-2.f, acc[m][0][e] + acc[m][1][e], fmaf(-reach[r], (e & 1) ? bias.w : bias.y, (e & 1) ? bias.z : bias.x));
+                    some |= low[m][e] < upper[r];
+                }
+            if (some) {
+                const int col = base + nt * 8 + 2 * c;
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int r = 2 * m + (e >> 1);
+                        if (low[m][e] < upper[r]) {
+                            // (1.0001: the stored constant is |c|^2 (1 - kNearErr), rounded)
+                            const float wide = fmaf(1.0001f * kNearErr, (e & 1) ? bias.z : bias.x, reach[r] * ((e & 1) ? bias.w : bias.y));
+                            upper[r] = fminf(upper[r], fmaf(2.f, wide, low[m][e] + shared[r]));
+                            insert(r, low[m][e], col + (e & 1));
+                        }
+                    }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {                       // the four lanes of a point share its upper bound
+            upper[r] = fminf(upper[r], __shfl_xor_sync(0xFFFFFFFFu, upper[r], 1));
+            upper[r] = fminf(upper[r], __shfl_xor_sync(0xFFFFFFFFu, upper[r], 2));
         }
         __syncthreads();                                    // the stage may be filled again
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
+        NearTop top = load(r);
 #pragma unroll
         for (int o = 1; o <= 2; o <<= 1) {
             NearTop n;
-            n.t1 = __shfl_xor_sync(0xFFFFFFFFu, top[r].t1, o);
-            n.t2 = __shfl_xor_sync(0xFFFFFFFFu, top[r].t2, o);
-            n.t3 = __shfl_xor_sync(0xFFFFFFFFu, top[r].t3, o);
-            n.i1 = __shfl_xor_sync(0xFFFFFFFFu, top[r].i1, o);
-            n.i2 = __shfl_xor_sync(0xFFFFFFFFu, top[r].i2, o);
-            near_merge(top[r], n);
+            n.t1 = __shfl_xor_sync(0xFFFFFFFFu, top.t1, o);
+            n.t2 = __shfl_xor_sync(0xFFFFFFFFu, top.t2, o);
+            n.t3 = __shfl_xor_sync(0xFFFFFFFFu, top.t3, o);
+            n.t4 = __shfl_xor_sync(0xFFFFFFFFu, top.t4, o);
+            n.upper = top.upper;
+            n.i1 = __shfl_xor_sync(0xFFFFFFFFu, top.i1, o);
+            n.i2 = __shfl_xor_sync(0xFFFFFFFFu, top.i2, o);
+            n.i3 = __shfl_xor_sync(0xFFFFFFFFu, top.i3, o);
+            near_merge(top, n);
         }
-        if (c == 0) sm.top[warp * 32 + 8 * r + (lane >> 2)] = top[r];
+        if (c == 0) sm.top[warp * 32 + 8 * r + (lane >> 2)] = top;
     }
     __syncwarp();                                           // a warp's points are its own rows
 }

@@ -173,3 +173,22 @@ def test_fit_random_small_configurations(case):
     _fit_both(spec, n_centres, batch_size=int(rng.choice([16, 100, 512, 4096])), max_iter=int(rng.choice([1, 3, 100])),
               patience=int(rng.choice([1, 3, 10])), reassignment_ratio=float(rng.choice([0.0, 0.01, 0.5])),
               seed=int(rng.integers(1 << 62)), stream_base=int(rng.integers(1 << 30)))
+
+
+@pytest.mark.parametrize("n", [300, 12800, 17000])
+def test_fit_with_a_centre_per_key_returns_the_keys(n):
+    """k = N on distinct points: every greedy pick is a point that is no centre yet, every minibatch point is
+    its own centre, and with an inertia of zero the fit stops after one step and `patience` more. The sizes
+    take the start in one kernel, the start for samples beyond shared memory, and labels beyond 14 bits."""
+    bits = (np.arange(n)[:, None] >> np.arange(15)) & 1
+    rows = np.zeros((1, n, 128), dtype=np.float32)
+    rows[0, :, :15] = 3.0 * bits - 1.0
+    geom = sp.Geometry(1, 1, 1, 128, 16, 4)
+    k = torch.from_numpy(rows).cuda().to(torch.bfloat16)
+    centres, steps = sp.santapp_kmeans_fit(geom, [n], [n], k, reassignment_ratio=0.0, patience=3)
+    torch.cuda.synchronize()
+    assert int(steps[0, 0]) == 4
+    got = centres[0].cpu().numpy()
+    order = (((got[:, :15] + 1.0) / 3.0) @ (2.0 ** np.arange(15))).astype(np.int64)
+    assert np.array_equal(np.sort(order), np.arange(n))
+    assert np.array_equal(got, rows[0][order])
