@@ -567,7 +567,7 @@ int kmeans_layout(const santapp_geom *geom, const int32_t *prompt_len_host, cons
     L->centre_hi = take(sizeof(uint16_t) * H * (size_t)L->centres_total * kHeadDim);
     L->centre_bias = take(sizeof(float2) * H * (size_t)L->centres_total);
     // the pairs' scans share the blocks that 148 SMs hold at once (two each); no block takes less than a tile
-    const int tiles = (o->batch_size + 255) / 256, k_tiles = (L->k_max + 63) / 64;
+    const int tiles = (o->batch_size + 127) / 128, k_tiles = (L->k_max + 127) / 128;
     L->scan_blocks = std::max(1, std::min((int)(2 * 148 / pairs), tiles * k_tiles));
     L->scan_segs = L->scan_blocks / tiles + 2;
     L->near_top = take(kNearTopBytes * pairs * (size_t)L->scan_segs * (size_t)o->batch_size);

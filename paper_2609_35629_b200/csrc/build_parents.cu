@@ -27,15 +27,15 @@ constexpr int kThreads = 256;
 __device__ __forceinline__ int clamp_label(int v, int n) { return min(max(v, 0), n - 1); }
 
 // ---- Algorithm 3, assignment step: b_i = argmin_u |k_i - mu_u|^2, ties to the smaller u ----
-// A block takes 256 tokens and scans all centres (nearest.cuh), which it rounds to 16 bits as it
-// brings them into shared memory (a quarter of a row per thread). Only tokens whose bounds leave more than
-// one centre see fp64. 4 x 32768 tokens, 2048 centres: 6.7 ms with every distance in fp64.
+// A block takes 128 tokens and scans all centres (nearest.cuh), which it rounds to 16 bits as it brings them into shared
+// memory (half a row per thread). Only tokens whose bounds leave more than one centre see fp64. 4 x 32768 tokens,
+// 2048 centres: 6.7 ms with every distance in fp64.
 template <bool kHalf>
 __global__ void __launch_bounds__(kNearThreads, 2)
 assign_parents_kernel(AssignParams p)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    NearSmem &sm = *reinterpret_cast<NearSmem *>(smem_raw);
+    extern __shared__ __align__(1024) unsigned char near_smem[];
+    NearSmem &sm = *reinterpret_cast<NearSmem *>(near_smem);
     step_wait();
     const int b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
     const int64_t row0 = p.seq_row_off[b];
@@ -45,71 +45,81 @@ assign_parents_kernel(AssignParams p)
     const int k = (int)(p.seq_centre_off[b + 1] - c0off);
     const uint16_t *keys = p.k_prompt + ((size_t)j * p.rows_total + row0) * kHeadDim;
     const float *cen = p.centres + ((size_t)j * p.centres_total + c0off) * kHeadDim;
-    uint32_t a[2][8][4];
-    near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)min(i0 + i, N - 1) * kHeadDim; }, a);
-    near_scan<kHalf>(sm, a, 0, k, [&](int stage, int base, int n) {
-        const int row = tid >> 2, part = tid & 3;            // 32 values: four 16-byte pieces of each half
-        float nc = 0.f, m = 0.f;
-        if (row < n) {
-            const float *src = cen + (size_t)(base + row) * kHeadDim + part * 32;
-            const bool wide = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+    uint32_t uses[2] = {0u, 0u};
+    near_open_block(sm);
+    near_scan<kHalf>(sm, [&](int i) { return keys + (size_t)min(i0 + i, N - 1) * kHeadDim; }, 0, k, uses,
+                     [&](int stage, int slot, int base, int n) {
+        // eight lanes share a row: lane part takes pieces part and part + 8, a 32-byte run of the centre each
+        const int part = tid & 7;
+#pragma unroll 2
+        for (int r0 = 0; r0 < kNearTile; r0 += kNearThreads / 8) {
+            const int row = r0 + (tid >> 3);
+            float nc = 0.f, m = 0.f;
+            uint4 out[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+            if (row < n) {
+                const float *src = cen + (size_t)(base + row) * kHeadDim;
+                const bool wide = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float v[8];
-                if (wide) {
-                    const float4 v0 = __ldg(reinterpret_cast<const float4 *>(src + 8 * c)), v1 = __ldg(reinterpret_cast<const float4 *>(src + 8 * c + 4));
-                    v[0] = v0.x; v[1] = v0.y; v[2] = v0.z; v[3] = v0.w; v[4] = v1.x; v[5] = v1.y; v[6] = v1.z; v[7] = v1.w;
-                } else {
+                for (int c = 0; c < 2; ++c) {
+                    const float *from = src + 8 * (part + 8 * c);
+                    float v[8];
+                    if (wide) {
+                        const float4 v0 = __ldg(reinterpret_cast<const float4 *>(from)), v1 = __ldg(reinterpret_cast<const float4 *>(from + 4));
+                        v[0] = v0.x; v[1] = v0.y; v[2] = v0.z; v[3] = v0.w; v[4] = v1.x; v[5] = v1.y; v[6] = v1.z; v[7] = v1.w;
+                    } else {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) v[e] = __ldg(src + 8 * c + e);
+                        for (int e = 0; e < 8; ++e) v[e] = __ldg(from + e);
+                    }
+                    uint32_t hi[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        hi[e] = pack_elems<kHalf>(v[2 * e], v[2 * e + 1]);
+                        const float r0v = v[2 * e] - elem_lo<kHalf>(hi[e]), r1v = v[2 * e + 1] - elem_hi<kHalf>(hi[e]);
+                        nc = fmaf(v[2 * e], v[2 * e], fmaf(v[2 * e + 1], v[2 * e + 1], nc));
+                        m = fmaf(r0v, r0v, fmaf(r1v, r1v, m));
+                    }
+                    out[c] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                 }
-                uint32_t hi[4];
+            }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    hi[e] = pack_elems<kHalf>(v[2 * e], v[2 * e + 1]);
-                    const float r0 = v[2 * e] - elem_lo<kHalf>(hi[e]), r1 = v[2 * e + 1] - elem_hi<kHalf>(hi[e]);
-                    nc = fmaf(v[2 * e], v[2 * e], fmaf(v[2 * e + 1], v[2 * e + 1], nc));
-                    m = fmaf(r0, r0, fmaf(r1, r1, m));
-                }
-                sm.ring[stage][near_piece(row, part * 4 + c)] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            for (int o = 1; o <= 4; o <<= 1) {
+                nc += __shfl_xor_sync(0xFFFFFFFFu, nc, o);
+                m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
+            }
+            const float bias = row < n ? centre_bias<kHalf>(nc) : kNearFar;
+            const bool fits = row < n && bias > -kNearFar;  // else: no part in the products
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                *reinterpret_cast<uint4 *>(sm.centres[stage] + near_byte(row, part + 8 * c)) = fits ? out[c] : make_uint4(0u, 0u, 0u, 0u);
+            if (part == 0) sm.bias[slot][row] = make_float2(bias, fits ? 1.00001f * sqrtf(m) : 0.f);
+        }
+    });
+    if (tid < kNearPoints) {
+        const int i = i0 + tid;
+        const bool live = i < N;
+        const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)min(i, N - 1) * kHeadDim);
+        const NearTop top = sm.top[tid];
+        int arg = top.i1;
+        const bool all = near_open(top, sm.nx[tid]);
+        if (live && !all && !(top.t2 > top.upper)) {
+            double best = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim);
+            const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
+            if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
+            if (!(top.t3 > top.upper)) {
+                const double d3 = near_exact<kHalf>(x, cen + (size_t)top.i3 * kHeadDim);
+                if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
             }
         }
-#pragma unroll
-        for (int o = 1; o <= 2; o <<= 1) {
-            nc += __shfl_xor_sync(0xFFFFFFFFu, nc, o);
-            m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
+        for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
+            const int l = __ffs(left) - 1;
+            const uint4 *xl = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)x, l));
+            double d;
+            const int u = near_scan_exact<kHalf>(xl, cen, k, d);
+            if (lane == l) arg = u;
         }
-        const float bias = row < n ? centre_bias<kHalf>(nc) : CUDART_INF_F;
-        const bool fits = bias > -CUDART_INF_F;              // else: no part in the products
-        if (row < n && !fits)
-            for (int c = 0; c < 4; ++c) sm.ring[stage][near_piece(row, part * 4 + c)] = make_uint4(0u, 0u, 0u, 0u);
-        m = fits ? 1.00001f * sqrtf(m) : 0.f;
-        if (part == 0) sm.bias[stage][row] = make_float2(bias, m);
-    });
-    __syncthreads();
-    const int i = i0 + tid;
-    const bool live = i < N;
-    const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)min(i, N - 1) * kHeadDim);
-    const NearTop top = sm.top[tid];
-    int arg = top.i1;
-    const bool all = near_open(top, sm.nx[tid]);
-    if (live && !all && !(top.t2 > top.upper)) {
-        double best = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim);
-        const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
-        if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
-        if (!(top.t3 > top.upper)) {
-            const double d3 = near_exact<kHalf>(x, cen + (size_t)top.i3 * kHeadDim);
-            if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
-        }
+        if (live) p.parent_of[(size_t)j * p.rows_total + row0 + i] = arg;
     }
-    for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
-        const int l = __ffs(left) - 1;
-        const uint4 *xl = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)x, l));
-        double d;
-        const int u = near_scan_exact<kHalf>(xl, cen, k, d);
-        if (lane == l) arg = u;
-    }
-    if (live) p.parent_of[(size_t)j * p.rows_total + row0 + i] = arg;
+    near_close_block(sm);
 }
 
 // ---- member lists ----

@@ -853,7 +853,7 @@ __device__ __forceinline__ void store_centre(const KmeansParams &p, size_t centr
     n = warp_sum(n);
     m = 1.00001f * sqrtf(warp_sum(m));
     const float bias = centre_bias<kHalf>(n);
-    const bool fits = bias > -CUDART_INF_F;
+    const bool fits = bias > -kNearFar;
     double2 *to = reinterpret_cast<double2 *>(p.centres64 + centre * kHeadDim + 4 * lane);
     to[0] = make_double2(v[0], v[1]);
     to[1] = make_double2(v[2], v[3]);
@@ -921,7 +921,7 @@ km_last_inertia_kernel(KmeansParams p, int t)
     km_inertia(p, pair_of(p, blockIdx.x / p.n_kv, blockIdx.x % p.n_kv), t, 2, kInertiaParts, term_s);
 }
 
-// A pair's minibatch as tiles of 256 points, its centres as tiles of 64: their products in row-major order are cut
+// A pair's minibatch as tiles of 128 points, its centres as tiles of 128: their products in row-major order are cut
 // into equal ranges, one per block of the pair. A block leaves one NearTop per point and tile of points it touches.
 struct ScanSplit {
     int k_tiles, units, blocks;
@@ -942,14 +942,13 @@ template <bool kHalf>
 __global__ void __launch_bounds__(kNearThreads, 2)
 km_scan_kernel(KmeansParams p, int t)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    NearSmem &sm = *reinterpret_cast<NearSmem *>(smem_raw);
-    __shared__ int idx_s[kNearPoints];
+    extern __shared__ __align__(1024) unsigned char near_smem[];
+    NearSmem &sm = *reinterpret_cast<NearSmem *>(near_smem);
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     const int tid = threadIdx.x;
     if ((int)blockIdx.x == p.scan_blocks) {
-        km_inertia(p, q, t - 1, 2, 3, reinterpret_cast<double *>(smem_raw));
+        km_inertia(p, q, t - 1, 2, 3, reinterpret_cast<double *>(near_smem));
         return;
     }
     if (!pair_active(p, q, t)) return;
@@ -959,30 +958,34 @@ km_scan_kernel(KmeansParams p, int t)
     const uint4 *hi = reinterpret_cast<const uint4 *>(p.centre_hi + q.cplane * kHeadDim);
     const float2 *bias = p.centre_bias + q.cplane;
     const int end = sp.start(blockIdx.x + 1);
+    uint32_t uses[2] = {0u, 0u};
+    near_open_block(sm);
     for (int unit = sp.start(blockIdx.x); unit < end;) {
         const int tile = unit / sp.k_tiles, k0 = unit - tile * sp.k_tiles, k1 = min(sp.k_tiles, k0 + end - unit);
         const int s = tile * kNearPoints + tid;
-        idx_s[tid] = km_index(km_word(p, (uint32_t)(s < p.batch ? s : 0), kTagBatch, q.stream, (uint32_t)t), q.N);
-        if (k0 == 0 && s < p.batch) p.idx[(size_t)q.id * p.batch + s] = idx_s[tid];
-        __syncwarp();
-        uint32_t a[2][8][4];
-        near_load_points<kHalf>(sm, [&](int i) { return keys + (size_t)idx_s[i] * kHeadDim; }, a);
-        near_scan<kHalf>(sm, a, k0 * kNearTile, min(k1 * kNearTile, q.k), [&](int stage, int base, int n) {
+        if (tid < kNearPoints) {
+            sm.idx[tid] = km_index(km_word(p, (uint32_t)(s < p.batch ? s : 0), kTagBatch, q.stream, (uint32_t)t), q.N);
+            if (k0 == 0 && s < p.batch) p.idx[(size_t)q.id * p.batch + s] = sm.idx[tid];
+        }
+        __syncthreads();
+        near_scan<kHalf>(sm, [&](int i) { return keys + (size_t)sm.idx[i] * kHeadDim; }, k0 * kNearTile, min(k1 * kNearTile, q.k), uses,
+                         [&](int stage, int slot, int base, int n) {
 #pragma unroll
-            for (int m = 0; m < kNearTile * 16 / kNearThreads; ++m) {
-                const int e = m * kNearThreads + tid, row = e >> 4;
-                if (row < n) copy16_async(shared_addr(&sm.ring[stage][near_piece(row, e & 15)]), hi + (size_t)base * 16 + e);
-            }
-            if (tid < kNearTile) sm.bias[stage][tid] = tid < n ? bias[base + tid] : make_float2(CUDART_INF_F, 0.f);
-        });
-        if (s < p.batch) {
+                             for (int m = 0; m < kNearTile * 16 / kNearThreads; ++m) {
+                                 const int e = m * kNearThreads + tid, row = e >> 4;
+                                 copy16_or_zero(shared_addr(sm.centres[stage] + near_byte(row, e & 15)), hi + (size_t)(base + min(row, n - 1)) * 16 + (e & 15), row < n);
+                             }
+                             if (tid < kNearTile) sm.bias[slot][tid] = tid < n ? bias[base + tid] : make_float2(kNearFar, 0.f);
+                         });
+        if (tid < kNearPoints && s < p.batch) {
             const int seg = (int)blockIdx.x - sp.block_of(tile * sp.k_tiles);
             p.near_top[((size_t)q.id * p.scan_segs + seg) * p.batch + s] = sm.top[tid];
             if (k0 == 0) p.near_nx[(size_t)q.id * p.batch + s] = sm.nx[tid];
         }
         unit += k1 - k0;
-        __syncthreads();                                    // sm.top, sm.nx and idx_s are read
+        __syncthreads();                                    // sm.top, sm.nx and sm.idx are read
     }
+    near_close_block(sm);
 }
 
 // The nearest centre of each minibatch point and the fp64 distance to it: the scan's results merged, the

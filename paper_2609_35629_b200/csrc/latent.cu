@@ -30,6 +30,7 @@
 #include "santapp_latent.h"
 #include "score_tile.cuh"
 #include "select_rows.cuh"
+#include "tc.cuh"
 
 using namespace santapp;
 

@@ -47,30 +47,6 @@ constexpr int kTcWaitLimit = 1 << 22;
 
 enum { kBarFull = 0, kBarPvDone = 2, kBarSReady = 4, kBarSFree = 6, kBarPReady = 8 };
 
-__device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t leading_bytes, uint32_t stride_bytes)
-{
-    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((leading_bytes >> 4) & 0x3FFFu) << 16)
-           | ((uint64_t)((stride_bytes >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);      // version 1, no swizzle
-}
-__device__ __forceinline__ uint64_t tc_desc_sw128(uint32_t saddr, uint32_t leading_bytes, uint32_t stride_bytes)
-{
-    return tc_desc(saddr, leading_bytes, stride_bytes) | ((uint64_t)2 << 61);                // 128-byte swizzle
-}
-__device__ __forceinline__ uint32_t tc_idesc(int M, int N, int a_mn_major, int b_mn_major)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16)
-           | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);                       // fp32 accumulate, bf16 x bf16
-}
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-                 : "memory");
-}
-__device__ __forceinline__ void tc_commit(uint32_t bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -85,13 +61,6 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&v)[16])
                  "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
                  "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
                  : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // Wait until the phase of `bar` with index `use` (0, 1, 2, ... in the order the phases complete) is
 // over. The waiter is never more than one phase behind, so the parity identifies the phase.

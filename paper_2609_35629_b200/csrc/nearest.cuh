@@ -4,26 +4,33 @@
 //
 // A centre is rounded to a 16-bit vector `hi` (the points' element type); m = |c - hi|. With x.hi from tensor cores,
 //   s_c = |c|^2 - 2 x.hi      (the squared distance less |x|^2, the same for every centre)
-// orders the centres up to an error: what the rounding leaves out is at most 2 |x| m, eight MMAs of 16 values in a
-// row cost at most 8 * 17 * 2^-23 of sum |x_d hi_d| <= (1 + 2^-8) (|x|^2 + |c|^2) / 2 (see select_rows.cuh): together at most
-// E_c = kNearErr (|x|^2 + |c|^2) + 2 |x| m. The scan keeps, per point, the smallest upper bound so far, and of the centres
-// whose lower bound does not exceed it the three smallest lower bounds with their centres and the fourth smallest.
-// Usually one is left at the end; where two or three are, they are compared in fp64, where there are more all centres
-// are (with early exit). (A second product with c - hi would leave fewer open, for twice the MMAs. Keeping the
-// smallest lower bounds whatever the upper one took 79 us instead of 70 for 4 x 4096 points and 2048 centres:
-// every centre was inserted somewhere in a warp.) Products that underflow fp32 add less than 1e-34.
+// orders the centres up to an error: what the rounding leaves out is at most 2 |x| m; eight MMAs of 16 values in a
+// row cost at most 8 * 17 * 2^-23 of sum |x_d hi_d| <= (1 + 2^-8) (|x|^2 + |c|^2) / 2 (see select_rows.cuh), twice that for the
+// distance; the column of a centre, kept in the last five bits of its bound, 2^-18 of at most 2.04 (|x|^2 + |c|^2).
+// Together at most E_c = kNearErr (|x|^2 + |c|^2) + 2 |x| m. A centre can be nearest only if its lower bound does not exceed the
+// smallest upper bound; where that leaves two or three they are compared in fp64, where it leaves more all
+// centres are (with early exit). Products that underflow fp32 add less than 1e-34.
+//
+// The products are a GEMM (tcgen05, 128 points x 128 centres x 128 dimensions a tile, 512 cycles at the measured rate);
+// looking at 16384 results takes the block's eight warps about twice that, since every one costs two FMAs and four
+// minimum or logic operations at half rate, so two blocks share an SM and the tensor core is busy half the time. The
+// search is free of branches over a chunk of 32 centres (its two smallest bounds), because in a warp of 32
+// points some lane would take any branch that a new minimum takes: mma.sync with such a branch per value took
+// 70 us for 4 x 4096 points and 2048 centres, this 37.
 #pragma once
 #include <math_constants.h>
 
 #include "common.cuh"
 #include "select_rows.cuh"
+#include "tc.cuh"
 
 namespace santapp {
 
-constexpr float kNearErr = 2.2e-5f;
-constexpr int kNearPoints = 256;         // points per block
-constexpr int kNearThreads = 256;        // 8 warps of 32 points
-constexpr int kNearTile = 64;            // centres per shared-memory stage
+constexpr float kNearErr = 3.0e-5f;
+constexpr float kNearFar = 3.0e38f;      // a bound that says nothing: below -1e38, all centres have to be compared; above 1e38, no centre
+constexpr int kNearPoints = 128;         // points per block: the rows of an accumulator
+constexpr int kNearThreads = 256;        // warps w and w + 4 look at the two halves of the columns of points 32 (w & 3) ..
+constexpr int kNearTile = 128;           // centres per shared-memory stage: the columns
 
 // Bounds leave out what all centres of a point share (its kNearErr |x|^2): lower s_c - kNearErr |c|^2 - 2 |x| m, and the
 // upper bound with that part counted twice.
@@ -34,7 +41,7 @@ struct NearTop {                         // smallest lower bounds of a point, th
 static_assert(sizeof(NearTop) == kNearTopBytes, "the fit's workspace holds these");
 __device__ __forceinline__ NearTop near_none(int i)
 {
-    return {CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, CUDART_INF_F, i, i, i};
+    return {kNearFar, kNearFar, kNearFar, kNearFar, kNearFar, i, i, i};
 }
 __device__ __forceinline__ void near_insert(NearTop &n, float s, int i)
 {
@@ -62,12 +69,12 @@ __device__ __forceinline__ void near_merge(NearTop &n, const NearTop &o)
     n.upper = fminf(n.upper, o.upper);
 }
 // Whether the bounds say too little, and all centres have to be compared.
-__device__ __forceinline__ bool near_open(const NearTop &n, float nx) { return !(nx <= 1e37f) || !(fabsf(n.t1) < CUDART_INF_F) || !(n.t4 > n.upper); }
+__device__ __forceinline__ bool near_open(const NearTop &n, float nx) { return !(nx <= 1e37f) || !(fabsf(n.t1) < 1e38f) || !(n.t4 > n.upper); }
 
 // A centre with components beyond the element type, or whose squared norm fp32 cannot hold, is stored as zeros with
-// a bound of -inf: it is a candidate of every point. Else: the lower bound's constant.
+// a bound of -kNearFar: every point compares all centres. Else: the lower bound's constant.
 template <bool kHalf>
-__device__ __forceinline__ float centre_bias(float nc) { return nc <= (kHalf ? 4.2e9f : 1e37f) ? nc * (1.f - kNearErr) : -CUDART_INF_F; }
+__device__ __forceinline__ float centre_bias(float nc) { return nc <= (kHalf ? 4.2e9f : 1e37f) ? nc * (1.f - kNearErr) : -kNearFar; }
 template <bool kHalf>
 __device__ __forceinline__ uint32_t pack_elems(float lo, float hi)
 {
@@ -78,178 +85,172 @@ __device__ __forceinline__ uint32_t pack_elems(float lo, float hi)
 }
 
 struct NearSmem {
-    uint4 ring[4][kNearTile * 16];       // stages (and, all of it, the points before the scan): rows of 256 bytes, 16-byte pieces XOR-swizzled
-    float2 bias[2][kNearTile];           // constant of the lower bound, m
-    float list[7][kNearThreads * 4];     // a thread's four points (of which it sees a quarter of the centres): t1 .. t4, i1 .. i3
-    NearTop top[kNearPoints];
+    // K-major operands with the tensor core's 128-byte swizzle (near_byte)
+    alignas(1024) unsigned char points[kNearPoints * 256];
+    unsigned char centres[2][kNearTile * 256];
+    float2 bias[3][kNearTile];           // constant of the lower bound and m, by tile
     float nx[kNearPoints];
+    int idx[kNearPoints];                // for the caller: tokens of the points
+    NearTop top[kNearPoints];
+    uint64_t done[2];                    // mbarriers: the products in an accumulator buffer are there
+    uint32_t tmem;
+    int failed;                          // a wait ran out (never expected): all centres are compared
 };
-__device__ __forceinline__ int near_piece(int row, int chunk) { return row * 16 + (chunk ^ (row & 7)); }
-
-// The block's points as MMA operands: `row_of(i)` points to the 256 bytes of point i < kNearPoints (any valid
-// row for a point past the end). Every thread of the block calls it.
-template <bool kHalf, typename RowOf>
-__device__ __forceinline__ void near_load_points(NearSmem &sm, RowOf row_of, uint32_t (&a)[2][8][4])
+static_assert(kNearTile == kNearPoints, "both operands have one layout");
+// Byte of 16-byte piece ch of row r: atoms of 64 values of eight rows, pieces XOR-swizzled inside.
+__device__ __forceinline__ int near_byte(int r, int ch) { return (ch >> 3) * (kNearPoints * 128) + (r >> 3) * 1024 + (r & 7) * 128 + (((ch & 7) ^ (r & 7)) << 4); }
+__device__ __forceinline__ void copy16_or_zero(uint32_t dst, const void *src, bool real)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint4 *rows = &sm.ring[0][0];                           // 64 KB: the whole ring
-#pragma unroll 4
-    for (int m = 0; m < 16; ++m) {                          // a warp copies its own 32 rows, two per step
-        const int i = warp * 32 + 2 * m + (lane >> 4), ch = lane & 15;
-        copy16_async(shared_addr(rows + near_piece(i, ch)), reinterpret_cast<const uint4 *>(row_of(i)) + ch);
-    }
-    copy_async_wait();
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-        for (int s = 0; s < 8; ++s)
-            ldmatrix4(a[m][s], shared_addr(rows + near_piece(warp * 32 + 16 * m + (lane & 15), 2 * s + (lane >> 4))));
-    // squared norms, from the fragments: rows g and g + 8 of each group of 16
-    float n[2][2];
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-        n[m][0] = n[m][1] = 0.f;
-#pragma unroll
-        for (int s = 0; s < 8; ++s)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float x0 = elem_lo<kHalf>(a[m][s][r]), x1 = elem_hi<kHalf>(a[m][s][r]);
-                n[m][r & 1] = fmaf(x0, x0, fmaf(x1, x1, n[m][r & 1]));
-            }
-    }
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            n[m][h] += __shfl_xor_sync(0xFFFFFFFFu, n[m][h], 1);
-            n[m][h] += __shfl_xor_sync(0xFFFFFFFFu, n[m][h], 2);
-            if ((lane & 3) == 0) sm.nx[warp * 32 + 16 * m + 8 * h + (lane >> 2)] = n[m][h];
-        }
-    __syncthreads();                                        // the ring is free
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(real ? 16 : 0) : "memory");
 }
 
-// The scan over centres [k_lo, k_hi): `fill(stage, base, n)` brings centres [base, base + n) into a stage
-// (asynchronous copies of it are waited for here). Leaves the points' NearTop in sm.top.
-template <bool kHalf, typename Fill>
-__device__ __forceinline__ void near_scan(NearSmem &sm, const uint32_t (&a)[2][8][4], int k_lo, int k_hi, Fill fill)
+// Tensor memory (two accumulator buffers of kNearTile columns) and barriers; every thread of the block, at its
+// beginning and its end.
+__device__ __forceinline__ void near_open_block(NearSmem &sm)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane & 3;
-    // The thread's points are rows g, g + 8, g + 16, g + 24 of the warp's 32. Their lists are in shared memory: they are
-    // touched rarely, and would not fit in registers beside the points.
-    float reach[4], shared[4], upper[4];                    // 2 |x|, the part of the upper bound that all centres share
-    auto slot = [&](int r) { return &sm.list[0][r * kNearThreads + threadIdx.x]; };
-    constexpr int kWord = kNearThreads * 4;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        float *l = slot(r);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) l[w * kWord] = CUDART_INF_F;
-#pragma unroll
-        for (int w = 4; w < 7; ++w) l[w * kWord] = __int_as_float(k_lo);
-        const float nx = sm.nx[warp * 32 + 8 * r + (lane >> 2)];
-        reach[r] = 2.000002f * sqrtf(nx);
-        shared[r] = fmaf(2.f * kNearErr, nx, 1e-34f);
-        upper[r] = CUDART_INF_F;
+    if (threadIdx.x == 0) {
+        sm.failed = 0;
+        for (int i = 0; i < 2; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&sm.done[i])), "r"(1));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    auto load = [&](int r) {
-        const float *l = slot(r);
-        return NearTop{l[0], l[kWord], l[2 * kWord], l[3 * kWord], upper[r], __float_as_int(l[4 * kWord]), __float_as_int(l[5 * kWord]),
-                       __float_as_int(l[6 * kWord])};
-    };
-    auto insert = [&](int r, float s, int i) {
-        NearTop n = load(r);
-        near_insert(n, s, i);
-        float *l = slot(r);
-        l[0] = n.t1;
-        l[kWord] = n.t2;
-        l[2 * kWord] = n.t3;
-        l[3 * kWord] = n.t4;
-        l[4 * kWord] = __int_as_float(n.i1);
-        l[5 * kWord] = __int_as_float(n.i2);
-        l[6 * kWord] = __int_as_float(n.i3);
-    };
-    fill(0, k_lo, min(kNearTile, k_hi - k_lo));
-    asm volatile("cp.async.commit_group;");
-    int stage = 0;
-    for (int base = k_lo; base < k_hi; base += kNearTile, stage ^= 1) {
-        if (base + kNearTile < k_hi) fill(stage ^ 1, base + kNearTile, min(kNearTile, k_hi - base - kNearTile));
-        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(shared_addr(&sm.tmem)), "r"(2 * kNearTile) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+}
+__device__ __forceinline__ void near_close_block(NearSmem &sm)
+{
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(2 * kNearTile));
+}
+__device__ __forceinline__ void near_wait(NearSmem &sm, int buf, uint32_t parity)
+{
+    if (*reinterpret_cast<volatile int *>(&sm.failed)) return;
+    for (int i = 0; i < (1 << 20); ++i) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}\n"
+                     : "=r"(done) : "r"(shared_addr(&sm.done[buf])), "r"(parity) : "memory");
+        if (done) return;
+    }
+    sm.failed = 1;
+}
+
+// One point against 32 consecutive centres from `first` on: v their products with it, bias their constants.
+__device__ __forceinline__ void near_look(NearTop &n, const uint32_t (&v)[32], const float2 *bias, int first, float reach, float shared)
+{
+    float key[32], t1 = kNearFar, t2 = kNearFar;
+#pragma unroll
+    for (int c = 0; c < 32; c += 2) {
+        const float4 b = *reinterpret_cast<const float4 *>(bias + c);
+        const float l0 = fmaf(-2.f, __uint_as_float(v[c]), fmaf(-reach, b.y, b.x));
+        const float l1 = fmaf(-2.f, __uint_as_float(v[c + 1]), fmaf(-reach, b.w, b.z));
+        key[c] = __uint_as_float((__float_as_uint(l0) & ~31u) | (uint32_t)c);
+        key[c + 1] = __uint_as_float((__float_as_uint(l1) & ~31u) | (uint32_t)(c + 1));
+        t2 = fminf(t2, fmaxf(t1, key[c]));
+        t1 = fminf(t1, key[c]);
+        t2 = fminf(t2, fmaxf(t1, key[c + 1]));
+        t1 = fminf(t1, key[c + 1]);
+    }
+    if (t1 <= n.upper) {
+        const float2 b = bias[__float_as_uint(t1) & 31u];
+        // (1.0001: the stored constant is |c|^2 (1 - kNearErr), rounded)
+        n.upper = fminf(n.upper, fmaf(2.f, fmaf(1.0001f * kNearErr, b.x, reach * b.y), t1 + shared));
+    }
+    if (t1 <= n.upper) near_insert(n, t1, first + (int)(__float_as_uint(t1) & 31u));
+    while (__any_sync(0xFFFFFFFFu, t2 <= n.upper)) {         // some point of the warp has another candidate here
+        if (t2 <= n.upper) near_insert(n, t2, first + (int)(__float_as_uint(t2) & 31u));
+        float next = kNearFar;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) next = fminf(next, key[c] > t2 ? key[c] : kNearFar);
+        t2 = next < kNearFar ? next : CUDART_INF_F;
+    }
+}
+
+// The nearest centres among [k_lo, k_hi) of the block's points, left in sm.top (for all threads to read). `row_of(i)`
+// points to the 256 bytes of point i < kNearPoints (any valid row for a point past the end); `fill(stage, slot, base, n)`
+// brings centres [base, base + n) into a stage and their constants into a slot of the bias table, by asynchronous copies
+// or plain stores, with zeros and kNearFar behind them. `uses`: how often the accumulator buffers have been
+// waited for, kept by the caller, 0 at first.
+template <bool kHalf, typename RowOf, typename Fill>
+__device__ __forceinline__ void near_scan(NearSmem &sm, RowOf row_of, int k_lo, int k_hi, uint32_t (&uses)[2], Fill fill)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n_tiles = (k_hi - k_lo + kNearTile - 1) / kNearTile, row = 32 * (warp & 3) + lane;
+    fill(0, 0, k_lo, min(kNearTile, k_hi - k_lo));
+#pragma unroll
+    for (int m = 0; m < kNearPoints * 16 / kNearThreads; ++m) {
+        const int e = m * kNearThreads + tid;
+        copy16_async(shared_addr(sm.points + near_byte(e >> 4, e & 15)), reinterpret_cast<const uint4 *>(row_of(e >> 4)) + (e & 15));
+    }
+    NearTop top = near_none(k_lo);
+    float reach = 0.f, shared = 0.f;                        // 2 |x|, the part of the upper bound that all centres share
+    for (int i = 0; i <= n_tiles; ++i) {
+        if (i < n_tiles) {
+            copy_async_wait();
+            proxy_fence();
+        }
+        tc_fence_before();
         __syncthreads();
-        const uint32_t hi_a = shared_addr(&sm.ring[stage][0]);
-#pragma unroll 2
-        for (int nt = 0; nt < kNearTile / 8; ++nt) {
-            float acc[2][2][4];                             // two chains of four MMAs each per group of 16 points
+        tc_fence_after();
+        if (i < n_tiles && tid == 0) {
+            const uint64_t da = tc_desc_sw128(shared_addr(sm.points), 16, 1024), db = tc_desc_sw128(shared_addr(sm.centres[i & 1]), 16, 1024);
+            const uint32_t idesc = tc_idesc(kNearPoints, kNearTile, 0, 0, kHalf);
 #pragma unroll
-            for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) acc[m][h][0] = acc[m][h][1] = acc[m][h][2] = acc[m][h][3] = 0.f;
-#pragma unroll
-            for (int s2 = 0; s2 < 4; ++s2) {
-                uint32_t bh[4];
-                ldmatrix4(bh, hi_a + (uint32_t)near_piece(nt * 8 + (lane & 7), 4 * s2 + (lane >> 3)) * 16u);
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-                        const uint32_t(&f)[4] = a[m][2 * s2 + h];
-                        mma_rows<kHalf>(acc[m][h], f[0], f[1], f[2], f[3], bh[2 * h], bh[2 * h + 1]);
-                    }
+            for (int s = 0; s < 8; ++s) {
+                const uint64_t at = (uint64_t)(((s >> 2) * (kNearPoints * 128) + (s & 3) * 32) >> 4);
+                tc_mma(sm.tmem + kNearTile * (i & 1), da + at, db + at, idesc, s > 0 ? 1u : 0u);
             }
-            const float4 bias = *reinterpret_cast<const float4 *>(&sm.bias[stage][nt * 8 + 2 * c]);
-            float low[2][4];
-            bool some = false;
+            tc_commit(shared_addr(&sm.done[i & 1]));
+        }
+        if (i == 0) {                                       // beside the first product: the points' norms
+            float n = 0.f;
+#pragma unroll 4
+            for (int ch = 0; ch < 16; ++ch) {
+                const uint4 w4 = *reinterpret_cast<const uint4 *>(sm.points + near_byte(row, ch));
+                const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-            for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int r = 2 * m + (e >> 1);
-                    low[m][e] = fmaf(-2.f, acc[m][0][e] + acc[m][1][e], fmaf(-reach[r], (e & 1) ? bias.w : bias.y, (e & 1) ? bias.z : bias.x));
-                    some |= low[m][e] < upper[r];
+                for (int t = 0; t < 4; ++t) {
+                    const float x0 = elem_lo<kHalf>(w[t]), x1 = elem_hi<kHalf>(w[t]);
+                    n = fmaf(x0, x0, fmaf(x1, x1, n));
                 }
-            if (some) {
-                const int col = base + nt * 8 + 2 * c;
+            }
+            if (warp < 4) sm.nx[row] = n;
+            reach = 2.000002f * sqrtf(n);
+            shared = fmaf(2.f * kNearErr, n, 1e-34f);
+        } else {
+            const int buf = (i - 1) & 1;
+            near_wait(sm, buf, uses[buf] & 1u);
+            ++uses[buf];
+            tc_fence_after();
+        }
+        if (i + 1 < n_tiles) {                              // the product before this one has left the stage
+            const int base = k_lo + (i + 1) * kNearTile;
+            fill((i + 1) & 1, (i + 1) % 3, base, min(kNearTile, k_hi - base));
+        }
+        if (i > 0) {
+            const int col = 64 * (warp >> 2);
 #pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int r = 2 * m + (e >> 1);
-                        if (low[m][e] < upper[r]) {
-                            // (1.0001: the stored constant is |c|^2 (1 - kNearErr), rounded)
-                            const float wide = fmaf(1.0001f * kNearErr, (e & 1) ? bias.z : bias.x, reach[r] * ((e & 1) ? bias.w : bias.y));
-                            upper[r] = fminf(upper[r], fmaf(2.f, wide, low[m][e] + shared[r]));
-                            insert(r, low[m][e], col + (e & 1));
-                        }
-                    }
+            for (int half = 0; half < 2; ++half) {
+                uint32_t v[32];
+                tc_ld32(sm.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(kNearTile * ((i - 1) & 1) + col + 32 * half), v);
+                near_look(top, v, sm.bias[(i - 1) % 3] + col + 32 * half, k_lo + (i - 1) * kNearTile + col + 32 * half, reach, shared);
             }
         }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {                       // the four lanes of a point share its upper bound
-            upper[r] = fminf(upper[r], __shfl_xor_sync(0xFFFFFFFFu, upper[r], 1));
-            upper[r] = fminf(upper[r], __shfl_xor_sync(0xFFFFFFFFu, upper[r], 2));
-        }
-        __syncthreads();                                    // the stage may be filled again
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        NearTop top = load(r);
-#pragma unroll
-        for (int o = 1; o <= 2; o <<= 1) {
-            NearTop n;
-            n.t1 = __shfl_xor_sync(0xFFFFFFFFu, top.t1, o);
-            n.t2 = __shfl_xor_sync(0xFFFFFFFFu, top.t2, o);
-            n.t3 = __shfl_xor_sync(0xFFFFFFFFu, top.t3, o);
-            n.t4 = __shfl_xor_sync(0xFFFFFFFFu, top.t4, o);
-            n.upper = top.upper;
-            n.i1 = __shfl_xor_sync(0xFFFFFFFFu, top.i1, o);
-            n.i2 = __shfl_xor_sync(0xFFFFFFFFu, top.i2, o);
-            n.i3 = __shfl_xor_sync(0xFFFFFFFFu, top.i3, o);
-            near_merge(top, n);
-        }
-        if (c == 0) sm.top[warp * 32 + 8 * r + (lane >> 2)] = top;
+    if (sm.failed) top.t1 = -kNearFar;
+    if (warp >= 4) sm.top[row] = top;
+    __syncthreads();
+    if (warp < 4) {
+        near_merge(top, sm.top[row]);
+        sm.top[row] = top;
     }
-    __syncwarp();                                           // a warp's points are its own rows
+    __syncthreads();
 }
 
 // The defining distance of a point (128 packed 16-bit values) and a centre of doubles or floats.

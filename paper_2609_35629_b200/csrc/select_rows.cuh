@@ -56,6 +56,9 @@ __device__ __forceinline__ float dist_error(float largest_norm)
 }
 __device__ __forceinline__ float norm_or_inf(float n) { return n <= 1e37f ? n : CUDART_INF_F; }
 
+// Rows of 256 bytes in shared memory, 16-byte pieces XOR-swizzled: ldmatrix without bank conflicts.
+__device__ __forceinline__ int near_piece(int row, int chunk) { return row * 16 + (chunk ^ (row & 7)); }
+
 // The defining distance of two rows (words of two 16-bit values each); not a number counts as infinitely far.
 template <bool kHalf>
 __device__ __forceinline__ double exact_dist(const uint32_t *a, const uint32_t *b, int n_words)
