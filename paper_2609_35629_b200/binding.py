@@ -8,6 +8,7 @@ the first call raises.
 The functions keep the names of the C entry points (include/santapp.h, include/santapp_latent.h).
 """
 import ctypes
+import functools
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -188,12 +189,20 @@ def _ptr(t: Optional[torch.Tensor]):
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise SantappError(SANTAPP_ERR_INVALID_ARG, "tensors must be contiguous CUDA tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream_ptr(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    # (the raw handle: making torch's Stream object costs more than a kernel launch's share of a call)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+@functools.lru_cache(maxsize=256)
+def _geom_ref(cls, *fields):
+    """Reference to a geometry struct (read only, kept for the next call with the same fields)."""
+    return ctypes.byref(cls(*fields))
 
 
 @dataclass
@@ -209,6 +218,10 @@ class Geometry:
     def c(self) -> CGeom:
         return CGeom(self.n_seqs, self.n_q_heads, self.n_kv_heads, self.head_dim, self.parent_size,
                      self.reps_per_parent, self.elem_type)
+
+    def ref(self):
+        return _geom_ref(CGeom, self.n_seqs, self.n_q_heads, self.n_kv_heads, self.head_dim, self.parent_size,
+                         self.reps_per_parent, self.elem_type)
 
     @property
     def torch_dtype(self):
@@ -265,8 +278,7 @@ def santapp_build_teams_sizes(geom: Geometry, prompt_len) -> Sizes:
     n = len(prompt_len)
     arr = (ctypes.c_int32 * n)(*[int(x) for x in prompt_len])
     out = CSizes()
-    g = geom.c()
-    _check(L.santapp_build_teams_sizes(ctypes.byref(g), arr, ctypes.byref(out)))
+    _check(L.santapp_build_teams_sizes(geom.ref(), arr, ctypes.byref(out)))
     return Sizes(out.rows_total, out.teams_total, out.max_teams_per_seq, out.max_rows_per_seq,
                  out.team_row_start_elems, out.build_workspace_bytes)
 
@@ -287,8 +299,7 @@ def santapp_build_teams(geom: Geometry, prompt_len, k_prompt: torch.Tensor, v_pr
     ws = torch.empty(max(sizes.build_workspace_bytes, 256), dtype=torch.uint8, device=k_prompt.device)
     n = len(prompt_len)
     arr = (ctypes.c_int32 * n)(*[int(x) for x in prompt_len])
-    g = geom.c()
-    _check(getattr(L, _entry)(ctypes.byref(g), arr, _ptr(k_prompt), _ptr(v_prompt), ctypes.byref(teams.c),
+    _check(getattr(L, _entry)(geom.ref(), arr, _ptr(k_prompt), _ptr(v_prompt), ctypes.byref(teams.c),
                               _ptr(ws), ws.numel(), _stream_ptr(stream)))
     teams._build_ws = ws      # keep alive until the stream has consumed it
     return teams
@@ -309,17 +320,16 @@ def santapp_kmeans_fit(geom: Geometry, prompt_len, n_centres, k_prompt: torch.Te
     """Minibatch k-means fit per (sequence, KV head); the defaults are the paper's settings.
     Returns (centres fp32 [n_kv_heads, sum(n_centres), d], steps int32 [n_kv_heads, n_seqs])."""
     L = load_library()
-    g = geom.c()
     o = CKmeansOpts(batch_size, max_iter, patience, 1 if no_host_poll else 0, reassignment_ratio, seed, stream_base, 0)
     n, c = _i32_array(prompt_len), _i32_array(n_centres)
-    need = int(L.santapp_kmeans_fit_workspace_bytes(ctypes.byref(g), n, c, ctypes.byref(o)))
+    need = int(L.santapp_kmeans_fit_workspace_bytes(geom.ref(), n, c, ctypes.byref(o)))
     if need == 0:
         raise SantappError(SANTAPP_ERR_INVALID_ARG, "k-means fit arguments")
     dev = k_prompt.device
     ws = torch.empty(need, dtype=torch.uint8, device=dev)
     centres = torch.empty((geom.n_kv_heads, int(sum(n_centres)), geom.head_dim), dtype=torch.float32, device=dev)
     steps = torch.zeros((geom.n_kv_heads, geom.n_seqs), dtype=torch.int32, device=dev)
-    _check(L.santapp_kmeans_fit(ctypes.byref(g), n, c, _ptr(k_prompt), ctypes.byref(o), _ptr(centres), _ptr(steps),
+    _check(L.santapp_kmeans_fit(geom.ref(), n, c, _ptr(k_prompt), ctypes.byref(o), _ptr(centres), _ptr(steps),
                                 _ptr(ws), ws.numel(), _stream_ptr(stream)))
     centres._ws = ws
     return centres, steps
@@ -330,13 +340,12 @@ def santapp_assign_parents(geom: Geometry, prompt_len, n_centres, k_prompt: torc
     """Nearest-centre label of every token. centres: fp32 CUDA tensor [n_kv_heads, sum(n_centres), d].
     Returns int32 [n_kv_heads, rows_total]."""
     L = load_library()
-    g = geom.c()
     if centres.dtype != torch.float32:
         raise SantappError(SANTAPP_ERR_INVALID_ARG, "centres must be float32")
     parent_of = torch.empty((geom.n_kv_heads, k_prompt.shape[1]), dtype=torch.int32, device=k_prompt.device)
-    ws = torch.empty(max(int(L.santapp_assign_parents_workspace_bytes(ctypes.byref(g))), 256), dtype=torch.uint8,
+    ws = torch.empty(max(int(L.santapp_assign_parents_workspace_bytes(geom.ref())), 256), dtype=torch.uint8,
                      device=k_prompt.device)
-    _check(L.santapp_assign_parents(ctypes.byref(g), _i32_array(prompt_len), _i32_array(n_centres), _ptr(k_prompt),
+    _check(L.santapp_assign_parents(geom.ref(), _i32_array(prompt_len), _i32_array(n_centres), _ptr(k_prompt),
                                     _ptr(centres), _ptr(parent_of), _ptr(ws), ws.numel(), _stream_ptr(stream)))
     parent_of._ws = ws
     return parent_of
@@ -345,8 +354,7 @@ def santapp_assign_parents(geom: Geometry, prompt_len, n_centres, k_prompt: torc
 def santapp_parent_teams_sizes(geom: Geometry, prompt_len, n_parents) -> Sizes:
     L = load_library()
     out = CSizes()
-    g = geom.c()
-    _check(L.santapp_parent_teams_sizes(ctypes.byref(g), _i32_array(prompt_len), _i32_array(n_parents),
+    _check(L.santapp_parent_teams_sizes(geom.ref(), _i32_array(prompt_len), _i32_array(n_parents),
                                         ctypes.byref(out)))
     return Sizes(out.rows_total, out.teams_total, out.max_teams_per_seq, out.max_rows_per_seq,
                  out.team_row_start_elems, out.build_workspace_bytes)
@@ -367,10 +375,9 @@ def santapp_build_teams_parents(geom: Geometry, prompt_len, n_parents, k_prompt:
     sizes = santapp_parent_teams_sizes(geom, prompt_len, n_parents)
     teams = Teams(geom, sizes, k_prompt.device)
     ws = torch.empty(max(sizes.build_workspace_bytes, 256), dtype=torch.uint8, device=k_prompt.device)
-    g = geom.c()
     if parent_of.dtype != torch.int32:
         raise SantappError(SANTAPP_ERR_INVALID_ARG, "parent_of must be int32")
-    _check(getattr(L, _entry)(ctypes.byref(g), _i32_array(prompt_len), _i32_array(n_parents),
+    _check(getattr(L, _entry)(geom.ref(), _i32_array(prompt_len), _i32_array(n_parents),
                               _ptr(k_prompt), _ptr(v_prompt), _ptr(parent_of), ctypes.byref(teams.c),
                               _ptr(ws), ws.numel(), _stream_ptr(stream)))
     teams._build_ws = ws      # keep alive until the stream has consumed it
@@ -378,13 +385,11 @@ def santapp_build_teams_parents(geom: Geometry, prompt_len, n_parents, k_prompt:
 
 
 def santapp_decode_workspace_bytes(geom: Geometry, teams: Teams, n_sample: int) -> int:
-    g = geom.c()
-    return int(load_library().santapp_decode_workspace_bytes(ctypes.byref(g), ctypes.byref(teams.c), n_sample))
+    return int(load_library().santapp_decode_workspace_bytes(geom.ref(), ctypes.byref(teams.c), n_sample))
 
 
 def santapp_dense_workspace_bytes(geom: Geometry, teams: Teams) -> int:
-    g = geom.c()
-    return int(load_library().santapp_dense_workspace_bytes(ctypes.byref(g), ctypes.byref(teams.c)))
+    return int(load_library().santapp_dense_workspace_bytes(geom.ref(), ctypes.byref(teams.c)))
 
 
 class DebugBuffers:
@@ -418,9 +423,8 @@ def santapp_decode_attn(geom: Geometry, teams: Teams, q: torch.Tensor, k_suffix:
         workspace = torch.empty(santapp_decode_workspace_bytes(geom, teams, n_sample), dtype=torch.uint8,
                                 device=q.device)
     cap = 0 if k_suffix is None else int(k_suffix.shape[2])
-    g = geom.c()
-    _check(L.santapp_decode_attn(ctypes.byref(g), ctypes.byref(teams.c), _ptr(q), _ptr(k_suffix), _ptr(v_suffix),
-                                 _ptr(suffix_len), cap, n_sample, ctypes.c_uint64(seed), step, _ptr(step_dev),
+    _check(L.santapp_decode_attn(geom.ref(), ctypes.byref(teams.c), _ptr(q), _ptr(k_suffix), _ptr(v_suffix),
+                                 _ptr(suffix_len), cap, n_sample, int(seed), step, _ptr(step_dev),
                                  stream_base, scale, _ptr(out), ctypes.byref(debug.c) if debug is not None else None,
                                  _ptr(workspace), workspace.numel(), _stream_ptr(stream)))
     return out
@@ -436,8 +440,7 @@ def santapp_dense_decode_attn(geom: Geometry, teams: Teams, q: torch.Tensor, k_s
     if workspace is None:
         workspace = torch.empty(santapp_dense_workspace_bytes(geom, teams), dtype=torch.uint8, device=q.device)
     cap = 0 if k_suffix is None else int(k_suffix.shape[2])
-    g = geom.c()
-    _check(L.santapp_dense_decode_attn(ctypes.byref(g), ctypes.byref(teams.c), _ptr(q), _ptr(k_suffix),
+    _check(L.santapp_dense_decode_attn(geom.ref(), ctypes.byref(teams.c), _ptr(q), _ptr(k_suffix),
                                        _ptr(v_suffix), _ptr(suffix_len), cap, scale, _ptr(out), _ptr(workspace),
                                        workspace.numel(), _stream_ptr(stream)))
     return out
@@ -457,8 +460,7 @@ def santapp_dense_decode_attn_noalloc(geom: Geometry, teams: Teams, q: torch.Ten
     if out is None:
         out = torch.empty((geom.n_seqs, geom.n_q_heads, geom.head_dim), dtype=torch.float32, device=q.device)
     cap = 0 if k_suffix is None else int(k_suffix.shape[2])
-    g = geom.c()
-    _check(L.santapp_dense_decode_attn_noalloc(ctypes.byref(g), ctypes.byref(teams.c), _ptr(q), _ptr(k_suffix),
+    _check(L.santapp_dense_decode_attn_noalloc(geom.ref(), ctypes.byref(teams.c), _ptr(q), _ptr(k_suffix),
                                                _ptr(v_suffix), _ptr(suffix_len), cap, scale, _ptr(out),
                                                _stream_ptr(stream)))
     return out
@@ -476,6 +478,9 @@ class LatentGeometry:
 
     def c(self) -> CLatentGeom:
         return CLatentGeom(self.n_seqs, self.n_heads, self.parent_size, self.reps_per_parent)
+
+    def ref(self):
+        return _geom_ref(CLatentGeom, self.n_seqs, self.n_heads, self.parent_size, self.reps_per_parent)
 
 
 class LatentTeams:
@@ -500,8 +505,7 @@ class LatentTeams:
 def santapp_latent_sizes(geom: LatentGeometry, prompt_len) -> Sizes:
     L = load_library()
     out = CSizes()
-    g = geom.c()
-    _check(L.santapp_latent_sizes(ctypes.byref(g), _i32_array(prompt_len), ctypes.byref(out)))
+    _check(L.santapp_latent_sizes(geom.ref(), _i32_array(prompt_len), ctypes.byref(out)))
     return Sizes(out.rows_total, out.teams_total, out.max_teams_per_seq, out.max_rows_per_seq,
                  out.team_row_start_elems, out.build_workspace_bytes)
 
@@ -512,22 +516,19 @@ def santapp_latent_build_teams(geom: LatentGeometry, prompt_len, rows_prompt: to
     sizes = santapp_latent_sizes(geom, prompt_len)
     teams = LatentTeams(geom, sizes, rows_prompt.device)
     ws = torch.empty(max(sizes.build_workspace_bytes, 256), dtype=torch.uint8, device=rows_prompt.device)
-    g = geom.c()
-    _check(L.santapp_latent_build_teams(ctypes.byref(g), _i32_array(prompt_len), _ptr(rows_prompt), ctypes.byref(teams.c),
+    _check(L.santapp_latent_build_teams(geom.ref(), _i32_array(prompt_len), _ptr(rows_prompt), ctypes.byref(teams.c),
                                         _ptr(ws), ws.numel(), _stream_ptr(stream)))
     teams._build_ws = ws
     return teams
 
 
 def santapp_latent_decode_workspace_bytes(geom: LatentGeometry, teams: LatentTeams, n_sample: int, suffix_cap: int) -> int:
-    g = geom.c()
-    return int(load_library().santapp_latent_decode_workspace_bytes(ctypes.byref(g), ctypes.byref(teams.c), n_sample,
+    return int(load_library().santapp_latent_decode_workspace_bytes(geom.ref(), ctypes.byref(teams.c), n_sample,
                                                                     suffix_cap))
 
 
 def santapp_latent_dense_workspace_bytes(geom: LatentGeometry, teams: LatentTeams) -> int:
-    g = geom.c()
-    return int(load_library().santapp_latent_dense_workspace_bytes(ctypes.byref(g), ctypes.byref(teams.c)))
+    return int(load_library().santapp_latent_dense_workspace_bytes(geom.ref(), ctypes.byref(teams.c)))
 
 
 class LatentDebugBuffers(DebugBuffers):
@@ -551,9 +552,8 @@ def santapp_latent_decode_attn(geom: LatentGeometry, teams: LatentTeams, q: torc
     if workspace is None:
         workspace = torch.empty(santapp_latent_decode_workspace_bytes(geom, teams, n_sample, cap), dtype=torch.uint8,
                                 device=q.device)
-    g = geom.c()
-    _check(L.santapp_latent_decode_attn(ctypes.byref(g), ctypes.byref(teams.c), _ptr(q), _ptr(suffix_rows),
-                                        _ptr(suffix_len), cap, n_sample, ctypes.c_uint64(seed), step, _ptr(step_dev),
+    _check(L.santapp_latent_decode_attn(geom.ref(), ctypes.byref(teams.c), _ptr(q), _ptr(suffix_rows),
+                                        _ptr(suffix_len), cap, n_sample, int(seed), step, _ptr(step_dev),
                                         stream_base, scale, _ptr(out),
                                         ctypes.byref(debug.c) if debug is not None else None, _ptr(workspace),
                                         workspace.numel(), _stream_ptr(stream)))
@@ -570,8 +570,7 @@ def santapp_latent_dense_decode_attn(geom: LatentGeometry, teams: LatentTeams, q
         out = torch.empty((geom.n_seqs, geom.n_heads, LATENT_DIM), dtype=torch.float32, device=q.device)
     if workspace is None:
         workspace = torch.empty(santapp_latent_dense_workspace_bytes(geom, teams), dtype=torch.uint8, device=q.device)
-    g = geom.c()
-    _check(L.santapp_latent_dense_decode_attn(ctypes.byref(g), ctypes.byref(teams.c), _ptr(q), _ptr(suffix_rows),
+    _check(L.santapp_latent_dense_decode_attn(geom.ref(), ctypes.byref(teams.c), _ptr(q), _ptr(suffix_rows),
                                               _ptr(suffix_len), cap, scale, _ptr(out), _ptr(workspace),
                                               workspace.numel(), _stream_ptr(stream)))
     return out

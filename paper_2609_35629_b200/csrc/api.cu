@@ -141,6 +141,14 @@ DecodeLayout decode_layout(const santapp_geom *g, const santapp_teams *t, int K,
     return L;
 }
 
+// Blocks per pair of the fixed split: no more than the longest sequence has shares of min_rows (the others would only
+// leave empty partials for the merge to read: 3.5 us for 148 of them).
+int ctas_per_pair(const DecodeLayout &L, const santapp_teams *t, int suffix_cap, int min_rows)
+{
+    const int64_t shares = ((int64_t)t->max_rows_per_seq + suffix_cap + min_rows - 1) / min_rows;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(L.ctas_per_pair, shares));
+}
+
 void fill_plan(const DecodeLayout &L, char *ws, PlanView &plan)
 {
     plan.seg_cap = L.seg_cap;
@@ -851,16 +859,16 @@ int santapp_decode_attn(const santapp_geom *geom, const santapp_teams *teams, co
 #ifdef SANTAPP_TUNE
     if (const char *e = getenv("SANTAPP_SPAN_PENALTY")) ap.span_penalty_rows = atoi(e);
 #endif
-    ap.ctas_per_pair = L.ctas_per_pair;
+    ap.ctas_per_pair = ctas_per_pair(L, teams, suffix_cap, ap.min_rows_per_cta);
     ap.max_words = (teams->max_teams_per_seq + 31) / 32;
     if (g_stage_mask & SANTAPP_STAGE_ATTEND) {
-        const int launch_grid = L.static_split ? L.n_pairs * L.ctas_per_pair : grid;
+        const int launch_grid = L.static_split ? L.n_pairs * ap.ctas_per_pair : grid;
         err = launch_attend(ap, false, L.static_split, launch_grid, s);
         if (err != cudaSuccess) return cuda_fail(err, "attend launch");
         ++g_launches;
     }
     if (g_stage_mask & SANTAPP_STAGE_MERGE) {
-        const int launch_grid = L.static_split ? L.n_pairs * L.ctas_per_pair : grid;
+        const int launch_grid = L.static_split ? L.n_pairs * ap.ctas_per_pair : grid;
         err = launch_merge(ap, L.static_split, launch_grid, s);
         if (err != cudaSuccess) return cuda_fail(err, "merge launch");
         ++g_launches;
@@ -935,8 +943,8 @@ int santapp_dense_decode_attn(const santapp_geom *geom, const santapp_teams *tea
 #ifdef SANTAPP_TUNE
     if (const char *e = getenv("SANTAPP_SPAN_PENALTY_DENSE")) ap.span_penalty_rows = atoi(e);
 #endif
-    ap.ctas_per_pair = L.ctas_per_pair;
-    const int launch_grid = L.static_split ? L.n_pairs * L.ctas_per_pair : grid;
+    ap.ctas_per_pair = ctas_per_pair(L, teams, suffix_cap, ap.min_rows_per_cta);
+    const int launch_grid = L.static_split ? L.n_pairs * ap.ctas_per_pair : grid;
     err = launch_attend(ap, true, L.static_split, launch_grid, s);
     if (err != cudaSuccess) return cuda_fail(err, "attend launch");
     ++g_launches;

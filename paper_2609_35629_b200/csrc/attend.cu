@@ -695,9 +695,15 @@ cudaError_t launch_attend_g(const AttendParams &p, bool all_heads, bool static_s
 
 int attend_grid_size()
 {
+    static std::atomic<int> known[64];                     // per device: asked several times in every call
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > kMaxAttendGrid ? kMaxAttendGrid : sms;
+    if (cudaGetDevice(&dev) != cudaSuccess) return sms;
+    if (dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+    sms = 148;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 148;
+    sms = sms > kMaxAttendGrid ? kMaxAttendGrid : sms;
+    if (dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+    return sms;
 }
 
 int attend_max_segments() { return kSegMax; }

@@ -20,6 +20,8 @@
 
 #include <stddef.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace santapp {
@@ -33,7 +35,7 @@ constexpr int kWindow = 255;            // histogram bins per pass of the bound
 // kDim: values per routing key (128 for K rows, 576 for shared-latent rows); a multiple of 64.
 template <int kDim>
 struct alignas(16) HeadSmemT {
-    double q64[kDotLanes][kDim / kDotLanes + 2];   // query in fp64: [slice of kDim / 8 dims][+ pad] (pad: conflict-free LDS.128)
+    double q64[kDotLanes][kDim / kDotLanes + 2];   // query in fp64: [lane of a key's eight][its dims, + pad] (pad: conflict-free LDS.128)
     double cand_y[kCandCap + 2];        // dot products, then exact Y; read in pairs
     double cand_phi[kCandCap];          // log n_g, then phi_g
     double cand_g[kCandCap];            // Gumbel term
@@ -103,6 +105,12 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
     for (int i = 0; i < kQRegs; ++i)
         q_val[i] = tid + i * kT < kDim ? elem_to_float<kHalf>(in.q[(size_t)hq * kDim + tid + i * kT]) : 0.f;
     const float k_abs_max = in.rep_abs_max[(size_t)j * in.bv.n_seqs + b];
+    // fp32 -> fp64 conversions run at 16 per clock and SM, a quarter of the fp64 rate, and are what the exact dot products
+    // wait for. Finite bf16 keys convert the upper value of a word with two integer instructions instead: its bits,
+    // moved to where a double has them, are the value times 2^-896 (subnormals included). The query's odd
+    // values are held times 2^700 and the odd sums end with 2^196: exact scalings, the same sums bit for bit.
+    const bool shifted = !kHalf && k_abs_max <= 3.4e38f;
+    constexpr double kShiftUp = 0x1p700, kShiftDown = 0x1p196;
 
     const int64_t team0 = in.bv.seq_team_off[b];
     const int M = pair_team_count(in.bv, b, j);
@@ -152,7 +160,7 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
 #pragma unroll
         for (int i = 0; i < kQRegs; ++i) {
             const int d = tid + i * kT;
-            if (d < kDim) sm.q64[d / kSlice][d % kSlice] = (double)q_val[i];
+            if (d < kDim) sm.q64[(d >> 3) & 7][(d >> 6) * 8 + (d & 7)] = (double)q_val[i] * (shifted && (d & 1) ? kShiftUp : 1.0);
         }
         if (lane == 0) { sm.red_sum[warp] = a; sm.red_max[warp] = top; }
         if (tid == 0) sm.n_cand = 0;
@@ -283,9 +291,16 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
         //          log n_g and the Gumbel term on the other warps (one thread per candidate) ----
         // Long keys (kAllDot): every warp takes part in the dot products (their round trips to memory
         // are the longest chain of the kernel), then every thread takes a candidate's other terms.
-        if (kAllDot || warp < kDotWarps) {
+        auto dot_products = [&](auto by_bits) {
+            constexpr bool kBits = decltype(by_bits)::value;
+            auto widen_odd = [](uint32_t w) {
+                if constexpr (kBits) return __hiloint2double(((int)w >> 3) & (int)0x8FFFE000, 0);
+                else return (double)elem_hi<kHalf>(w);
+            };
             const int sub = lane & (kDotLanes - 1);
             const double *qs = sm.q64[sub];
+            // (piece sub + 8 pc for each pc: a key's eight lanes read whole 128-byte lines together; with slices of consecutive
+            // pieces instead, 576-value keys touched 32 lines an instruction and the kernel was bound by line accesses)
             // a few candidates per thread group at a time: all their key pieces are requested before
             // the first product, so a chunk costs one memory round trip
             constexpr int kPerPass = kDotWarps * 32 / kDotLanes, kChunk = kPieces > 2 ? 1 : (kT >= 512 ? 2 : 4);
@@ -295,9 +310,9 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
                 for (int u = 0; u < kChunk; ++u) {
                     const int cand = c0 + u * kPerPass + (tid >> 3);
                     if (cand < n_cand) {
-                        const uint4 *kr = reinterpret_cast<const uint4 *>(rep + (size_t)sm.cand_id[cand] * kDim) + sub * kPieces;
+                        const uint4 *kr = reinterpret_cast<const uint4 *>(rep + (size_t)sm.cand_id[cand] * kDim) + sub;
 #pragma unroll
-                        for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = __ldg(kr + pc);
+                        for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = __ldg(kr + kDotLanes * pc);
                     } else {
 #pragma unroll
                         for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = make_uint4(0u, 0u, 0u, 0u);
@@ -311,20 +326,27 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
                     for (int pc = 0; pc < kPieces; ++pc) {
                         const uint4 wv = w[u][pc];
                         d0 = fma((double)elem_lo<kHalf>(wv.x), qs[8 * pc + 0], d0);
-                        d1 = fma((double)elem_hi<kHalf>(wv.x), qs[8 * pc + 1], d1);
+                        d1 = fma(widen_odd(wv.x), qs[8 * pc + 1], d1);
                         d0 = fma((double)elem_lo<kHalf>(wv.y), qs[8 * pc + 2], d0);
-                        d1 = fma((double)elem_hi<kHalf>(wv.y), qs[8 * pc + 3], d1);
+                        d1 = fma(widen_odd(wv.y), qs[8 * pc + 3], d1);
                         d0 = fma((double)elem_lo<kHalf>(wv.z), qs[8 * pc + 4], d0);
-                        d1 = fma((double)elem_hi<kHalf>(wv.z), qs[8 * pc + 5], d1);
+                        d1 = fma(widen_odd(wv.z), qs[8 * pc + 5], d1);
                         d0 = fma((double)elem_lo<kHalf>(wv.w), qs[8 * pc + 6], d0);
-                        d1 = fma((double)elem_hi<kHalf>(wv.w), qs[8 * pc + 7], d1);
+                        d1 = fma(widen_odd(wv.w), qs[8 * pc + 7], d1);
                     }
-                    double d = d0 + d1;
+                    double d = kBits ? fma(d1, kShiftDown, d0) : d0 + d1;
                     d += __shfl_xor_sync(0xFFFFFFFFu, d, 1);
                     d += __shfl_xor_sync(0xFFFFFFFFu, d, 2);
                     d += __shfl_xor_sync(0xFFFFFFFFu, d, 4);
                     if (cand < n_cand && sub == 0) sm.cand_y[cand] = d;
                 }
+            }
+        };
+        if (kAllDot || warp < kDotWarps) {
+            if (shifted) {
+                if constexpr (!kHalf) dot_products(std::true_type{});
+            } else {
+                dot_products(std::false_type{});
             }
         }
         if (kAllDot || warp >= kDotWarps) {
