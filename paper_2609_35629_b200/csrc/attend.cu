@@ -712,11 +712,13 @@ int attend_pairs_staged() { return kPairMax; }
 
 cudaError_t launch_merge(const AttendParams &p, bool static_split, int attend_grid, cudaStream_t s)
 {
-    // few pairs: many partials each (16 warps share them); many pairs: a handful each
+    // few pairs: many partials each (16 warps share them); more pairs: a block's range and its tail chunks make about
+    // 3 * blocks / pairs, which eight warps request at once, or four where they are a handful
     const dim3 blocks(p.bv.group, p.n_pairs);
     const bool wide = static_split || p.n_pairs * 8 <= attend_grid;
     if (static_split) return launch_step(merge_kernel<16, true>, blocks, dim3(16 * 32), 0, s, p, attend_grid);
     if (wide) return launch_step(merge_kernel<16, false>, blocks, dim3(16 * 32), 0, s, p, attend_grid);
+    if (p.n_pairs * 8 <= 3 * attend_grid) return launch_step(merge_kernel<8, false>, blocks, dim3(8 * 32), 0, s, p, attend_grid);
     return launch_step(merge_kernel<4, false>, blocks, dim3(4 * 32), 0, s, p, attend_grid);
 }
 

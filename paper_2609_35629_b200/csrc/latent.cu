@@ -888,8 +888,22 @@ latent_merge_kernel(const float *partials, const uint32_t *pair_prefix, int n_se
     const int c_lo = (int)(lo / per), c_hi = hi > lo ? (int)((hi - 1) / per) : c_lo - 1;
     const float *base = partials + ((size_t)b * kHeads + h) * kLatPartialStride;      // slot c + b
     const size_t slot = (size_t)kHeads * kLatPartialStride;
-    float M = -CUDART_INF_F;
-    for (int c = c_lo + tid; c <= c_hi; c += kLmThreads) M = fmaxf(M, __ldcg(base + c * slot));
+    // Two partials a thread are requested whole before anything else (a sequence rarely has more than eight); the maxima are
+    // exchanged while they travel
+    constexpr int kAhead = 2;
+    float m[kAhead], l[kAhead];
+    float4 v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+        const int c = c_lo + part + 4 * u;
+        const bool there = c <= c_hi;
+        const float *p = base + (there ? c : c_lo) * slot;
+        m[u] = there ? __ldcg(p) : -CUDART_INF_F;
+        l[u] = there ? __ldcg(p + 1) : 0.f;
+        v[u] = there ? __ldcg(reinterpret_cast<const float4 *>(p + 4) + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float M = fmaxf(m[0], m[1]);
+    for (int c = c_lo + 4 * kAhead + tid; c <= c_hi; c += kLmThreads) M = fmaxf(M, __ldcg(base + c * slot));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
     if ((tid & 31) == 0) red[tid >> 5] = M;
@@ -899,19 +913,20 @@ latent_merge_kernel(const float *partials, const uint32_t *pair_prefix, int n_se
     const float Mu = M == -CUDART_INF_F ? 0.f : M;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float L = 0.f;
-    for (int c = c_lo + part; c <= c_hi; c += 8) {
-        const float *p0 = base + c * slot, *p1 = p0 + 4 * slot;
-        const bool two = c + 4 <= c_hi;
-        const float m0 = __ldcg(p0), l0 = __ldcg(p0 + 1);
-        const float4 v0 = __ldcg(reinterpret_cast<const float4 *>(p0 + 4) + col);
-        const float m1 = two ? __ldcg(p1) : -CUDART_INF_F, l1 = two ? __ldcg(p1 + 1) : 0.f;
-        const float4 v1 = two ? __ldcg(reinterpret_cast<const float4 *>(p1 + 4) + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float w0 = ex2(m0 - Mu), w1 = ex2(m1 - Mu);
-        L += w0 * l0 + w1 * l1;
-        acc.x += w0 * v0.x + w1 * v1.x;
-        acc.y += w0 * v0.y + w1 * v1.y;
-        acc.z += w0 * v0.z + w1 * v1.z;
-        acc.w += w0 * v0.w + w1 * v1.w;
+    auto add = [&](float pm, float pl, const float4 &pv) {
+        const float w = ex2(pm - Mu);
+        L += w * pl;
+        acc.x += w * pv.x;
+        acc.y += w * pv.y;
+        acc.z += w * pv.z;
+        acc.w += w * pv.w;
+    };
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+        if (c_lo + part + 4 * u <= c_hi) add(m[u], l[u], v[u]);
+    for (int c = c_lo + part + 4 * kAhead; c <= c_hi; c += 4) {
+        const float *p = base + c * slot;
+        add(__ldcg(p), __ldcg(p + 1), __ldcg(reinterpret_cast<const float4 *>(p + 4) + col));
     }
     if (part > 0) { part_acc[part - 1][col] = acc; part_l[part - 1][col] = L; }
     __syncthreads();
