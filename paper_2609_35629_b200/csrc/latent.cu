@@ -504,28 +504,49 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
-// One block per SM. The rows to read of all sequences form one line, cut into equal ranges, one per
-// block; a block walks the sequences its range touches, 32 rows (a tile) at a time, and leaves one
+// The rows to read of all sequences form one line, cut into equal ranges, one per block; a block walks the sequences its range touches, 32 rows (a tile) at a time, and leaves one
 // partial result per sequence. Eight warps in two roles. Four compute S = Q Rows^T of a tile with
 // the contraction split between them (each keeps its 144 of the 576 query values as A fragments in
 // registers), add the four partial S tiles up through shared memory, take a quarter of the tile's
 // rows each through the softmax step (tile maxima exchanged through shared memory) and hand P (two
 // bf16 terms, already laid out as the A fragments of the next product) and the factors by which the
 // running maxima moved over through shared memory. The other four copy the rows from global memory
-// into a ring of four tiles (eight lanes copy 128 contiguous bytes of a row into one XOR-swizzled
+// into a ring of tiles (eight lanes copy 128 contiguous bytes of a row into one XOR-swizzled
 // line, so ldmatrix is conflict-free and a global sector lands in one piece) and accumulate
-// O += P V for their 128 of the 512 value columns. S of a tile runs beside P V of the tile before it
-// while two more tiles are on their way from memory; named barriers order the hand-overs.
+// O += P V for their 128 of the 512 value columns. Named barriers order the hand-overs.
+//
+// What bounds it is the chain of a tile (barrier, products, two exchanges, softmax, barrier, products):
+// neither memory nor the tensor cores are busy while one block walks it. So there are two forms. With
+// one block per SM the ring holds four tiles and S of a tile runs beside P V of the tile before it.
+// With two, each block has a ring of two tiles and walks its chain in order; the other block fills the
+// gaps, and the SM keeps as many tiles on their way. That costs twice the partial results for the
+// merge. 32 sequences of 8192 rows, this kernel and the merge, one block -> two blocks: 66.0 -> 60.1 us
+// behind the sampler, 70.5 -> 69.1 over all rows; at 4 sequences 16.5 -> 19.1 and 20.2 -> 25.8.
 constexpr int kLfThreads = 256;
-constexpr int kLfStages = 4;
-constexpr int kLfOffBias = kLfStages * kTileBytes;                              // [stage][32 rows][kBiasPitch] floats
-constexpr int kLfOffXch = kLfOffBias + kLfStages * kTileRows * kBiasPitch * 4;  // [tile parity][4 warps][4][32 lanes] float4
-constexpr int kLfOffP = kLfOffXch + 2 * 4 * 4 * 32 * 16 + 2 * 64 * 4;            // (+ the warps' tile maxima [parity][4][16]); P: [tile parity][16 registers][32 lanes]
-constexpr int kLfOffAlpha = kLfOffP + 2 * 16 * 32 * 4;                          // [tile parity][16 heads]
-constexpr int kLfOffMl = kLfOffAlpha + 2 * 16 * 4;                              // [m 16 | l of each S warp 4 x 16]
-constexpr int kLfOffPrefix = kLfOffMl + 80 * 4;
-constexpr int kLfOffScan = kLfOffPrefix + (kMaxLatentSeqs + 4) * 4;
-constexpr int kLfSmemBytes = kLfOffScan + 48 * 4;
+template <int kBlocks>
+struct LfShape {
+    static constexpr int stages = kBlocks == 1 ? 4 : 2;
+    static constexpr int max_seqs = kBlocks == 1 ? kMaxLatentSeqs : 512;
+    static constexpr int key_steps = kBlocks == 1 ? 9 : 3;                          // k-steps whose key fragments are in registers at once
+    static constexpr int off_bias = stages * kTileBytes;                            // [stage][32 rows][kBiasPitch] floats
+    static constexpr int off_xch = off_bias + stages * kTileRows * kBiasPitch * 4;  // [tile parity][4 warps][4][32 lanes] float4
+    static constexpr int off_p = off_xch + 2 * 4 * 4 * 32 * 16 + 2 * 64 * 4;        // (+ the warps' tile maxima [parity][4][16]); P: [tile parity][16 registers][32 lanes]
+    static constexpr int off_alpha = off_p + 2 * 16 * 32 * 4;                       // [tile parity][16 heads]
+    static constexpr int off_ml = off_alpha + 2 * 16 * 4;                           // [m 16 | l of each S warp 4 x 16]
+    static constexpr int off_prefix = off_ml + 80 * 4;
+    static constexpr int off_scan = off_prefix + (max_seqs + 4) * 4;
+    static constexpr int smem_bytes = off_scan + 48 * 4;
+};
+static_assert(LfShape<1>::smem_bytes <= 227 * 1024 && LfShape<2>::smem_bytes <= 113 * 1024, "shared memory of an SM");
+
+// Blocks per SM. The second one pays once a block still has enough tiles to walk (about 1024 rows an SM where the
+// sampler's scattered rows are read, 1536 where all rows are) and a sequence's partial results stay few (at 1 and 2
+// sequences of 100000 rows the merge made the step 10 and 5 us slower); its table of sequences is the shorter one.
+inline int latent_blocks_per_sm(int64_t rows_total, int n_seqs, int sms, bool dense)
+{
+    if (n_seqs < 16 || n_seqs > LfShape<2>::max_seqs) return 1;
+    return rows_total >= (int64_t)(dense ? 1536 : 1024) * sms ? 2 : 1;
+}
 
 __device__ __forceinline__ void named_sync(int id, int count) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory"); }
 __device__ __forceinline__ void named_arrive(int id, int count) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory"); }
@@ -541,17 +562,19 @@ __device__ __forceinline__ void lf_mark(unsigned long long *trace, bool on, int 
     }
 }
 
-template <bool kAll>
-__global__ void __launch_bounds__(kLfThreads, 1)
+template <bool kAll, int kBlocks>
+__global__ void __launch_bounds__(kLfThreads, kBlocks)
 latent_attend_kernel(LatentAttendParams p)
 {
     step_wait();
+    using Sh = LfShape<kBlocks>;
+    constexpr int kStages = Sh::stages;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int pv_role = warp >> 2, gw = warp & 3, gt = gw * 32 + lane;
     const int r = lane >> 2, t = lane & 3;
-    uint32_t *prefix = reinterpret_cast<uint32_t *>(smem + kLfOffPrefix);
-    int *scan = reinterpret_cast<int *>(smem + kLfOffScan);
+    uint32_t *prefix = reinterpret_cast<uint32_t *>(smem + Sh::off_prefix);
+    int *scan = reinterpret_cast<int *>(smem + Sh::off_scan);
     const int n = p.lv.n_seqs, H = p.lv.n_heads;
     {
         uint32_t carry = 0;
@@ -590,11 +613,11 @@ latent_attend_kernel(LatentAttendParams p)
         pr = a;
     }
     const uint32_t smem_base = (uint32_t)__cvta_generic_to_shared(smem);
-    const float *bias_all = reinterpret_cast<const float *>(smem + kLfOffBias);
-    float4 *xch_all = reinterpret_cast<float4 *>(smem + kLfOffXch);
-    uint32_t *p_all = reinterpret_cast<uint32_t *>(smem + kLfOffP);
-    float *alpha_all = reinterpret_cast<float *>(smem + kLfOffAlpha);
-    float *ml = reinterpret_cast<float *>(smem + kLfOffMl);
+    const float *bias_all = reinterpret_cast<const float *>(smem + Sh::off_bias);
+    float4 *xch_all = reinterpret_cast<float4 *>(smem + Sh::off_xch);
+    uint32_t *p_all = reinterpret_cast<uint32_t *>(smem + Sh::off_p);
+    float *alpha_all = reinterpret_cast<float *>(smem + Sh::off_alpha);
+    float *ml = reinterpret_cast<float *>(smem + Sh::off_ml);
     const uint4 *rows_g = reinterpret_cast<const uint4 *>(p.rows_packed);
     const uint4 *suffix_g = reinterpret_cast<const uint4 *>(p.suffix_rows);
 
@@ -623,7 +646,7 @@ latent_attend_kernel(LatentAttendParams p)
             }
 #pragma unroll 1
             for (int j = 0; j < n_tiles; ++j) {
-                const int par = j & 1, stage = j & (kLfStages - 1);
+                const int par = j & 1, stage = j & (kStages - 1);
                 const bool tr = j >= 4 && j <= 5 && gt == 0;
                 lf_mark(p.trace, tr && j == 4, 0);
                 named_sync(kLfBarData + par, 256);          // the tile's rows (and corrections) have landed
@@ -635,25 +658,31 @@ latent_attend_kernel(LatentAttendParams p)
 #pragma unroll
                 for (int nt = 0; nt < 4; ++nt) x[nt][0] = x[nt][1] = x[nt][2] = x[nt][3] = 0.f;
                 {
-                    // all of the warp's key fragments first (the loads pipeline; an MMA right behind its own
-                    // load would wait out the load's latency every time), then the 36 MMAs
-                    uint32_t kb[9][2][4];
+                    // many key fragments first (the loads pipeline; an MMA right behind its own load would wait
+                    // out the load's latency every time), then their MMAs; two blocks per SM leave registers for three
+                    // k-steps of them
+                    constexpr int kSteps = Sh::key_steps;
 #pragma unroll
-                    for (int ks = 0; ks < 9; ++ks) {
+                    for (int k0 = 0; k0 < 9; k0 += kSteps) {
+                        uint32_t kb[kSteps][2][4];
 #pragma unroll
-                        for (int ntp = 0; ntp < 2; ++ntp) {
-                            const int row = 16 * ntp + ((lane >> 4) << 3) + (lane & 7);
-                            const int chunk = 18 * gw + 2 * ks + ((lane >> 3) & 1);
-                            ldmatrix_x4(kb[ks][ntp][0], kb[ks][ntp][1], kb[ks][ntp][2], kb[ks][ntp][3],
-                                        tile_addr + row * kRowBytes + ((chunk ^ (lane & 7)) << 4));
+                        for (int ks = 0; ks < kSteps; ++ks) {
+#pragma unroll
+                            for (int ntp = 0; ntp < 2; ++ntp) {
+                                const int row = 16 * ntp + ((lane >> 4) << 3) + (lane & 7);
+                                const int chunk = 18 * gw + 2 * (k0 + ks) + ((lane >> 3) & 1);
+                                ldmatrix_x4(kb[ks][ntp][0], kb[ks][ntp][1], kb[ks][ntp][2], kb[ks][ntp][3],
+                                            tile_addr + row * kRowBytes + ((chunk ^ (lane & 7)) << 4));
+                            }
                         }
-                    }
 #pragma unroll
-                    for (int ks = 0; ks < 9; ++ks) {
+                        for (int ks = 0; ks < kSteps; ++ks) {
+                            const uint32_t(&a)[4] = qa[k0 + ks];
 #pragma unroll
-                        for (int ntp = 0; ntp < 2; ++ntp) {
-                            mma_bf16(x[2 * ntp], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], kb[ks][ntp][0], kb[ks][ntp][1]);
-                            mma_bf16(x[2 * ntp + 1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], kb[ks][ntp][2], kb[ks][ntp][3]);
+                            for (int ntp = 0; ntp < 2; ++ntp) {
+                                mma_bf16(x[2 * ntp], a[0], a[1], a[2], a[3], kb[ks][ntp][0], kb[ks][ntp][1]);
+                                mma_bf16(x[2 * ntp + 1], a[0], a[1], a[2], a[3], kb[ks][ntp][2], kb[ks][ntp][3]);
+                            }
                         }
                     }
                 }
@@ -759,7 +788,7 @@ latent_attend_kernel(LatentAttendParams p)
             // permutes pieces inside it); rows past the share's end are zero-filled
             auto issue = [&](int j, int4 meta) {
                 if (j < n_tiles) {
-                    const int jl = gt & 7, stage = j & (kLfStages - 1);
+                    const int jl = gt & 7, stage = j & (kStages - 1);
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         const int i = (gt >> 3) + 16 * half;
@@ -774,7 +803,7 @@ latent_attend_kernel(LatentAttendParams p)
 #pragma unroll
                         for (int c = 0; c < kRowChunks / 8; ++c) cp_async16(dst + c * 128, g + 8 * c + jl, bytes);
                         if (!kAll && jl < 4) {
-                            const uint32_t bdst = smem_base + kLfOffBias + (stage * kTileRows * kBiasPitch + i * kBiasPitch + 4 * jl) * 4;
+                            const uint32_t bdst = smem_base + Sh::off_bias + (stage * kTileRows * kBiasPitch + i * kBiasPitch + 4 * jl) * 4;
                             cp_async16(bdst, valid ? bias_g + (size_t)mseg * kHeads + 4 * jl : reinterpret_cast<const float *>(rows_g), bytes);
                         }
                     }
@@ -782,65 +811,75 @@ latent_attend_kernel(LatentAttendParams p)
                 asm volatile("cp.async.commit_group;" ::: "memory");
             };
 #pragma unroll
-            for (int j = 0; j < kLfStages; ++j) issue(j, load_meta(j));
-            asm volatile("cp.async.wait_group 3;" ::: "memory");
+            for (int j = 0; j < kStages; ++j) issue(j, load_meta(j));
+            asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
             named_arrive(kLfBarData, 256);                  // tile 0 is there
-            int4 meta_next = load_meta(kLfStages);
+            int4 meta_next = load_meta(kStages);
 #pragma unroll 1
             for (int j = 0; j < n_tiles; ++j) {
                 const int par = j & 1;
                 const int4 meta_cur = meta_next;            // of the tile issued at the end of this round
-                meta_next = load_meta(j + kLfStages + 1);
+                meta_next = load_meta(j + kStages + 1);
                 const bool tr = j == 4 && gt == 0;
                 lf_mark(p.trace, tr, 6);
-                if (j + 1 < n_tiles) {                      // tile j + 1 was requested three rounds ago: tell the S warps
+                if (kBlocks == 1 && j + 1 < n_tiles) {      // tile j + 1 was requested three rounds ago: tell the S warps
                     asm volatile("cp.async.wait_group 2;" ::: "memory");
                     named_arrive(kLfBarData + (par ^ 1), 256);
                 }
                 lf_mark(p.trace, tr, 7);
                 named_sync(kLfBarP + par, 256);             // P of tile j is there
                 lf_mark(p.trace, tr, 8);
-                uint32_t pf[16];
                 const uint32_t *pb = p_all + par * (16 * 32);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) pf[i] = pb[i * 32 + lane];
                 const float a0 = alpha_all[par * 16 + r], a1 = alpha_all[par * 16 + r + 8];
                 if (__any_sync(0xFFFFFFFFu, a0 != 1.f || a1 != 1.f)) {        // most tiles leave the maxima where they were
 #pragma unroll
                     for (int j2 = 0; j2 < 16; ++j2) { o[j2][0] *= a0; o[j2][1] *= a0; o[j2][2] *= a1; o[j2][3] *= a1; }
                 }
-                const uint32_t tile_addr = smem_base + (j & (kLfStages - 1)) * kTileBytes;
-                {
-                    uint32_t vb[2][8][4];                   // V fragments of the 16 column tiles, both k-steps: all loads first
+                const uint32_t tile_addr = smem_base + (j & (kStages - 1)) * kTileBytes;
+                auto load_v = [&](uint32_t (&vb)[8][4], int ks2) {              // V fragments of the 16 column tiles, one k-step
 #pragma unroll
-                    for (int ks2 = 0; ks2 < 2; ++ks2) {
+                    for (int j2 = 0; j2 < 8; ++j2) {
+                        const int mi = lane >> 3;
+                        const int row = 16 * ks2 + ((mi & 1) << 3) + (lane & 7);
+                        const int chunk = 16 * gw + 2 * j2 + (mi >> 1);
+                        ldmatrix_x4_trans(vb[j2][0], vb[j2][1], vb[j2][2], vb[j2][3], tile_addr + row * kRowBytes + ((chunk ^ (lane & 7)) << 4));
+                    }
+                };
+                auto add_pv = [&](const uint32_t (&vb)[8][4], int ks2) {
+#pragma unroll
+                    for (int term = 0; term < 2; ++term) {                      // 16 independent accumulators per term
+                        uint32_t pf[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) pf[i] = pb[(8 * term + 4 * ks2 + i) * 32 + lane];
 #pragma unroll
                         for (int j2 = 0; j2 < 8; ++j2) {
-                            const int mi = lane >> 3;
-                            const int row = 16 * ks2 + ((mi & 1) << 3) + (lane & 7);
-                            const int chunk = 16 * gw + 2 * j2 + (mi >> 1);
-                            ldmatrix_x4_trans(vb[ks2][j2][0], vb[ks2][j2][1], vb[ks2][j2][2], vb[ks2][j2][3],
-                                              tile_addr + row * kRowBytes + ((chunk ^ (lane & 7)) << 4));
+                            mma_bf16(o[2 * j2], pf[0], pf[1], pf[2], pf[3], vb[j2][0], vb[j2][1]);
+                            mma_bf16(o[2 * j2 + 1], pf[0], pf[1], pf[2], pf[3], vb[j2][2], vb[j2][3]);
                         }
                     }
+                };
+                if constexpr (kBlocks == 1) {
+                    uint32_t v0[8][4], v1[8][4];                                // all loads first
+                    load_v(v0, 0);
+                    load_v(v1, 1);
+                    add_pv(v0, 0);
+                    add_pv(v1, 1);
+                } else {
 #pragma unroll
                     for (int ks2 = 0; ks2 < 2; ++ks2) {
-#pragma unroll
-                        for (int term = 0; term < 2; ++term) {      // 16 independent accumulators per term
-#pragma unroll
-                            for (int j2 = 0; j2 < 8; ++j2) {
-                                mma_bf16(o[2 * j2], pf[8 * term + 4 * ks2], pf[8 * term + 4 * ks2 + 1], pf[8 * term + 4 * ks2 + 2],
-                                         pf[8 * term + 4 * ks2 + 3], vb[ks2][j2][0], vb[ks2][j2][1]);
-                                mma_bf16(o[2 * j2 + 1], pf[8 * term + 4 * ks2], pf[8 * term + 4 * ks2 + 1], pf[8 * term + 4 * ks2 + 2],
-                                         pf[8 * term + 4 * ks2 + 3], vb[ks2][j2][2], vb[ks2][j2][3]);
-                            }
-                        }
+                        uint32_t v[8][4];
+                        load_v(v, ks2);
+                        add_pv(v, ks2);
                     }
                 }
                 lf_mark(p.trace, tr, 9);
                 named_sync(kLfBarV, 128);                   // every P V warp is done with this stage
                 lf_mark(p.trace, tr, 10);
-                issue(j + kLfStages, meta_cur);
+                issue(j + kStages, meta_cur);
+                if (kBlocks == 2 && j + 1 < n_tiles) {      // a ring of two: only now is it time to wait for tile j + 1
+                    asm volatile("cp.async.wait_group 1;" ::: "memory");
+                    named_arrive(kLfBarData + (par ^ 1), 256);
+                }
                 lf_mark(p.trace, tr, 11);
             }
             asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -999,14 +1038,16 @@ LatentView make_latent_view(const santapp_latent_geom *g, const santapp_latent_t
 // Workspace of the decode calls. Offsets in bytes.
 struct LatentLayout {
     size_t y32, sel_team, sel_logc, sel_rows, row_meta, seg_bias, pair_rows, pair_prefix, partials, total;
-    int seg_cap, grid;
+    int seg_cap, sms, blocks, grid;        // attention: blocks per SM and blocks in all
     int64_t y_stride;
 };
 
 LatentLayout latent_layout(const santapp_latent_geom *g, const santapp_latent_teams *t, int K, int suffix_cap, bool dense)
 {
     LatentLayout L;
-    L.grid = attend_grid_size();
+    L.sms = attend_grid_size();
+    L.blocks = latent_blocks_per_sm(t->rows_total, g->n_seqs, L.sms, dense);
+    L.grid = L.blocks * L.sms;
     int64_t cap = (int64_t)g->n_heads * K;
     if (cap > t->max_teams_per_seq) cap = t->max_teams_per_seq;
     L.seg_cap = (int)cap + 1;
@@ -1047,41 +1088,39 @@ int latent_attend_and_merge(const santapp_latent_geom *geom, const santapp_laten
     ap.partials = reinterpret_cast<float *>(ws + L.partials);
     ap.pair_prefix = reinterpret_cast<uint32_t *>(ws + L.pair_prefix);
     ap.trace = trace;
+    // The tcgen05 variant (latent_tc.cuh) computes the same thing on the 5th-generation tensor cores; it is
+    // slower here (a tcgen05.mma of N = 16 columns costs as much as one of 64, and one thread issues 68 of
+    // them per 64 rows), so the mma.sync kernel is the default and the other is chosen by the environment
+    // (SANTAPP_LATENT_ATTEND=tcgen05).
+    const char *which = getenv("SANTAPP_LATENT_ATTEND");
+    const bool tc = which != nullptr && strcmp(which, "tcgen05") == 0;
     cudaError_t err;
     if (mask & SANTAPP_STAGE_ATTEND) {
         static std::atomic<unsigned long long> done_tc_all, done_tc_sel;
-        // The tcgen05 variant (latent_tc.cuh) computes the same thing on the 5th-generation tensor cores; it is
-        // slower here (a tcgen05.mma of N = 16 columns costs as much as one of 64, and one thread issues 68 of
-        // them per 64 rows), so the mma.sync kernel is the default and the other is chosen by the environment
-        // (SANTAPP_LATENT_ATTEND=tcgen05).
-        const char *which = getenv("SANTAPP_LATENT_ATTEND");
-        const bool tc = which != nullptr && strcmp(which, "tcgen05") == 0;
-        static std::atomic<unsigned long long> done_sp_all, done_sp_sel;
         if (!tc) {
-            if (dense) {
-                if ((err = ensure_dynamic_smem((const void *)latent_attend_kernel<true>, kLfSmemBytes, done_sp_all)) != cudaSuccess)
-                    return note_cuda_failure(err, "latent attend attribute");
-                err = launch_step(latent_attend_kernel<true>, dim3(L.grid), dim3(kLfThreads), kLfSmemBytes, s, ap);
-            } else {
-                if ((err = ensure_dynamic_smem((const void *)latent_attend_kernel<false>, kLfSmemBytes, done_sp_sel)) != cudaSuccess)
-                    return note_cuda_failure(err, "latent attend attribute");
-                err = launch_step(latent_attend_kernel<false>, dim3(L.grid), dim3(kLfThreads), kLfSmemBytes, s, ap);
-            }
+            static const struct { void (*run)(LatentAttendParams); int smem; } forms[2][2] = {
+                {{latent_attend_kernel<false, 1>, LfShape<1>::smem_bytes}, {latent_attend_kernel<false, 2>, LfShape<2>::smem_bytes}},
+                {{latent_attend_kernel<true, 1>, LfShape<1>::smem_bytes}, {latent_attend_kernel<true, 2>, LfShape<2>::smem_bytes}}};
+            static std::atomic<unsigned long long> done[2][2];
+            const auto &form = forms[dense][L.blocks - 1];
+            if ((err = ensure_dynamic_smem((const void *)form.run, form.smem, done[dense][L.blocks - 1])) != cudaSuccess)
+                return note_cuda_failure(err, "latent attend attribute");
+            err = launch_step(form.run, dim3(L.grid), dim3(kLfThreads), form.smem, s, ap);
         } else if (dense) {
             if ((err = ensure_dynamic_smem((const void *)latent_attend_tc_kernel<true>, kTcSmemBytes, done_tc_all)) != cudaSuccess)
                 return note_cuda_failure(err, "latent attend attribute");
-            err = launch_step(latent_attend_tc_kernel<true>, dim3(L.grid), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
+            err = launch_step(latent_attend_tc_kernel<true>, dim3(L.sms), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
         } else {
             if ((err = ensure_dynamic_smem((const void *)latent_attend_tc_kernel<false>, kTcSmemBytes, done_tc_sel)) != cudaSuccess)
                 return note_cuda_failure(err, "latent attend attribute");
-            err = launch_step(latent_attend_tc_kernel<false>, dim3(L.grid), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
+            err = launch_step(latent_attend_tc_kernel<false>, dim3(L.sms), dim3(kTcThreads), kTcSmemBytes, s, ap, status);
         }
         if (err != cudaSuccess) return note_cuda_failure(err, "latent attend launch");
         ++launches;
     }
     if (mask & SANTAPP_STAGE_MERGE) {
         err = launch_step(latent_merge_kernel, dim3(geom->n_heads, geom->n_seqs), dim3(kLmThreads), 0, s,
-                            (const float *)ap.partials, (const uint32_t *)ap.pair_prefix, geom->n_seqs, geom->n_heads, L.grid, out,
+                            (const float *)ap.partials, (const uint32_t *)ap.pair_prefix, geom->n_seqs, geom->n_heads, tc ? L.sms : L.grid, out,
                             status);
         if (err != cudaSuccess) return note_cuda_failure(err, "latent merge launch");
         ++launches;
@@ -1279,7 +1318,7 @@ int santapp_latent_decode_attn(const santapp_latent_geom *geom, const santapp_la
         in.dbg_union_rows = nullptr;
         in.trace = dbg ? reinterpret_cast<unsigned long long *>(dbg->trace) : nullptr;
         const int n_heads = geom->n_seqs * geom->n_heads;
-        if (n_heads <= L.grid) err = launch_step(latent_select_kernel<512>, dim3(n_heads), dim3(512), 0, s, in);
+        if (n_heads <= L.sms) err = launch_step(latent_select_kernel<512>, dim3(n_heads), dim3(512), 0, s, in);
         else                   err = launch_step(latent_select_kernel<256>, dim3(n_heads), dim3(256), 0, s, in);
         if (err != cudaSuccess) return note_cuda_failure(err, "latent select launch");
         ++launches;

@@ -224,6 +224,22 @@ def test_step_ragged_batch_with_several_tiles_per_scoring_warp():
     check_step(layer, 0, seqs=[0, 7, 40, 71])
 
 
+@pytest.mark.parametrize("n,lo,hi", [(15, 15200, 15900), (16, 14250, 15000), (512, 1, 920), (513, 1, 920)])
+def test_step_attention_with_one_and_two_blocks_per_sm(n, lo, hi):
+    """Enough rows for two blocks per SM at the fewest and the most sequences that take them, and one sequence
+    beside either limit: shares of many tiles, and shares of part of one; the shortest and the longest sequence,
+    the first and the last against the oracle."""
+    rng = np.random.default_rng(n)
+    lens = [int(x) for x in rng.integers(lo, hi, size=n)]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lens[n // 2] += max(0, 1536 * sms - sum(lens))          # the larger of the two limits on the rows
+    layer = LatentLayer(synth.LatentSpec("blocks", lens, n_sample=48, suffix_cap=4,
+                                         suffix_len0=[int(x) for x in rng.integers(0, 5, size=n)], suffix_growth=0))
+    seqs = sorted({0, n - 1, int(np.argmin(lens)), int(np.argmax(lens))})
+    check_step(layer, 1, seqs=seqs)
+    check_dense(layer, 1, seqs=seqs)
+
+
 def test_two_hundred_steps_of_the_sampler():
     """Many draws on one layer (a different seed every step, K = 96 of 512 and 375 teams): now and
     then two candidates' scores agree in the upper half of their integer keys, which sends a head
