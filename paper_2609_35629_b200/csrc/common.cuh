@@ -190,19 +190,7 @@ inline cudaError_t ensure_dynamic_smem(const void *fn, int bytes, std::atomic<un
     return err;
 }
 
-// Launch through cudaLaunchKernelEx so that the launch's own status comes back (no sticky-error read).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
-// Launch of a kernel of a decode step: it may be set up while the kernel before it on the stream is still
+// Launch of a kernel of a decode step (through cudaLaunchKernelEx, so that the launch's own status comes back): it may be set up while the kernel before it on the stream is still
 // running (programmatic stream serialisation), and starts with step_wait(), which returns once that
 // kernel has completed. Outside a CUDA graph a plain launch behind a running kernel cost 1.5 us more than
 // inside one; with this the eager step takes what the graph takes (28 layers of batch 1 at 32K: 903 ->
@@ -367,9 +355,8 @@ cudaError_t launch_kmeans_tables(const KmTableChunk &c, int64_t *row_off, int64_
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 __device__ __forceinline__ float bf16_to_float(uint16_t b) { return __uint_as_float(((uint32_t)b) << 16); }
-__device__ __forceinline__ double bf16_to_double(uint16_t b) { return (double)bf16_to_float(b); }
 
-// The same three conversions for either 16-bit element type (kHalf: IEEE fp16, else bf16).
+// The same conversions for either 16-bit element type (kHalf: IEEE fp16, else bf16).
 template <bool kHalf>
 __device__ __forceinline__ float elem_to_float(uint16_t b)
 {
@@ -499,11 +486,6 @@ __device__ __forceinline__ unsigned long long sortable_key(double v)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     return (b & 0x8000000000000000ull) ? ~b : (b | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double key_to_double(unsigned long long k)
-{
-    const unsigned long long b = (k & 0x8000000000000000ull) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k;
-    return __longlong_as_double((long long)b);
 }
 
 // Exclusive prefix sum of one int per thread over the block; returns the thread's offset and the

@@ -104,9 +104,9 @@ struct TileScores {
 // c + 4 i of the key of team base + 8 t + g), in two halves so that a kernel walking many tiles can
 // run the tensor-core instructions of one tile beside the arithmetic of the previous one.
 // The 16 teams are the M rows of the tensor-core tile and the query heads its 8 columns, so one
-// instruction per 16 dimensions covers the whole tile (the legacy tensor-core instruction is slow
-// on this GPU, and a tile's time is mostly spent waiting for them). A lane ends up with the
-// scores of teams g and g + 8 for heads 2 c and 2 c + 1.
+// instruction per 16 dimensions covers the whole tile (the instruction issues every
+// 8 cycles and takes 21, and the eight of a tile depend on one another: fewer of them shorten the chain). A lane
+// ends up with the scores of teams g and g + 8 for heads 2 c and 2 c + 1.
 // csr_tile points at the 17 row offsets of the tile's teams (global or shared memory);
 // words_smem: 128 words of this warp's own shared memory (the tile's Philox words, [head][team]);
 // the caller orders writes and reads of that buffer (__syncwarp) between the two halves.
