@@ -427,6 +427,18 @@ def test_decode_many_short_sequences():
     check_dense_step(layer, 0)
 
 
+@pytest.mark.parametrize("n_seqs,K", [(2, 100), (2, 128), (12, 128), (24, 60), (24, 100), (24, 127), (24, 128)])
+@pytest.mark.parametrize("gain", [1.0, 16.0])
+def test_decode_candidates_around_a_thread_each(n_seqs, K, gain):
+    """The sampler ranks in one pass with a candidate per thread: budgets whose candidates are fewer than, as many as
+    and more than the 512, 256 or 128 threads of a head, and scores spread beyond the range of its keys."""
+    spec = synth.spec_small_gqa(n_seqs=n_seqs, prompt=tuple(500 + 37 * (i % 5) for i in range(n_seqs)), parent_size=32, reps=32,
+                                suffix0=tuple(i % 4 for i in range(n_seqs)))
+    layer = pu.GpuLayer(spec, synth.make_layer(spec))
+    bits = synth.make_queries(spec, layer.data, 3)
+    _check_with_queries(layer, synth.f32_to_bf16_bits(np.float32(gain) * synth.bf16_to_f32(bits)), K=K, step=3)
+
+
 @pytest.mark.parametrize("n_q,n_kv", [(32, 4), (8, 2), (6, 6), (3, 1)])
 def test_decode_other_group_sizes(n_q, n_kv):
     """GQA groups of 8, 4, 1 and 3 query heads per KV head (the tensor-core tile holds up to 8)."""
