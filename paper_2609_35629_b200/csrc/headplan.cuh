@@ -125,37 +125,50 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
     const int n4 = (M + 3) >> 2;                                      // 16-byte pieces that hold teams
     const int need = K + 1;
 
-    // f(x, team, valid) for every score slot this thread owns, the same number of calls in every
-    // thread of the block (so f may use warp-wide votes); x = -inf where valid is false
-    auto each_score = [&](auto &&f) {
+    // what lies behind the last team becomes -inf; pm: a piece's largest score, gm: that of a group of 16 teams (four
+    // neighbouring lanes' pieces), formed here, where the shuffles of the pieces overlap
+    auto mask_piece = [&](float4 &v, int at) {
+        if (4 * at + 3 >= M) {
+            if (4 * at >= M) v.x = -CUDART_INF_F;
+            if (4 * at + 1 >= M) v.y = -CUDART_INF_F;
+            if (4 * at + 2 >= M) v.z = -CUDART_INF_F;
+            v.w = -CUDART_INF_F;
+        }
+        return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
+    };
+    auto group_max = [&](float x) {
+        x = fmaxf(x, __shfl_xor_sync(0xFFFFFFFFu, x, 1));
+        return fmaxf(x, __shfl_xor_sync(0xFFFFFFFFu, x, 2));
+    };
+    float pm[kScoreRegs], gm[kScoreRegs];
+#pragma unroll
+    for (int i = 0; i < kScoreRegs; ++i) pm[i] = mask_piece(yv[i], tid + i * kT);
+#pragma unroll
+    for (int i = 0; i < kScoreRegs; ++i) gm[i] = group_max(pm[i]);
+    // f(piece, its largest score, its group's, piece index) for every piece this thread owns, the same number of calls in
+    // every thread of the block
+    auto each_piece = [&](auto &&f) {
 #pragma unroll
         for (int i = 0; i < kScoreRegs; ++i) {
             if (4 * i * kT >= M) break;                               // the same for every thread: no team in this piece or later ones
-            const int at = tid + i * kT;
-            const float4 v = yv[i];
-            f(4 * at < M ? v.x : -CUDART_INF_F, 4 * at, 4 * at < M);
-            f(4 * at + 1 < M ? v.y : -CUDART_INF_F, 4 * at + 1, 4 * at + 1 < M);
-            f(4 * at + 2 < M ? v.z : -CUDART_INF_F, 4 * at + 2, 4 * at + 2 < M);
-            f(4 * at + 3 < M ? v.w : -CUDART_INF_F, 4 * at + 3, 4 * at + 3 < M);
+            f(yv[i], pm[i], gm[i], tid + i * kT);
         }
         for (int base = kScoreRegs * kT; base < n4; base += kT) {
             const int at = base + tid;
-            const float4 v = at < n4 ? __ldcg(y4 + at) : kNone;
-            f(4 * at < M ? v.x : -CUDART_INF_F, 4 * at, 4 * at < M);
-            f(4 * at + 1 < M ? v.y : -CUDART_INF_F, 4 * at + 1, 4 * at + 1 < M);
-            f(4 * at + 2 < M ? v.z : -CUDART_INF_F, 4 * at + 2, 4 * at + 2 < M);
-            f(4 * at + 3 < M ? v.w : -CUDART_INF_F, 4 * at + 3, 4 * at + 3 < M);
+            float4 v = at < n4 ? __ldcg(y4 + at) : kNone;
+            const float x = mask_piece(v, at);
+            f(v, x, group_max(x), at);
         }
     };
     {
         float a = 0.f, top = -CUDART_INF_F;
 #pragma unroll
         for (int i = 0; i < kQRegs; ++i) a += fabsf(q_val[i]);
-        each_score([&](float x, int, bool) { top = fmaxf(top, x); });
+        each_piece([&](const float4 &, float, float g, int) { top = fmaxf(top, g); });
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-            top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+            if (o >= 4) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
         }
         trace_mark(in.trace, 1, 8);
         __syncthreads();                                              // the shared structure is free (block reuse)
@@ -196,24 +209,16 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
                 const int gb = score_bin(top, x);
                 if (gb >= win) atomicAdd(&sm.hist[min(gb - win, kWindow)], 1);
             };
-            float grp = -CUDART_INF_F;
-            bool any = false;
-            each_score([&](float x, int team, bool valid) {
-                if (level == 0) {
-                    if (valid) count(x);
+            each_piece([&](const float4 &v, float x, float g, int at) {
+                if (level == 2) {
+                    if ((lane & 3) == 0 && 4 * at < M) count(g);
+                } else if (level == 1) {
+                    if (4 * at < M) count(x);
                 } else {
-                    grp = fmaxf(grp, x);
-                    any = any || valid;
-                    if ((team & 3) == 3) {                            // the piece is complete
-                        if (level == 2) {                             // four neighbouring lanes hold one group of 16
-                            grp = fmaxf(grp, __shfl_xor_sync(0xFFFFFFFFu, grp, 1));
-                            grp = fmaxf(grp, __shfl_xor_sync(0xFFFFFFFFu, grp, 2));
-                            any = __shfl_sync(0xFFFFFFFFu, (int)any, lane & ~3) != 0 && (lane & 3) == 0;
-                        }
-                        if (any) count(grp);
-                        grp = -CUDART_INF_F;
-                        any = false;
-                    }
+                    if (4 * at < M) count(v.x);
+                    if (4 * at + 1 < M) count(v.y);
+                    if (4 * at + 2 < M) count(v.z);
+                    if (4 * at + 3 < M) count(v.w);
                 }
             });
             trace_mark(in.trace, 1, 9);
@@ -253,22 +258,28 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
     const float t_lo = t_lb - 2.f * guard;
     trace_mark(in.trace, 1, 3);
 
-    // ---- 2. candidates: teams whose score reaches t_lo; a warp reserves its slots with one atomic ----
+    // ---- 2. candidates: teams whose score reaches t_lo; a thread that has some reserves their slots with one atomic ----
     {
-        int cnt = 0;
-        each_score([&](float x, int, bool valid) { cnt += __popc(__ballot_sync(0xFFFFFFFFu, valid && x >= t_lo)); });
-        int base = 0;
-        if (lane == 0 && cnt > 0) base = atomicAdd(&sm.n_cand, cnt);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        each_score([&](float x, int team, bool valid) {
-            const bool mine = valid && x >= t_lo;
-            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, mine);
-            if (mine) {
-                const int slot = base + __popc(votes & ((1u << lane) - 1u));
-                if (slot < kCandCap) sm.cand_id[slot] = team;
-            }
-            base += __popc(votes);
-        });
+        auto reach = [&](const float4 &v, float x, int at) {              // bit e: score e of the piece (teams behind the last one hold -inf)
+            if (!(x >= t_lo) || 4 * at >= M) return 0u;
+            const uint32_t bits = (v.x >= t_lo ? 1u : 0u) | (v.y >= t_lo ? 2u : 0u) | (v.z >= t_lo ? 4u : 0u) | (v.w >= t_lo ? 8u : 0u);
+            return 4 * at + 3 < M ? bits : bits & ((1u << (M - 4 * at)) - 1u);
+        };
+        uint32_t hits = 0u;                                               // the register pieces', four bits each
+#pragma unroll
+        for (int i = 0; i < kScoreRegs; ++i) hits |= reach(yv[i], pm[i], tid + i * kT) << (4 * i);
+        auto take = [&](uint32_t bits, auto &&team_of) {
+            if (bits == 0u) return;
+            int slot = atomicAdd(&sm.n_cand, __popc(bits));
+            for (; bits != 0u; bits &= bits - 1u, ++slot)
+                if (slot < kCandCap) sm.cand_id[slot] = team_of(__ffs((int)bits) - 1);
+        };
+        take(hits, [&](int bit) { return 4 * (tid + (bit >> 2) * kT) + (bit & 3); });
+        for (int at = kScoreRegs * kT + tid; at < n4; at += kT) {
+            float4 v = __ldcg(y4 + at);
+            const float x = mask_piece(v, at);
+            take(reach(v, x, at), [&](int bit) { return 4 * at + bit; });
+        }
     }
     __syncthreads();
     trace_mark(in.trace, 1, 4);
