@@ -100,10 +100,7 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
 #pragma unroll
     for (int i = 0; i < kScoreRegs; ++i) {
         const int at = tid + i * kT;
-        yv[i] = kNone;
-        if (at < n4_row)                                              // (volatile: the compiler would ask only after the early return below)
-            asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(yv[i].x), "=f"(yv[i].y), "=f"(yv[i].z), "=f"(yv[i].w) : "l"(y4 + at));
+        yv[i] = at < n4_row ? __ldcg(y4 + at) : kNone;
     }
     float q_val[kQRegs];
 #pragma unroll
@@ -212,19 +209,18 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
                 const int gb = score_bin(top, x);
                 if (gb >= win) atomicAdd(&sm.hist[min(gb - win, kWindow)], 1);
             };
-            if (level != 0) {
-                const bool counts = level == 1 || (lane & 3) == 0;
-                each_piece([&](const float4 &, float x, float g, int at) {
-                    if (counts && 4 * at < M) count(level == 2 ? g : x);
-                });
-            } else {
-                each_piece([&](const float4 &v, float, float, int at) {
+            each_piece([&](const float4 &v, float x, float g, int at) {
+                if (level == 2) {
+                    if ((lane & 3) == 0 && 4 * at < M) count(g);
+                } else if (level == 1) {
+                    if (4 * at < M) count(x);
+                } else {
                     if (4 * at < M) count(v.x);
                     if (4 * at + 1 < M) count(v.y);
                     if (4 * at + 2 < M) count(v.z);
                     if (4 * at + 3 < M) count(v.w);
-                });
-            }
+                }
+            });
             trace_mark(in.trace, 1, 9);
             __syncthreads();
             trace_mark(in.trace, 1, 10);
