@@ -159,10 +159,11 @@ __device__ __forceinline__ void near_look(NearTop &n, const uint32_t (&v)[32], c
     }
     if (t1 <= n.upper) {
         const float2 b = bias[__float_as_uint(t1) & 31u];
-        // (1.0001: the stored constant is |c|^2 (1 - kNearErr), rounded)
-        n.upper = fminf(n.upper, fmaf(2.f, fmaf(1.0001f * kNearErr, b.x, reach * b.y), t1 + shared));
+        // (1.0001: the stored constant is |c|^2 (1 - kNearErr), rounded. The mark of a centre that the products say nothing about
+        // bounds nothing from above: it stays the smallest key, and near_open finds it.)
+        if (t1 > -1e38f) n.upper = fminf(n.upper, fmaf(2.f, fmaf(1.0001f * kNearErr, b.x, reach * b.y), t1 + shared));
+        near_insert(n, t1, first + (int)(__float_as_uint(t1) & 31u));
     }
-    if (t1 <= n.upper) near_insert(n, t1, first + (int)(__float_as_uint(t1) & 31u));
     while (__any_sync(0xFFFFFFFFu, t2 <= n.upper)) {         // some point of the warp has another candidate here
         if (t2 <= n.upper) near_insert(n, t2, first + (int)(__float_as_uint(t2) & 31u));
         float next = kNearFar;

@@ -192,3 +192,29 @@ def test_fit_with_a_centre_per_key_returns_the_keys(n):
     order = (((got[:, :15] + 1.0) / 3.0) @ (2.0 ** np.arange(15))).astype(np.int64)
     assert np.array_equal(np.sort(order), np.arange(n))
     assert np.array_equal(got, rows[0][order])
+
+
+def _fit_keys_both(keys, elem, k, **opts):
+    """A fit of one sequence's keys [n_kv][N][128] on the GPU and by the oracle, pair by pair."""
+    bits = synth.round_bits(keys, elem)
+    n_kv, N = keys.shape[:2]
+    geom = sp.Geometry(1, n_kv, n_kv, 128, 16, 4, sp.SANTAPP_FP16 if elem == "fp16" else sp.SANTAPP_BF16)
+    centres, steps = sp.santapp_kmeans_fit(geom, [N], [k], sp.bf16_bits_to_cuda(bits, dtype=geom.torch_dtype), **opts)
+    torch.cuda.synchronize()
+    o = {"batch": opts["batch_size"], "max_iter": opts["max_iter"], "patience": opts["patience"], "seed": opts["seed"]}
+    for j in range(n_kv):
+        want, want_steps = orc.minibatch_kmeans(synth.to_f64(bits[j], elem), k, stream=j, ratio=opts["reassignment_ratio"], **o)
+        assert int(steps[j, 0]) == want_steps, f"steps of pair {j}"
+        assert np.array_equal(centres[j].cpu().numpy(), want.astype(np.float32)), f"centres of pair {j}"
+
+
+@pytest.mark.parametrize("elem,far", [("fp16", 6000.0), ("fp16", 60000.0), ("bf16", 1e20)])
+def test_fit_with_outlier_keys_beyond_the_range_of_the_bounds(elem, far):
+    """Two keys so long that the greedy start makes them centres and no product bounds their distances
+    (squared norm beyond 4.2e9 for fp16, 1e37 for bf16): the minibatch steps of the ordinary keys are the oracle's."""
+    rng = np.random.default_rng(17)
+    keys = rng.standard_normal((2, 900, 128)).astype(np.float32)
+    for j, rows in enumerate([(3, 600), (450, 899)]):
+        keys[j, rows[0]] = far
+        keys[j, rows[1]] = -far
+    _fit_keys_both(keys, elem, 200, batch_size=256, max_iter=3, patience=4, seed=2, reassignment_ratio=0.0)

@@ -260,3 +260,23 @@ def test_null_team_count_means_every_slot_is_a_team():
     dense_a, _ = pu.gpu_step(layer, q_bits, sl, 0, 0, 0, dense=True)
     assert np.array_equal(out_a, out_b) and np.array_equal(dense_a, dense_b)
     assert torch.equal(dbg_a.sel_idx, dbg_b.sel_idx)
+
+
+@pytest.mark.parametrize("elem,far", [("fp16", 6000.0), ("fp16", 60000.0), ("bf16", 1e20), ("bf16", np.inf), ("bf16", np.nan)])
+@pytest.mark.parametrize("at", [(0,), (40,), (97,), (150,), (299,), (5, 6, 33, 290)])
+def test_assignment_with_centres_whose_norm_the_products_cannot_bound(elem, far, at):
+    """Centres far outside the range of the bounds (squared norm beyond 4.2e9 for fp16 calls, 1e37 for bf16), or not
+    numbers, among 300 ordinary ones, in every column half and tile of the scan: ordinary tokens still go to
+    the nearest of all centres, exact ties to the smaller index (the last 30 ordinary centres repeat earlier ones)."""
+    rng = np.random.default_rng([len(at), at[0]])
+    N, k = 700, 300
+    cen = rng.standard_normal((1, k, 128)).astype(np.float32)
+    cen[0, 270:] = cen[0, rng.permutation(270)[:30]]
+    keys = cen[0, rng.integers(0, k, size=N)] + 0.7 * rng.standard_normal((N, 128)).astype(np.float32)
+    cen[0, list(at)] = np.float32(far)
+    bits = synth.round_bits(keys[None], elem)
+    geom = sp.Geometry(1, 1, 1, 128, 16, 4, sp.SANTAPP_FP16 if elem == "fp16" else sp.SANTAPP_BF16)
+    lab = sp.santapp_assign_parents(geom, [N], [k], sp.bf16_bits_to_cuda(bits, dtype=geom.torch_dtype), torch.from_numpy(cen).cuda())
+    want, _, _ = orc.nearest_centre_parents(synth.to_f64(bits[0], elem), cen[0].astype(np.float64))
+    assert np.array_equal(lab[0].cpu().numpy(), want)
+    assert len(set(want.tolist())) > 200 and not set(at) & set(want.tolist())
