@@ -1079,7 +1079,8 @@ km_sort_batch_kernel(KmeansParams p, int t)
         km_inertia(p, q, t - 1, 4, 5, reinterpret_cast<double *>(smem_raw));
         return;
     }
-    if (!pair_active(p, q, t)) return;
+    // one look at the flag for the block: beside it the block above may be stopping this very fit
+    if (!__syncthreads_or(threadIdx.x == 0 && pair_active(p, q, t))) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t *idx = p.idx + (size_t)q.id * p.batch;
     uint32_t key[4];                                        // the warp's 128 entries, 32 at a time in order

@@ -218,3 +218,25 @@ def test_fit_with_outlier_keys_beyond_the_range_of_the_bounds(elem, far):
         keys[j, rows[0]] = far
         keys[j, rows[1]] = -far
     _fit_keys_both(keys, elem, 200, batch_size=256, max_iter=3, patience=4, seed=2, reassignment_ratio=0.0)
+
+
+def test_fits_that_stop_beside_their_own_sorting_blocks():
+    """The stopping rule of a step is settled beside the ordering of the next minibatch, in other blocks of one launch.
+    192 fits that stop at many different steps, every step enqueued: ten runs, each with the oracle's step counts
+    and the first run's centres."""
+    rng = np.random.default_rng(21)
+    B, kv, k = 96, 2, 5
+    lens = [int(x) for x in rng.integers(40, 90, size=B)]
+    bits = synth.round_bits(rng.standard_normal((kv, sum(lens), 128)).astype(np.float32))
+    geom, keys = sp.Geometry(B, kv, kv, 128, 16, 4), sp.bf16_bits_to_cuda(bits)
+    opts = dict(batch_size=16, max_iter=12, patience=2, seed=6, no_host_poll=True)
+    off = np.concatenate([[0], np.cumsum(lens)])
+    want = [[orc.minibatch_kmeans(synth.to_f64(bits[j, off[b]:off[b + 1]]), k, batch=16, max_iter=12, patience=2, seed=6, stream=b * kv + j)[1]
+             for b in range(B)] for j in range(kv)]
+    first = None
+    for _ in range(10):
+        centres, steps = sp.santapp_kmeans_fit(geom, lens, [k] * B, keys, **opts)
+        assert steps.cpu().tolist() == want
+        first = centres if first is None else first
+        assert torch.equal(centres, first)
+    assert len(set(np.ravel(want).tolist())) > 8
