@@ -494,7 +494,7 @@ km_start_kernel(KmeansParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StartSmem &sm = *reinterpret_cast<StartSmem *>(smem_raw);
-    constexpr float kPairErr = 0.5f * kDistErr;             // times the sum of the two squared norms
+    constexpr float kPairErr = 0.5f * kDistErr;             // times the sum of the two squared norms, plus kUnderflow
     const int n_blk = (int)cluster_size(), rank = (int)cluster_rank();
     const int pair = blockIdx.x / n_blk, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, c4 = lane & 3;
     const Pair q = pair_of(p, pair / p.n_kv, pair % p.n_kv);
@@ -585,18 +585,18 @@ km_start_kernel(KmeansParams p)
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {
                             val[h][v] = fmaf(-2.f, acc[k][v >> 1][2 * h + (v & 1)], bar + ny[v]);
-                            if (!(val[h][v] > 1e-34f)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));     // (1e-34: products that underflow)
+                            if (!(val[h][v] > kUnderflow)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));
                         }
                         if (!(bar < CUDART_INF_F)) bits[h] = 0u;     // past the end of the sample
                     }
                     if (__any_sync(0xFFFFFFFFu, (bits[0] | bits[1]) != 0u)) {
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const float e = 2.f * kPairErr * sm.norm[mt[k] * 16 + g + 8 * h];
+                            const float e = fmaf(2.f * kPairErr, sm.norm[mt[k] * 16 + g + 8 * h], kUnderflow);
 #pragma unroll
                             for (int v = 0; v < 4; ++v)
                                 if ((bits[h] >> ((v >> 1) * 8 + 2 * c4 + (v & 1))) & 1u) {
-                                    hi[v] -= val[h][v];
+                                    hi[v] += kUnderflow - val[h][v];
                                     lo[v] += fmaxf(-val[h][v] - (e + err[v]), 0.f);
                                 }
                             bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 1);

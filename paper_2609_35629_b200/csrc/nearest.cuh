@@ -9,7 +9,7 @@
 // distance; the column of a centre, kept in the last five bits of its bound, 2^-18 of at most 2.04 (|x|^2 + |c|^2).
 // Together at most E_c = kNearErr (|x|^2 + |c|^2) + 2 |x| m. A centre can be nearest only if its lower bound does not exceed the
 // smallest upper bound; where that leaves two or three they are compared in fp64, where it leaves more all
-// centres are (with early exit). Products that underflow fp32 add less than 1e-34.
+// centres are (with early exit). Products that underflow fp32 add less than kUnderflow.
 //
 // The products are a GEMM (tcgen05, 128 points x 128 centres x 128 dimensions a tile, 512 cycles at the measured rate);
 // looking at 16384 results takes the block's eight warps about twice that, since every one costs two FMAs and four
@@ -223,7 +223,7 @@ __device__ __forceinline__ void near_scan(NearSmem &sm, RowOf row_of, int k_lo, 
             }
             if (warp < 4) sm.nx[row] = n;
             reach = 2.000002f * sqrtf(n);
-            shared = fmaf(2.f * kNearErr, n, 1e-34f);
+            shared = fmaf(2.f * kNearErr, n, kUnderflow);
         } else {
             const int buf = (i - 1) & 1;
             near_wait(sm, buf, uses[buf] & 1u);

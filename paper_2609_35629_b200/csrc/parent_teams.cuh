@@ -284,7 +284,7 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
     float best = CUDART_INF_F;
 #pragma unroll
     for (int k = 0; k < kRpt; ++k)
-        if ((live >> k) & 1u) best = fminf(best, mind[k] + kDistErr * (norm[k] + mean_norm));
+        if ((live >> k) & 1u) best = fminf(best, mind[k] + fmaf(kDistErr, norm[k] + mean_norm, kUnderflow));
     best = -warp_max(-best);
     if (lane == 0) sm.red[2][warp] = best;
     __syncthreads();
@@ -293,7 +293,7 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
     unsigned maybe = 0u;
 #pragma unroll
     for (int k = 0; k < kRpt; ++k)
-        if (((live >> k) & 1u) && !(mind[k] - kDistErr * (norm[k] + mean_norm) > best)) { maybe |= 1u << k; sm.rep_of[0] = (uint16_t)LARGE_ROW(k); }
+        if (((live >> k) & 1u) && !(mind[k] - fmaf(kDistErr, norm[k] + mean_norm, kUnderflow) > best)) { maybe |= 1u << k; sm.rep_of[0] = (uint16_t)LARGE_ROW(k); }
     const bool one = __syncthreads_count(maybe != 0u) == 1 && __syncthreads_count(__popc(maybe) > 1) == 0;
     int rep = one ? sm.rep_of[0] : nearest_mean_exact<kWarps, kRpt, kHalf>(sm, nC, maybe);
 
@@ -306,7 +306,7 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
         for (int s = 0; s < 8; ++s)
             ldmatrix4(a[m][s], rows_a + (uint32_t)((warp * 32 * kRpt + 16 * m + (lane & 15)) * kPitch * 4 + (lane >> 4) * 16 + s * 32));
 
-    constexpr float kPairErr = 0.5f * kDistErr;               // times the sum of the two squared norms
+    constexpr float kPairErr = 0.5f * kDistErr;               // times the sum of the two squared norms, plus kUnderflow
     int owner[kRpt], parity = 0, u = 0;
     unsigned open_owner = 0u;                                 // bit k: the bound leaves the nearest representative open
 #pragma unroll
@@ -391,7 +391,7 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
             int top_row = 0;
 #pragma unroll
             for (int k = 0; k < kRpt; ++k) {
-                const float d = sm.dist[col][LARGE_ROW(k)], e = kPairErr * (norm[k] + rep_norm);
+                const float d = sm.dist[col][LARGE_ROW(k)], e = fmaf(kPairErr, norm[k] + rep_norm, kUnderflow);
                 if (u == 0 || d + e < lo[k]) {                // certainly nearer than every earlier one
                     mind[k] = d; lo[k] = d - e; hi[k] = d + e; owner[k] = u;
                     open_owner &= ~(1u << k);

@@ -12,8 +12,10 @@
 // one and add it to an fp32 total). That is 8 * 17 * 2^-23 * B for a dot product and four times that,
 // plus the rounding of the last few operations, for a distance: 2^-13.85 B. kDistErr is 5 % above. A score
 // against the parent's mean (norm minus twice the mean of the row's dot products) has a smaller
-// error. The fp64 sums are within 2^-44 of the true values, which the 5 % covers as well. Where fp32 could
-// overflow or lose the products to underflow (B outside [1e-30, 1e37], or not a number) the bound is infinite:
+// error. The fp64 sums are within 2^-44 of the true values, which the 5 % covers as well. A product below the range of
+// normal fp32 numbers may lose up to 2^-126 whatever the size of its factors; a distance has at most 4 * 576 such
+// losses, 3e-35, and kUnderflow stands for them in every bound that is relative to the two rows at hand. Where fp32
+// could overflow or loses most products (B outside [1e-30, 1e37], or not a number) the bound is infinite:
 // then every comparison is made on the fp64 sums.
 #pragma once
 #include <limits.h>
@@ -24,6 +26,7 @@
 namespace santapp {
 
 constexpr float kDistErr = 7.2e-5f;      // error bound of an fp32 distance, in units of the largest squared norm
+constexpr float kUnderflow = 1e-34f;     // and in absolute terms: products and squares that fp32 holds as subnormals or loses
 
 template <bool kHalf>
 __device__ __forceinline__ void mma_rows(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
@@ -52,7 +55,7 @@ __device__ __forceinline__ void copy_async_wait()
 
 __device__ __forceinline__ float dist_error(float largest_norm)
 {
-    return largest_norm >= 1e-30f && largest_norm <= 1e37f ? kDistErr * largest_norm : CUDART_INF_F;
+    return largest_norm >= 1e-30f && largest_norm <= 1e37f ? fmaf(kDistErr, largest_norm, kUnderflow) : CUDART_INF_F;
 }
 __device__ __forceinline__ float norm_or_inf(float n) { return n <= 1e37f ? n : CUDART_INF_F; }
 

@@ -92,3 +92,22 @@ def test_shared_latent_records_at_every_parent_size(P, R, kind):
         assert np.array_equal(csr[t0 + b:t1 + b + 1], ts) and np.array_equal(token[off[b]:off[b + 1]], tm)
         assert np.array_equal(synth.to_f64(rep[t0:t1]), reps) and np.array_equal(packed[off[b]:off[b + 1]], rows[tm])
         assert t.rep_abs_max[b].item() == np.abs(synth.to_f32(rep[t0:t1])).max()
+
+
+@pytest.mark.parametrize("P,R", [(16, 4), (32, 8), (64, 16), (128, 16), (256, 16), (512, 32)])
+@pytest.mark.parametrize("scale", [1e-21, 1e-22, 3e-23])
+def test_records_of_parents_with_one_ordinary_row_among_rows_whose_products_underflow(P, R, scale):
+    """One row of every parent is of ordinary length, so that fp32 distances are used, and the products of the others are
+    subnormal in fp32: their distances are decided by the fp64 sums."""
+    rng = np.random.default_rng([P, R, int(1 / scale) & 0xFFFF])
+    lens, kv = [4 * P], 2
+    x = (scale * rng.standard_normal((kv, lens[0], 128))).astype(np.float32)
+    x[:, P // 3::P] = rng.standard_normal((kv, 4, 128))
+    k_bits = synth.round_bits(x)
+    geom = sp.Geometry(1, kv, kv, 128, P, R)
+    k = sp.bf16_bits_to_cuda(k_bits)
+    t = sp.santapp_build_teams(geom, lens, k, k)
+    csr, token = t.team_row_start.cpu().numpy(), t.row_token.cpu().numpy()
+    for j in range(kv):
+        ts, tm, _ = orc.build_teams_contiguous(synth.to_f64(k_bits[j]), P, R)
+        assert np.array_equal(csr[j, :len(ts)], ts) and np.array_equal(token[j], tm)

@@ -240,3 +240,9 @@ def test_fits_that_stop_beside_their_own_sorting_blocks():
         first = centres if first is None else first
         assert torch.equal(centres, first)
     assert len(set(np.ravel(want).tolist())) > 8
+
+
+@pytest.mark.parametrize("scale", [1e-18, 1e-20, 1e-21, 1e-22])
+def test_fit_of_keys_whose_products_underflow(scale):
+    keys = scale * np.random.default_rng(23).standard_normal((4, 800, 128))
+    _fit_keys_both(keys.astype(np.float32), "bf16", 40, batch_size=128, max_iter=2, patience=4, seed=5, reassignment_ratio=0.01)
