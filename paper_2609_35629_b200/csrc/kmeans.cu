@@ -334,8 +334,9 @@ km_accept_kernel(KmeansParams p, int c)
 constexpr int kStartThreads = 256, kStartWarps = kStartThreads / 32;
 constexpr int kStartBlocks = 6;          // blocks of the sums per thread block: 768 rows of 256 bytes
 constexpr int kStartRows = kStartBlocks * kSumBlock;
-constexpr int kStartTrials = 10;         // 2 + floor(ln k) for every k with a sample of at most 16 * kStartRows
 constexpr int kStartMaxCluster = 16, kStartSums = kStartBlocks * kStartMaxCluster;
+constexpr int kStartTrials = 11;         // 2 + floor(ln k) for every k with a sample of at most 16 * kStartRows: k <= 12288, ln k < 10
+static_assert(kStartMaxCluster * kStartRows < 22026, "e^10: from there on a centre has more trials");
 
 struct StartSmem {
     uint4 rows[kStartRows * 16];                            // 16-byte pieces XOR-swizzled (near_piece)
@@ -352,7 +353,6 @@ struct StartSmem {
     float trial_norm[kStartTrials];
     int pick[2][kStartTrials];                              // sample indices of the trial points
     uint32_t touched[kStartBlocks];                         // trials with a marked point in the block
-    int best;
     uint16_t mask[kStartRows];                              // trials that may lower the point's distance
 };
 static_assert(sizeof(StartSmem) <= 227 * 1024, "shared memory of one block");

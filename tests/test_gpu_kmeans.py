@@ -246,3 +246,9 @@ def test_fits_that_stop_beside_their_own_sorting_blocks():
 def test_fit_of_keys_whose_products_underflow(scale):
     keys = scale * np.random.default_rng(23).standard_normal((4, 800, 128))
     _fit_keys_both(keys.astype(np.float32), "bf16", 40, batch_size=128, max_iter=2, patience=4, seed=5, reassignment_ratio=0.01)
+
+
+@pytest.mark.parametrize("n", [8103, 8104, 12288])
+def test_start_with_ten_and_eleven_trials_a_centre(n):
+    """2 + floor(ln k) is 11 from k = 8104 on; samples of up to 12288 keys take the start in one kernel all the same."""
+    test_fit_with_a_centre_per_key_returns_the_keys(n)
