@@ -407,8 +407,8 @@ huge_parents_kernel(ParentBuildParams p)
     {
         ValIdx best = {INFINITY, INT_MAX};
         for (int i = tid; i < nC; i += kThreads) {
-            ValIdx c = {sqdist_grow_vec<kHalf>(kbase + (size_t)mem[i] * 16, mu), i};
-            best = pick<true>(best, c);
+            const double d = sqdist_grow_vec<kHalf>(kbase + (size_t)mem[i] * 16, mu);
+            best = pick<true>(best, {d == d ? d : INFINITY, i});       // (not a number counts as infinitely far)
         }
         best = block_arg<true>(best, scratch);
         if (tid == 0) { rep_pos[0] = best.i; is_rep[best.i] = 1; }

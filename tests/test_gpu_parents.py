@@ -280,3 +280,27 @@ def test_assignment_with_centres_whose_norm_the_products_cannot_bound(elem, far,
     want, _, _ = orc.nearest_centre_parents(synth.to_f64(bits[0], elem), cen[0].astype(np.float64))
     assert np.array_equal(lab[0].cpu().numpy(), want)
     assert len(set(want.tolist())) > 200 and not set(at) & set(want.tolist())
+
+
+@pytest.mark.parametrize("size", [20, 100, 400, 700])
+def test_records_of_parents_with_keys_that_are_not_numbers(size):
+    """One key of a parent that is not a number makes its mean, and so every distance to it, not a number: the first
+    representative is then the parent's first key, for parents of every kernel's sizes. The other parents'
+    records are the oracle's."""
+    rng = np.random.default_rng(size)
+    N, n_parents, R = 3 * size, 3, 6
+    labels = rng.permutation(np.repeat(np.arange(3), size)).astype(np.int32)
+    bits = synth.round_bits(rng.standard_normal((1, N, 128)).astype(np.float32))
+    bad = int(np.flatnonzero(labels == 1)[size // 2])
+    bits[0, bad, 77] = 0x7FC0
+    geom = sp.Geometry(1, 1, 1, 128, 3 * R, R)
+    k = sp.bf16_bits_to_cuda(bits)
+    t = sp.santapp_build_teams_parents(geom, [N], [n_parents], k, k, torch.from_numpy(labels[None]).cuda())
+    csr, token = t.team_row_start[0, :3 * R + 1].cpu().numpy(), t.row_token[0].cpu().numpy()
+    rep = t.rep_keys.view(torch.int16).cpu().numpy().view(np.uint16)[0]
+    assert np.array_equal(np.sort(token), np.arange(N)) and np.all(np.diff(csr) >= 0)
+    assert np.array_equal(rep[R], bits[0, np.flatnonzero(labels == 1)[0]])
+    for u in (0, 2):
+        rows = np.flatnonzero(labels == u).astype(np.int32)
+        ts, tm, _ = orc.build_teams(synth.to_f64(bits[0]), np.array([0, size], dtype=np.int32), rows, R)
+        assert np.array_equal(csr[u * R:u * R + R + 1] - u * size, ts) and np.array_equal(token[u * size:(u + 1) * size], tm[:size])
