@@ -30,6 +30,7 @@ __device__ __forceinline__ int clamp_label(int v, int n) { return min(max(v, 0),
 // A block takes 128 tokens and scans all centres (nearest.cuh), which it rounds to 16 bits as it brings them into shared
 // memory (half a row per thread). Only tokens whose bounds leave more than one centre see fp64. 4 x 32768 tokens,
 // 2048 centres: 6.7 ms with every distance in fp64.
+constexpr int kAssignFewOpen = 24;       // tokens of a block up to which they go through all centres one by one
 template <bool kHalf>
 __global__ void __launch_bounds__(kNearThreads, 2)
 assign_parents_kernel(AssignParams p)
@@ -37,10 +38,12 @@ assign_parents_kernel(AssignParams p)
     extern __shared__ __align__(1024) unsigned char near_smem[];
     NearSmem &sm = *reinterpret_cast<NearSmem *>(near_smem);
     step_wait();
-    const int b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
+    __shared__ int n_open;                                  // tokens that go through all centres
+    const int b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t row0 = p.seq_row_off[b];
     const int N = (int)(p.seq_row_off[b + 1] - row0), i0 = blockIdx.x * kNearPoints;
     if (i0 >= N) return;
+    if (tid == 0) n_open = 0;
     const int64_t c0off = p.seq_centre_off[b];
     const int k = (int)(p.seq_centre_off[b + 1] - c0off);
     const uint16_t *keys = p.k_prompt + ((size_t)j * p.rows_total + row0) * kHeadDim;
@@ -94,14 +97,15 @@ assign_parents_kernel(AssignParams p)
             if (part == 0) sm.bias[slot][row] = make_float2(bias, fits ? 1.00001f * sqrtf(m) : 0.f);
         }
     });
-    if (tid < kNearPoints) {
-        const int i = i0 + tid;
-        const bool live = i < N;
-        const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)min(i, N - 1) * kHeadDim);
-        const NearTop top = sm.top[tid];
+    const int point = tid % kNearPoints, i = i0 + point;
+    const NearTop top = sm.top[point];
+    const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)min(i, N - 1) * kHeadDim);
+    int32_t *labels = p.parent_of + (size_t)j * p.rows_total + row0;
+    const bool open = i < N && near_open(top, sm.nx[point]);
+    if (tid < kNearPoints && open) sm.idx[atomicAdd(&n_open, 1)] = i;
+    if (tid < kNearPoints && i < N && !open) {
         int arg = top.i1;
-        const bool all = near_open(top, sm.nx[tid]);
-        if (live && !all && !(top.t2 > top.upper)) {
+        if (!(top.t2 > top.upper)) {
             double best = near_exact<kHalf>(x, cen + (size_t)arg * kHeadDim);
             const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
             if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
@@ -110,14 +114,19 @@ assign_parents_kernel(AssignParams p)
                 if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
             }
         }
-        for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
-            const int l = __ffs(left) - 1;
-            const uint4 *xl = reinterpret_cast<const uint4 *>(__shfl_sync(0xFFFFFFFFu, (unsigned long long)x, l));
-            double d;
-            const int u = near_scan_exact<kHalf>(xl, cen, k, d);
-            if (lane == l) arg = u;
+        labels[i] = arg;
+    }
+    __syncthreads();
+    double d;
+    if (n_open > kAssignFewOpen) {
+        const int arg = near_scan_tiles<kHalf, kNearThreads, 2>(x, open, cen, k, reinterpret_cast<double (*)[kHeadDim]>(sm.centres[0]), d);
+        if (tid < kNearPoints && open) labels[i] = arg;
+    } else {
+        for (int e = warp; e < n_open; e += kNearThreads / 32) {
+            const int arg = near_scan_exact<kHalf>(reinterpret_cast<const uint4 *>(keys + (size_t)sm.idx[e] * kHeadDim), cen, k,
+                                                   reinterpret_cast<double *>(sm.points) + warp * kHeadDim, d);
+            if (lane == 0) labels[sm.idx[e]] = arg;
         }
-        if (live) p.parent_of[(size_t)j * p.rows_total + row0 + i] = arg;
     }
     near_close_block(sm);
 }

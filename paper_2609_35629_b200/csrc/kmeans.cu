@@ -992,11 +992,12 @@ km_scan_kernel(KmeansParams p, int t)
 // candidates that the bounds leave open compared in fp64. A warp takes 32 points: the terms of each distance are
 // formed by all lanes (coalesced reads, four conversions a lane), then every lane adds up its own point's in order.
 constexpr int kResolveWarps = 2, kTermPitch = kHeadDim + 1;
+constexpr int kResolveFewOpen = 8;       // points of a block up to which they go through all centres one by one
 template <bool kHalf>
 __global__ void __launch_bounds__(kResolveWarps * 32)
 km_resolve_kernel(KmeansParams p, int t)
 {
-    extern __shared__ double term_s[];                      // [warps][32][kTermPitch]
+    extern __shared__ __align__(16) double term_s[];        // [warps][32][kTermPitch]
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     if (blockIdx.x == gridDim.x - 1) {
@@ -1044,12 +1045,20 @@ km_resolve_kernel(KmeansParams p, int t)
             if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
         }
     }
-    for (unsigned left = __ballot_sync(0xFFFFFFFFu, live && all); left; left &= left - 1) {
-        const int l = __ffs(left) - 1;
-        const uint4 *xl = reinterpret_cast<const uint4 *>(keys + (size_t)__shfl_sync(0xFFFFFFFFu, point, l) * kHeadDim);
-        double d;
-        const int u = near_scan_exact<kHalf>(xl, cen, q.k, d);
-        if (lane == l) { best = d; arg = u; }
+    const bool open = live && all;
+    const int n_open = __syncthreads_count(open);
+    double d;
+    if (n_open > kResolveFewOpen) {
+        const int u = near_scan_tiles<kHalf, kResolveWarps * 32, 1>(reinterpret_cast<const uint4 *>(keys + (size_t)point * kHeadDim), open, cen, q.k,
+                                                                    reinterpret_cast<double (*)[kHeadDim]>(term_s), d);
+        if (open) { best = d; arg = u; }
+    } else {
+        for (unsigned left = __ballot_sync(0xFFFFFFFFu, open); left; left &= left - 1) {
+            const int l = __ffs(left) - 1;
+            const uint4 *xl = reinterpret_cast<const uint4 *>(keys + (size_t)__shfl_sync(0xFFFFFFFFu, point, l) * kHeadDim);
+            const int u = near_scan_exact<kHalf>(xl, cen, q.k, term, d);
+            if (lane == l) { best = d; arg = u; }
+        }
     }
     if (live) {
         p.label[at] = arg;

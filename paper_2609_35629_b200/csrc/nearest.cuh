@@ -8,8 +8,8 @@
 // row cost at most 8 * 17 * 2^-23 of sum |x_d hi_d| <= (1 + 2^-8) (|x|^2 + |c|^2) / 2 (see select_rows.cuh), twice that for the
 // distance; the column of a centre, kept in the last five bits of its bound, 2^-18 of at most 2.04 (|x|^2 + |c|^2).
 // Together at most E_c = kNearErr (|x|^2 + |c|^2) + 2 |x| m. A centre can be nearest only if its lower bound does not exceed the
-// smallest upper bound; where that leaves two or three they are compared in fp64, where it leaves more all
-// centres are (with early exit). Products that underflow fp32 add less than kUnderflow.
+// smallest upper bound; where that leaves two or three they are compared in fp64, where it leaves more the
+// point goes through all centres (near_scan_exact, near_scan_tiles). Products that underflow fp32 add less than kUnderflow.
 //
 // The products are a GEMM (tcgen05, 128 points x 128 centres x 128 dimensions a tile, 512 cycles at the measured rate);
 // looking at 16384 results takes the block's eight warps about twice that, since every one costs two FMAs and four
@@ -274,36 +274,132 @@ __device__ __forceinline__ double near_exact(const uint4 *x, const C *cen)
     return s;
 }
 
-// All centres in fp64, one point per warp (a lane takes every 32nd centre): for points the bounds leave open.
-// A lane gives a centre up once its partial sum exceeds the best so far (sums only grow). Every lane gets the
-// result; like the plain loop, distances that are not smaller than infinity leave centre 0.
+// Four consecutive values of a centre (rows of floats need not be 16-byte aligned).
+__device__ __forceinline__ void near_quad(const float *p, float (&v)[4])
+{
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+        const float4 w = __ldg(reinterpret_cast<const float4 *>(p));
+        v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = __ldg(p + e);
+    }
+}
+__device__ __forceinline__ void near_quad(const double *p, double (&v)[4])
+{
+    const double2 w0 = __ldg(reinterpret_cast<const double2 *>(p)), w1 = __ldg(reinterpret_cast<const double2 *>(p) + 1);
+    v[0] = w0.x; v[1] = w0.y; v[2] = w1.x; v[3] = w1.y;
+}
+
+// All centres of one point by a warp, where the bounds leave few points of a block open. The centres come eight at a time,
+// four dimensions per lane (whole lines; with a centre per lane a load touched 32). fp32 distances leave out
+// most of them: a sum of (x - c)^2 whose c is rounded to fp32 once is off by at most 13 * 2^-24 of itself and 2^-23
+// |x|^2. Of the rest, one equal to the best so far is no better, and the others are evaluated in fp64, terms by all
+// lanes and then the sum in order. `term`: 128 doubles of the warp, 16-byte aligned. Every lane gets the result; like
+// the plain loop, distances that are not smaller than infinity leave centre 0.
 template <bool kHalf, typename C>
-__device__ __noinline__ int near_scan_exact(const uint4 *x, const C *cen, int k, double &dist)
+__device__ __noinline__ int near_scan_exact(const uint4 *x, const C *cen, int k, double *term, double &dist)
 {
     const int lane = threadIdx.x & 31;
+    const uint2 w = __ldg(reinterpret_cast<const uint2 *>(x) + lane);
+    const float xf[4] = {elem_lo<kHalf>(w.x), elem_hi<kHalf>(w.x), elem_lo<kHalf>(w.y), elem_hi<kHalf>(w.y)};
+    const float slack = fmaf(1e-6f, warp_sum(fmaf(xf[0], xf[0], xf[1] * xf[1]) + fmaf(xf[2], xf[2], xf[3] * xf[3])), kUnderflow);
+    const C *mine = cen + 4 * lane;
     double best = CUDART_INF;
     int arg = INT_MAX;
-    for (int u = lane; u < k; u += 32) {
-        const C *cu = cen + (size_t)u * kHeadDim;
-        double s = 0.0;
-        for (int q = 0; q < 16 && !(s > best); ++q) {
-            const uint4 w4 = __ldg(x + q);
-            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+    C held[4] = {};                                         // the best centre's values
+    float up = CUDART_INF_F;                                // no nearest centre is farther
+    for (int base = 0; base < k; base += 8) {
+        float d[8];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const double e0 = __dsub_rn((double)elem_lo<kHalf>(w[t]), (double)cu[8 * q + 2 * t]);
-                const double e1 = __dsub_rn((double)elem_hi<kHalf>(w[t]), (double)cu[8 * q + 2 * t + 1]);
-                s = __dadd_rn(s, __dmul_rn(e0, e0));
-                s = __dadd_rn(s, __dmul_rn(e1, e1));
+        for (int c = 0; c < 8; ++c) {
+            C v[4];
+            near_quad(mine + (size_t)min(base + c, k - 1) * kHeadDim, v);
+            d[c] = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[c] = fmaf(xf[e] - (float)v[e], xf[e] - (float)v[e], d[c]);
+        }
+        // sums over the lanes, halving the centres a lane holds: lane l ends up with centre l >> 2
+#pragma unroll
+        for (int half = 4; half > 0; half >>= 1) {
+            const bool upper = lane & (4 * half);
+#pragma unroll
+            for (int m = 0; m < half; ++m) d[m] = (upper ? d[m + half] : d[m]) + __shfl_xor_sync(0xFFFFFFFFu, upper ? d[m] : d[m + half], 4 * half);
+        }
+        d[0] += __shfl_xor_sync(0xFFFFFFFFu, d[0], 2);
+        d[0] += __shfl_xor_sync(0xFFFFFFFFu, d[0], 1);
+        const bool there = base + (lane >> 2) < k;
+        up = fminf(up, __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, __float_as_uint(there ? fmaf(d[0], 2e-6f, d[0]) + slack : CUDART_INF_F))));
+        for (unsigned left = __ballot_sync(0xFFFFFFFFu, there && (lane & 3) == 0 && !(fmaf(d[0], -2e-6f, d[0]) - slack > up)); left; left &= left - 1) {
+            const int u = base + ((__ffs(left) - 1) >> 2);
+            C v[4];
+            near_quad(mine + (size_t)u * kHeadDim, v);
+            if (arg != INT_MAX && __all_sync(0xFFFFFFFFu, v[0] == held[0] && v[1] == held[1] && v[2] == held[2] && v[3] == held[3])) continue;
+            double t[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                t[e] = __dsub_rn((double)xf[e], (double)v[e]);
+                t[e] = __dmul_rn(t[e], t[e]);
+            }
+            __syncwarp();
+            *reinterpret_cast<double2 *>(term + 4 * lane) = make_double2(t[0], t[1]);
+            *reinterpret_cast<double2 *>(term + 4 * lane + 2) = make_double2(t[2], t[3]);
+            __syncwarp();
+            double s = 0.0;
+#pragma unroll 8
+            for (int q = 0; q < kHeadDim; q += 2) {
+                const double2 two = *reinterpret_cast<const double2 *>(term + q);
+                s = __dadd_rn(s, two.x);
+                s = __dadd_rn(s, two.y);
+            }
+            if (s < best) {
+                best = s;
+                arg = u;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) held[e] = v[e];
             }
         }
-        if (s < best) { best = s; arg = u; }
     }
+    __syncwarp();
+    dist = best;
+    return arg == INT_MAX ? 0 : arg;
+}
+
+// The same by a block for many open points (centres that repeat leave every point open), kShare threads per point: all
+// fp64 distances, sixteen centres at a time as doubles in shared memory (`tile`, 16-byte aligned), eight of
+// them per pass of a thread; a warp without open points only brings centres. Every thread of the block; `x` is
+// a valid row in any case. The first kThreads / kShare threads get the results.
+constexpr int kScanTile = 16;
+template <bool kHalf, int kThreads, int kShare, typename C>
+__device__ __noinline__ int near_scan_tiles(const uint4 *x, bool open, const C *cen, int k, double (*tile)[kHeadDim], double &dist)
+{
+    constexpr int kPoints = kThreads / kShare;
+    const int tid = threadIdx.x, part = tid / kPoints;
+    const bool busy = __any_sync(0xFFFFFFFFu, open);
+    double best = CUDART_INF;
+    int arg = INT_MAX;
+    for (int base = 0; base < k; base += kScanTile) {
+        __syncthreads();
+        for (int e = tid; e < kScanTile * kHeadDim; e += kThreads)
+            tile[e / kHeadDim][e % kHeadDim] = (double)__ldg(cen + (size_t)min(base + e / kHeadDim, k - 1) * kHeadDim + e % kHeadDim);
+        __syncthreads();
+        if (!busy) continue;
+        for (int t = 8 * part; t < kScanTile; t += 8 * kShare) {
+            const uint4 *const row[1] = {x};
+            double d[1][8] = {};
+            dist_points<kHalf, 1, 8, 8>(row, tile + t, d);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double w = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-        const int j = __shfl_xor_sync(0xFFFFFFFFu, arg, o);
-        if (w < best || (w == best && j < arg)) { best = w; arg = j; }
+            for (int v = 0; v < 8; ++v)
+                if (base + t + v < k && d[0][v] < best) { best = d[0][v]; arg = base + t + v; }
+        }
+    }
+    __syncthreads();
+    if constexpr (kShare == 2) {
+        double *half_best = tile[0];
+        int *half_arg = reinterpret_cast<int *>(tile[1]);
+        if (part == 1) { half_best[tid - kPoints] = best; half_arg[tid - kPoints] = arg; }
+        __syncthreads();
+        if (part == 0 && (half_best[tid] < best || (half_best[tid] == best && half_arg[tid] < arg))) { best = half_best[tid]; arg = half_arg[tid]; }
     }
     dist = best;
     return arg == INT_MAX ? 0 : arg;

@@ -252,3 +252,11 @@ def test_fit_of_keys_whose_products_underflow(scale):
 def test_start_with_ten_and_eleven_trials_a_centre(n):
     """2 + floor(ln k) is 11 from k = 8104 on; samples of up to 12288 keys take the start in one kernel all the same."""
     test_fit_with_a_centre_per_key_returns_the_keys(n)
+
+
+@pytest.mark.parametrize("kind", ["few", "same", "padded", "some", "integer"])
+def test_fit_of_keys_that_repeat(kind):
+    from test_gpu_parents import _repeated
+    rng = np.random.default_rng(31)
+    keys = np.stack([_repeated(kind, 1000, rng) for _ in range(2)])
+    _fit_keys_both(keys.astype(np.float32), "bf16", 150, batch_size=256, max_iter=4, patience=5, seed=9, reassignment_ratio=0.3)

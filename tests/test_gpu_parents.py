@@ -304,3 +304,59 @@ def test_records_of_parents_with_keys_that_are_not_numbers(size):
         rows = np.flatnonzero(labels == u).astype(np.int32)
         ts, tm, _ = orc.build_teams(synth.to_f64(bits[0]), np.array([0, size], dtype=np.int32), rows, R)
         assert np.array_equal(csr[u * R:u * R + R + 1] - u * size, ts) and np.array_equal(token[u * size:(u + 1) * size], tm[:size])
+
+
+def _repeated(kind, n, rng):
+    if kind == "few":                            # 40 distinct rows
+        return rng.standard_normal((40, 128))[rng.integers(0, 40, size=n)]
+    if kind == "same":
+        return np.repeat(rng.standard_normal((1, 128)), n, axis=0)
+    if kind == "padded":                         # half of them zero
+        return rng.standard_normal((n, 128)) * (np.arange(n) < n // 2)[:, None]
+    if kind == "some":                           # one in sixteen zero
+        return rng.standard_normal((n, 128)) * (np.arange(n) % 16 > 0)[:, None]
+    return rng.integers(-1, 2, size=(n, 128))    # "integer": many distinct rows at exactly equal distances
+
+
+@pytest.mark.parametrize("kind", ["few", "same", "padded", "some", "integer"])
+@pytest.mark.parametrize("elem,offset", [("bf16", 0), ("fp16", 1)])
+def test_assignment_to_centres_that_repeat(kind, elem, offset):
+    """Centres drawn from keys that repeat: the bounds leave every token, or few of a block, more candidates than are
+    compared one by one. The centres' rows start at a 16-byte boundary and beside one."""
+    rng = np.random.default_rng(len(kind))
+    N, k = 900, 333
+    bits = synth.round_bits(_repeated(kind, N, rng).astype(np.float32)[None], elem)
+    keys = synth.to_f64(bits[0], elem)
+    cen = keys[rng.integers(0, N, size=k)].astype(np.float32)
+    cen[5] += 1e-6
+    geom = sp.Geometry(1, 1, 1, 128, 16, 4, sp.SANTAPP_FP16 if elem == "fp16" else sp.SANTAPP_BF16)
+    room = torch.zeros(k * 128 + 4, device="cuda")
+    room[offset:offset + k * 128] = torch.from_numpy(cen.ravel())
+    lab = sp.santapp_assign_parents(geom, [N], [k], sp.bf16_bits_to_cuda(bits, dtype=geom.torch_dtype),
+                                    room[offset:offset + k * 128].view(1, k, 128))
+    want, _, _ = orc.nearest_centre_parents(keys, cen.astype(np.float64))
+    assert np.array_equal(lab[0].cpu().numpy(), want)
+
+
+def test_tokens_that_the_bounds_leave_open_cost_their_fp64_distances_and_no_more():
+    """512 centres of which eight and eight are equal, so that every token goes through all of them: about twelve times the
+    usual call (the distances in fp64, which the call took for any centres before the bounds); 150 when each
+    token's scan read its centres one lane each."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    N, k, geom = 8192, 512, sp.Geometry(1, 4, 4, 128, 16, 4)
+    rows = torch.randn(4, N, 128, generator=g, device="cuda").to(torch.bfloat16)
+
+    def microseconds(keys, cen):
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            sp.santapp_assign_parents(geom, [N], [k], keys, cen)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, 1e3 * a.elapsed_time(b))
+        return best
+
+    usual = microseconds(rows, rows[:, :k].float().contiguous())
+    repeated = rows[:, :64].repeat(1, N // 64, 1)
+    assert microseconds(repeated, repeated[:, :k].float().contiguous()) < 40 * usual
