@@ -348,9 +348,10 @@ int santapp_assign_parents(const santapp_geom *geom, const int32_t *prompt_len_h
     std::vector<int64_t> offs(2 * ((size_t)geom->n_seqs + 1));
     int64_t *row_off = offs.data(), *cen_off = offs.data() + geom->n_seqs + 1;
     row_off[0] = cen_off[0] = 0;
-    int max_rows = 0;
+    int max_rows = 0, max_centres = 0;
     for (int b = 0; b < geom->n_seqs; ++b) {
         if (prompt_len_host[b] < 1 || n_centres_host[b] < 1) return SANTAPP_ERR_INVALID_ARG;
+        max_centres = std::max(max_centres, n_centres_host[b]);
         row_off[b + 1] = row_off[b] + prompt_len_host[b];
         cen_off[b + 1] = cen_off[b] + n_centres_host[b];
         if (prompt_len_host[b] > max_rows) max_rows = prompt_len_host[b];
@@ -369,6 +370,7 @@ int santapp_assign_parents(const santapp_geom *geom, const int32_t *prompt_len_h
     p.n_kv = geom->n_kv_heads;
     p.elem = geom->elem_type;
     p.max_rows_per_seq = max_rows;
+    p.max_centres_per_seq = max_centres;
     p.rows_total = row_off[geom->n_seqs];
     p.centres_total = cen_off[geom->n_seqs];
     p.seq_row_off = d_row_off;

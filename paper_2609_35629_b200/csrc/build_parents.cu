@@ -131,6 +131,43 @@ assign_parents_kernel(AssignParams p)
     near_close_block(sm);
 }
 
+// At most eight centres: one pass of fp64 distances, two tokens per thread. Bound by fp64 additions, like the scan above
+// where centres lie close together, but without its set-up: 4 x 100000 tokens and two or eight centres 107 us, the scan
+// 130, or 180 and 250 when the centres are means of random tokens.
+constexpr int kFewCentres = 8, kFewThreads = 128, kFewPoints = 2;
+template <bool kHalf>
+__global__ void __launch_bounds__(kFewThreads)
+assign_few_kernel(AssignParams p)
+{
+    __shared__ __align__(16) double c[kFewCentres][kHeadDim];
+    step_wait();
+    const int b = blockIdx.y, j = blockIdx.z, tid = threadIdx.x;
+    const int64_t row0 = p.seq_row_off[b], c0off = p.seq_centre_off[b];
+    const int N = (int)(p.seq_row_off[b + 1] - row0), k = (int)(p.seq_centre_off[b + 1] - c0off), i0 = blockIdx.x * kFewPoints * kFewThreads;
+    if (i0 >= N) return;
+    const float *cen = p.centres + ((size_t)j * p.centres_total + c0off) * kHeadDim;
+    for (int e = tid; e < kFewCentres * kHeadDim; e += kFewThreads)
+        c[e / kHeadDim][e % kHeadDim] = (double)__ldg(cen + (size_t)min(e / kHeadDim, k - 1) * kHeadDim + e % kHeadDim);
+    const size_t plane = (size_t)j * p.rows_total + row0;
+    const uint4 *row[kFewPoints];
+#pragma unroll
+    for (int u = 0; u < kFewPoints; ++u)
+        row[u] = reinterpret_cast<const uint4 *>(p.k_prompt + (plane + min(i0 + u * kFewThreads + tid, N - 1)) * kHeadDim);
+    __syncthreads();
+    double d[kFewPoints][kFewCentres] = {};
+    dist_points<kHalf, kFewPoints, kFewCentres, kFewCentres>(row, c, d);
+#pragma unroll
+    for (int u = 0; u < kFewPoints; ++u) {
+        const int i = i0 + u * kFewThreads + tid;
+        double best = INFINITY;
+        int arg = 0;
+#pragma unroll
+        for (int v = 0; v < kFewCentres; ++v)
+            if (v < k && d[u][v] < best) { best = d[u][v]; arg = v; }
+        if (i < N) p.parent_of[plane + i] = arg;
+    }
+}
+
 // ---- member lists ----
 // One warp per (chunk of a sequence's tokens, sequence, KV head): the tokens 32 at a time in increasing index; lanes with
 // the same label form a group whose lowest lane moves the label's count, and each lane takes its rank in the
@@ -495,6 +532,9 @@ huge_parents_kernel(ParentBuildParams p)
 template <bool kHalf>
 static cudaError_t launch_assign(const AssignParams &p, cudaStream_t s)
 {
+    if (p.max_centres_per_seq <= kFewCentres)
+        return launch_step(assign_few_kernel<kHalf>, dim3((p.max_rows_per_seq + kFewPoints * kFewThreads - 1) / (kFewPoints * kFewThreads), p.n_seqs, p.n_kv),
+                           dim3(kFewThreads), 0, s, p);
     static std::atomic<unsigned long long> done;
     const cudaError_t err = ensure_dynamic_smem((const void *)assign_parents_kernel<kHalf>, (int)sizeof(NearSmem), done);
     if (err != cudaSuccess) return err;

@@ -257,7 +257,7 @@ cudaError_t launch_build_groups_mean(const BuildParams &p, cudaStream_t s);
 
 // Nearest-centre assignment (last step of Algorithm 3).
 struct AssignParams {
-    int n_seqs, n_kv, max_rows_per_seq, elem;
+    int n_seqs, n_kv, max_rows_per_seq, max_centres_per_seq, elem;
     int64_t rows_total, centres_total;
     const int64_t *seq_row_off;             // device [n_seqs + 1]
     const int64_t *seq_centre_off;          // device [n_seqs + 1]

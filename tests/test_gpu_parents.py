@@ -360,3 +360,21 @@ def test_tokens_that_the_bounds_leave_open_cost_their_fp64_distances_and_no_more
     usual = microseconds(rows, rows[:, :k].float().contiguous())
     repeated = rows[:, :64].repeat(1, N // 64, 1)
     assert microseconds(repeated, repeated[:, :k].float().contiguous()) < 40 * usual
+
+
+@pytest.mark.parametrize("n_centres", [[1, 2], [8, 3], [2, 9]])
+@pytest.mark.parametrize("elem", ["bf16", "fp16"])
+def test_assignment_to_few_centres(n_centres, elem):
+    """Up to eight centres in every sequence, and one more in one: the two kernels of the assignment on ragged sequences."""
+    rng = np.random.default_rng(n_centres)
+    lens = [257, 130]
+    bits = synth.round_bits(rng.standard_normal((2, sum(lens), 128)).astype(np.float32), elem)
+    cen = rng.standard_normal((2, sum(n_centres), 128)).astype(np.float32)
+    cen[0, -1] = cen[0, n_centres[0]]                                  # an exact tie, or the centre itself
+    cen[1, 0] = np.nan if n_centres[0] > 1 else cen[1, 0]              # never the nearest
+    geom = sp.Geometry(2, 2, 2, 128, 16, 4, sp.SANTAPP_FP16 if elem == "fp16" else sp.SANTAPP_BF16)
+    lab = sp.santapp_assign_parents(geom, lens, n_centres, sp.bf16_bits_to_cuda(bits, dtype=geom.torch_dtype), torch.from_numpy(cen).cuda())
+    for j in range(2):
+        for r0, c0, n, k in ((0, 0, lens[0], n_centres[0]), (lens[0], n_centres[0], lens[1], n_centres[1])):
+            want, _, _ = orc.nearest_centre_parents(synth.to_f64(bits[j, r0:r0 + n], elem), cen[j, c0:c0 + k].astype(np.float64))
+            assert np.array_equal(lab[j, r0:r0 + n].cpu().numpy(), want)
