@@ -341,14 +341,29 @@ large_parents_kernel(ParentBuildParams p, int kind)
     }
 }
 
-// K and V of one token to a row of the sequence's packed order, by a warp.
-__device__ __forceinline__ void copy_row(const ParentRows &t, int token, int row)
+// K and V of up to 32 tokens (one per lane, the first n of them) to rows of the sequence's packed order, by a warp: eight
+// tokens are on their way at a time, a half warp each. (One at a time, a block took 7 ms for 50000 tokens.)
+__device__ __forceinline__ void copy_rows(const ParentRows &t, int token, int row, int n)
 {
-    const int lane = threadIdx.x & 31;
-    const size_t from = (t.plane + token) * 32 + lane, to = (t.plane + row) * 32 + lane;
-    reinterpret_cast<uint2 *>(t.k_packed)[to] = reinterpret_cast<const uint2 *>(t.k_prompt)[from];
-    reinterpret_cast<uint2 *>(t.v_packed)[to] = reinterpret_cast<const uint2 *>(t.v_prompt)[from];
-    if (lane == 0) t.row_token[t.plane + row] = token;
+    const int lane = threadIdx.x & 31, q = lane & 15;
+    const uint4 *k = reinterpret_cast<const uint4 *>(t.k_prompt) + t.plane * 16 + q, *v = reinterpret_cast<const uint4 *>(t.v_prompt) + t.plane * 16 + q;
+    uint4 *kd = reinterpret_cast<uint4 *>(t.k_packed) + t.plane * 16 + q, *vd = reinterpret_cast<uint4 *>(t.v_packed) + t.plane * 16 + q;
+    for (int l0 = 0; l0 < n; l0 += 8) {
+        uint4 kr[4], vr[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int l = l0 + 2 * m + (lane >> 4);
+            const size_t at = (size_t)__shfl_sync(0xFFFFFFFFu, token, l) * 16;
+            if (l < n) { kr[m] = __ldg(k + at); vr[m] = __ldg(v + at); }
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int l = l0 + 2 * m + (lane >> 4);
+            const size_t at = (size_t)__shfl_sync(0xFFFFFFFFu, row, l) * 16;
+            if (l < n) { kd[at] = kr[m]; vd[at] = vr[m]; }
+        }
+    }
+    if (lane < n) t.row_token[t.plane + row] = token;
 }
 
 template <bool kHalf>
@@ -393,8 +408,9 @@ __device__ __forceinline__ double sqdist_grow_row(const uint4 *row, const uint32
 // Parents of more than 512 rows (and, for the centroid-guided baseline, all parents): rows are read through the member
 // list, the per-member state lives in global memory, every distance is taken in fp64. Blocks walk the list
 // of such parents (mean keys: one block per label).
+constexpr int kHugeBlocks = 2;          // per SM; with three or four the inner loops lack registers (8 % slower where each has a parent)
 template <bool kHalf>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kHugeBlocks)
 huge_parents_kernel(ParentBuildParams p)
 {
     __shared__ int scan_s[33], start_s[kMaxParent];
@@ -445,7 +461,7 @@ huge_parents_kernel(ParentBuildParams p)
         // element (fp64 -> fp32 to nearest, fp32 -> bf16 or fp16 to nearest even)
         if (tid == 0) t.csr[1] = s0 + nC;
         if (tid < kHeadDim) p.rep_keys[t.rep0 * kHeadDim + tid] = double_to_elem<kHalf>(mu[tid]);
-        for (int i = warp; i < nC; i += kThreads / 32) copy_row(t, mem[i], s0 + i);
+        for (int i = 32 * warp; i < nC; i += kThreads) copy_rows(t, mem[min(i + lane, nC - 1)], s0 + i + lane, min(32, nC - i));
         return;
     }
 
@@ -513,7 +529,7 @@ huge_parents_kernel(ParentBuildParams p)
             }
             __syncthreads();
         }
-        for (int l = 0; l < 32 && i0 + warp * 32 + l < nC; ++l) copy_row(t, mem[i0 + warp * 32 + l], s0 + __shfl_sync(0xFFFFFFFFu, pos, l));
+        copy_rows(t, mem[min(i, nC - 1)], s0 + pos, min(32, nC - (i0 + warp * 32)));
     }
     uint32_t m = 0u;
     uint32_t *rep_dst = reinterpret_cast<uint32_t *>(p.rep_keys) + t.rep0 * 64;
@@ -552,8 +568,10 @@ static cudaError_t launch_parents(const ParentBuildParams &p, cudaStream_t s)
     const int B = p.bv.n_seqs, H = p.bv.n_kv, sms = attend_grid_size();
     cudaError_t err;
     if (p.mean_keys) return launch_step(huge_parents_kernel<kHalf>, dim3(p.max_labels_per_seq, B, H), dim3(kThreads), 0, s, p);
-    // the few large parents first: theirs are the longest blocks
-    if ((err = launch_step(huge_parents_kernel<kHalf>, dim3(sms), dim3(kThreads), 0, s, p)) != cudaSuccess) return err;
+    // the few large parents first: theirs are the longest blocks. As many as are resident: a parent is a chain of reads
+    // that one block cannot keep an SM busy with (8 sequences of 32K tokens in 40 parents per KV head: 7.4 ms at one
+    // per SM, 3.6 at two, 4.1 with a block per parent)
+    if ((err = launch_step(huge_parents_kernel<kHalf>, dim3(kHugeBlocks * sms), dim3(kThreads), 0, s, p)) != cudaSuccess) return err;
     static std::atomic<unsigned long long> large_done, mid_done;
     using Large = LargeSmem<8, 2>;
     using Mid = LargeSmem<4, 1>;
