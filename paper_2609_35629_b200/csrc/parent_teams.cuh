@@ -117,6 +117,7 @@ struct LargeSmem {
     };
     float norm[kRows];
     double mu64[kHeadDim];
+    double near[kRows];                                       // fp64 distances to the owners, of the rows that a choice needed them of
     float mu[4][kHeadDim];
     LargeTop top[2][kWarps];
     uint32_t next_key[2 * kWarps];                            // two rows of each warp for the next candidates
@@ -202,8 +203,32 @@ __device__ __noinline__ void select_large_exact(LargeSmem<kWarps, kRpt> &sm, int
     __syncthreads();
 }
 
-// Rows a step may leave open before the parent goes to the fp64 evaluation.
-constexpr int kMaxOpen = 64;
+// What a parent's open comparisons may cost before it goes to the fp64 evaluation, which starts over: half of what
+// that takes. Unit: a warp's fp64 distances to one representative, of which the evaluation makes r for every 32 rows;
+// an open row takes one per 32 representatives, a choice among rows whose distances are known about kChoiceCost.
+constexpr int kChoiceCost = 1;
+
+// The first of a row's nearest representatives among the first n, by the defining distances: a warp, whose lanes take the
+// representatives. Every lane gets it and the distance.
+template <bool kHalf, int kWarps, int kRpt>
+__device__ __forceinline__ int nearest_rep(const LargeSmem<kWarps, kRpt> &sm, int i, int n, double &dist)
+{
+    const int lane = threadIdx.x & 31;
+    double near = CUDART_INF;
+    int who = INT_MAX;
+    for (int q = lane; q < n; q += 32) {
+        const double d = exact_dist<kHalf>(sm.rows + i * kPitch, sm.rows + sm.rep_of[q] * kPitch, kWords);
+        if (d < near || who == INT_MAX) { near = d; who = q; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double d = __shfl_xor_sync(0xFFFFFFFFu, near, o);
+        const int w = __shfl_xor_sync(0xFFFFFFFFu, who, o);
+        if (d < near || (d == near && w < who)) { near = d; who = w; }
+    }
+    dist = near;
+    return who;
+}
 
 template <int kWarps, int kRpt, bool kHalf>
 __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC, int r)
@@ -307,8 +332,10 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
             ldmatrix4(a[m][s], rows_a + (uint32_t)((warp * 32 * kRpt + 16 * m + (lane & 15)) * kPitch * 4 + (lane >> 4) * 16 + s * 32));
 
     constexpr float kPairErr = 0.5f * kDistErr;               // times the sum of the two squared norms, plus kUnderflow
-    int owner[kRpt], parity = 0, u = 0;
+    const int budget = max(16, r * kRpt * kWarps / 2);
+    int owner[kRpt], parity = 0, u = 0, spent = 0;
     unsigned open_owner = 0u;                                 // bit k: the bound leaves the nearest representative open
+    unsigned known = 0u;                                      // bit k: sm.near holds the row's distance
 #pragma unroll
     for (int k = 0; k < kRpt; ++k) {
         owner[k] = 0;
@@ -395,11 +422,13 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
                 if (u == 0 || d + e < lo[k]) {                // certainly nearer than every earlier one
                     mind[k] = d; lo[k] = d - e; hi[k] = d + e; owner[k] = u;
                     open_owner &= ~(1u << k);
-                } else if (!(d - e > hi[k])) {                // not certain: the minimum lies between the smaller bounds
+                    known &= ~(1u << k);
+                } else if (!(d - e > hi[k]) && hi[k] > 0.f) { // not certain: the minimum lies between the smaller bounds
                     if (d < mind[k]) { mind[k] = d; owner[k] = u; }
                     lo[k] = fminf(lo[k], d - e);
                     hi[k] = fminf(hi[k], d + e);
                     open_owner |= 1u << k;
+                    known &= ~(1u << k);
                 }
                 if (((live & ~is_rep) >> k) & 1u) {
                     if (lo[k] > top_lo || top_row == 0) {
@@ -434,30 +463,35 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
             if (!__any_sync(0xFFFFFFFFu, rival)) {
                 rep = __shfl_sync(0xFFFFFFFFu, t.row, wl);
             } else {
-                // the rows that may be the farthest, by their fp64 distance to the nearest representative
+                // the rows that may be the farthest, by their fp64 distance to the nearest representative (kept: rows that
+                // tie are asked again at the next choice)
                 maybe = 0u;
 #pragma unroll
                 for (int k = 0; k < kRpt; ++k)
                     if ((((live & ~is_rep) >> k) & 1u) && !(hi[k] < bar)) maybe |= 1u << k;
                 const int n_open = __syncthreads_count((maybe & open_owner) != 0u);
-                if (n_open > kMaxOpen) { select_large_exact<kWarps, kRpt, kHalf>(sm, nC, r); return; }
+                spent += kChoiceCost + n_open * ((u + 31) / 32);
+                if (spent > budget) { select_large_exact<kWarps, kRpt, kHalf>(sm, nC, r); return; }
                 ValIdx x = {-2.0, INT_MAX};
 #pragma unroll
                 for (int k = 0; k < kRpt; ++k) {
-                    double v = -2.0;
-                    if (((maybe & ~open_owner) >> k) & 1u)
-                        v = exact_dist<kHalf>(sm.rows + LARGE_ROW(k) * kPitch, sm.rows + sm.rep_of[owner[k]] * kPitch, kWords);
+                    double &near = sm.near[LARGE_ROW(k)];
+                    bool asked = ((maybe & ~open_owner & ~known) >> k) & 1u;
+                    if (asked) near = exact_dist<kHalf>(sm.rows + LARGE_ROW(k) * kPitch, sm.rows + sm.rep_of[owner[k]] * kPitch, kWords);
                     for (unsigned left = __ballot_sync(0xFFFFFFFFu, ((maybe & open_owner) >> k) & 1u); left; left &= left - 1) {
-                        const int l = __ffs(left) - 1;        // lanes take the representatives
-                        const uint32_t *row = sm.rows + (warp * 32 * kRpt + 32 * k + l) * kPitch;
-                        double near = CUDART_INF;
-                        for (int q = lane; q < u; q += 32) near = fmin(near, exact_dist<kHalf>(row, sm.rows + sm.rep_of[q] * kPitch, kWords));
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) near = fmin(near, __shfl_xor_sync(0xFFFFFFFFu, near, o));
-                        if (lane == l) v = near;
+                        const int l = __ffs(left) - 1;
+                        double dist;
+                        const int who = nearest_rep<kHalf>(sm, warp * 32 * kRpt + 32 * k + l, u, dist);
+                        if (lane == l) { near = dist; owner[k] = who; asked = true; }
                     }
-                    if ((maybe >> k) & 1u) x = pick<false>(x, {v, LARGE_ROW(k)});
+                    if (asked) {                              // certain from here on, and within a float's rounding
+                        lo[k] = __double2float_rd(near);
+                        mind[k] = hi[k] = __double2float_ru(near);
+                    }
+                    if ((maybe >> k) & 1u) x = pick<false>(x, {near, LARGE_ROW(k)});
                 }
+                open_owner &= ~maybe;
+                known |= maybe;
                 x = block_arg<false>(x, sm.arg);
                 rep = min(x.i, nC - 1);
             }
@@ -473,19 +507,13 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
     // rows whose two nearest representatives the bound leaves open: lanes take the representatives
     __syncthreads();
     const unsigned ask = live & open_owner & ~is_rep;
-    if (__syncthreads_count(ask != 0u) > 4 * kMaxOpen) { select_large_exact<kWarps, kRpt, kHalf>(sm, nC, r); return; }
+    if (__syncthreads_count(ask != 0u) * ((r + 31) / 32) > r * kRpt * kWarps) { select_large_exact<kWarps, kRpt, kHalf>(sm, nC, r); return; }
 #pragma unroll
     for (int k = 0; k < kRpt; ++k) {
         for (unsigned left = __ballot_sync(0xFFFFFFFFu, (ask >> k) & 1u); left; left &= left - 1) {
             const int l = __ffs(left) - 1;
-            const uint32_t *row = sm.rows + (warp * 32 * kRpt + 32 * k + l) * kPitch;
-            double near = CUDART_INF;
-            int who = INT_MAX;
-            for (int q = lane; q < r; q += 32) {
-                const double d = exact_dist<kHalf>(row, sm.rows + sm.rep_of[q] * kPitch, kWords);
-                if (d < near || who == INT_MAX) { near = d; who = q; }
-            }
-            who = warp_arg<true>(near, who, lane < r);
+            double dist;
+            const int who = nearest_rep<kHalf>(sm, warp * 32 * kRpt + 32 * k + l, r, dist);
             if (lane == l) owner[k] = who;
         }
         sm.owner[LARGE_ROW(k)] = (uint16_t)owner[k];
