@@ -202,6 +202,8 @@ __device__ __forceinline__ void select_small(const uint32_t *rows, float *dist, 
     float mind = CUDART_INF_F;
     int owner = 0;
     bool is_rep = false;
+    double near = 0.0;                                            // the fp64 distance to the owner, once a comparison needed it
+    bool known = false;
     for (int u = 0; u < r; ++u) {
         if (lane == 0) rep_of[u] = rep;
         is_rep |= lane == rep;
@@ -209,12 +211,14 @@ __device__ __forceinline__ void select_small(const uint32_t *rows, float *dist, 
         const float nr = dist[rep * kDp + rep];
         const float d = lane == rep ? 0.f : norm + nr - 2.f * dist[me * kDp + rep];
         bool closer = u == 0 || d < mind - 2.f * err;
-        const bool open = live && u > 0 && !closer && !(d > mind + 2.f * err);
+        const bool open = live && u > 0 && !closer && !(d > mind + 2.f * err) && !(known && near == 0.0);      // (nothing is nearer than zero)
         if (open) {
             const double d_new = exact_dist<kHalf>(my_row, rows + rep * kPitch, kWords);
-            const double d_old = exact_dist<kHalf>(my_row, rows + rep_of[owner] * kPitch, kWords);
-            closer = d_new < d_old;
+            if (!known) near = exact_dist<kHalf>(my_row, rows + rep_of[owner] * kPitch, kWords);
+            closer = d_new < near;
+            if (closer) near = d_new;
         }
+        known = open || (known && !closer);
         if (closer) owner = u;
         mind = open ? fminf(mind, d) : (closer ? d : mind);       // either value is within the bound of the smaller one
         if (u + 1 < r) {
@@ -225,8 +229,9 @@ __device__ __forceinline__ void select_small(const uint32_t *rows, float *dist, 
             if (__popc(who) == 1) {
                 rep = __ffs(who) - 1;
             } else {
-                const double v = maybe ? exact_dist<kHalf>(my_row, rows + rep_of[owner] * kPitch, kWords) : 0.0;
-                rep = min(warp_arg<false>(v, lane, maybe), nC - 1);
+                if (maybe && !known) near = exact_dist<kHalf>(my_row, rows + rep_of[owner] * kPitch, kWords);
+                known |= maybe;
+                rep = min(warp_arg<false>(near, lane, maybe), nC - 1);
             }
         }
     }

@@ -142,3 +142,31 @@ def test_records_of_one_repeated_row_cost_little_more_than_others(P, R):
         return best
 
     assert microseconds(rows[:, :1].repeat(1, N, 1)) < 6 * microseconds(rows)
+
+
+@pytest.mark.parametrize("P,R", [(8, 2), (16, 4), (17, 17), (32, 8), (32, 32)])
+@pytest.mark.parametrize("kind", ["same", "repeated", "integer"])
+def test_records_of_small_parents_whose_rows_tie(P, R, kind):
+    _check(P, R, kind, "fp16")
+    test_shared_latent_records_at_every_parent_size(P, R, kind)
+
+
+def test_shared_latent_records_of_zero_rows_cost_a_few_times_the_usual():
+    """About 3 times at 32 rows and 8 representatives (every comparison in fp64 once), 10 when each was made up to three
+    times."""
+    g = torch.Generator(device="cuda").manual_seed(6)
+    geom, N = sp.LatentGeometry(1, 16, 32, 8), 1 << 18
+    rows = torch.randn(N, sp.LATENT_ROW, generator=g, device="cuda").to(torch.bfloat16)
+
+    def microseconds(x):
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            sp.santapp_latent_build_teams(geom, [N], x)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, 1e3 * a.elapsed_time(b))
+        return best
+
+    assert microseconds(torch.zeros_like(rows)) < 5.5 * microseconds(rows)
