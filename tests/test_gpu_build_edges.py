@@ -170,3 +170,39 @@ def test_shared_latent_records_of_zero_rows_cost_a_few_times_the_usual():
         return best
 
     assert microseconds(torch.zeros_like(rows)) < 5.5 * microseconds(rows)
+
+
+@pytest.mark.parametrize("kind", ["contiguous", "parents", "latent"])
+def test_preparation_calls_can_be_captured_in_a_cuda_graph(kind):
+    """The tables made from host arrays travel inside kernel arguments: a captured call, replayed on other keys after its
+    host arrays are gone, leaves the records of a plain call on them."""
+    g = torch.Generator(device="cuda").manual_seed(8)
+    lens = [700, 333]
+    first, second = (torch.randn(2, sum(lens), 128, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    k = first.clone()
+    rows = torch.randn(sum(lens), sp.LATENT_ROW, generator=g, device="cuda").to(torch.bfloat16)
+    cen = torch.randn(2, 30, 128, generator=g, device="cuda")
+    geom = sp.Geometry(2, 4, 2, 128, 64, 8)
+
+    def call():
+        if kind == "contiguous":
+            t = sp.santapp_build_teams(geom, list(lens), k, k)
+        elif kind == "parents":
+            t = sp.santapp_build_teams_parents(geom, list(lens), [20, 10], k, k, sp.santapp_assign_parents(geom, list(lens), [20, 10], k, cen))
+        else:
+            t = sp.santapp_latent_build_teams(sp.LatentGeometry(2, 16, 16, 4), list(lens), rows)
+            return t, [t.rows_packed, t.rep_rows, t.team_row_start, t.row_token, t.seq_row_off, t.seq_team_off, t.rep_abs_max]
+        return t, [t.k_packed, t.rep_keys, t.team_row_start, t.row_token, t.seq_row_off, t.seq_team_off, t.rep_abs_max, t.team_count]
+
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        kept, got = call()
+    for other in (second, first):
+        k.copy_(other)
+        rows.mul_(-0.5)
+        graph.replay()
+        want = call()[1]
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -88,8 +88,8 @@ def test_fit_without_host_polling_can_be_captured_in_a_cuda_graph():
 
 
 def test_fit_on_a_sequence_too_long_for_the_shared_memory_shuffle():
-    """52000 keys beside 900: the long sequence's index list does not fit in shared memory, so its
-    initialisation sample is shuffled in global memory, the short one's in shared memory."""
+    """52000 keys beside 900: more indices than shared memory holds, of which the initialisation sample takes the head
+    of a shuffle (entries found one by one, without the list), beside a sequence whose sample is all of it."""
     spec = synth.spec_small_gqa(prompt=(52000, 900), suffix0=(0, 0))
     spec.n_clusters = 16
     _fit_both(spec, [11, 6], batch_size=192, seed=5, max_iter=3, patience=4)
