@@ -963,19 +963,23 @@ latent_merge_kernel(const float *partials, const uint32_t *pair_prefix, int n_se
 #pragma unroll
     for (int u = 0; u < kAhead; ++u)
         if (c_lo + part + 4 * u <= c_hi) add(m[u], l[u], v[u]);
-    for (int c0 = c_lo + part + 4 * kAhead; c0 <= c_hi; c0 += 16) {      // (a lone long sequence has one from every block)
+    int c = c_lo + part + 4 * kAhead;
+    for (; c + 12 <= c_hi; c += 16) {                       // (a lone long sequence has a partial from every block)
         float pm[4], pl[4];
         float4 pv[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const float *p = base + min(c0 + 4 * u, c_hi) * slot;
+            const float *p = base + (c + 4 * u) * slot;
             pm[u] = __ldcg(p);
             pl[u] = __ldcg(p + 1);
             pv[u] = __ldcg(reinterpret_cast<const float4 *>(p + 4) + col);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (c0 + 4 * u <= c_hi) add(pm[u], pl[u], pv[u]);
+        for (int u = 0; u < 4; ++u) add(pm[u], pl[u], pv[u]);
+    }
+    for (; c <= c_hi; c += 4) {
+        const float *p = base + c * slot;
+        add(__ldcg(p), __ldcg(p + 1), __ldcg(reinterpret_cast<const float4 *>(p + 4) + col));
     }
     if (part > 0) { part_acc[part - 1][col] = acc; part_l[part - 1][col] = L; }
     __syncthreads();
