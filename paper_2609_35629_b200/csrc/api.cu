@@ -576,9 +576,9 @@ int kmeans_layout(const santapp_geom *geom, const int32_t *prompt_len_host, cons
     L->dist = take(sizeof(double) * 2 * pairs * (size_t)o->batch_size);
     L->centre_hi = take(sizeof(uint16_t) * H * (size_t)L->centres_total * kHeadDim);
     L->centre_bias = take(sizeof(float2) * H * (size_t)L->centres_total);
-    // the pairs' scans share the blocks that 148 SMs hold at once (two each); no block takes less than a tile
+    // the pairs' scans share the blocks that are resident at once (two per SM); no block takes less than a tile
     const int tiles = (o->batch_size + 127) / 128, k_tiles = (L->k_max + 127) / 128;
-    L->scan_blocks = std::max(1, std::min((int)(2 * 148 / pairs), tiles * k_tiles));
+    L->scan_blocks = std::max(1, std::min((int)(2 * attend_grid_size() / pairs), tiles * k_tiles));
     L->scan_segs = L->scan_blocks / tiles + 2;
     L->near_top = take(kNearTopBytes * pairs * (size_t)L->scan_segs * (size_t)o->batch_size);
     L->near_nx = take(sizeof(float) * pairs * (size_t)o->batch_size);
