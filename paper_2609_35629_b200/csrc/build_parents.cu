@@ -328,7 +328,7 @@ small_parents_kernel(ParentBuildParams p)
 
 // Parents of 33 to 128 and of 129 to 512 rows: blocks walk the lists.
 template <int kWarps, int kRpt, bool kHalf>
-__global__ void __launch_bounds__(32 * kWarps, 1)
+__global__ void __launch_bounds__(32 * kWarps, large_blocks(kWarps, kRpt))
 large_parents_kernel(ParentBuildParams p, int kind)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -580,7 +580,7 @@ static cudaError_t launch_parents(const ParentBuildParams &p, cudaStream_t s)
     if ((err = ensure_dynamic_smem((const void *)large_parents_kernel<8, 2, kHalf>, (int)sizeof(Large), large_done)) != cudaSuccess) return err;
     if ((err = ensure_dynamic_smem((const void *)large_parents_kernel<4, 1, kHalf>, (int)sizeof(Mid), mid_done)) != cudaSuccess) return err;
     if ((err = launch_step(large_parents_kernel<8, 2, kHalf>, dim3(sms), dim3(256), sizeof(Large), s, p, 1)) != cudaSuccess) return err;
-    if ((err = launch_step(large_parents_kernel<4, 1, kHalf>, dim3(3 * sms), dim3(128), sizeof(Mid), s, p, 0)) != cudaSuccess) return err;
+    if ((err = launch_step(large_parents_kernel<4, 1, kHalf>, dim3(large_blocks(4, 1) * sms), dim3(128), sizeof(Mid), s, p, 0)) != cudaSuccess) return err;
     return launch_step(small_parents_kernel<kHalf>, dim3((p.max_labels_per_seq + kSmallParentWarps - 1) / kSmallParentWarps, B, H),
                        dim3(kSmallParentWarps * 32), 0, s, p);
 }

@@ -61,7 +61,7 @@ build_small_kernel(BuildParams p)
 }
 
 template <int kWarps, int kRpt, bool kHalf>
-__global__ void __launch_bounds__(32 * kWarps, 1)
+__global__ void __launch_bounds__(32 * kWarps, large_blocks(kWarps, kRpt))
 build_large_kernel(BuildParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];

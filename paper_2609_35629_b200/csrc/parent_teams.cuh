@@ -106,6 +106,10 @@ struct LargeTop {                        // a warp's farthest row: bounds of its
     float lo, hi, hi_others;             //   the warp's other rows, and its index
     int row;
 };
+// Up to 256 rows as many blocks share an SM as make sixteen warps: with a block or two, whatever registers the compiler takes
+// when it is not told (199 for 64 to 256 rows, where 125 do without spills), the chain of one block has nothing beside it.
+// 4 x 32K keys in parents of 256 / 128 / 64: 82 -> 60, 57 -> 44, 59 -> 44 us.
+__host__ __device__ constexpr int large_blocks(int warps, int rows_per_thread) { return rows_per_thread > 1 ? 1 : 16 / warps; }
 template <int kWarps, int kRpt>
 struct LargeSmem {
     static constexpr int kT = 32 * kWarps, kRows = kT * kRpt; // threads, rows
