@@ -827,8 +827,8 @@ cudaError_t launch_start(const KmeansParams &p, int pairs, int n_blk, cudaStream
 // A step is five kernels: the scan for the nearest centres (nearest.cuh), the fp64 distance to the one found,
 // the minibatch ordered by centre, the update, the reassignment of starved centres. The inertia of a
 // minibatch is a sum of `batch` terms in order -- 4096 dependent additions, 18 us -- and only decides whether
-// the next step's update is still made. An extra block per pair in each of the five kernels from the update on takes
-// a fifth of it, so it is over when the next update starts and costs no time of its own; from then on a fit
+// the next step's update is still made. An extra block per pair in four of the kernels from the update on takes
+// a part of it, so it is over when the next update starts and costs no time of its own; from then on a fit
 // that has stopped does nothing. At 4 pairs, batch 4096 and 2048 centres a step was 0.94 ms (0.84 of it fp64
 // distances to every centre).
 __device__ __forceinline__ bool pair_active(const KmeansParams &p, const Pair &q, int t)
@@ -881,7 +881,16 @@ km_prepare_kernel(KmeansParams p)
 
 // Parts [part, part_end) of kInertiaParts of the inertia of step t, one block per pair; after the last part the averaged
 // inertia and the stopping rule. A part's terms go through shared memory: one thread adds them in order.
-constexpr int kInertiaParts = 5, kInertiaTerms = 4096 / kInertiaParts + 1;
+// The parts ride on the update, the reassignment, the next step's resolve and its sorting kernel, in sixteenths of the minibatch
+// by what these kernels take without them (16, 5, 20, 12 us; a sixteenth takes 1.2). None rides on the scan, whose blocks
+// fill the device: a fifth of the terms there made 300 blocks for 296 places, and the four that waited for one
+// doubled the kernel's time.
+constexpr int kInertiaParts = 4, kInertiaTerms = 4096 * 6 / 16 + 1;
+__device__ __forceinline__ int inertia_cut(int part, int batch)
+{
+    const int sixteenths = part <= 0 ? 0 : part == 1 ? 6 : part == 2 ? 7 : part == 3 ? 12 : 16;
+    return (int)((long long)sixteenths * batch / 16);
+}
 __device__ __forceinline__ void km_inertia(const KmeansParams &p, const Pair &q, int t, int part, int part_end, double *term_s)
 {
     if (t < 0 || !pair_active(p, q, t)) return;
@@ -889,7 +898,7 @@ __device__ __forceinline__ void km_inertia(const KmeansParams &p, const Pair &q,
     const double *dist = p.dist + ((size_t)(t & 1) * p.n_seqs * p.n_kv + q.id) * p.batch;
     double sum = part > 0 ? st.partial : 0.0;
     for (; part < part_end; ++part) {
-        const int lo = (int)((long long)part * p.batch / kInertiaParts), n = (int)((long long)(part + 1) * p.batch / kInertiaParts) - lo;
+        const int lo = inertia_cut(part, p.batch), n = inertia_cut(part + 1, p.batch) - lo;
         __syncthreads();
         for (int s = threadIdx.x; s < n; s += blockDim.x) term_s[s] = dist[lo + s];
         __syncthreads();
@@ -947,10 +956,6 @@ km_scan_kernel(KmeansParams p, int t)
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     const int tid = threadIdx.x;
-    if ((int)blockIdx.x == p.scan_blocks) {
-        km_inertia(p, q, t - 1, 2, 3, reinterpret_cast<double *>(near_smem));
-        return;
-    }
     if (!pair_active(p, q, t)) return;
     const ScanSplit sp = scan_split(p, q);
     if ((int)blockIdx.x >= sp.blocks) return;
@@ -989,78 +994,121 @@ km_scan_kernel(KmeansParams p, int t)
 }
 
 // The nearest centre of each minibatch point and the fp64 distance to it: the scan's results merged, the
-// candidates that the bounds leave open compared in fp64. A warp takes 32 points: the terms of each distance are
-// formed by all lanes (coalesced reads, four conversions a lane), then every lane adds up its own point's in order.
-constexpr int kResolveWarps = 2, kTermPitch = kHeadDim + 1;
-// Points of a block up to which they go through all centres one by one: two warps at about 37 us a point and 512 centres, against 200
+// candidates that the bounds leave open compared in fp64. A block takes 64 points, eight per warp: the terms of each distance
+// are formed by all lanes (coalesced reads, four conversions a lane), then a thread per point adds them up in order. Bound by the
+// latency of scattered reads: with 32 points per warp, one after another, 5 % of the warps were resident.
+constexpr int kResolveThreads = 256, kResolveWarps = kResolveThreads / 32, kResolvePoints = 64, kTermPitch = kHeadDim + 1;
+// Points of a block up to which they go through all centres one by one: eight warps at about 37 us a point and 512 centres, against 200
 // for all of the block's together.
-constexpr int kResolveFewOpen = 8;
+constexpr int kResolveFewOpen = 24;
+struct ResolveSmem {
+    double term[kResolvePoints][kTermPitch];
+    __align__(16) double tmp[kResolveWarps][kHeadDim];
+    double dist[2 * kResolvePoints];                        // of the listed candidates, or of the open points
+    int2 list[2 * kResolvePoints];                          // (point, centre)
+    int found[kResolvePoints];                              // nearest centres of the open points
+    int point[kResolvePoints], centre[kResolvePoints];
+    int n_list, n_open;
+};
+// Squared differences of a row (16-bit values) and a centre in each dimension, by a warp.
 template <bool kHalf>
-__global__ void __launch_bounds__(kResolveWarps * 32)
+__device__ __forceinline__ void resolve_terms(const uint16_t *x, const double *c, double *term)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const double d = __dsub_rn(elem_to_double<kHalf>(__ldg(x + 32 * e + lane)), c[32 * e + lane]);
+        term[32 * e + lane] = __dmul_rn(d, d);
+    }
+}
+template <bool kHalf>
+__global__ void __launch_bounds__(kResolveThreads)
 km_resolve_kernel(KmeansParams p, int t)
 {
-    extern __shared__ __align__(16) double term_s[];        // [warps][32][kTermPitch]
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ResolveSmem &sm = *reinterpret_cast<ResolveSmem *>(smem_raw);
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     if (blockIdx.x == gridDim.x - 1) {
-        km_inertia(p, q, t - 1, 3, 4, term_s);
+        km_inertia(p, q, t - 1, 2, 3, &sm.term[0][0]);
         return;
     }
     if (!pair_active(p, q, t)) return;
-    const int lane = threadIdx.x & 31, s = blockIdx.x * kResolveWarps * 32 + threadIdx.x;
-    const bool live = s < p.batch;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, s = blockIdx.x * kResolvePoints + tid;
+    const bool live = tid < kResolvePoints && s < p.batch;
     const size_t at = (size_t)q.id * p.batch + (live ? s : 0);
-    const int point = p.idx[at];
     const double *cen = p.centres64 + q.cplane * kHeadDim;
-    const ScanSplit sp = scan_split(p, q);
-    const int tile = (live ? s : 0) / kNearPoints;
-    const int segs = sp.block_of(tile * sp.k_tiles + sp.k_tiles - 1) - sp.block_of(tile * sp.k_tiles) + 1;
-    NearTop top = near_none(0);
-    for (int seg = 0; seg < segs; ++seg) near_merge(top, p.near_top[((size_t)q.id * p.scan_segs + seg) * p.batch + (live ? s : 0)]);
-    const float nx = p.near_nx[at];
-    const bool all = near_open(top, nx);
-    int arg = top.i1;
-    double *term = term_s + (size_t)(threadIdx.x >> 5) * 32 * kTermPitch;
     const uint16_t *keys = p.k_prompt + q.plane * kHeadDim;
-#pragma unroll 4
-    for (int l = 0; l < 32; ++l) {
-        const uint16_t *x = keys + (size_t)__shfl_sync(0xFFFFFFFFu, point, l) * kHeadDim;
-        const double *c = cen + (size_t)__shfl_sync(0xFFFFFFFFu, arg, l) * kHeadDim;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const double d = __dsub_rn(elem_to_double<kHalf>(__ldg(x + 32 * e + lane)), c[32 * e + lane]);
-            term[l * kTermPitch + 32 * e + lane] = __dmul_rn(d, d);
+    if (tid == 0) sm.n_list = sm.n_open = 0;
+    __syncthreads();
+    const int point = p.idx[at];
+    int arg = 0, second = -1, third = -1, open_at = -1;     // places in the lists
+    NearTop top = near_none(0);
+    if (tid < kResolvePoints) {
+        const ScanSplit sp = scan_split(p, q);
+        const int tile = (live ? s : 0) / kNearPoints;
+        const int segs = sp.block_of(tile * sp.k_tiles + sp.k_tiles - 1) - sp.block_of(tile * sp.k_tiles) + 1;
+        for (int seg = 0; seg < segs; ++seg) near_merge(top, p.near_top[((size_t)q.id * p.scan_segs + seg) * p.batch + (live ? s : 0)]);
+        arg = top.i1;
+        sm.point[tid] = point;
+        sm.centre[tid] = arg;
+        if (live) {
+            if (near_open(top, p.near_nx[at])) {
+                open_at = atomicAdd(&sm.n_open, 1);
+            } else {
+                if (!(top.t2 > top.upper)) sm.list[second = atomicAdd(&sm.n_list, 1)] = make_int2(point, top.i2);
+                if (!(top.t3 > top.upper)) sm.list[third = atomicAdd(&sm.n_list, 1)] = make_int2(point, top.i3);
+            }
         }
     }
-    __syncwarp();
-    double best = 0.0;
+    __syncthreads();
+#pragma unroll 4
+    for (int l = 0; l < kResolvePoints / kResolveWarps; ++l) {
+        const int i = warp * (kResolvePoints / kResolveWarps) + l;
+        resolve_terms<kHalf>(keys + (size_t)sm.point[i] * kHeadDim, cen + (size_t)sm.centre[i] * kHeadDim, sm.term[i]);
+    }
+    const int n_list = sm.n_list, n_open = sm.n_open;
+    for (int e = warp; e < n_list; e += kResolveWarps) {    // second and third candidates, a warp each
+        resolve_terms<kHalf>(keys + (size_t)sm.list[e].x * kHeadDim, cen + (size_t)sm.list[e].y * kHeadDim, sm.tmp[warp]);
+        __syncwarp();
+        if (lane == 0) {
+            double d = 0.0;
 #pragma unroll 16
-    for (int d = 0; d < kHeadDim; ++d) best = __dadd_rn(best, term[lane * kTermPitch + d]);
-    if (live && !all) {
-        const uint4 *x = reinterpret_cast<const uint4 *>(keys + (size_t)point * kHeadDim);
-        if (!(top.t2 > top.upper)) {
-            const double d2 = near_exact<kHalf>(x, cen + (size_t)top.i2 * kHeadDim);
+            for (int u = 0; u < kHeadDim; ++u) d = __dadd_rn(d, sm.tmp[warp][u]);
+            sm.dist[e] = d;
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    double best = 0.0;
+    if (tid < kResolvePoints) {
+#pragma unroll 16
+        for (int d = 0; d < kHeadDim; ++d) best = __dadd_rn(best, sm.term[tid][d]);
+        if (second >= 0) {
+            const double d2 = sm.dist[second];
             if (d2 < best || (d2 == best && top.i2 < arg)) { best = d2; arg = top.i2; }
         }
-        if (!(top.t3 > top.upper)) {
-            const double d3 = near_exact<kHalf>(x, cen + (size_t)top.i3 * kHeadDim);
+        if (third >= 0) {
+            const double d3 = sm.dist[third];
             if (d3 < best || (d3 == best && top.i3 < arg)) { best = d3; arg = top.i3; }
         }
     }
-    const bool open = live && all;
-    const int n_open = __syncthreads_count(open);
-    double d;
     if (n_open > kResolveFewOpen) {
-        const int u = near_scan_tiles<kHalf, kResolveWarps * 32, 1>(reinterpret_cast<const uint4 *>(keys + (size_t)point * kHeadDim), open, cen, q.k,
-                                                                    reinterpret_cast<double (*)[kHeadDim]>(term_s), d);
-        if (open) { best = d; arg = u; }
-    } else {
-        for (unsigned left = __ballot_sync(0xFFFFFFFFu, open); left; left &= left - 1) {
-            const int l = __ffs(left) - 1;
-            const uint4 *xl = reinterpret_cast<const uint4 *>(keys + (size_t)__shfl_sync(0xFFFFFFFFu, point, l) * kHeadDim);
-            const int u = near_scan_exact<kHalf>(xl, cen, q.k, term, d);
-            if (lane == l) { best = d; arg = u; }
+        double d;
+        const int u = near_scan_tiles<kHalf, kResolveThreads, 1>(reinterpret_cast<const uint4 *>(keys + (size_t)point * kHeadDim), open_at >= 0, cen, q.k,
+                                                                 reinterpret_cast<double (*)[kHeadDim]>(smem_raw), d);
+        if (open_at >= 0) { best = d; arg = u; }
+    } else if (n_open > 0) {
+        __syncthreads();                                    // the terms and the candidates' distances have been read
+        if (open_at >= 0) sm.point[open_at] = point;
+        __syncthreads();
+        for (int e = warp; e < n_open; e += kResolveWarps) {
+            double d;
+            const int u = near_scan_exact<kHalf>(reinterpret_cast<const uint4 *>(keys + (size_t)sm.point[e] * kHeadDim), cen, q.k, sm.tmp[warp], d);
+            if (lane == 0) { sm.dist[e] = d; sm.found[e] = u; }
         }
+        __syncthreads();
+        if (open_at >= 0) { best = sm.dist[open_at]; arg = sm.found[open_at]; }
     }
     if (live) {
         p.label[at] = arg;
@@ -1087,7 +1135,7 @@ km_sort_batch_kernel(KmeansParams p, int t)
     const int pairs = p.n_seqs * p.n_kv, pair = blockIdx.x % pairs;
     const Pair q = pair_of(p, pair / p.n_kv, pair % p.n_kv);
     if ((int)blockIdx.x >= pairs) {
-        km_inertia(p, q, t - 1, 4, 5, reinterpret_cast<double *>(smem_raw));
+        km_inertia(p, q, t - 1, 3, 4, reinterpret_cast<double *>(smem_raw));
         return;
     }
     // one look at the flag for the block: beside it the block above may be stopping this very fit
@@ -1154,9 +1202,11 @@ km_sort_batch_kernel(KmeansParams p, int t)
 }
 
 // Cumulative-count update, a warp per centre (four dimensions per lane): the centre's new points are added in
-// minibatch order; c <- (c * count + sum) / (count + n). The next 16 rows are on their way while 16 are added.
-template <bool kHalf>
-__global__ void __launch_bounds__(128)
+// minibatch order; c <- (c * count + sum) / (count + n). The next kAhead rows are on their way while kAhead are added:
+// 16 for centres of many points; 4 where a centre has less than eight on average, since 16 take the registers of
+// three of four warps (2048 centres of two points were three and a half waves of blocks).
+template <bool kHalf, int kAhead>
+__global__ void __launch_bounds__(128, kAhead > 4 ? 4 : 8)
 km_batch_update_kernel(KmeansParams p, int t)
 {
     __shared__ double term_s[kInertiaTerms];
@@ -1178,7 +1228,6 @@ km_batch_update_kernel(KmeansParams p, int t)
     const double2 *from = reinterpret_cast<const double2 *>(p.centres64 + (q.cplane + u) * kHeadDim + 4 * lane);
     const double2 c0 = from[0], c1 = from[1];
     double sum[4] = {0.0, 0.0, 0.0, 0.0};
-    constexpr int kAhead = 16;
     int id = point[min(lo + lane, hi - 1)];                 // tokens of the 32 points from `lo` on
     uint2 next[kAhead];
 #pragma unroll
@@ -1190,11 +1239,11 @@ km_batch_update_kernel(KmeansParams p, int t)
         uint2 w[kAhead];
 #pragma unroll
         for (int i = 0; i < kAhead; ++i) w[i] = next[i];
-        const bool second = ((i0 - lo) & kAhead) == 0;      // the next 16 are the second half of `id`
-        if (!second) id = point[min(i0 + kAhead + lane, hi - 1)];
+        const int place = (i0 - lo + kAhead) & 31;          // place of the next ones among the 32 of `id`
+        if (place == 0) id = point[min(i0 + kAhead + lane, hi - 1)];
 #pragma unroll
         for (int i = 0; i < kAhead; ++i) {
-            const int tok = __shfl_sync(0xFFFFFFFFu, id, second ? kAhead + i : i);
+            const int tok = __shfl_sync(0xFFFFFFFFu, id, place + i);
             if (i0 + kAhead + i < hi) next[i] = __ldg(keys + (size_t)tok * 32);
         }
 #pragma unroll
@@ -1346,18 +1395,20 @@ cudaError_t run_fit(const KmeansParams &p, cudaStream_t s)
     const dim3 threads(kThreads);
     if ((err = launch_step(km_prepare_kernel<kHalf>, dim3((p.k_max + kThreads / 32 - 1) / (kThreads / 32), pairs), threads, 0, s, p)) != cudaSuccess) return err;
     static std::atomic<unsigned long long> scan_done, resolve_done, sort_done;
-    const size_t resolve_smem = sizeof(double) * kResolveWarps * 32 * kTermPitch;
     if ((err = ensure_dynamic_smem((const void *)km_scan_kernel<kHalf>, (int)sizeof(NearSmem), scan_done)) != cudaSuccess) return err;
-    if ((err = ensure_dynamic_smem((const void *)km_resolve_kernel<kHalf>, (int)resolve_smem, resolve_done)) != cudaSuccess) return err;
+    if ((err = ensure_dynamic_smem((const void *)km_resolve_kernel<kHalf>, (int)sizeof(ResolveSmem), resolve_done)) != cudaSuccess) return err;
     if ((err = ensure_dynamic_smem((const void *)km_sort_batch_kernel, (int)sizeof(SortSmem), sort_done)) != cudaSuccess) return err;
     const size_t move_smem = std::max(sizeof(int32_t) * ((size_t)p.batch + (size_t)p.batch / 2 + 1), sizeof(double) * (size_t)kInertiaTerms);
-    const dim3 resolve_grid((p.batch + kResolveWarps * 32 - 1) / (kResolveWarps * 32) + 1, pairs);
+    const dim3 resolve_grid((p.batch + kResolvePoints - 1) / kResolvePoints + 1, pairs);
     int t = 0;
     for (; t < p.t_max_max; ++t) {
-        if ((err = launch_step(km_scan_kernel<kHalf>, dim3(p.scan_blocks + 1, pairs), dim3(kNearThreads), sizeof(NearSmem), s, p, t)) != cudaSuccess) return err;
-        if ((err = launch_step(km_resolve_kernel<kHalf>, resolve_grid, dim3(kResolveWarps * 32), resolve_smem, s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_scan_kernel<kHalf>, dim3(p.scan_blocks, pairs), dim3(kNearThreads), sizeof(NearSmem), s, p, t)) != cudaSuccess) return err;
+        if ((err = launch_step(km_resolve_kernel<kHalf>, resolve_grid, dim3(kResolveThreads), sizeof(ResolveSmem), s, p, t)) != cudaSuccess) return err;
         if ((err = launch_step(km_sort_batch_kernel, dim3(2 * pairs), dim3(kSortThreads), sizeof(SortSmem), s, p, t)) != cudaSuccess) return err;
-        if ((err = launch_step(km_batch_update_kernel<kHalf>, dim3((p.k_max + 3) / 4 + 1, pairs), dim3(128), 0, s, p, t)) != cudaSuccess) return err;
+        const dim3 update_grid((p.k_max + 3) / 4 + 1, pairs);
+        err = p.batch < 8 * p.k_max ? launch_step(km_batch_update_kernel<kHalf, 4>, update_grid, dim3(128), 0, s, p, t)
+                                    : launch_step(km_batch_update_kernel<kHalf, 16>, update_grid, dim3(128), 0, s, p, t);
+        if (err != cudaSuccess) return err;
         if ((err = launch_step(km_reassign_kernel<kHalf>, dim3(B, H, 2), threads, move_smem, s, p, t)) != cudaSuccess) return err;
         if (!p.no_host_poll && (t + 1) % kPollEvery == 0 && t + 1 < p.t_max_max) {
             // most fits stop long before the step limit: ask the device how many are still running

@@ -254,6 +254,13 @@ def test_start_with_ten_and_eleven_trials_a_centre(n):
     test_fit_with_a_centre_per_key_returns_the_keys(n)
 
 
+@pytest.mark.parametrize("batch,k", [(1, 2), (63, 7), (64, 8), (65, 9), (128, 16), (129, 16), (129, 17)])
+def test_steps_at_the_edges_of_their_blocks_and_of_the_update_rule(batch, k):
+    """64 points a block of the resolving kernel; fewer or more than eight points a centre in the update."""
+    keys = np.random.default_rng(37).standard_normal((2, 400, 128))
+    _fit_keys_both(keys.astype(np.float32), "bf16", k, batch_size=batch, max_iter=2, patience=30, seed=8, reassignment_ratio=0.01)
+
+
 @pytest.mark.parametrize("kind", ["few", "same", "padded", "some", "integer"])
 def test_fit_of_keys_that_repeat(kind):
     from test_gpu_parents import _repeated
