@@ -354,13 +354,16 @@ struct LatentPlanSmem {
     int scan[40];
 };
 
+// Grid (sequences, parts): every block finds the sequence's union for itself (its tables are a few KB of shared
+// memory) and writes its share of the segments. What a sequence has to write, 64 bytes of bias a segment and 8 a row,
+// is what the kernel takes its time for, and a batch has fewer sequences than the device has SMs.
 __global__ void __launch_bounds__(kLpThreads)
 latent_plan_kernel(LatentPlanParams p)
 {
     step_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LatentPlanSmem &sm = *reinterpret_cast<LatentPlanSmem *>(smem_raw);
-    const int b = blockIdx.x, tid = threadIdx.x;
+    const int b = blockIdx.x, tid = threadIdx.x, part = blockIdx.y, parts = gridDim.y;
     const int H = p.lv.n_heads, K = p.n_sample;
     const int64_t row0 = p.lv.seq_row_off[b];
     const int N = (int)(p.lv.seq_row_off[b + 1] - row0);
@@ -374,7 +377,8 @@ latent_plan_kernel(LatentPlanParams p)
 
     if (K >= M) {
         // every team is read with correction one; nothing was drawn
-        for (int i = tid; i < N; i += kLpThreads) line[i] = make_int2((int)(row0 + i), 0);
+        for (int i = part * kLpThreads + tid; i < N; i += parts * kLpThreads) line[i] = make_int2((int)(row0 + i), 0);
+        if (part > 0) return;
         for (int i = tid; i < t_suffix; i += kLpThreads) line[N + i] = make_int2((int)(kSrcSuffix | (uint32_t)(b * p.suffix_cap + i)), 0);
         if (tid < kHeads) bias[tid] = 0.f;
         if (tid == 0) {
@@ -421,15 +425,17 @@ latent_plan_kernel(LatentPlanParams p)
         int run = block_exclusive_scan(sum, sm.scan, nseg);
         for (int w = lo; w < hi; ++w) { sm.wprefix[w] = run; run += __popc(sm.bitmap[w]); }
     }
-    for (int i = tid; i < nseg * kHeads; i += kLpThreads) bias[i] = -CUDART_INF_F;
-    if (tid < kHeads) bias[(size_t)nseg * kHeads + tid] = 0.f;              // the suffix segment
+    const int seg_lo = nseg * part / parts, seg_hi = nseg * (part + 1) / parts;            // the block's segments
+    for (int i = seg_lo * (kHeads / 4) + tid; i < seg_hi * (kHeads / 4); i += kLpThreads)
+        reinterpret_cast<float4 *>(bias)[i] = make_float4(-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F);
+    if (part == 0 && tid < kHeads) bias[(size_t)nseg * kHeads + tid] = 0.f;  // the suffix segment
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < kLpPerThread; ++u) {
         const int team = my_team[u], e = tid + u * kLpThreads;
         if (team < 0) continue;
         const int seg = sm.wprefix[team >> 5] + __popc(sm.bitmap[team >> 5] & ((1u << (team & 31)) - 1u));
-        bias[(size_t)seg * kHeads + e / K] = -kLog2e * my_logc[u];             // weight e^s / c_g
+        if (seg >= seg_lo && seg < seg_hi) bias[(size_t)seg * kHeads + e / K] = -kLog2e * my_logc[u];      // weight e^s / c_g
         sm.seg_start[seg] = my_rows[u].x;                                      // the same from every selecting head
         sm.seg_n[seg] = my_rows[u].y;
     }
@@ -445,10 +451,11 @@ latent_plan_kernel(LatentPlanParams p)
     }
     __syncthreads();
     total = min(total, N);                                                     // distinct teams cannot hold more rows
-    for (int sg = tid; sg < nseg; sg += kLpThreads) {
+    for (int sg = seg_lo + tid; sg < seg_hi; sg += kLpThreads) {
         const int at = sm.seg_prefix[sg], n = sm.seg_n[sg], start = sm.seg_start[sg];
         for (int i = 0; i < n && at + i < N; ++i) line[at + i] = make_int2((int)(row0 + min(start + i, N - 1)), sg);
     }
+    if (part > 0) return;
     for (int i = tid; i < t_suffix; i += kLpThreads)
         line[total + i] = make_int2((int)(kSrcSuffix | (uint32_t)(b * p.suffix_cap + i)), nseg);
     if (tid == 0) {
@@ -1356,7 +1363,7 @@ int santapp_latent_decode_attn(const santapp_latent_geom *geom, const santapp_la
         static std::atomic<unsigned long long> done_plan;
         if ((err = ensure_dynamic_smem((const void *)latent_plan_kernel, (int)sizeof(LatentPlanSmem), done_plan)) != cudaSuccess)
             return note_cuda_failure(err, "latent plan attribute");
-        if ((err = launch_step(latent_plan_kernel, dim3(geom->n_seqs), dim3(kLpThreads), sizeof(LatentPlanSmem), s, pp)) != cudaSuccess)
+        if ((err = launch_step(latent_plan_kernel, dim3(geom->n_seqs, std::clamp(attend_grid_size() / geom->n_seqs, 1, 8)), dim3(kLpThreads), sizeof(LatentPlanSmem), s, pp)) != cudaSuccess)
             return note_cuda_failure(err, "latent plan launch");
         ++launches;
     }
