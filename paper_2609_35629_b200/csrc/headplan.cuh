@@ -108,9 +108,9 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
         q_val[i] = tid + i * kT < kDim ? elem_to_float<kHalf>(in.q[(size_t)hq * kDim + tid + i * kT]) : 0.f;
     const float k_abs_max = in.rep_abs_max[(size_t)j * in.bv.n_seqs + b];
     // fp32 -> fp64 conversions run at 16 per clock and SM, a quarter of the fp64 rate, and are what the exact dot products
-    // wait for. Finite bf16 keys convert the upper value of a word with two integer instructions instead: its bits,
-    // moved to where a double has them, are the value times 2^-896 (subnormals included). The query's odd
-    // values are held times 2^700 and the odd sums end with 2^196: exact scalings, the same sums bit for bit.
+    // wait for. Finite bf16 keys are widened by two or three integer instructions instead: a value's bits, moved to
+    // where a double has them, are the value times 2^-896 (subnormals included). The query is held times 2^700
+    // and the sums end with 2^196: exact scalings, the same sums bit for bit.
     const bool shifted = !kHalf && k_abs_max <= 3.4e38f;
     constexpr double kShiftUp = 0x1p700, kShiftDown = 0x1p196;
 
@@ -175,7 +175,7 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
 #pragma unroll
         for (int i = 0; i < kQRegs; ++i) {
             const int d = tid + i * kT;
-            if (d < kDim) sm.q64[(d >> 3) & 7][(d >> 6) * 8 + (d & 7)] = (double)q_val[i] * (shifted && (d & 1) ? kShiftUp : 1.0);
+            if (d < kDim) sm.q64[(d >> 3) & 7][(d >> 6) * 8 + (d & 7)] = (double)q_val[i] * (shifted ? kShiftUp : 1.0);
         }
         if (lane == 0) { sm.red_sum[warp] = a; sm.red_max[warp] = top; }
         if (tid == 0) { sm.n_cand = 0; sm.rank_sum = 0; }
@@ -321,6 +321,10 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
         // are the longest chain of the kernel), then every thread takes a candidate's other terms.
         auto dot_products = [&](auto by_bits) {
             constexpr bool kBits = decltype(by_bits)::value;
+            auto widen_even = [](uint32_t w) {
+                if constexpr (kBits) return __hiloint2double(((int)(w << 16) >> 3) & (int)0x8FFFE000, 0);
+                else return (double)elem_lo<kHalf>(w);
+            };
             auto widen_odd = [](uint32_t w) {
                 if constexpr (kBits) return __hiloint2double(((int)w >> 3) & (int)0x8FFFE000, 0);
                 else return (double)elem_hi<kHalf>(w);
@@ -329,44 +333,90 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
             const double *qs = sm.q64[sub];
             // (piece sub + 8 pc for each pc: a key's eight lanes read whole 128-byte lines together; with slices of consecutive
             // pieces instead, 576-value keys touched 32 lines an instruction and the kernel was bound by line accesses)
-            // a few candidates per thread group at a time: all their key pieces are requested before
-            // the first product, so a chunk costs one memory round trip
-            constexpr int kPerPass = kDotWarps * 32 / kDotLanes, kChunk = kPieces > 2 ? 1 : (kT >= 512 ? 2 : 4);
-            for (int c0 = 0; c0 < n_cand; c0 += kPerPass * kChunk) {
-                uint4 w[kChunk][kPieces];
+            constexpr int kPerPass = kDotWarps * 32 / kDotLanes;
+            if constexpr (kPieces > 2) {
+                // two candidates per thread group, kDepth pieces of each on their way: a query value read from shared memory, which
+                // takes as long as four products of it, serves both
+                constexpr int kDepth = 3;
+                auto key_of = [&](int cand) { return reinterpret_cast<const uint4 *>(rep + (size_t)sm.cand_id[min(cand, n_cand - 1)] * kDim) + sub; };
+                for (int c0 = 0; c0 < n_cand; c0 += 2 * kPerPass) {
+                    const int cand = c0 + (tid >> 3);
+                    const uint4 *ka = key_of(cand), *kb = key_of(cand + kPerPass);
+                    uint4 w[2][kDepth];
 #pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    const int cand = c0 + u * kPerPass + (tid >> 3);
-                    if (cand < n_cand) {
-                        const uint4 *kr = reinterpret_cast<const uint4 *>(rep + (size_t)sm.cand_id[cand] * kDim) + sub;
-#pragma unroll
-                        for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = __ldg(kr + kDotLanes * pc);
-                    } else {
-#pragma unroll
-                        for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = make_uint4(0u, 0u, 0u, 0u);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    const int cand = c0 + u * kPerPass + (tid >> 3);
-                    double d0 = 0.0, d1 = 0.0;                        // even and odd dims of the slice, in order
+                    for (int pc = 0; pc < kDepth; ++pc) { w[0][pc] = __ldg(ka + kDotLanes * pc); w[1][pc] = __ldg(kb + kDotLanes * pc); }
+                    double d[2][2] = {};                              // even and odd dims of the slices, in order
 #pragma unroll
                     for (int pc = 0; pc < kPieces; ++pc) {
-                        const uint4 wv = w[u][pc];
-                        d0 = fma((double)elem_lo<kHalf>(wv.x), qs[8 * pc + 0], d0);
-                        d1 = fma(widen_odd(wv.x), qs[8 * pc + 1], d1);
-                        d0 = fma((double)elem_lo<kHalf>(wv.y), qs[8 * pc + 2], d0);
-                        d1 = fma(widen_odd(wv.y), qs[8 * pc + 3], d1);
-                        d0 = fma((double)elem_lo<kHalf>(wv.z), qs[8 * pc + 4], d0);
-                        d1 = fma(widen_odd(wv.z), qs[8 * pc + 5], d1);
-                        d0 = fma((double)elem_lo<kHalf>(wv.w), qs[8 * pc + 6], d0);
-                        d1 = fma(widen_odd(wv.w), qs[8 * pc + 7], d1);
+                        double qv[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) qv[e] = qs[8 * pc + e];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const uint4 wv = w[u][pc % kDepth];
+                            d[u][0] = fma(widen_even(wv.x), qv[0], d[u][0]);
+                            d[u][1] = fma(widen_odd(wv.x), qv[1], d[u][1]);
+                            d[u][0] = fma(widen_even(wv.y), qv[2], d[u][0]);
+                            d[u][1] = fma(widen_odd(wv.y), qv[3], d[u][1]);
+                            d[u][0] = fma(widen_even(wv.z), qv[4], d[u][0]);
+                            d[u][1] = fma(widen_odd(wv.z), qv[5], d[u][1]);
+                            d[u][0] = fma(widen_even(wv.w), qv[6], d[u][0]);
+                            d[u][1] = fma(widen_odd(wv.w), qv[7], d[u][1]);
+                        }
+                        if (pc + kDepth < kPieces) {
+                            w[0][pc % kDepth] = __ldg(ka + kDotLanes * (pc + kDepth));
+                            w[1][pc % kDepth] = __ldg(kb + kDotLanes * (pc + kDepth));
+                        }
                     }
-                    double d = kBits ? fma(d1, kShiftDown, d0) : d0 + d1;
-                    d += __shfl_xor_sync(0xFFFFFFFFu, d, 1);
-                    d += __shfl_xor_sync(0xFFFFFFFFu, d, 2);
-                    d += __shfl_xor_sync(0xFFFFFFFFu, d, 4);
-                    if (cand < n_cand && sub == 0) sm.cand_y[cand] = d;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        double y = kBits ? (d[u][0] + d[u][1]) * kShiftDown : d[u][0] + d[u][1];
+                        y += __shfl_xor_sync(0xFFFFFFFFu, y, 1);
+                        y += __shfl_xor_sync(0xFFFFFFFFu, y, 2);
+                        y += __shfl_xor_sync(0xFFFFFFFFu, y, 4);
+                        if (cand + u * kPerPass < n_cand && sub == 0) sm.cand_y[cand + u * kPerPass] = y;
+                    }
+                }
+            } else {
+                // a few candidates per thread group at a time: all their key pieces are requested before
+                // the first product, so a chunk costs one memory round trip
+                constexpr int kChunk = kT >= 512 ? 2 : 4;
+                for (int c0 = 0; c0 < n_cand; c0 += kPerPass * kChunk) {
+                    uint4 w[kChunk][kPieces];
+#pragma unroll
+                    for (int u = 0; u < kChunk; ++u) {
+                        const int cand = c0 + u * kPerPass + (tid >> 3);
+                        if (cand < n_cand) {
+                            const uint4 *kr = reinterpret_cast<const uint4 *>(rep + (size_t)sm.cand_id[cand] * kDim) + sub;
+#pragma unroll
+                            for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = __ldg(kr + kDotLanes * pc);
+                        } else {
+#pragma unroll
+                            for (int pc = 0; pc < kPieces; ++pc) w[u][pc] = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kChunk; ++u) {
+                        const int cand = c0 + u * kPerPass + (tid >> 3);
+                        double d0 = 0.0, d1 = 0.0;                        // even and odd dims of the slice, in order
+#pragma unroll
+                        for (int pc = 0; pc < kPieces; ++pc) {
+                            const uint4 wv = w[u][pc];
+                            d0 = fma(widen_even(wv.x), qs[8 * pc + 0], d0);
+                            d1 = fma(widen_odd(wv.x), qs[8 * pc + 1], d1);
+                            d0 = fma(widen_even(wv.y), qs[8 * pc + 2], d0);
+                            d1 = fma(widen_odd(wv.y), qs[8 * pc + 3], d1);
+                            d0 = fma(widen_even(wv.z), qs[8 * pc + 4], d0);
+                            d1 = fma(widen_odd(wv.z), qs[8 * pc + 5], d1);
+                            d0 = fma(widen_even(wv.w), qs[8 * pc + 6], d0);
+                            d1 = fma(widen_odd(wv.w), qs[8 * pc + 7], d1);
+                        }
+                        double d = kBits ? (d0 + d1) * kShiftDown : d0 + d1;
+                        d += __shfl_xor_sync(0xFFFFFFFFu, d, 1);
+                        d += __shfl_xor_sync(0xFFFFFFFFu, d, 2);
+                        d += __shfl_xor_sync(0xFFFFFFFFu, d, 4);
+                        if (cand < n_cand && sub == 0) sm.cand_y[cand] = d;
+                    }
                 }
             }
         };
