@@ -27,10 +27,9 @@ static cudaError_t launch_headplan_t(const PlanInputs &in, cudaStream_t s)
 {
     const int n_heads = in.bv.n_seqs * in.bv.n_q;
     const int sms = attend_grid_size();
-    // up to 1024 scores a head 256 threads are faster than 512: a replayed step 15.1 against 15.9 us at 256 teams, 18.9 and
-    // 19.7 at 1024. At 2048 they are too by now (21.2 and 21.8; 7.6 and 7.4 us of kernel before the one-pass ranking, when
-    // this line was drawn); longer rows have not been measured again
-    if (n_heads <= sms && in.y_stride > 1024) return launch_step(headplan_kernel<512, kHalf>, dim3(n_heads), dim3(512), 0, s, in);
+    // up to 2048 scores a head 256 threads are faster than 512 (28 layers of 28 heads, 2048 teams: 675 against 693 us), above
+    // they are slower (8192 teams: 715 against 592, 4 x 8192: 37.4 against 32.8)
+    if (n_heads <= sms && in.y_stride > 2048) return launch_step(headplan_kernel<512, kHalf>, dim3(n_heads), dim3(512), 0, s, in);
     if (n_heads <= 4 * sms) return launch_step(headplan_kernel<256, kHalf>, dim3(n_heads), dim3(256), 0, s, in);
     return launch_step(headplan_kernel<128, kHalf>, dim3(n_heads), dim3(128), 0, s, in);
 }
