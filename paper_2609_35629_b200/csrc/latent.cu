@@ -66,11 +66,11 @@ struct LatentBuildParams {
 
 // A warp per parent (at most 32 rows), everything in one kernel: the parent's rows keep their range of the packed
 // order, so its owners give its row offsets and packed rows at once. Rows go through shared memory (asynchronous
-// copies, 18 KB of 16 rows on their way per warp, ten warps per SM); distances over the latent columns and the
+// copies, 18 KB of 16 rows on their way per warp, eleven warps per SM); distances over the latent columns and the
 // selection: select_rows.cuh. Bound by memory: 1152 bytes in and 1152 * (1 + R / P) out per row. The fp64
 // version in three kernels (block per parent, scan, pack) took 1309 us for 32 sequences of 8192.
 constexpr int kLbPitch = kRowDim / 2 + 4;                   // words per staged row: ldmatrix without bank conflicts
-constexpr int kLbWarps = 2;
+constexpr int kLbWarps = 1;                                 // (of two, ten instead of eleven warps share an SM: 127 against 122 us)
 template <int kRows>
 struct LatentBuildSmem {
     __align__(16) uint32_t rows[kRows * kLbPitch];
