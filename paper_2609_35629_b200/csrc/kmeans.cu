@@ -323,37 +323,56 @@ km_accept_kernel(KmeansParams p, int c)
 // of what it takes off their nearest-centre distance, and the products of the rows with the trial points give every
 // such gain within a bound (select_rows.cuh). Per centre the cluster's blocks
 //   1. multiply their rows with the trial points on tensor cores, mark the points that a trial may lower, add up
-//      each trial's largest and smallest possible gain, and exchange the sums (distributed shared memory);
+//      each trial's largest and smallest possible gain, and send one another the sums;
 //   2. take the trial whose smallest gain exceeds every other's largest; if there is none, the potentials are
 //      summed in fp64 for all trials (a few centres in two thousand; trials that drew the same point do not count);
 //   3. evaluate the winner's marked points in fp64 (a handful, after the first hundred centres), lower the
-//      distances, renew the running sums of the blocks of the sums they lie in, and exchange those blocks' sums;
+//      distances, renew the running sums of the blocks of the sums they lie in, and send those blocks' sums;
 //   4. add up the blocks and draw the next trial points: the block that owns a drawn point sends its row to all.
-// Left are three cluster barriers a centre and the serial sums (128 terms of a distance, of a block, the blocks;
-// 8 cycles a term). The two kernels per centre took 38 us, 24 of them fp64 distances of every point to every trial.
-constexpr int kStartThreads = 256, kStartWarps = kStartThreads / 32;
+// Bound by the chain of a centre, 13000 cycles of 12288 points and nine trials: 4700 for the marks (1500 of them products at the
+// tensor cores' rate, the rest their operands, the look at the results and the slowest warp), 3900 for the slowest
+// block's distances and its running sums (128 terms in order, 11 cycles each), 1100 for the blocks' (96 terms), three
+// messages of 700. Messages are stores that count their bytes on an mbarrier of the block they go to; with cluster
+// barriers behind remote stores, three of 1900 cycles, all of a block's threads waiting for the slowest block's, and a
+// distance summed in order by one lane (1100 cycles a point), a centre took 8.2 us, now 6.6. Sixteen warps, so that three
+// tiles a warp and four warps a scheduler overlap operands, products and marks (eight warps: 6.9). The operands wait in tensor
+// memory: read from shared memory they are as long on their way as the products take. (tcgen05 itself: sixteen
+// columns take as long as 128, 9 us a centre.) The two kernels per centre took 38 us, 24 of them fp64 distances of
+// every point to every trial.
+constexpr int kStartThreads = 512, kStartWarps = kStartThreads / 32;
 constexpr int kStartBlocks = 6;          // blocks of the sums per thread block: 768 rows of 256 bytes
 constexpr int kStartRows = kStartBlocks * kSumBlock;
+constexpr int kStartTmp = 4;             // warps that sum potentials
+enum { kGains, kSums, kDraws };          // the messages of a centre
 constexpr int kStartMaxCluster = 16, kStartSums = kStartBlocks * kStartMaxCluster;
 constexpr int kStartTrials = 11;         // 2 + floor(ln k) for every k with a sample of at most 16 * kStartRows: k <= 12288, ln k < 10
+static_assert(kStartTrials <= kStartWarps, "a warp per draw");
 static_assert(kStartMaxCluster * kStartRows < 22026, "e^10: from there on a centre has more trials");
 
+struct StartDraw {                       // a drawn trial point: squared norm, index in the sample, unit (elem_unit of its row)
+    float norm;
+    int pick, unit, pad;
+};
 struct StartSmem {
-    uint4 rows[kStartRows * 16];                            // 16-byte pieces XOR-swizzled (near_piece)
+    alignas(16) uint4 rows[kStartRows * 16];                // 16-byte pieces XOR-swizzled (near_piece)
     uint4 trial[kStartTrials * 16];
     double closest[kStartRows];
     double run[kStartRows];                                 // running sums of the distances inside each block of the sums
-    double tmp[kStartWarps][kSumBlock];
+    double tmp[kStartTmp][kSumBlock];
     double raw[kStartSums];                                 // sums of all the pair's blocks
     double pre[kStartSums];                                 // ... and their running sums
     float norm[kStartRows];                                 // squared norms
-    float bar[kStartRows];                                  // norm * (1 - error) - nearest-centre distance
-    float2 gain[kStartMaxCluster][kStartTrials];            // (smallest, largest) gain of a trial over each block's points
-    float2 warp_gain[kStartWarps][kStartTrials];
-    float trial_norm[kStartTrials];
-    int pick[2][kStartTrials];                              // sample indices of the trial points
+    float bar[kStartRows];                                  // norm * (1 - error) - nearest-centre distance; infinite where no centre is nearer
+    float2 gain[2][kStartMaxCluster][kStartTrials];         // (smallest, largest) gain of a trial over each block's points, by the centre's parity
+    float own_gain[2][kStartTrials][2];                     // of this block, by the centre's parity
+    alignas(16) StartDraw draw[2][kStartTrials];            // the trial points, by the centre's parity
+    uint64_t arrived[3];                                    // mbarriers: every block's gains, block sums, trial points
     uint32_t touched[kStartBlocks];                         // trials with a marked point in the block
+    uint32_t tmem;
+    int failed;                                             // a wait ran out (never expected)
     uint16_t mask[kStartRows];                              // trials that may lower the point's distance
+    int8_t unit[kStartRows];                                // every value of the row is a multiple of 2^unit; -128: not known
+    uint8_t list[kStartWarps][kSumBlock];                   // marked points of a warp's block
 };
 static_assert(sizeof(StartSmem) <= 227 * 1024, "shared memory of one block");
 
@@ -384,16 +403,41 @@ __device__ __forceinline__ void cluster_barrier()
     __syncwarp();
 }
 
-// Four of a row's values (dimensions 4 * lane ..) as doubles.
+// Messages between the blocks of a cluster: stores into another block's shared memory that count their bytes on an mbarrier there.
+__device__ __forceinline__ void send2(uint32_t to, uint32_t bar, float x, float y)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(to), "f"(x), "f"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send_double(uint32_t to, uint32_t bar, double x)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(to), "d"(x), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send4(uint32_t to, uint32_t bar, uint4 v)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(to), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void expect_bytes(uint64_t *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(shared_addr(bar)), "r"(bytes) : "memory");
+}
+
+// The exponent of a 16-bit value's lowest set bit; 127 for zero, -128 where it is -128 or below.
 template <bool kHalf>
-__device__ __forceinline__ void row_quad(const uint4 *rows, int i, double (&v)[4])
+__device__ __forceinline__ int elem_unit(uint32_t v)
+{
+    constexpr int kMan = kHalf ? 10 : 7, kLow = kHalf ? -24 : -133;         // mantissa bits, exponent of the smallest subnormal
+    const int e = (int)((v & 0x7FFFu) >> kMan), m = (int)(v & ((1u << kMan) - 1u)) | (e > 0 ? 1 << kMan : 0);
+    return m == 0 ? 127 : max(kLow + max(e, 1) - 1 + __ffs(m) - 1, -128);
+}
+// The smallest of a row's, by a warp.
+template <bool kHalf>
+__device__ __forceinline__ int row_unit(const uint4 *rows, int i)
 {
     const int lane = threadIdx.x & 31;
     const uint2 w = reinterpret_cast<const uint2 *>(rows + near_piece(i, lane >> 1))[lane & 1];
-    v[0] = (double)elem_lo<kHalf>(w.x);
-    v[1] = (double)elem_hi<kHalf>(w.x);
-    v[2] = (double)elem_lo<kHalf>(w.y);
-    v[3] = (double)elem_hi<kHalf>(w.y);
+    return __reduce_min_sync(0xFFFFFFFFu, min(min(elem_unit<kHalf>(w.x & 0xFFFFu), elem_unit<kHalf>(w.x >> 16)),
+                                              min(elem_unit<kHalf>(w.y & 0xFFFFu), elem_unit<kHalf>(w.y >> 16))));
 }
 // Squared norm of a row by a warp (an fp32 sum; every lane gets it).
 template <bool kHalf>
@@ -451,50 +495,53 @@ __device__ __forceinline__ double start_dist(const uint4 *rows, int i, const uin
     }
     return s;
 }
-// The same by a warp: every lane widens and squares four dimensions (widening is what a lane on its own would wait
-// for: 8 cycles a value), one adds them up in order. `tmp`: 128 doubles of the warp. Every lane gets it.
+// Eight consecutive values as doubles.
 template <bool kHalf>
-__device__ __forceinline__ double start_dist_warp(const uint4 *rows, int i, const double (&y)[4], double *tmp)
+__device__ __forceinline__ void widen8(const uint4 &w4, double (&v)[8])
 {
-    const int lane = threadIdx.x & 31;
-    double x[4];
-    row_quad<kHalf>(rows, i, x);
+    const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        x[e] = __dsub_rn(x[e], y[e]);
-        x[e] = __dmul_rn(x[e], x[e]);
+    for (int t = 0; t < 4; ++t) {
+        v[2 * t] = (double)elem_lo<kHalf>(w[t]);
+        v[2 * t + 1] = (double)elem_hi<kHalf>(w[t]);
     }
-    *reinterpret_cast<double2 *>(tmp + 4 * lane) = make_double2(x[0], x[1]);
-    *reinterpret_cast<double2 *>(tmp + 4 * lane + 2) = make_double2(x[2], x[3]);
-    __syncwarp();
-    double s = 0.0;
-    if (lane == 0) {
-        double t[8];
+}
+// An eighth of that distance in any order: pieces `part` and `part + 8` of row i against a trial point's, y.
+template <bool kHalf>
+__device__ __forceinline__ double start_dist_part(const uint4 *rows, int i, int part, const double (&y)[2][8])
+{
+    double s[2] = {0.0, 0.0};
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(&t[e]) = *reinterpret_cast<const double2 *>(tmp + e);
+    for (int h = 0; h < 2; ++h) {
+        double x[8];
+        widen8<kHalf>(rows[near_piece(i, part + 8 * h)], x);
 #pragma unroll
-        for (int u = 0; u < kHeadDim; u += 8) {
-            double n[8];
-#pragma unroll
-            for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2 *>(&n[e]) = *reinterpret_cast<const double2 *>(tmp + (u + 8 < kHeadDim ? u + 8 : u) + e);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) s = __dadd_rn(s, t[e]);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) t[e] = n[e];
+        for (int t = 0; t < 8; ++t) {
+            const double e = x[t] - y[h][t];
+            s[h] = fma(e, e, s[h]);
         }
     }
-    s = __shfl_sync(0xFFFFFFFFu, s, 0);
-    __syncwarp();
-    return s;
+    return s[0] + s[1];
+}
+// A lane of every eight gets the sum of the eight lanes' parts (all eight do).
+__device__ __forceinline__ double sum_parts(double s)
+{
+    s += __shfl_xor_sync(0xFFFFFFFFu, s, 1);
+    s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
+    return s + __shfl_xor_sync(0xFFFFFFFFu, s, 4);
 }
 
 template <bool kHalf>
 __global__ void __launch_bounds__(kStartThreads, 1)
 km_start_kernel(KmeansParams p)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    StartSmem &sm = *reinterpret_cast<StartSmem *>(smem_raw);
+    extern __shared__ __align__(128) unsigned char start_smem[];
+    StartSmem &sm = *reinterpret_cast<StartSmem *>(start_smem);
     constexpr float kPairErr = 0.5f * kDistErr;             // times the sum of the two squared norms, plus kUnderflow
+    // The rows as mma.sync's first operands (a word per lane, tile of 16 rows, step of 16 values: 32 columns a tile) in tensor memory,
+    // a warp's tiles m = warp, warp + 16, ... behind one another, four warps to a quarter of the lanes.
+    constexpr int kTiles = kStartRows / 16 / kStartWarps, kTmemCols = 512;
+    static_assert(kStartWarps / 4 * kTiles * 32 <= kTmemCols, "operands in tensor memory");
     const int n_blk = (int)cluster_size(), rank = (int)cluster_rank();
     const int pair = blockIdx.x / n_blk, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, c4 = lane & 3;
     const Pair q = pair_of(p, pair / p.n_kv, pair % p.n_kv);
@@ -510,26 +557,78 @@ km_start_kernel(KmeansParams p)
     for (int e = tid; e < n_rows * 16; e += kStartThreads)
         copy16_async(shared_addr(&sm.rows[near_piece(e >> 4, e & 15)]), keys + (size_t)perm[row0 + (e >> 4)] * 16 + (e & 15));
     const int first = p.pick[(size_t)q.id * p.trials_max];
-    if (tid < 16) copy16_async(shared_addr(&sm.trial[near_piece(0, tid)]), keys + (size_t)perm[first] * 16 + tid);
+    if (tid == 0) {
+        sm.failed = 0;
+        for (int t = 0; t < 3; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&sm.arrived[t])), "r"(1));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(shared_addr(&sm.tmem)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
+    }
     copy_async_wait();
+    for (int e = n_rows * 16 + tid; e < mb * kSumBlock * 16; e += kStartThreads) sm.rows[near_piece(e >> 4, e & 15)] = make_uint4(0u, 0u, 0u, 0u);
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
+    const int tiles = mb * (kSumBlock / 16);
+    const uint32_t operands = sm.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * kTiles * 32);
+    for (int n = 0; warp + kStartWarps * n < tiles; ++n)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t w[16];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t f[4];
+                ldmatrix4(f, shared_addr(&sm.rows[near_piece((warp + kStartWarps * n) * 16 + (lane & 15), 8 * h + 2 * e + (lane >> 4))]));
+                w[4 * e] = f[0]; w[4 * e + 1] = f[1]; w[4 * e + 2] = f[2]; w[4 * e + 3] = f[3];
+            }
+            tc_st16(operands + (uint32_t)(32 * n + 16 * h), w);
+        }
     for (int i = warp; i < mb * kSumBlock; i += kStartWarps) {
         const float n = i < n_rows ? row_norm<kHalf>(sm.rows, i) : 0.f;
+        const int unit = i < n_rows ? row_unit<kHalf>(sm.rows, i) : 0;
         if (lane == 0) {
             sm.norm[i] = n;
+            sm.unit[i] = (int8_t)unit;
             sm.closest[i] = i < n_rows ? CUDART_INF : 0.0;
             sm.bar[i] = i < n_rows ? 0.f : CUDART_INF_F;    // (set with the first distances)
             sm.mask[i] = i < n_rows ? 1 : 0;
         }
     }
+    if (warp == 0) {
+        const uint4 piece = __ldg(keys + (size_t)perm[first] * 16 + (lane & 15));
+        if (lane < 16) sm.trial[near_piece(0, lane)] = piece;
+        const uint32_t w[4] = {piece.x, piece.y, piece.z, piece.w};
+        int unit = 127;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) unit = min(unit, min(elem_unit<kHalf>(w[t] & 0xFFFFu), elem_unit<kHalf>(w[t] >> 16)));
+        unit = __reduce_min_sync(0xFFFFFFFFu, unit);
+        if (lane == 0) { sm.draw[0][0].unit = unit; sm.draw[0][0].pick = first; }
+    }
     if (tid < kStartBlocks) sm.touched[tid] = tid < mb ? 1u : 0u;
-    if (tid == 0) sm.pick[0][0] = first;
-    for (int e = tid; e < kStartMaxCluster * kStartTrials; e += kStartThreads) sm.gain[0][e] = make_float2(0.f, 0.f);
+    for (int e = tid; e < 2 * kStartMaxCluster * kStartTrials; e += kStartThreads) sm.gain[0][0][e] = make_float2(0.f, 0.f);
+    if (tid < 4 * kStartTrials) sm.own_gain[0][0][tid] = 0.f;
     cluster_barrier();                                      // every block of the cluster runs: its shared memory may be written
 
+    auto await = [&](int what, uint32_t parity) {
+        if (!*reinterpret_cast<volatile int *>(&sm.failed) && !tc_wait(shared_addr(&sm.arrived[what]), parity)) sm.failed = 1;
+        __syncwarp();
+    };
+    // a thread sends one trial's gains to one block
+    const int gain_of = tid % q.L, gain_to = tid / q.L;
+    const uint32_t gain_at = in_block(shared_addr(&sm.gain[0][rank][gain_of]), min(gain_to, n_blk - 1));
+    const uint32_t gain_bar = in_block(shared_addr(&sm.arrived[kGains]), min(gain_to, n_blk - 1));
     for (int c = 0; c < q.k; ++c) {
-        const int L = c == 0 ? 1 : q.L;
+        const int L = c == 0 ? 1 : q.L, par = c & 1;
         int best = 0;
+        if (tid == 0) {                                     // the centre's messages to come (the ones before have all been waited for)
+            if (c > 0) expect_bytes(&sm.arrived[kGains], (uint32_t)(n_blk * L * sizeof(float2)));
+            if (c + 1 < q.k) {
+                expect_bytes(&sm.arrived[kSums], (uint32_t)(nb * sizeof(double)));
+                expect_bytes(&sm.arrived[kDraws], (uint32_t)(q.L * (kHeadDim * 2 + sizeof(StartDraw))));
+            }
+        }
         if (c > 0) {
             // ---- 1. which points a trial may lower, and by how much ----
             uint32_t bf[2][8][2];                           // the trial points as MMA columns (two groups of eight)
@@ -547,108 +646,94 @@ km_start_kernel(KmeansParams p)
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 const int t = (v >> 1) * 8 + 2 * c4 + (v & 1);
-                const float n = t < L ? sm.trial_norm[t] : 0.f;
+                const float n = t < L ? sm.draw[par][t].norm : 0.f;
                 // (a column that is no trial is never marked; of a norm that fp32 does not hold the product decides nothing)
                 ny[v] = t >= L ? CUDART_INF_F : (n <= 1e37f ? n * (1.f - kPairErr) : -CUDART_INF_F);
                 err[v] = 2.f * kPairErr * n;
                 lo[v] = hi[v] = 0.f;
             }
-            const int tiles = mb * (kSumBlock / 16);        // a multiple of 8: every warp has the same number, two at a time
-            for (int m0 = warp; m0 < tiles; m0 += 2 * kStartWarps) {
-                const bool two = m0 + kStartWarps < tiles;
-                const int mt[2] = {m0, two ? m0 + kStartWarps : m0};
-                float acc[2][2][4];
-#pragma unroll
-                for (int k = 0; k < 2; ++k)
-#pragma unroll
-                    for (int n = 0; n < 2; ++n) acc[k][n][0] = acc[k][n][1] = acc[k][n][2] = acc[k][n][3] = 0.f;
+            for (int n = 0; warp + kStartWarps * n < tiles; ++n) {
+                const int i0 = (warp + kStartWarps * n) * 16;
+                float acc[2][4] = {};
+                uint32_t a[32];
+                tc_ld32(operands + (uint32_t)(32 * n), a);
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
-                    uint32_t a[2][4];
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) ldmatrix4(a[k], shared_addr(&sm.rows[near_piece(mt[k] * 16 + (lane & 15), 2 * s + (lane >> 4))]));
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        mma_rows<kHalf>(acc[k][0], a[k][0], a[k][1], a[k][2], a[k][3], bf[0][s][0], bf[0][s][1]);
-                        if (L > 8) mma_rows<kHalf>(acc[k][1], a[k][0], a[k][1], a[k][2], a[k][3], bf[1][s][0], bf[1][s][1]);
-                    }
+                    mma_rows<kHalf>(acc[0], a[4 * s], a[4 * s + 1], a[4 * s + 2], a[4 * s + 3], bf[0][s][0], bf[0][s][1]);
+                    if (L > 8) mma_rows<kHalf>(acc[1], a[4 * s], a[4 * s + 1], a[4 * s + 2], a[4 * s + 3], bf[1][s][0], bf[1][s][1]);
                 }
+                uint32_t bits[2];
+                float val[2][4];
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    if (k == 1 && !two) break;
-                    uint32_t bits[2];
-                    float val[2][4];
+                for (int h = 0; h < 2; ++h) {
+                    const float bar = sm.bar[i0 + g + 8 * h];
+                    bits[h] = 0u;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        val[h][v] = fmaf(-2.f, acc[v >> 1][2 * h + (v & 1)], bar + ny[v]);
+                        if (!(val[h][v] > kUnderflow)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));
+                    }
+                    if (!(bar < CUDART_INF_F)) bits[h] = 0u;         // a centre, or past the end of the sample
+                }
+                if (__any_sync(0xFFFFFFFFu, (bits[0] | bits[1]) != 0u)) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const float bar = sm.bar[mt[k] * 16 + g + 8 * h];
-                        bits[h] = 0u;
+                        const float e = fmaf(2.f * kPairErr, sm.norm[i0 + g + 8 * h], kUnderflow);
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            val[h][v] = fmaf(-2.f, acc[k][v >> 1][2 * h + (v & 1)], bar + ny[v]);
-                            if (!(val[h][v] > kUnderflow)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));
-                        }
-                        if (!(bar < CUDART_INF_F)) bits[h] = 0u;     // past the end of the sample
+                        for (int v = 0; v < 4; ++v)
+                            if ((bits[h] >> ((v >> 1) * 8 + 2 * c4 + (v & 1))) & 1u) {
+                                hi[v] += kUnderflow - val[h][v];
+                                lo[v] += fmaxf(-val[h][v] - (e + err[v]), 0.f);
+                            }
+                        bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 1);
+                        bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 2);
                     }
-                    if (__any_sync(0xFFFFFFFFu, (bits[0] | bits[1]) != 0u)) {
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const float e = fmaf(2.f * kPairErr, sm.norm[mt[k] * 16 + g + 8 * h], kUnderflow);
-#pragma unroll
-                            for (int v = 0; v < 4; ++v)
-                                if ((bits[h] >> ((v >> 1) * 8 + 2 * c4 + (v & 1))) & 1u) {
-                                    hi[v] += kUnderflow - val[h][v];
-                                    lo[v] += fmaxf(-val[h][v] - (e + err[v]), 0.f);
-                                }
-                            bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 1);
-                            bits[h] |= __shfl_xor_sync(0xFFFFFFFFu, bits[h], 2);
-                        }
-                        const uint32_t any = __reduce_or_sync(0xFFFFFFFFu, bits[0] | bits[1]);
-                        if (lane == 0) atomicOr(&sm.touched[mt[k] / (kSumBlock / 16)], any);
-                    }
-                    if (c4 < 2) sm.mask[mt[k] * 16 + g + 8 * c4] = (uint16_t)(c4 ? bits[1] : bits[0]);
+                    const uint32_t any = __reduce_or_sync(0xFFFFFFFFu, bits[0] | bits[1]);
+                    if (lane == 0) atomicOr(&sm.touched[i0 / kSumBlock], any);
                 }
+                if (c4 < 2) sm.mask[i0 + g + 8 * c4] = (uint16_t)(c4 ? bits[1] : bits[0]);
             }
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                if (v >= 2 && L <= 8) break;
+            for (int v = 0; v < 4; ++v) {                   // (most columns have no marked point in the warp's rows)
+                if (!__any_sync(0xFFFFFFFFu, hi[v] != 0.f)) continue;
 #pragma unroll
                 for (int o = 4; o <= 16; o <<= 1) {
                     lo[v] += __shfl_xor_sync(0xFFFFFFFFu, lo[v], o);
                     hi[v] += __shfl_xor_sync(0xFFFFFFFFu, hi[v], o);
                 }
                 const int t = (v >> 1) * 8 + 2 * c4 + (v & 1);
-                if (g == 0 && t < L) sm.warp_gain[warp][t] = make_float2(lo[v], hi[v]);
+                if (g == 0 && hi[v] != 0.f) {               // (the order of these sums is covered by the 1e-5 below)
+                    atomicAdd(&sm.own_gain[par][t][0], lo[v]);
+                    atomicAdd(&sm.own_gain[par][t][1], hi[v]);
+                }
             }
             __syncthreads();
-            for (int e = tid; e < L * n_blk; e += kStartThreads) {
-                const int l = e % L, to = e / L;
-                float2 s = sm.warp_gain[0][l];
-#pragma unroll
-                for (int w = 1; w < kStartWarps; ++w) { s.x += sm.warp_gain[w][l].x; s.y += sm.warp_gain[w][l].y; }
-                asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(in_block(shared_addr(&sm.gain[rank][l]), to)), "f"(s.x), "f"(s.y) : "memory");
-            }
-            cluster_barrier();
+            if (gain_to < n_blk) send2(gain_at + (uint32_t)(par * sizeof(sm.gain[0])), gain_bar, sm.own_gain[par][gain_of][0], sm.own_gain[par][gain_of][1]);
+            const float slack = (float)(1e-11 * sm.pre[nb - 1]);
+            const int mine = sm.draw[par][min(lane, L - 1)].pick;
+            await(kGains, (uint32_t)(c - 1) & 1u);
             // ---- 2. the winner ----
             {
                 // every warp for itself; 1e-5: rounding of the fp32 sums; 1e-11: of the fp64 sums that define the potentials
                 float gl = 0.f, gh = 0.f;
 #pragma unroll
-                for (int r = 0; r < kStartMaxCluster; ++r) {     // (zero past the cluster's blocks)
-                    const float2 v = sm.gain[r][min(lane, L - 1)];
+                for (int r = 0; r < kStartMaxCluster / 2; ++r) {     // half the blocks each half of the warp (zero past the cluster's)
+                    const float2 v = sm.gain[par][(lane & 16) / 2 + r][min(lane & 15, L - 1)];
                     gl += v.x;
                     gh += v.y;
                 }
-                const float slack = (float)(1e-11 * sm.pre[nb - 1]);
+                gl += __shfl_xor_sync(0xFFFFFFFFu, gl, 16);
+                gh += __shfl_xor_sync(0xFFFFFFFFu, gh, 16);
                 gl = lane < L ? gl * (1.f - 1e-5f) - slack : -CUDART_INF_F;
                 gh = gh * (1.f + 1e-5f);
                 const float top = warp_max(gl);
                 const unsigned at = __ballot_sync(0xFFFFFFFFu, gl == top);
                 best = at ? __ffs(at) - 1 : 0;
-                const int mine = sm.pick[c & 1][min(lane, L - 1)], its = __shfl_sync(0xFFFFFFFFu, mine, best);
+                const int its = __shfl_sync(0xFFFFFFFFu, mine, best);
                 const bool open = lane < L && !(gh < top) && mine != its;
                 if (__any_sync(0xFFFFFFFFu, open)) {
                     // all potentials in fp64: each block of the sums in order, then the blocks in order
-                    for (int v = warp; v < L * mb; v += kStartWarps) {
+                    for (int v = warp; warp < kStartTmp && v < L * mb; v += kStartTmp) {
                         const int l = v / mb, blk = v - l * mb, base = blk * kSumBlock;
                         double w = sm.raw[b0 + blk];
                         if ((sm.touched[blk] >> l) & 1u) {
@@ -682,95 +767,103 @@ km_start_kernel(KmeansParams p)
                 }
             }
         }
-        if (rank == 0 && tid == 0) p.chosen[q.cplane + c] = sm.pick[c & 1][best];
+        if (rank == 0 && tid == kStartThreads - 1) p.chosen[q.cplane + c] = sm.draw[par][best].pick;
         if (c + 1 == q.k) break;
-        // ---- 3. the winner's distances, a warp per touched block of the sums ----
+        // ---- 3. the winner's distances, a warp per block of the sums, eight lanes per point; the block's sum to all ----
         for (int blk = warp; blk < mb; blk += kStartWarps) {
-            if (!((sm.touched[blk] >> best) & 1u)) continue;
-            const int base = blk * kSumBlock, cnt = min(kSumBlock, n_rows - base);
-            unsigned who[4];
-            int m = 0;
+            double w = sm.raw[b0 + blk];
+            if ((sm.touched[blk] >> best) & 1u) {
+                const int base = blk * kSumBlock, cnt = min(kSumBlock, n_rows - base), eighth = lane & 7;
+                double y[2][8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                who[e] = __ballot_sync(0xFFFFFFFFu, (sm.mask[base + e * 32 + lane] >> best) & 1);
-                m += __popc(who[e]);
-            }
-            int first_at = kSumBlock;                       // first point that gets a smaller distance
-            auto lower = [&](int i, double d) {             // one lane
-                if (!(d < sm.closest[i]) && c > 0) return false;
-                sm.closest[i] = d;
-                // (a norm that fp32 does not hold: the product decides nothing)
-                sm.bar[i] = sm.norm[i] <= 1e37f ? sm.norm[i] * (1.f - kPairErr) - __double2float_ru(d) : -CUDART_INF_F;
-                return true;
-            };
-            if (m <= 3) {
-                double y[4];
-                row_quad<kHalf>(sm.trial, best, y);
+                for (int h = 0; h < 2; ++h) widen8<kHalf>(sm.trial[near_piece(best, eighth + 8 * h)], y[h]);
+                int m = 0;
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    for (unsigned w = who[e]; w; w &= w - 1) {
-                        const int i = base + e * 32 + __ffs(w) - 1;
-                        const double d = start_dist_warp<kHalf>(sm.rows, i, y, sm.tmp[warp]);
-                        const bool did = lane == 0 && lower(i, d);
-                        if (__any_sync(0xFFFFFFFFu, did)) first_at = min(first_at, i - base);
-                    }
-            } else {
-#pragma unroll 1
                 for (int e = 0; e < 4; ++e) {
+                    const bool marked = (sm.mask[base + e * 32 + lane] >> best) & 1;
+                    const unsigned who = __ballot_sync(0xFFFFFFFFu, marked);
+                    if (marked) sm.list[warp][m + __popc(who & ((1u << lane) - 1u))] = (uint8_t)(e * 32 + lane);
+                    m += __popc(who);
+                }
+                __syncwarp();
+                const int unit = sm.draw[par][best].unit;
+                int first_at = kSumBlock;                       // first point that gets a smaller distance
+#pragma unroll 2
+                for (int j0 = 0; j0 < m; j0 += 4) {
+                    const int j = j0 + (lane >> 3), at = sm.list[warp][min(j, m - 1)], i = base + at;
+                    double d = sum_parts(start_dist_part<kHalf>(sm.rows, i, eighth, y));
                     bool did = false;
-                    if ((sm.mask[base + e * 32 + lane] >> best) & 1)
-                        did = lower(base + e * 32 + lane, start_dist<kHalf>(sm.rows, base + e * 32 + lane, sm.trial, best));
-                    const unsigned any = __ballot_sync(0xFFFFFFFFu, did);
-                    if (any) first_at = min(first_at, e * 32 + __ffs(any) - 1);
+                    if (j < m && eighth == 0) {
+                        // Rows that are multiples of 2^u: their distance is one of 2^2u, and so is every partial sum. Below 2^(53 + 2u)
+                        // none of them is rounded, and the order of the sum does not matter; else the defining order.
+                        const int u = min(unit, (int)sm.unit[i]);
+                        const double exact_below = u > -128 ? __hiloint2double((1023 + 52 + 2 * u) << 20, 0) : 0.0;
+                        if (!(d < exact_below)) d = start_dist<kHalf>(sm.rows, i, sm.trial, best);
+                        if (d < sm.closest[i] || c == 0) {
+                            did = true;
+                            sm.closest[i] = d;
+                            // (a norm that fp32 does not hold: the product decides nothing; nothing is nearer than zero)
+                            sm.bar[i] = d == 0.0 ? CUDART_INF_F
+                                      : sm.norm[i] <= 1e37f ? sm.norm[i] * (1.f - kPairErr) - __double2float_ru(d) : -CUDART_INF_F;
+                        }
+                    }
+                    first_at = min(first_at, did ? at : kSumBlock);
+                }
+                first_at = __reduce_min_sync(0xFFFFFFFFu, first_at);
+                __syncwarp();
+                if (first_at < kSumBlock) {
+                    if (lane == 0) w = run_sums(sm.closest + base, sm.run + base, first_at, cnt, first_at > 0 ? sm.run[base + first_at - 1] : 0.0);
+                    w = __shfl_sync(0xFFFFFFFFu, w, 0);
                 }
             }
-            __syncwarp();
-            if (first_at == kSumBlock) continue;
-            double w = 0.0;
-            if (lane == 0) w = run_sums(sm.closest + base, sm.run + base, first_at, cnt, first_at > 0 ? sm.run[base + first_at - 1] : 0.0);
-            w = __shfl_sync(0xFFFFFFFFu, w, 0);
-            if (lane < n_blk)
-                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(in_block(shared_addr(&sm.raw[b0 + blk]), lane)), "d"(w) : "memory");
+            if (lane < n_blk) send_double(in_block(shared_addr(&sm.raw[b0 + blk]), lane), in_block(shared_addr(&sm.arrived[kSums]), lane), w);
         }
-        cluster_barrier();
-        // ---- 4. the blocks' running sums; the next trial points: a warp per draw, in the block that owns it ----
-        if (tid < kStartBlocks) sm.touched[tid] = 0u;
+        // ---- 4. the blocks' running sums; the next trial points, a warp per draw: the block that owns a drawn point sends
+        // its row to all ----
+        const int l = warp;
+        const uint32_t word = km_word(p, (uint32_t)l, kTagStart, q.stream, (uint32_t)(c + 1));
+        await(kSums, (uint32_t)par);
         if (tid == 0) run_sums(sm.raw, sm.pre, 0, nb, 0.0);
         __syncthreads();
-        const double total = sm.pre[nb - 1];
-        for (int l = warp; l < q.L; l += kStartWarps) {
-            const uint32_t w = km_word(p, (uint32_t)l, kTagStart, q.stream, (uint32_t)(c + 1));
-            const double target = __dmul_rn(((double)w + 0.5) * (1.0 / 4294967296.0), total);
+        if (tid < kStartBlocks) sm.touched[tid] = 0u;
+        if (tid >= 32 && tid < 32 + 2 * kStartTrials) sm.own_gain[par][0][tid - 32] = 0.f;      // (for the centre after the next)
+        if (l < q.L) {
+            const double target = __dmul_rn(((double)word + 0.5) * (1.0 / 4294967296.0), sm.pre[nb - 1]);
             int blk = nb;                                   // first block whose running sum exceeds the target
-            for (int o = 0; o < nb; o += 32) {
+#pragma unroll
+            for (int o = kStartSums - 32; o >= 0; o -= 32) {
                 const unsigned over = __ballot_sync(0xFFFFFFFFu, o + lane < nb && sm.pre[min(o + lane, nb - 1)] > target);
-                if (over) { blk = o + __ffs(over) - 1; break; }
+                if (over) blk = o + __ffs(over) - 1;
             }
             const bool none = blk == nb;                    // rounding left no point beyond the target: the last one
             if (none) blk = nb - 1;
-            if (blk < b0 || blk >= b0 + mb) continue;
-            const int base = (blk - b0) * kSumBlock, cnt = min(kSumBlock, n_rows - base);
-            int at = cnt - 1;
-            if (!none) {                                    // first point of the block with offset + running sum beyond it
+            if (blk >= b0 && blk < b0 + mb) {
+                const int base = (blk - b0) * kSumBlock, cnt = min(kSumBlock, n_rows - base), h = lane & 15;
                 const double before = blk > 0 ? sm.pre[blk - 1] : 0.0;
+                int at = cnt - 1;                           // first point of the block with offset + running sum beyond it
 #pragma unroll
-                for (int e = 3; e >= 0; --e) {
-                    const unsigned over = __ballot_sync(0xFFFFFFFFu, e * 32 + lane < cnt && __dadd_rn(before, sm.run[base + e * 32 + lane]) > target);
+                for (int e = kSumBlock / 32 - 1; e >= 0; --e) {
+                    const unsigned over = __ballot_sync(0xFFFFFFFFu, !none && e * 32 + lane < cnt && __dadd_rn(before, sm.run[base + e * 32 + lane]) > target);
                     if (over) at = e * 32 + __ffs(over) - 1;
                 }
-            }
-            const uint4 piece = sm.rows[near_piece(base + at, lane & 15)];
-            const uint32_t row_to = shared_addr(&sm.trial[near_piece(l, lane & 15)]);
-            for (int to = lane >> 4; to < n_blk; to += 2)
-                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(in_block(row_to, to)), "r"(piece.x), "r"(piece.y), "r"(piece.z),
-                             "r"(piece.w) : "memory");
-            if (lane < n_blk) {
-                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(in_block(shared_addr(&sm.trial_norm[l]), lane)), "f"(sm.norm[base + at]) : "memory");
-                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(in_block(shared_addr(&sm.pick[(c + 1) & 1][l]), lane)), "r"(row0 + base + at) : "memory");
+                const uint4 piece = sm.rows[near_piece(base + at, h)];
+                const uint32_t to = shared_addr(&sm.trial[near_piece(l, h)]), bar = shared_addr(&sm.arrived[kDraws]);
+#pragma unroll
+                for (int b = 0; b < kStartMaxCluster; b += 2)       // half a warp a block
+                    if (b + (lane >> 4) < n_blk) send4(in_block(to, b + (lane >> 4)), in_block(bar, b + (lane >> 4)), piece);
+                if (lane < n_blk)
+                    send4(in_block(shared_addr(&sm.draw[par ^ 1][l]), lane), in_block(bar, lane),
+                          make_uint4(__float_as_uint(sm.norm[base + at]), (uint32_t)(row0 + base + at), (uint32_t)(int)sm.unit[base + at], 0u));
             }
         }
-        cluster_barrier();
+        await(kDraws, (uint32_t)par);
+        __syncthreads();
     }
+    tc_fence_before();
+    cluster_barrier();                                      // (a block's shared memory stays while another may send to it)
+    tc_fence_after();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(kTmemCols));
+    if (tid == 0 && sm.failed) p.chosen[q.cplane] = -1;
 }
 
 // How many blocks share a pair's sample in km_start_kernel; 0: the sample does not fit, or the device has no room for
@@ -872,9 +965,11 @@ km_prepare_kernel(KmeansParams p)
     const int u = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0.0, 0, 0, 0, 0};
     if (u >= q.k) return;
-    const int row = p.perm[q.plane + p.chosen[q.cplane + u]];
+    const bool lost = p.chosen[q.cplane] < 0;               // the start gave up on a message (never expected): no centres
+    const int row = p.perm[q.plane + (lost ? 0 : p.chosen[q.cplane + u])];
     const uint2 w = reinterpret_cast<const uint2 *>(p.k_prompt + (q.plane + row) * kHeadDim)[lane];
-    const double v[4] = {(double)elem_lo<kHalf>(w.x), (double)elem_hi<kHalf>(w.x), (double)elem_lo<kHalf>(w.y), (double)elem_hi<kHalf>(w.y)};
+    double v[4] = {(double)elem_lo<kHalf>(w.x), (double)elem_hi<kHalf>(w.x), (double)elem_lo<kHalf>(w.y), (double)elem_hi<kHalf>(w.y)};
+    if (lost) v[0] = v[1] = v[2] = v[3] = CUDART_NAN;
     store_centre<kHalf>(p, q.cplane + u, v);
     if (lane == 0) p.count[q.cplane + u] = 0.0;
 }

@@ -132,13 +132,7 @@ __device__ __forceinline__ void near_close_block(NearSmem &sm)
 __device__ __forceinline__ void near_wait(NearSmem &sm, int buf, uint32_t parity)
 {
     if (*reinterpret_cast<volatile int *>(&sm.failed)) return;
-    for (int i = 0; i < (1 << 20); ++i) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}\n"
-                     : "=r"(done) : "r"(shared_addr(&sm.done[buf])), "r"(parity) : "memory");
-        if (done) return;
-    }
-    sm.failed = 1;
+    if (!tc_wait(shared_addr(&sm.done[buf]), parity)) sm.failed = 1;
 }
 
 // One point against 32 consecutive centres from `first` on: v their products with it, bias their constants.

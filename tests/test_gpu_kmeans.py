@@ -248,6 +248,19 @@ def test_fit_of_keys_whose_products_underflow(scale):
     _fit_keys_both(keys.astype(np.float32), "bf16", 40, batch_size=128, max_iter=2, patience=4, seed=5, reassignment_ratio=0.01)
 
 
+@pytest.mark.parametrize("elem,n,spread,tiny", [("bf16", 1000, 0, 0.0), ("bf16", 129, 14, 0.0), ("bf16", 1000, 14, 0.0), ("bf16", 900, 3, 1e-39),
+                                                ("fp16", 1000, 0, 0.0), ("fp16", 700, 9, 0.0), ("fp16", 900, 2, 1e-7)])
+def test_start_on_values_of_many_magnitudes(elem, n, spread, tiny):
+    """A distance whose terms are multiples of one power of two, of which it has fewer than 2^53, is summed in any order,
+    another in the defining one: keys of which all, some and hardly any distances are of the first kind, zeros
+    and subnormal values among them."""
+    rng = np.random.default_rng(29)
+    keys = rng.standard_normal((2, n, 128)) * 2.0 ** -rng.integers(0, spread + 1, size=(2, n, 128))
+    rows = rng.random((2, n)) < 0.5
+    keys[rows] = np.where(rng.random((int(rows.sum()), 128)) < 0.05, tiny * rng.integers(-3, 4, size=(int(rows.sum()), 128)), keys[rows])
+    _fit_keys_both(keys.astype(np.float32), elem, min(150, n // 2), batch_size=128, max_iter=1, patience=4, seed=4, reassignment_ratio=0.0)
+
+
 @pytest.mark.parametrize("n", [8103, 8104, 12288])
 def test_start_with_ten_and_eleven_trials_a_centre(n):
     """2 + floor(ln k) is 11 from k = 8104 on; samples of up to 12288 keys take the start in one kernel all the same."""
