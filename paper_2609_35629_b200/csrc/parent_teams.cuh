@@ -240,20 +240,19 @@ __device__ __forceinline__ void select_large(LargeSmem<kWarps, kRpt> &sm, int nC
     constexpr int kT = 32 * kWarps;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, c = lane & 3;
     // the mean, approximately (fp32 sums), then every row's norm and its distance to the mean
-    constexpr int kParts = kT >= kHeadDim ? kT / kHeadDim : 1;
-    for (int d = tid; d < kParts * kHeadDim; d += kT) {
-        const int dim = d & (kHeadDim - 1), part = d / kHeadDim;
-        float s0 = 0.f, s1 = 0.f;                             // chains of at most 128 additions
-#pragma unroll 4
-        for (int i = part; i < nC; i += 2 * kParts) {
-            const uint32_t w = sm.rows[i * kPitch + (dim >> 1)];
-            s0 += (dim & 1) ? elem_hi<kHalf>(w) : elem_lo<kHalf>(w);
-            if (i + kParts < nC) {
-                const uint32_t v = sm.rows[(i + kParts) * kPitch + (dim >> 1)];
-                s1 += (dim & 1) ? elem_hi<kHalf>(v) : elem_lo<kHalf>(v);
-            }
+    constexpr int kParts = kT / kWords;
+    static_assert(kParts >= 1 && kParts <= 4 && kParts * 128 >= LargeSmem<kWarps, kRpt>::kRows, "a word per thread; chains of at most 128 additions");
+    {
+        const int word = tid & (kWords - 1), part = tid / kWords;
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+        for (int i = part; i < nC; i += kParts) {
+            const uint32_t w = sm.rows[i * kPitch + word];
+            s0 += elem_lo<kHalf>(w);
+            s1 += elem_hi<kHalf>(w);
         }
-        sm.mu[part][dim] = s0 + s1;
+        sm.mu[part][2 * word] = s0;
+        sm.mu[part][2 * word + 1] = s1;
     }
     __syncthreads();
     for (int d = tid; d < kHeadDim; d += kT) {
