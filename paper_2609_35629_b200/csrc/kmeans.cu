@@ -803,8 +803,8 @@ km_start_kernel(KmeansParams p)
                             did = true;
                             sm.closest[i] = d;
                             // (a norm that fp32 does not hold: the product decides nothing; nothing is nearer than zero)
-                            sm.bar[i] = d == 0.0 ? CUDART_INF_F
-                                      : sm.norm[i] <= 1e37f ? sm.norm[i] * (1.f - kPairErr) - __double2float_ru(d) : -CUDART_INF_F;
+                            sm.bar[i] = !(sm.norm[i] <= 1e37f) ? -CUDART_INF_F
+                                      : d == 0.0 ? CUDART_INF_F : sm.norm[i] * (1.f - kPairErr) - __double2float_ru(d);
                         }
                     }
                     first_at = min(first_at, did ? at : kSumBlock);
