@@ -75,9 +75,9 @@ __device__ __forceinline__ ScoreCtx score_ctx(const ScoreParams &p)
     return c;
 }
 
-// Small grids: one warp per tile of 16 teams, keys straight into registers (the shortest path).
-template <int G, bool kHalf>
-__global__ void __launch_bounds__(kScoreThreads, 2)
+// Small grids: one warp per tile of 16 teams, keys straight into registers (the shortest path); kBlocks of them fit an SM.
+template <int G, bool kHalf, int kBlocks>
+__global__ void __launch_bounds__(kScoreThreads, kBlocks)
 score32_kernel(ScoreParams p)
 {
     step_wait();
@@ -329,9 +329,13 @@ template <int G, bool kHalf>
 cudaError_t launch_score32_g(const ScoreParams &p, int max_teams, cudaStream_t s)
 {
     const long long ctas1 = (long long)((max_teams + kScoreTeamsPerCta - 1) / kScoreTeamsPerCta) * p.n_pairs;
-    if (ctas1 < 2 * attend_grid_size()) {
-        dim3 grid((max_teams + kScoreTeamsPerCta - 1) / kScoreTeamsPerCta, p.n_pairs);
-        return launch_step(score32_kernel<G, kHalf>, grid, dim3(kScoreThreads), 0, s, p);
+    // A tile per warp as long as all of them are resident: with up to two blocks per SM at 78 registers, four at 64 (28 layers of one
+    // block per SM: 669.6 and 670.6 us). Walking two tiles a warp through the ring instead: 8 x 32K keys 91.0 against 90.1 us a step,
+    // 16 x 16K 105 against 102.9; more blocks than are resident: 4 x 128K the same, 32 ragged sequences 210.6 against 214.1.
+    if (ctas1 <= 4 * attend_grid_size()) {
+        const dim3 grid((max_teams + kScoreTeamsPerCta - 1) / kScoreTeamsPerCta, p.n_pairs);
+        return ctas1 < 2 * attend_grid_size() ? launch_step(score32_kernel<G, kHalf, 2>, grid, dim3(kScoreThreads), 0, s, p)
+                                              : launch_step(score32_kernel<G, kHalf, 4>, grid, dim3(kScoreThreads), 0, s, p);
     }
     static std::atomic<unsigned long long> done;
     cudaError_t e = ensure_dynamic_smem((const void *)score32_flat_kernel<G, kHalf>, kScoreRingBytes, done);

@@ -439,6 +439,14 @@ def test_decode_candidates_around_a_thread_each(n_seqs, K, gain):
     _check_with_queries(layer, synth.f32_to_bf16_bits(np.float32(gain) * synth.bf16_to_f32(bits)), K=K, step=3)
 
 
+@pytest.mark.parametrize("most", [128, 129, 257, 512, 513])
+def test_decode_at_the_edges_of_the_scorers_forms(most):
+    """A scoring block takes 128 teams of a pair: fewer than two blocks per SM, two to four, more."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count // 4          # sequences of four pairs: a block of each pair per SM
+    spec = synth.spec_small_gqa(n_seqs=n, prompt=tuple(most - 7 * (i % 4) for i in range(n)), parent_size=32, reps=32, suffix0=(1,) * n)
+    check_sparse_step(pu.GpuLayer(spec, synth.make_layer(spec)), 0, K=8, seqs=[0, n // 2, n - 1])
+
+
 @pytest.mark.parametrize("n_q,n_kv", [(32, 4), (8, 2), (6, 6), (3, 1)])
 def test_decode_other_group_sizes(n_q, n_kv):
     """GQA groups of 8, 4, 1 and 3 query heads per KV head (the tensor-core tile holds up to 8)."""
