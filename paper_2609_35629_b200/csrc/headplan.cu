@@ -31,7 +31,11 @@ static cudaError_t launch_headplan_t(const PlanInputs &in, cudaStream_t s)
     // they are slower (8192 teams: 715 against 592, 4 x 8192: 37.4 against 32.8)
     if (n_heads <= sms && in.y_stride > 2048) return launch_step(headplan_kernel<512, kHalf>, dim3(n_heads), dim3(512), 0, s, in);
     if (n_heads <= 4 * sms) return launch_step(headplan_kernel<256, kHalf>, dim3(n_heads), dim3(256), 0, s, in);
-    return launch_step(headplan_kernel<128, kHalf>, dim3(n_heads), dim3(128), 0, s, in);
+    // Seven blocks share an SM where that saves a wave of them, else six: 32 sequences of 28 heads, 896 for 888 places, at 4096 / 8192 tokens
+    // 82.6 -> 78.7 and 104.9 -> 102.1 us a step (lengths from 8K to 64K: 211.6, 212.1); 48 sequences, two waves in any case, take 78.0
+    // with six and 78.7 with seven. The shared memory asked for on top leaves room for six.
+    const bool seven = n_heads > 6 * sms && n_heads <= 7 * sms;
+    return launch_step(headplan_kernel<128, kHalf>, dim3(n_heads), dim3(128), seven ? 0 : 7168, s, in);
 }
 
 cudaError_t launch_headplan(const PlanInputs &in, cudaStream_t s)

@@ -28,13 +28,16 @@ namespace santapp {
 
 constexpr int kMaxHeadWarps = 32;        // blocks of up to 1024 threads
 constexpr int kCandCap = 512;           // candidates refined at a time
-constexpr int kListCap = 260;           // running top list: K + 1 <= 257 entries (+ pad); K <= 128 for K/V rows, <= 256 for shared-latent rows
+// Running top list: K + 1 entries (+ pad); K <= 128 for K/V rows, <= 256 for shared-latent rows. (A K/V block is 28 KB: seven fit an SM,
+// with 260 entries six.)
+template <int kDim> constexpr int kListCapOf = kDim > kHeadDim ? 260 : 132;
 constexpr int kDotLanes = 8;            // threads that share one candidate's dot product
 constexpr int kWindow = 255;            // histogram bins per pass of the bound
 
 // kDim: values per routing key (128 for K rows, 576 for shared-latent rows); a multiple of 64.
 template <int kDim>
 struct alignas(16) HeadSmemT {
+    static constexpr int kListCap = kListCapOf<kDim>;
     double q64[kDotLanes][kDim / kDotLanes + 2];   // query in fp64: [lane of a key's eight][its dims, + pad] (pad: conflict-free LDS.128)
     double cand_y[kCandCap + 2];        // dot products, then exact Y; read in pairs
     double cand_phi[kCandCap];          // log n_g, then phi_g
@@ -80,6 +83,7 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
 {
     static_assert(kDim % 64 == 0, "eight lanes share a key, each takes whole 16-byte pieces");
     constexpr bool kAllDot = kDim > 128;
+    constexpr int kListCap = kListCapOf<kDim>;
     constexpr int kHeadWarps = kT / 32, kDotWarps = kAllDot ? kHeadWarps : kHeadWarps / 2;
     constexpr int kSlice = kDim / kDotLanes;                          // dims per lane of a dot product
     constexpr int kPieces = kSlice / 8;                               // 16-byte pieces per lane
@@ -450,8 +454,8 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
             // ranks again on whole scores. (The upper halves of the doubles as keys, 1e-5 apart, tied in one head of
             // ten at 180 candidates.) Two barriers instead of seven and no lists: kernel at 32K tokens, K = 32, 7.3 -> 6.7 us;
             // 8192 teams, K = 31, 9.6 -> 8.9; 512 latent heads, K = 128, 37.1 -> 34.1.
-            uint32_t *keys = reinterpret_cast<uint32_t *>(sm.list_y[0]);  // (no list yet; room for kCandCap keys)
-            static_assert(2 * kListCap >= kCandCap, "the keys borrow a list");
+            uint32_t *keys = reinterpret_cast<uint32_t *>(sm.list_y);     // (no list yet; room for kCandCap keys)
+            static_assert(sizeof(sm.list_y) >= sizeof(uint32_t) * kCandCap, "the keys borrow the lists");
             double y = 0.0, phi = 0.0;
             uint32_t yh = 0u;                                             // padding: larger than no key
             if (tid < n_cand) {
