@@ -334,12 +334,14 @@ km_accept_kernel(KmeansParams p, int c)
 // block's distances and its running sums (128 terms in order, 11 cycles each), 1100 for the blocks' (96 terms), three
 // messages of 700. Messages are stores that count their bytes on an mbarrier of the block they go to; with cluster
 // barriers behind remote stores, three of 1900 cycles, all of a block's threads waiting for the slowest block's, and a
-// distance summed in order by one lane (1100 cycles a point), a centre took 8.2 us, now 6.6. Sixteen warps, so that three
-// tiles a warp and four warps a scheduler overlap operands, products and marks (eight warps: 6.9). The operands wait in tensor
+// distance summed in order by one lane (1100 cycles a point), a centre took 8.2 us, now 6.4. Twelve warps, four tiles each, so
+// that three warps a scheduler overlap operands, products and marks (eight warps: 6.9; sixteen, with which the cycles above were
+// counted: 6.6, a fit to 2048 centres 18.25 -> 17.75 ms, to 256 and 64 centres 5.32 -> 5.25 and 4.91 -> 4.86: a barrier and the
+// slowest warp of fewer). The operands wait in tensor
 // memory: read from shared memory they are as long on their way as the products take. (tcgen05 itself: sixteen
 // columns take as long as 128, 9 us a centre.) The two kernels per centre took 38 us, 24 of them fp64 distances of
 // every point to every trial.
-constexpr int kStartThreads = 512, kStartWarps = kStartThreads / 32;
+constexpr int kStartThreads = 384, kStartWarps = kStartThreads / 32;
 constexpr int kStartBlocks = 6;          // blocks of the sums per thread block: 768 rows of 256 bytes
 constexpr int kStartRows = kStartBlocks * kSumBlock;
 constexpr int kStartTmp = 4;             // warps that sum potentials
