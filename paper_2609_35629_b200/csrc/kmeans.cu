@@ -675,7 +675,9 @@ km_start_kernel(KmeansParams p)
                         val[h][v] = fmaf(-2.f, acc[v >> 1][2 * h + (v & 1)], bar + ny[v]);
                         if (!(val[h][v] > kUnderflow)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));
                     }
-                    if (!(bar < CUDART_INF_F)) bits[h] = 0u;         // a centre, or past the end of the sample
+                    // nothing of a centre or past the end of the sample; of a row that the products say nothing about every trial, but no
+                    // column that is none (minus and plus infinity above are not a number, which compares like a mark)
+                    bits[h] = bar < CUDART_INF_F ? bits[h] & ((1u << L) - 1u) : 0u;
                 }
                 if (__any_sync(0xFFFFFFFFu, (bits[0] | bits[1]) != 0u)) {
 #pragma unroll
@@ -704,7 +706,7 @@ km_start_kernel(KmeansParams p)
                     hi[v] += __shfl_xor_sync(0xFFFFFFFFu, hi[v], o);
                 }
                 const int t = (v >> 1) * 8 + 2 * c4 + (v & 1);
-                if (g == 0 && hi[v] != 0.f) {               // (the order of these sums is covered by the 1e-5 below)
+                if (g == 0 && t < L && hi[v] != 0.f) {      // (the order of these sums is covered by the 1e-5 below)
                     atomicAdd(&sm.own_gain[par][t][0], lo[v]);
                     atomicAdd(&sm.own_gain[par][t][1], hi[v]);
                 }
@@ -729,8 +731,8 @@ km_start_kernel(KmeansParams p)
                 gl = lane < L ? gl * (1.f - 1e-5f) - slack : -CUDART_INF_F;
                 gh = gh * (1.f + 1e-5f);
                 const float top = warp_max(gl);
-                const unsigned at = __ballot_sync(0xFFFFFFFFu, gl == top);
-                best = at ? __ffs(at) - 1 : 0;
+                const unsigned at = __ballot_sync(0xFFFFFFFFu, lane < L && gl == top);
+                best = at ? __ffs(at) - 1 : 0;              // (gains that do not compare leave the first trial)
                 const int its = __shfl_sync(0xFFFFFFFFu, mine, best);
                 const bool open = lane < L && !(gh < top) && mine != its;
                 if (__any_sync(0xFFFFFFFFu, open)) {

@@ -220,6 +220,19 @@ def test_fit_with_outlier_keys_beyond_the_range_of_the_bounds(elem, far):
     _fit_keys_both(keys, elem, 200, batch_size=256, max_iter=3, patience=4, seed=2, reassignment_ratio=0.0)
 
 
+@pytest.mark.parametrize("k,n", [(5, 900), (20, 900), (54, 900), (7, 2100), (54, 2100)])
+def test_start_with_few_trials_beside_rows_without_a_bound(k, n):
+    """Three to five trials a centre and four keys of different magnitudes whose squared norms fp32 does not hold: such a row is
+    marked for every trial and for no column of the products beyond them, and where all trials drew one of these
+    rows, which outweigh the rest, the centre is that row. 2100 keys are 17 blocks of the sums: a cluster of 16 has blocks without any."""
+    rng = np.random.default_rng(41)
+    keys = rng.standard_normal((2, n, 128)).astype(np.float32)
+    for j in range(2):
+        for row, far in zip(rng.choice(n, 4, replace=False), (2e18, 3e19, 5e20, -4e21)):
+            keys[j, row] *= far
+    _fit_keys_both(keys, "bf16", k, batch_size=700, max_iter=2, patience=4, seed=3, reassignment_ratio=0.0)
+
+
 def test_fits_that_stop_beside_their_own_sorting_blocks():
     """The stopping rule of a step is settled beside the ordering of the next minibatch, in other blocks of one launch.
     192 fits that stop at many different steps, every step enqueued: ten runs, each with the oracle's step counts
