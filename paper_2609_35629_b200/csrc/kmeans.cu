@@ -711,10 +711,12 @@ km_start_kernel(KmeansParams p)
                     atomicAdd(&sm.own_gain[par][t][1], hi[v]);
                 }
             }
-            __syncthreads();
-            if (gain_to < n_blk) send2(gain_at + (uint32_t)(par * sizeof(sm.gain[0])), gain_bar, sm.own_gain[par][gain_of][0], sm.own_gain[par][gain_of][1]);
+            // (read ahead of the barrier: behind it thread 0 writes these sums again once the messages are there, which wait for the warps that
+            // send some and not for the others)
             const float slack = (float)(1e-11 * sm.pre[nb - 1]);
             const int mine = sm.draw[par][min(lane, L - 1)].pick;
+            __syncthreads();
+            if (gain_to < n_blk) send2(gain_at + (uint32_t)(par * sizeof(sm.gain[0])), gain_bar, sm.own_gain[par][gain_of][0], sm.own_gain[par][gain_of][1]);
             await(kGains, (uint32_t)(c - 1) & 1u);
             // ---- 2. the winner ----
             {

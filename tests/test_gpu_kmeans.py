@@ -233,6 +233,19 @@ def test_start_with_few_trials_beside_rows_without_a_bound(k, n):
     _fit_keys_both(keys, "bf16", k, batch_size=700, max_iter=2, patience=4, seed=3, reassignment_ratio=0.0)
 
 
+@pytest.mark.parametrize("n", [129, 2100])
+def test_start_in_which_most_warps_send_nothing(n):
+    """Two and 17 blocks of the sums on clusters of 16: a thread block has sums on none to two of its warps and sends gains from
+    two or three; the others are held by barriers alone. Thirty runs with the oracle's centres."""
+    keys = np.random.default_rng(43).standard_normal((2, n, 128))
+    bits = synth.round_bits(keys.astype(np.float32))
+    geom, k = sp.Geometry(1, 2, 2, 128, 16, 4), sp.bf16_bits_to_cuda(bits)
+    want = np.stack([orc.minibatch_kmeans(synth.to_f64(bits[j], "bf16"), 100, batch=700, max_iter=1, patience=4, seed=12, stream=j)[0] for j in range(2)])
+    for _ in range(30):
+        centres, _ = sp.santapp_kmeans_fit(geom, [n], [100], k, batch_size=700, max_iter=1, patience=4, seed=12)
+        assert np.array_equal(centres.cpu().numpy(), want.astype(np.float32))
+
+
 def test_fits_that_stop_beside_their_own_sorting_blocks():
     """The stopping rule of a step is settled beside the ordering of the next minibatch, in other blocks of one launch.
     192 fits that stop at many different steps, every step enqueued: ten runs, each with the oracle's step counts
