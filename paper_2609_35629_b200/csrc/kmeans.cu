@@ -345,7 +345,10 @@ constexpr int kStartThreads = 384, kStartWarps = kStartThreads / 32;
 constexpr int kStartBlocks = 6;          // blocks of the sums per thread block: 768 rows of 256 bytes
 constexpr int kStartRows = kStartBlocks * kSumBlock;
 constexpr int kStartTmp = 4;             // warps that sum potentials
-enum { kGains, kSums, kDraws };          // the messages of a centre
+// The messages of a centre. A block that owns sums sends them when it has all gains, so nobody starts the next centre before; one that owns
+// none is not waited for, and the next centre's gains can reach it ahead of the last of this one's: gains have a barrier for each parity of
+// the centre (those of the centre after the next follow the gains that this block sends for the next).
+enum { kGains, kSums = 2, kDraws, kMessages };
 constexpr int kStartMaxCluster = 16, kStartSums = kStartBlocks * kStartMaxCluster;
 constexpr int kStartTrials = 11;         // 2 + floor(ln k) for every k with a sample of at most 16 * kStartRows: k <= 12288, ln k < 10
 static_assert(kStartTrials <= kStartWarps, "a warp per draw");
@@ -368,7 +371,7 @@ struct StartSmem {
     float2 gain[2][kStartMaxCluster][kStartTrials];         // (smallest, largest) gain of a trial over each block's points, by the centre's parity
     float own_gain[2][kStartTrials][2];                     // of this block, by the centre's parity
     alignas(16) StartDraw draw[2][kStartTrials];            // the trial points, by the centre's parity
-    uint64_t arrived[3];                                    // mbarriers: every block's gains, block sums, trial points
+    uint64_t arrived[kMessages];                            // mbarriers: every block's gains, block sums, trial points
     uint32_t touched[kStartBlocks];                         // trials with a marked point in the block
     uint32_t tmem;
     int failed;                                             // a wait ran out (never expected)
@@ -561,7 +564,7 @@ km_start_kernel(KmeansParams p)
     const int first = p.pick[(size_t)q.id * p.trials_max];
     if (tid == 0) {
         sm.failed = 0;
-        for (int t = 0; t < 3; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&sm.arrived[t])), "r"(1));
+        for (int t = 0; t < kMessages; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&sm.arrived[t])), "r"(1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -625,7 +628,7 @@ km_start_kernel(KmeansParams p)
         const int L = c == 0 ? 1 : q.L, par = c & 1;
         int best = 0;
         if (tid == 0) {                                     // the centre's messages to come (the ones before have all been waited for)
-            if (c > 0) expect_bytes(&sm.arrived[kGains], (uint32_t)(n_blk * L * sizeof(float2)));
+            if (c > 0) expect_bytes(&sm.arrived[kGains + par], (uint32_t)(n_blk * L * sizeof(float2)));
             if (c + 1 < q.k) {
                 expect_bytes(&sm.arrived[kSums], (uint32_t)(nb * sizeof(double)));
                 expect_bytes(&sm.arrived[kDraws], (uint32_t)(q.L * (kHeadDim * 2 + sizeof(StartDraw))));
@@ -716,8 +719,8 @@ km_start_kernel(KmeansParams p)
             const float slack = (float)(1e-11 * sm.pre[nb - 1]);
             const int mine = sm.draw[par][min(lane, L - 1)].pick;
             __syncthreads();
-            if (gain_to < n_blk) send2(gain_at + (uint32_t)(par * sizeof(sm.gain[0])), gain_bar, sm.own_gain[par][gain_of][0], sm.own_gain[par][gain_of][1]);
-            await(kGains, (uint32_t)(c - 1) & 1u);
+            if (gain_to < n_blk) send2(gain_at + (uint32_t)(par * sizeof(sm.gain[0])), gain_bar + (uint32_t)(par * sizeof(uint64_t)), sm.own_gain[par][gain_of][0], sm.own_gain[par][gain_of][1]);
+            await(kGains + par, (uint32_t)((c - 1) >> 1) & 1u);
             // ---- 2. the winner ----
             {
                 // every warp for itself; 1e-5: rounding of the fp32 sums; 1e-11: of the fp64 sums that define the potentials
