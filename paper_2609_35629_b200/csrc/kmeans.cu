@@ -617,7 +617,7 @@ km_start_kernel(KmeansParams p)
     cluster_barrier();                                      // every block of the cluster runs: its shared memory may be written
 
     auto await = [&](int what, uint32_t parity) {
-        if (!*reinterpret_cast<volatile int *>(&sm.failed) && !tc_wait(shared_addr(&sm.arrived[what]), parity)) sm.failed = 1;
+        if (!*reinterpret_cast<volatile int *>(&sm.failed) && !tc_wait<true>(shared_addr(&sm.arrived[what]), parity)) sm.failed = 1;
         __syncwarp();
     };
     // a thread sends one trial's gains to one block

@@ -210,8 +210,8 @@ def _fit_keys_both(keys, elem, k, **opts):
 
 @pytest.mark.parametrize("n", [100, 1153, 8200])
 def test_start_in_clusters_with_blocks_without_keys(n):
-    """1, 10 and 65 blocks of the sums: of 16 (n = 1153 in nine pairs: 8) thread blocks 15, 6 (3) and 3 own none and take part in the
-    messages all the same."""
+    """1, 10 and 65 blocks of the sums: 15 of 16, 3 of 8 (nine pairs) and 3 of 16 thread blocks own none and take part in the messages
+    all the same."""
     pairs = 9 if n == 1153 else 1
     keys = np.random.default_rng(47).standard_normal((pairs, n, 128))
     _fit_keys_both(keys.astype(np.float32), "bf16", 60, batch_size=4096, max_iter=1, patience=1, seed=14, reassignment_ratio=0.0)
