@@ -243,7 +243,9 @@ int32_t santapp_kmeans_parent_count(int32_t prompt_len, int32_t parent_size);
  *   k_prompt         device [n_kv_heads][rows_total][d], token order, in
  *   centres          device fp32 [n_kv_heads][sum_b k_b][d], out (the fp64 centres rounded to nearest);
  *                    the layout santapp_assign_parents takes
- *   steps_run        device int32 [n_kv_heads][n_seqs] or NULL, out: minibatch steps each fit ran
+ *   steps_run        device int32 [n_kv_heads][n_seqs] or NULL, out: minibatch steps each fit ran; -1: its start
+ *                    gave up on a message between thread blocks after about a second (never expected), its centres are
+ *                    not numbers
  *   workspace        device, >= santapp_kmeans_fit_workspace_bytes(...)
  * batch_size > 4096, or an initialisation sample above 28544 keys (more than 9514 centres in a
  * sequence): SANTAPP_ERR_UNSUPPORTED. The call enqueues a few kernels per centre and per

@@ -318,7 +318,8 @@ def santapp_kmeans_fit(geom: Geometry, prompt_len, n_centres, k_prompt: torch.Te
                        max_iter: int = 100, patience: int = 10, reassignment_ratio: float = 0.01, seed: int = 0,
                        stream_base: int = 0, stream=None, no_host_poll: bool = False):
     """Minibatch k-means fit per (sequence, KV head); the defaults are the paper's settings.
-    Returns (centres fp32 [n_kv_heads, sum(n_centres), d], steps int32 [n_kv_heads, n_seqs])."""
+    Returns (centres fp32 [n_kv_heads, sum(n_centres), d], steps int32 [n_kv_heads, n_seqs]; -1: the
+    fit's start gave up, see santapp.h)."""
     L = load_library()
     o = CKmeansOpts(batch_size, max_iter, patience, 1 if no_host_poll else 0, reassignment_ratio, seed, stream_base, 0)
     n, c = _i32_array(prompt_len), _i32_array(n_centres)

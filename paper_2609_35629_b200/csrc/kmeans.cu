@@ -348,7 +348,8 @@ constexpr int kStartTmp = 4;             // warps that sum potentials
 // The messages of a centre. A block that owns sums sends them when it has all gains, so nobody starts the next centre before; one that owns
 // none is not waited for, and the next centre's gains can reach it ahead of the last of this one's: gains have a barrier for each parity of
 // the centre (those of the centre after the next follow the gains that this block sends for the next).
-enum { kGains, kSums = 2, kDraws, kMessages };
+// Potentials lie in global memory; kPotentials counts the warps of the cluster that have written theirs.
+enum { kGains, kSums = 2, kDraws, kPotentials, kMessages };
 constexpr int kStartMaxCluster = 16, kStartSums = kStartBlocks * kStartMaxCluster;
 constexpr int kStartTrials = 11;         // 2 + floor(ln k) for every k with a sample of at most 16 * kStartRows: k <= 12288, ln k < 10
 static_assert(kStartTrials <= kStartWarps, "a warp per draw");
@@ -371,7 +372,7 @@ struct StartSmem {
     float2 gain[2][kStartMaxCluster][kStartTrials];         // (smallest, largest) gain of a trial over each block's points, by the centre's parity
     float own_gain[2][kStartTrials][2];                     // of this block, by the centre's parity
     alignas(16) StartDraw draw[2][kStartTrials];            // the trial points, by the centre's parity
-    uint64_t arrived[kMessages];                            // mbarriers: every block's gains, block sums, trial points
+    uint64_t arrived[kMessages];                            // mbarriers: every block's gains, block sums, trial points, potentials
     uint32_t touched[kStartBlocks];                         // trials with a marked point in the block
     uint32_t tmem;
     int failed;                                             // a wait ran out (never expected)
@@ -421,6 +422,11 @@ __device__ __forceinline__ void send4(uint32_t to, uint32_t bar, uint4 v)
 {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                  ::"r"(to), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
+// Arrival at a barrier of another block of the cluster, behind what the warp's lanes have written.
+__device__ __forceinline__ void arrive_at(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void expect_bytes(uint64_t *bar, uint32_t bytes)
 {
@@ -564,7 +570,8 @@ km_start_kernel(KmeansParams p)
     const int first = p.pick[(size_t)q.id * p.trials_max];
     if (tid == 0) {
         sm.failed = 0;
-        for (int t = 0; t < kMessages; ++t) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&sm.arrived[t])), "r"(1));
+        for (int t = 0; t < kMessages; ++t)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&sm.arrived[t])), "r"(t == kPotentials ? n_blk * kStartTmp : 1));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -616,6 +623,8 @@ km_start_kernel(KmeansParams p)
     if (tid < 4 * kStartTrials) sm.own_gain[0][0][tid] = 0.f;
     cluster_barrier();                                      // every block of the cluster runs: its shared memory may be written
 
+    // Where a wait runs out the block's later ones return at once, and the block leaves the loop with the centre; what its warps decide
+    // until then may differ, so between here and there stands no wait without a limit but the block's own barriers.
     auto await = [&](int what, uint32_t parity) {
         if (!*reinterpret_cast<volatile int *>(&sm.failed) && !tc_wait<true>(shared_addr(&sm.arrived[what]), parity)) sm.failed = 1;
         __syncwarp();
@@ -624,6 +633,7 @@ km_start_kernel(KmeansParams p)
     const int gain_of = tid % q.L, gain_to = tid / q.L;
     const uint32_t gain_at = in_block(shared_addr(&sm.gain[0][rank][gain_of]), min(gain_to, n_blk - 1));
     const uint32_t gain_bar = in_block(shared_addr(&sm.arrived[kGains]), min(gain_to, n_blk - 1));
+    uint32_t summed = 0u;                                   // centres whose potentials were summed
     for (int c = 0; c < q.k; ++c) {
         const int L = c == 0 ? 1 : q.L, par = c & 1;
         int best = 0;
@@ -762,7 +772,9 @@ km_start_kernel(KmeansParams p)
                         }
                         if (lane == 0) part[(size_t)l * n_part + b0 + blk] = w;
                     }
-                    cluster_barrier();                      // (the same decision in every warp of the cluster)
+                    __syncwarp();
+                    if (warp < kStartTmp && lane < n_blk) arrive_at(in_block(shared_addr(&sm.arrived[kPotentials]), lane));
+                    await(kPotentials, summed++ & 1u);      // (the same decision in every warp of the cluster)
                     double pot = 0.0;
                     if (lane < L)
 #pragma unroll 8
@@ -866,11 +878,13 @@ km_start_kernel(KmeansParams p)
             }
         }
         await(kDraws, (uint32_t)par);
-        __syncthreads();
+        if (__syncthreads_or(sm.failed)) break;
     }
     tc_fence_before();
     cluster_barrier();                                      // (a block's shared memory stays while another may send to it)
     tc_fence_after();
+    if (sm.failed)                                          // messages that were not waited for: they take a microsecond
+        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem), "r"(kTmemCols));
     if (tid == 0 && sm.failed) p.chosen[q.cplane] = -1;
 }
@@ -972,9 +986,9 @@ km_prepare_kernel(KmeansParams p)
     step_wait();
     const Pair q = pair_of(p, blockIdx.y / p.n_kv, blockIdx.y % p.n_kv);
     const int u = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0.0, 0, 0, 0, 0};
+    const bool lost = p.chosen[q.cplane] < 0;               // the start gave up on a message (never expected): no centres, no steps
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.state[q.id] = KmeansState{0.0, 0.0, 0.0, 0, lost ? -1 : 0, lost ? 1 : 0, 0};
     if (u >= q.k) return;
-    const bool lost = p.chosen[q.cplane] < 0;               // the start gave up on a message (never expected): no centres
     const int row = p.perm[q.plane + (lost ? 0 : p.chosen[q.cplane + u])];
     const uint2 w = reinterpret_cast<const uint2 *>(p.k_prompt + (q.plane + row) * kHeadDim)[lane];
     double v[4] = {(double)elem_lo<kHalf>(w.x), (double)elem_hi<kHalf>(w.x), (double)elem_lo<kHalf>(w.y), (double)elem_hi<kHalf>(w.y)};
