@@ -340,11 +340,12 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
             constexpr int kPerPass = kDotWarps * 32 / kDotLanes;
             if constexpr (kPieces > 2) {
                 // two candidates per thread group, three pieces of each on their way: a query value read from shared memory, which
-                // takes as long as four products of it, serves both. Where only one is left for every group, all pieces of it
-                // at once, one round trip (72 heads of up to 2047 rows, K = 32: 30.5 us a step with two always, 30.0 so).
+                // takes as long as four products of it, serves both. Every warp for itself: where a warp's groups have only one left, all
+                // pieces of it at once, one round trip, and a warp without any has nothing to do. Kernel at 32 x 8192 rows, K = 128, and
+                // 128 x 512 rows, K = 8: 29.6 and 27.2 us with one always, 24.2 and 29.1 with all warps in every pass, 23.9 and 24.2 so.
                 auto products = [&](auto two, int c0) {
                     constexpr int kKeys = decltype(two)::value ? 2 : 1, kDepth = kKeys > 1 ? 3 : kPieces;
-                    const int cand = c0 + (tid >> 3);
+                    const int cand = c0 + (lane >> 3);
                     const uint4 *key[kKeys];
 #pragma unroll
                     for (int u = 0; u < kKeys; ++u)
@@ -385,9 +386,10 @@ __device__ __forceinline__ void select_head(const PlanInputs &in, int hq, HeadSm
                         if (cand + u * kPerPass < n_cand && sub == 0) sm.cand_y[cand + u * kPerPass] = y;
                     }
                 };
-                int c0 = 0;
-                for (; c0 + kPerPass < n_cand; c0 += 2 * kPerPass) products(std::true_type(), c0);
-                if (c0 < n_cand) products(std::false_type(), c0);
+                for (int c0 = 4 * warp; c0 < n_cand; c0 += 2 * kPerPass) {
+                    if (c0 + kPerPass < n_cand) products(std::true_type(), c0);
+                    else products(std::false_type(), c0);
+                }
             } else {
                 // a few candidates per thread group at a time: all their key pieces are requested before
                 // the first product, so a chunk costs one memory round trip

@@ -240,6 +240,16 @@ def test_step_attention_with_one_and_two_blocks_per_sm(n, lo, hi):
     check_dense(layer, 1, seqs=seqs)
 
 
+@pytest.mark.parametrize("n_seqs", [2, 20])
+@pytest.mark.parametrize("K", [1, 2, 4, 8, 13, 16, 24, 40])
+def test_step_sampler_with_none_one_or_two_candidates_left_for_a_warp(n_seqs, K):
+    """Blocks of sixteen and of eight warps, four candidates a warp and pass: of 32 and 320 heads with some ten to
+    hundred candidates, the last pass of a head leaves its warps two, one or none each."""
+    layer = LatentLayer(synth.LatentSpec("few", [512 + 48 * i for i in range(n_seqs)], n_sample=K))
+    for step in range(3):
+        check_step(layer, step, seed=K + step, seqs=[0, n_seqs - 1])
+
+
 def test_two_hundred_steps_of_the_sampler():
     """Many draws on one layer (a different seed every step, K = 96 of 512 and 375 teams): now and
     then two candidates' scores agree in the upper half of their integer keys, which sends a head
