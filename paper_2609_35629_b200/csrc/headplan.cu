@@ -8,7 +8,7 @@ namespace {
 
 // Few heads: 512 threads each, so that every per-thread loop is short (the kernel is a chain of
 // dependent steps, not a throughput problem); more heads: 256 threads and four resident blocks per
-// SM, then 128 threads and eight.
+// SM, then 128 threads and six or seven.
 template <int kHeadThreads, bool kHalf>
 __global__ void __launch_bounds__(kHeadThreads, kHeadThreads >= 512 ? 1 : 1024 / kHeadThreads)
 headplan_kernel(PlanInputs in)
@@ -31,10 +31,12 @@ static cudaError_t launch_headplan_t(const PlanInputs &in, cudaStream_t s)
     // they are slower (8192 teams: 715 against 592, 4 x 8192: 37.4 against 32.8)
     if (n_heads <= sms && in.y_stride > 2048) return launch_step(headplan_kernel<512, kHalf>, dim3(n_heads), dim3(512), 0, s, in);
     if (n_heads <= 4 * sms) return launch_step(headplan_kernel<256, kHalf>, dim3(n_heads), dim3(256), 0, s, in);
-    // Seven blocks share an SM where that saves a wave of them, else six: 32 sequences of 28 heads, 896 for 888 places, at 4096 / 8192 tokens
-    // 82.6 -> 78.7 and 104.9 -> 102.1 us a step (lengths from 8K to 64K: 211.6, 212.1); 48 sequences, two waves in any case, take 78.0
-    // with six and 78.7 with seven. The shared memory asked for on top leaves room for six.
-    const bool seven = n_heads > 6 * sms && n_heads <= 7 * sms;
+    // Seven blocks share an SM where that saves a wave of them, else six (the shared memory asked for on top leaves room for six): kernel at
+    // 32 / 64 / 96 sequences of 28 heads and 2048 tokens, 896, 1792 and 2688 for 888 places with six: 12.8 -> 9.6, 19.9 -> 17.1 and 26.1 -> 23.3 us,
+    // lengths from 500 to 16000 13.4 -> 10.1, 19.9 -> 17.1, 26.3 -> 23.6; where both need as many waves seven are slower by up to a
+    // hundredth of the step (48 sequences).
+    auto waves = [&](int per_sm) { return (n_heads + per_sm * sms - 1) / (per_sm * sms); };
+    const bool seven = waves(7) < waves(6);
     return launch_step(headplan_kernel<128, kHalf>, dim3(n_heads), dim3(128), seven ? 0 : 7168, s, in);
 }
 

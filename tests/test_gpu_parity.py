@@ -427,6 +427,16 @@ def test_decode_many_short_sequences():
     check_dense_step(layer, 0)
 
 
+@pytest.mark.parametrize("per_sm", [6, 7, 12, 14])
+@pytest.mark.parametrize("beyond", [0, 1])
+def test_decode_around_six_and_seven_heads_per_sm_and_wave(per_sm, beyond):
+    """The sampler's smallest blocks share an SM by six or seven: the most sequences whose heads are no more than a wave or two of
+    either, and one sequence more."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count // 28 + beyond
+    spec = synth.spec_small_gqa(n_seqs=n, prompt=tuple(300 + 16 * (i % 3) for i in range(n)), parent_size=32, reps=8, suffix0=(1,) * n)
+    check_sparse_step(pu.GpuLayer(spec, synth.make_layer(spec)), 0, K=8, seqs=[0, n // 2, n - 1])
+
+
 @pytest.mark.parametrize("n_seqs,K", [(2, 100), (2, 128), (12, 128), (24, 60), (24, 100), (24, 127), (24, 128)])
 @pytest.mark.parametrize("gain", [1.0, 16.0])
 def test_decode_candidates_around_a_thread_each(n_seqs, K, gain):
