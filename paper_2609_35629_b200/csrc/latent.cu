@@ -66,11 +66,10 @@ struct LatentBuildParams {
 
 // A warp per parent (at most 32 rows), everything in one kernel: the parent's rows keep their range of the packed
 // order, so its owners give its row offsets and packed rows at once. Rows go through shared memory (asynchronous
-// copies, 18 KB of 16 rows on their way per warp, eleven warps per SM); distances over the latent columns and the
+// copies, 18 KB of 16 rows on their way per warp, ten or eleven warps per SM); distances over the latent columns and the
 // selection: select_rows.cuh. Bound by memory: 1152 bytes in and 1152 * (1 + R / P) out per row. The fp64
 // version in three kernels (block per parent, scan, pack) took 1309 us for 32 sequences of 8192.
 constexpr int kLbPitch = kRowDim / 2 + 4;                   // words per staged row: ldmatrix without bank conflicts
-constexpr int kLbWarps = 1;                                 // (of two, ten instead of eleven warps share an SM: 127 against 122 us)
 template <int kRows>
 struct LatentBuildSmem {
     __align__(16) uint32_t rows[kRows * kLbPitch];
@@ -78,7 +77,7 @@ struct LatentBuildSmem {
     int rep_of[kMaxP];
 };
 
-template <int kRows>
+template <int kRows, int kLbWarps>
 __global__ void __launch_bounds__(kLbWarps * 32)
 latent_build_kernel(LatentBuildParams p)
 {
@@ -132,15 +131,25 @@ latent_build_kernel(LatentBuildParams p)
     if (lane == 0) atomicMax(reinterpret_cast<uint32_t *>(p.rep_abs_max + b), m << 16);
 }
 
-template <int kRows>
-cudaError_t launch_latent_build(const LatentBuildParams &p, cudaStream_t s)
+template <int kRows, int kLbWarps>
+cudaError_t launch_latent_build_t(const LatentBuildParams &p, cudaStream_t s)
 {
     static std::atomic<unsigned long long> done;
     const int smem = (int)sizeof(LatentBuildSmem<kRows>) * kLbWarps;
-    const cudaError_t err = ensure_dynamic_smem((const void *)latent_build_kernel<kRows>, smem, done);
+    const cudaError_t err = ensure_dynamic_smem((const void *)latent_build_kernel<kRows, kLbWarps>, smem, done);
     if (err != cudaSuccess) return err;
-    return launch_step(latent_build_kernel<kRows>, dim3((p.max_parents_per_seq + kLbWarps - 1) / kLbWarps, p.lv.n_seqs),
+    return launch_step(latent_build_kernel<kRows, kLbWarps>, dim3((p.max_parents_per_seq + kLbWarps - 1) / kLbWarps, p.lv.n_seqs),
                        dim3(kLbWarps * 32), smem, s, p);
+}
+// One warp a block: eleven share an SM, of blocks of two ten warps do, and what one leaves the next takes at once (32 x 8192 rows, P = 16:
+// 137 -> 131 us; P = 32, where six warps share an SM in either case, 224 -> 186). Blocks of two are ahead by 3 to 6 % while the parents, of at most
+// 16 rows, are few enough for four rounds of the SMs and a block of one would not save the busiest SM a parent: 9 x 2047 rows 38.2 -> 36.5 us, 4 x 8192
+// 33.9 -> 31.3, 16 x 2048 33.9 -> 31.3; at 1 x 16384, seven parents against eight, one warp takes 23.9 and two take 27.5.
+cudaError_t launch_latent_build(const LatentBuildParams &p, cudaStream_t s)
+{
+    if (p.parent_size > 16) return launch_latent_build_t<kMaxP, 1>(p, s);
+    const long long sms = attend_grid_size(), per_sm = ((long long)p.max_parents_per_seq * p.lv.n_seqs + sms - 1) / sms;
+    return per_sm % 2 == 0 && per_sm <= 4 * 11 ? launch_latent_build_t<16, 2>(p, s) : launch_latent_build_t<16, 1>(p, s);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1227,7 +1236,7 @@ int santapp_latent_build_teams(const santapp_latent_geom *geom, const int32_t *p
     p.row_token = teams->row_token;
     p.rep_abs_max = teams->rep_abs_max;
     p.max_parents_per_seq = max_parents;
-    err = p.parent_size <= 16 ? launch_latent_build<16>(p, s) : launch_latent_build<kMaxP>(p, s);
+    err = launch_latent_build(p, s);
     if (err != cudaSuccess) return note_cuda_failure(err, "latent build launch");
     return SANTAPP_OK;
 }

@@ -138,6 +138,14 @@ def test_records_other_parent_shapes():
         check_records(LatentLayer(synth.LatentSpec(f"p{P}r{R}", [333, 64], parent_size=P, reps_per_parent=R, n_sample=4)))
 
 
+@pytest.mark.parametrize("per_sm,beyond", [(1, 0), (1, 1), (2, 1), (44, 0), (44, 1)])
+def test_records_by_blocks_of_one_and_two_parents(per_sm, beyond):
+    """An even number of parents per SM goes in blocks of two up to 44 per SM; the last parent is short, and alone in its block where the
+    number of parents is odd."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + beyond
+    check_records(LatentLayer(synth.LatentSpec("blocks", [16 * n - 5], n_sample=4)))
+
+
 def test_records_identical_rows_tie_rules():
     spec = synth.LatentSpec("ties", [200, 45], n_sample=4)
     data = synth.make_latent_layer(spec)
