@@ -363,9 +363,12 @@ struct LatentPlanSmem {
     int scan[40];
 };
 
-// Grid (sequences, parts): every block finds the sequence's union for itself (its tables are a few KB of shared
-// memory) and writes its share of the segments. What a sequence has to write, 64 bytes of bias a segment and 8 a row,
-// is what the kernel takes its time for, and a batch has fewer sequences than the device has SMs.
+// Grid (sequences, parts): every block reads the sequence's samples (up to 64 KB, L2 hits) and finds its union for itself, in
+// 64 KB of shared memory of its own, and writes its share of the segments. What a sequence has to write, 64 bytes of
+// bias a segment and 8 a row, is what the kernel takes its time for, and a batch has fewer sequences than the device has SMs:
+// 32 x 8192 rows 10.4 -> 6.6 us in four parts (K = 128), 5.4 -> 4.7 (K = 16); 1 x 32768, K = 256, 20.0 -> 7.7 in eight. With
+// 128 samples (K = 8) there is little to share: 4.8 -> 4.6 in four parts, 4.4 -> 4.5 in eight, 4.6 -> 5.0 in two (one part for those:
+// the same within 0.1 us).
 __global__ void __launch_bounds__(kLpThreads)
 latent_plan_kernel(LatentPlanParams p)
 {

@@ -302,6 +302,22 @@ def test_start_with_ten_and_eleven_trials_a_centre(n):
     test_fit_with_a_centre_per_key_returns_the_keys(n)
 
 
+def test_start_with_eleven_trials_rows_without_a_bound_and_blocks_without_keys():
+    """k = N = 8200: eleven trials, 65 blocks of the sums on a cluster of 16, three of whose blocks own none, and five keys
+    whose squared norms fp32 does not hold. All keys differ, so every one becomes a centre."""
+    n = 8200
+    bits = (np.arange(n)[:, None] >> np.arange(15)) & 1
+    rows = np.zeros((1, n, 128), dtype=np.float32)
+    rows[0, :, :15] = 3.0 * bits - 1.0
+    rows[0, [7, 1000, 4099, 8063, 8199]] *= np.float32([[2.0 ** 61], [2.0 ** 64], [-2.0 ** 66], [2.0 ** 70], [-2.0 ** 75]])
+    geom = sp.Geometry(1, 1, 1, 128, 16, 4)
+    k = torch.from_numpy(rows).cuda().to(torch.bfloat16)
+    centres, steps = sp.santapp_kmeans_fit(geom, [n], [n], k, batch_size=256, reassignment_ratio=0.0, patience=3)
+    torch.cuda.synchronize()
+    assert int(steps[0, 0]) == 4
+    assert np.array_equal(np.unique(centres[0].cpu().numpy(), axis=0), np.unique(rows[0], axis=0))
+
+
 @pytest.mark.parametrize("batch,k", [(1, 2), (63, 7), (64, 8), (65, 9), (128, 16), (129, 16), (129, 17)])
 def test_steps_at_the_edges_of_their_blocks_and_of_the_update_rule(batch, k):
     """64 points a block of the resolving kernel; fewer or more than eight points a centre in the update."""

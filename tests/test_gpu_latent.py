@@ -258,6 +258,15 @@ def test_step_sampler_with_none_one_or_two_candidates_left_for_a_warp(n_seqs, K)
         check_step(layer, step, seed=K + step, seqs=[0, n_seqs - 1])
 
 
+@pytest.mark.parametrize("H,K,n_seqs", [(1, 1, 1), (1, 3, 1), (2, 2, 3), (16, 1, 1), (3, 5, 19), (1, 1, 37), (2, 3, 75)])
+def test_step_with_fewer_segments_than_parts_of_the_plan(H, K, n_seqs):
+    """A sequence's plan is written by one to eight blocks (by the number of sequences): one segment, a few, and more than the parts."""
+    layer = LatentLayer(synth.LatentSpec("parts", [200 + 31 * (i % 4) for i in range(n_seqs)], n_heads=H, n_sample=K, suffix_cap=3,
+                                         suffix_len0=[i % 4 for i in range(n_seqs)], suffix_growth=0))
+    for step in range(3):
+        check_step(layer, step, seqs=sorted({0, n_seqs // 2, n_seqs - 1}))
+
+
 def test_two_hundred_steps_of_the_sampler():
     """Many draws on one layer (a different seed every step, K = 96 of 512 and 375 teams): now and
     then two candidates' scores agree in the upper half of their integer keys, which sends a head
