@@ -550,7 +550,7 @@ km_start_kernel(KmeansParams p)
     StartSmem &sm = *reinterpret_cast<StartSmem *>(start_smem);
     constexpr float kPairErr = 0.5f * kDistErr;             // times the sum of the two squared norms, plus kUnderflow
     // The rows as mma.sync's first operands (a word per lane, tile of 16 rows, step of 16 values: 32 columns a tile) in tensor memory,
-    // a warp's tiles m = warp, warp + 16, ... behind one another, four warps to a quarter of the lanes.
+    // a warp's tiles m = warp, warp + kStartWarps, ... behind one another, three warps to a quarter of the lanes.
     constexpr int kTiles = kStartRows / 16 / kStartWarps, kTmemCols = 512;
     static_assert(kStartWarps / 4 * kTiles * 32 <= kTmemCols, "operands in tensor memory");
     const int n_blk = (int)cluster_size(), rank = (int)cluster_rank();
@@ -634,6 +634,7 @@ km_start_kernel(KmeansParams p)
     const uint32_t gain_at = in_block(shared_addr(&sm.gain[0][rank][gain_of]), min(gain_to, n_blk - 1));
     const uint32_t gain_bar = in_block(shared_addr(&sm.arrived[kGains]), min(gain_to, n_blk - 1));
     uint32_t summed = 0u;                                   // centres whose potentials were summed
+    float slack = 0.f;                                      // rounding of the sums that define the potentials
     for (int c = 0; c < q.k; ++c) {
         const int L = c == 0 ? 1 : q.L, par = c & 1;
         int best = 0;
@@ -686,11 +687,11 @@ km_start_kernel(KmeansParams p)
 #pragma unroll
                     for (int v = 0; v < 4; ++v) {
                         val[h][v] = fmaf(-2.f, acc[v >> 1][2 * h + (v & 1)], bar + ny[v]);
-                        if (!(val[h][v] > kUnderflow)) bits[h] |= 1u << ((v >> 1) * 8 + 2 * c4 + (v & 1));
+                        // (a column that is no trial beside a row without a bound: plus and minus infinity, not a number)
+                        const int t = (v >> 1) * 8 + 2 * c4 + (v & 1);
+                        if (!(val[h][v] > kUnderflow) && t < L) bits[h] |= 1u << t;
                     }
-                    // nothing of a centre or past the end of the sample; of a row that the products say nothing about every trial, but no
-                    // column that is none (minus and plus infinity above are not a number, which compares like a mark)
-                    bits[h] = bar < CUDART_INF_F ? bits[h] & ((1u << L) - 1u) : 0u;
+                    if (!(bar < CUDART_INF_F)) bits[h] = 0u;         // a centre, or past the end of the sample
                 }
                 if (__any_sync(0xFFFFFFFFu, (bits[0] | bits[1]) != 0u)) {
 #pragma unroll
@@ -724,12 +725,9 @@ km_start_kernel(KmeansParams p)
                     atomicAdd(&sm.own_gain[par][t][1], hi[v]);
                 }
             }
-            // (read ahead of the barrier: behind it thread 0 writes these sums again once the messages are there, which wait for the warps that
-            // send some and not for the others)
-            const float slack = (float)(1e-11 * sm.pre[nb - 1]);
-            const int mine = sm.draw[par][min(lane, L - 1)].pick;
             __syncthreads();
             if (gain_to < n_blk) send2(gain_at + (uint32_t)(par * sizeof(sm.gain[0])), gain_bar + (uint32_t)(par * sizeof(uint64_t)), sm.own_gain[par][gain_of][0], sm.own_gain[par][gain_of][1]);
+            const int mine = sm.draw[par][min(lane, L - 1)].pick;
             await(kGains + par, (uint32_t)((c - 1) >> 1) & 1u);
             // ---- 2. the winner ----
             {
@@ -877,6 +875,9 @@ km_start_kernel(KmeansParams p)
                           make_uint4(__float_as_uint(sm.norm[base + at]), (uint32_t)(row0 + base + at), (uint32_t)(int)sm.unit[base + at], 0u));
             }
         }
+        // (read here: in the next centre thread 0 writes these sums again once the messages are there, which wait for the warps that send some
+        // and not for the others)
+        slack = (float)(1e-11 * sm.pre[nb - 1]);
         await(kDraws, (uint32_t)par);
         if (__syncthreads_or(sm.failed)) break;
     }
