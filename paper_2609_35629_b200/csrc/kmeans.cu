@@ -329,15 +329,15 @@ km_accept_kernel(KmeansParams p, int c)
 //   3. evaluate the winner's marked points in fp64 (a handful, after the first hundred centres), lower the
 //      distances, renew the running sums of the blocks of the sums they lie in, and send those blocks' sums;
 //   4. add up the blocks and draw the next trial points: the block that owns a drawn point sends its row to all.
-// Bound by the chain of a centre, 13000 cycles of 12288 points and nine trials: 4700 for the marks (1500 of them products at the
-// tensor cores' rate, the rest their operands, the look at the results and the slowest warp), 3900 for the slowest
-// block's distances and its running sums (128 terms in order, 11 cycles each), 1100 for the blocks' (96 terms), three
-// messages of 700. Messages are stores that count their bytes on an mbarrier of the block they go to; with cluster
-// barriers behind remote stores, three of 1900 cycles, all of a block's threads waiting for the slowest block's, and a
-// distance summed in order by one lane (1100 cycles a point), a centre took 8.2 us, now 6.4. Twelve warps, four tiles each, so
-// that three warps a scheduler overlap operands, products and marks (eight warps: 6.9; sixteen, with which the cycles above were
-// counted: 6.6, a fit to 2048 centres 18.25 -> 17.75 ms, to 256 and 64 centres 5.32 -> 5.25 and 4.91 -> 4.86: a barrier and the
-// slowest warp of fewer). The operands wait in tensor
+// Bound by the chain of a centre, 12300 cycles (6.4 us) of 12288 points and nine trials: 4000 for the marks (1500 of them products at the
+// tensor cores' rate, the rest their operands, the look at the results and the slowest warp) and the gains' sums, 2000 for the gains'
+// message and the winner, 3600 until the slowest block's distances and running sums (128 terms in order, 11 cycles each) are
+// there, 1100 for the blocks' sums (96 terms), 1600 for the draws and their rows. Messages are stores that count their bytes on an
+// mbarrier of the block they go to, 700 cycles; with cluster barriers behind remote stores, three of 1900 cycles, all of
+// a block's threads waiting for the slowest block's, and a distance summed in order by one lane (1100 cycles a point), a
+// centre took 8.2 us. Twelve warps, four tiles each, so that three warps a scheduler overlap operands, products and
+// marks (eight warps: 6.9 us a centre; sixteen: 6.6, with a barrier and the slowest warp of more): fits of 32768 keys to 2048, 256 and 64
+// centres 22.1 -> 18.2, 6.35 -> 5.10 and 4.63 -> 3.81 ms with the steps below. The operands wait in tensor
 // memory: read from shared memory they are as long on their way as the products take. (tcgen05 itself: sixteen
 // columns take as long as 128, 9 us a centre.) The two kernels per centre took 38 us, 24 of them fp64 distances of
 // every point to every trial.
